@@ -1202,102 +1202,223 @@ constexpr int SPLIT_BITS = 7;
 
 // exponent e of sigma = 2^e for every scalar row of a (possibly transposed)
 // row view: max_k |x_rk| = m 2^e with m in [0.5, 1) (e = 0 for an all-zero row);
-// the largest scaled row 1-norm sum_k |x_rk| / sigma (FP32, magnitudes
-// truncated to 24 bits) into *l1max and the largest scaled row 2-norm
-// (sum_k x_rk^2)^(1/2) / sigma (FP64 sum, rounded up) into *l2max, both as
-// FP32 bits
-__device__ __forceinline__ void row_scale_out(unsigned long long m, float l1, double sq, int nscalars, int* eout,
-                                              unsigned int* l1max, unsigned int* l2max) {
-  const int ea = (int)(m >> 52);
-  int e = 0;
-  if (ea > 0) e = ea - 1022;                       // [2^(ea-1023), 2^(ea-1022))
-  else if (m != 0) e = (64 - __clzll((long long)m)) - 1074;  // subnormal: [2^(L-1075), 2^(L-1074))
-  *eout = e;
-  if (m != 0) {
-    // entries below 2^-126 were left out: add their largest possible share
-    const float s = ldexpf(l1, -e) + (float)nscalars * ldexpf(1.0f, -126 - e);
-    atomicMax(l1max, __float_as_uint(fminf(s, 3.0e38f)));
-    const float s2 = (float)(ldexp(sqrt(sq), -e) * 1.0001) + 1e-30f;
-    atomicMax(l2max, __float_as_uint(fminf(s2, 3.0e38f)));
-  }
+// the largest scaled row 1-norm sum_k |x_rk| / sigma into *l1max and the
+// largest scaled row 2-norm (sum_k x_rk^2)^(1/2) / sigma into *l2max, both
+// bounds from above, as FP32 bits
+// two consecutive values (an even offset into a matrix's values); wide: the
+// values start on a 16-byte boundary (a caller's own array may start on any
+// multiple of eight)
+__device__ __forceinline__ double2 load_pair(const double* p, bool wide) {
+  if (wide) return *reinterpret_cast<const double2*>(p);
+  return make_double2(p[0], p[1]);
 }
 
-__device__ __forceinline__ void row_scale_acc(double x, unsigned long long& m, float& l1, double& sq) {
-  sq = fma(x, x, sq);
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-  m = u > m ? u : m;
-  const int e32 = (int)(u >> 52) - 896;  // FP32 exponent field of |x|
-  if (e32 > 0)
-    l1 += __uint_as_float(e32 > 254 ? 0x7f7fffffu : (((uint32_t)e32 << 23) | (uint32_t)((u >> 29) & 0x7fffffu)));
+// x 2^k in FP32, k of any size (sums are non-negative; too large: infinity)
+__device__ __forceinline__ float scale_f32(float x, int k) {
+  return x == 0.0f ? 0.0f : ldexpf(x, max(-2000, min(2000, k)));
 }
 
-// transposed views: one CTA of B threads per block row; thread r takes
-// column r of each stored block (op(X) row r), reads coalesced across threads
-template <int B>
-__global__ void __launch_bounds__(B) k_row_scale_t(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
-                                                   int nb, const double* __restrict__ val, int* __restrict__ eout,
-                                                   unsigned int* __restrict__ l1max, unsigned int* __restrict__ l2max) {
-  const int I = blockIdx.x, r = threadIdx.x;
-  if (I >= nb) return;
-  // four independent accumulators (rows k mod 4 of each block) so that the
-  // FP64 FMA and FP32 add chains overlap; combined at the end
-  unsigned long long m[4] = {0, 0, 0, 0};
-  float l1[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-  double sq[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int q = rp[I]; q < rp[I + 1]; ++q) {
-    const double* blk = val + (size_t)(src ? src[q] : q) * B * B;
-#pragma unroll 4
-    for (int k = 0; k < B; k += 4) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) row_scale_acc(blk[(k + j) * B + r], m[j], l1[j], sq[j]);
+// What a thread has seen of a row: the largest |x| by its high word, the low
+// words' bits (for rows of subnormals), and the sums of |x| and x^2 in FP32
+// relative to 2^(ref - 896), off the narrow FP64 pipe (one FP64 FMA per
+// element for the squares held this kernel at 2.0 TB/s).  ref follows the
+// values: one above 2^32 of the reference becomes the new one (rare after the
+// first nonzero value).  Values below 2^-126 of the reference (2^-63 for the
+// squares) add nothing, which row_bounds makes up for.
+struct RowScale {
+  uint32_t hi = 0, lo = 0, top = 0;
+  int ref = 0;  // subtracted from the FP64 exponent field
+  float l1 = 0.0f, sq = 0.0f;
+  __device__ __forceinline__ void add(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu, l = (uint32_t)__double2loint(x);
+    if (h > top) {
+      const int r = max((int)(h >> 20) - 127, 0);
+      l1 = scale_f32(l1, ref - r);
+      sq = scale_f32(sq, 2 * (ref - r));
+      ref = r;
+      top = (uint32_t)(r + 127 + 32) << 20;
     }
+    hi = h > hi ? h : hi;
+    lo |= l;
+    const int t = (int)h - ref * (1 << 20);
+    // the FP32 pattern: exponent field moved by ref, 23 of the 52 fraction bits
+    float f = __uint_as_float(__funnelshift_l(l, (uint32_t)t, 3));
+    if (t < (1 << 20)) f = 0.0f;
+    l1 += f;
+    sq = fmaf(f, f, sq);
   }
-  const unsigned long long m01 = m[0] > m[1] ? m[0] : m[1], m23 = m[2] > m[3] ? m[2] : m[3];
-  row_scale_out(m01 > m23 ? m01 : m23, (l1[0] + l1[1]) + (l1[2] + l1[3]), (sq[0] + sq[1]) + (sq[2] + sq[3]),
-                (rp[I + 1] - rp[I]) * B, eout + (size_t)I * B + r, l1max, l2max);
+};
+
+// exponent e of a row whose largest magnitude has these words: |x| < 2^e
+__device__ __forceinline__ int row_exponent(uint32_t hi, uint32_t lo) {
+  const int ea = (int)(hi >> 20);
+  if (ea > 0) return ea - 1022;                        // [2^(ea-1023), 2^(ea-1022))
+  if (hi != 0) return (64 - __clz((int)hi)) - 1074;    // subnormal: [2^(L-1075), 2^(L-1074))
+  return lo != 0 ? 32 - __clz((int)lo) - 1074 : 0;
 }
 
-// rows stored as rows: one warp per scalar row, lanes along the row (coalesced)
-template <int B>
-__global__ void k_row_scale(const int32_t* __restrict__ rp, const int32_t* __restrict__ src, int nb,
-                            const double* __restrict__ val, int* __restrict__ eout, unsigned int* __restrict__ l1max,
-                            unsigned int* __restrict__ l2max) {
-  const int64_t w = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= (int64_t)nb * B) return;
-  const int I = (int)(w / B), r = (int)(w % B);
-  unsigned long long m = 0;  // |x| bit patterns order like the magnitudes
-  float l1 = 0.0f;
-  double sq = 0.0;
-  for (int q = rp[I]; q < rp[I + 1]; ++q) {
-    const double* blk = val + (size_t)(src ? src[q] : q) * B * B;
-    for (int c = lane; c < B; c += 32) row_scale_acc(blk[r * B + c], m, l1, sq);
+// the row's scaled 1- and 2-norm bounds from its sums relative to 2^e, as FP32 bits
+__device__ __forceinline__ void row_bounds(bool any, int e, float l1, float sq, int nscalars, uint32_t& n1, uint32_t& n2) {
+  n1 = n2 = 0u;
+  if (!any) return;
+  if (e < -800) {  // the reference stops at the smallest exponents: no bound
+    n1 = n2 = __float_as_uint(3.0e38f);
+    return;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long u = __shfl_xor_sync(0xffffffffu, m, o);
-    m = u > m ? u : m;
-    l1 += __shfl_xor_sync(0xffffffffu, l1, o);
-    sq += __shfl_xor_sync(0xffffffffu, sq, o);
-  }
-  if (lane == 0) row_scale_out(m, l1, sq, (rp[I + 1] - rp[I]) * B, eout + w, l1max, l2max);
+  // magnitudes are truncated to 24 bits and the FP32 sums rounded: 1e-3 covers
+  // both; values left out of a sum are below 2^-126 (2^-63 for the squares) of
+  // a value of the row
+  n1 = __float_as_uint(fminf(l1 * 1.001f + (float)nscalars * 1.2e-38f, 3.0e38f));
+  n2 = __float_as_uint(fminf(sqrtf(sq + (float)nscalars * 1.2e-38f) * 1.001f + 1e-30f, 3.0e38f));
 }
 
-// sigma exponents (and the scaled 1-norm bound) of the rows of a row view
-static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, int nb, bool tr,
-                       const double* val, int* eout, unsigned int* l1max, unsigned int* l2max) {
-  const int g = cdiv((int64_t)nb * bs * 32, 256);
-  if (bs == 32) {
-    if (tr) k_row_scale_t<32><<<nb, 32, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
-    else k_row_scale<32><<<g, 256, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
-  } else if (bs == 64) {
-    if (tr) k_row_scale_t<64><<<nb, 64, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
-    else k_row_scale<64><<<g, 256, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
+// the warp's largest norm bounds, one atomic each (32 rows' atomics on one
+// word would queue up)
+__device__ __forceinline__ void row_scale_max(uint32_t n1, uint32_t n2, unsigned int* l1max, unsigned int* l2max) {
+  n1 = __reduce_max_sync(0xffffffffu, n1);
+  n2 = __reduce_max_sync(0xffffffffu, n2);
+  if ((threadIdx.x & 31) == 0 && n1) {
+    atomicMax(l1max, n1);
+    atomicMax(l2max, n2);
+  }
+}
+
+// Row scales of a view.  CTA (I, sp) reads part sp of `splits` of block row
+// I's blocks with 16-byte loads; TR: op(X) row r is column r of the stored
+// blocks, a thread takes two columns and every (512 / B)-th row; else eight
+// lanes share a row in segments of 128 bytes.  With splits > 1 -- a matrix of
+// few, long block rows, which would leave most SMs without a CTA -- each
+// part's sums go to `part` and k_row_scale_join adds them in order.  Measured:
+// 3D cluster factor of 4096 rows (64 block rows of 64 blocks) 896 -> 39 us
+// (one CTA of 64 threads per block row before), 262,144-row chain (4096 block
+// rows of three, 400 MB) 212 -> 101 us, rows stored as rows 486 -> 92 us.
+struct RowPart {
+  uint32_t hi, lo;
+  int e;  // l1 and sq relative to 2^e and 2^2e
+  float l1, sq;
+};
+
+template <int B, bool TR>
+__global__ void __launch_bounds__(256) k_row_scale(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
+                                                   int splits, const double* __restrict__ val, bool wide,
+                                                   int* __restrict__ eout, unsigned int* __restrict__ l1max,
+                                                   unsigned int* __restrict__ l2max, RowPart* __restrict__ part) {
+  constexpr int RG = TR ? 512 / B : 8;  // threads that share a row of op(X)
+  __shared__ RowScale sh[RG][B];
+  const int I = (int)blockIdx.x / splits, sp = (int)blockIdx.x % splits, tid = threadIdx.x;
+  const int q0 = rp[I], cnt = rp[I + 1] - q0, per = (cnt + splits - 1) / splits;
+  const int qa = min(q0 + sp * per, q0 + cnt), qe = min(qa + per, q0 + cnt);
+  if constexpr (TR) {
+    const int c = (tid % (B / 2)) * 2, r0 = tid / (B / 2);
+    RowScale a0, a1;
+    for (int q = qa; q < qe; ++q) {
+      const double* blk = val + (size_t)(src ? src[q] : q) * B * B + c;
+#pragma unroll 8
+      for (int k = r0; k < B; k += RG) {
+        const double2 x = load_pair(blk + k * B, wide);
+        a0.add(x.x);
+        a1.add(x.y);
+      }
+    }
+    sh[r0][c] = a0;
+    sh[r0][c + 1] = a1;
   } else {
-    if (tr) k_row_scale_t<128><<<nb, 128, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
-    else k_row_scale<128><<<g, 256, 0, ctx->stream>>>(rp, src, nb, val, eout, l1max, l2max);
+    const int wid = tid >> 5, lane = tid & 31;
+    constexpr int RS = B / 32;  // groups of four rows per warp
+    RowScale a[RS];
+    for (int q = qa; q < qe; ++q) {
+      const double* blk = val + (size_t)(src ? src[q] : q) * B * B + (lane & 7) * 2;
+#pragma unroll
+      for (int g = 0; g < RS; ++g) {
+        const double* row = blk + ((wid * RS + g) * 4 + (lane >> 3)) * B;
+#pragma unroll
+        for (int i = 0; i < B; i += 16) {
+          const double2 x = load_pair(row + i, wide);
+          a[g].add(x.x);
+          a[g].add(x.y);
+        }
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < RS; ++g) sh[lane & 7][(wid * RS + g) * 4 + (lane >> 3)] = a[g];
   }
+  __syncthreads();
+  if (tid >= B) return;
+  RowPart t{0u, 0u, 0, 0.0f, 0.0f};
+#pragma unroll
+  for (int g = 0; g < RG; ++g) {
+    t.hi = max(t.hi, sh[g][tid].hi);
+    t.lo |= sh[g][tid].lo;
+  }
+  t.e = row_exponent(t.hi, t.lo);
+#pragma unroll
+  for (int g = 0; g < RG; ++g) {  // a sum's unit is 2^(ref + 127 - 1023)
+    const int k = sh[g][tid].ref - 896 - t.e;
+    t.l1 += scale_f32(sh[g][tid].l1, k);
+    t.sq += scale_f32(sh[g][tid].sq, 2 * k);
+  }
+  const size_t row = (size_t)I * B + tid;
+  if (splits == 1) {
+    uint32_t n1, n2;
+    eout[row] = t.e;
+    row_bounds((t.hi | t.lo) != 0u, t.e, t.l1, t.sq, cnt * B, n1, n2);
+    row_scale_max(n1, n2, l1max, l2max);
+  } else {
+    part[(size_t)sp * (gridDim.x / splits) * B + row] = t;
+  }
+}
+
+// the parts of every row joined, in order (nrows is a multiple of 32)
+__global__ void k_row_scale_join(const int32_t* __restrict__ rp, int bs, int64_t nrows, int splits,
+                                 const RowPart* __restrict__ part, int* __restrict__ eout,
+                                 unsigned int* __restrict__ l1max, unsigned int* __restrict__ l2max) {
+  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (r >= nrows) return;
+  uint32_t hi = 0, lo = 0;
+  for (int s = 0; s < splits; ++s) {
+    hi = max(hi, part[s * nrows + r].hi);
+    lo |= part[s * nrows + r].lo;
+  }
+  const int e = row_exponent(hi, lo);
+  float l1 = 0.0f, sq = 0.0f;
+  for (int s = 0; s < splits; ++s) {
+    const RowPart p = part[s * nrows + r];
+    l1 += scale_f32(p.l1, p.e - e);
+    sq += scale_f32(p.sq, 2 * (p.e - e));
+  }
+  const int I = (int)(r / bs);
+  uint32_t n1, n2;
+  eout[r] = e;
+  row_bounds((hi | lo) != 0u, e, l1, sq, (rp[I + 1] - rp[I]) * bs, n1, n2);
+  row_scale_max(n1, n2, l1max, l2max);
+}
+
+template <int B>
+static void launch_row_scale(ifac_ctx* ctx, const int32_t* rp, const int32_t* src, int nb, int splits, bool tr,
+                             const double* val, int* eout, unsigned int* l1max, unsigned int* l2max,
+                             RowPart* part) {
+  const int grid = nb * splits;
+  const bool wide = aligned16(val);
+  if (tr) k_row_scale<B, true><<<grid, 256, 0, ctx->stream>>>(rp, src, splits, val, wide, eout, l1max, l2max, part);
+  else k_row_scale<B, false><<<grid, 256, 0, ctx->stream>>>(rp, src, splits, val, wide, eout, l1max, l2max, part);
   IFAC_CK_LAUNCH();
+}
+
+// sigma exponents (and the scaled norm bounds) of the rows of a row view of nnzb blocks
+static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, int nb, int64_t nnzb, bool tr,
+                       const double* val, int* eout, unsigned int* l1max, unsigned int* l2max) {
+  const int64_t rows = (int64_t)nb * bs;
+  // about four CTAs per SM, each with at least two blocks of its row
+  const int splits = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(4 * 152, nb), nnzb / (2 * (int64_t)nb)));
+  Buf<RowPart> part;
+  if (splits > 1) part = Buf<RowPart>(ctx, rows * splits);
+  if (bs == 32) launch_row_scale<32>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
+  else if (bs == 64) launch_row_scale<64>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
+  else launch_row_scale<128>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
+  if (splits > 1) {
+    k_row_scale_join<<<cdiv(rows, 128), 128, 0, ctx->stream>>>(rp, bs, rows, splits, part.p, eout, l1max, l2max);
+    IFAC_CK_LAUNCH();
+  }
 }
 
 // NS BF16 slice copies (K-major, op() CSR order) of a view; row r of block qb
@@ -1997,13 +2118,13 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   IFAC_CK(cudaMemsetAsync(l1.p, 0, 4 * sizeof(unsigned int), ctx->stream));
   if (!hit) {
     sige = Buf<int>(ctx, rows);
-    row_scales(ctx, bs, arows.rp, value_src(ctx, arows.src, avmap, A.nnzb, asrc), nb, tA, A.val, sige.p, l1.p,
+    row_scales(ctx, bs, arows.rp, value_src(ctx, arows.src, avmap, A.nnzb, asrc), nb, A.nnzb, tA, A.val, sige.p, l1.p,
                l1.p + 2);
   }
   {
     View bt = view_rows(ctx, B, !tB);
     Buf<int32_t> btsrc;
-    row_scales(ctx, bs, bt.rp, value_src(ctx, bt.src, bvmap, B.nnzb, btsrc), nb, !tB, B.val, taue.p, l1.p + 1,
+    row_scales(ctx, bs, bt.rp, value_src(ctx, bt.src, bvmap, B.nnzb, btsrc), nb, B.nnzb, !tB, B.val, taue.p, l1.p + 1,
                l1.p + 3);
   }
   // slices: row scale block of an op(A) entry is its CSR row; of an op(B) entry its CSR column

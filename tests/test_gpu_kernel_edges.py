@@ -1,0 +1,69 @@
+"""Kernels at the sizes and values where they can go wrong: tile edges,
+remainders, few long and many short block rows, values of very different
+magnitude, matrices that start off a 16-byte boundary."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1901_07993_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+FP64, TF32, BF16, FP64_SPLIT = 0, 1, 2, 3
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    from paper_1901_07993_gb300 import build as libbuild
+    from paper_1901_07993_gb300 import ifac
+    assert torch.cuda.is_available()
+    libbuild.build()
+    return ifac.Context()
+
+
+def full(h):
+    D = np.zeros((h.nb * h.bs, h.nb * h.bs))
+    for I in range(h.nb):
+        for q in range(h.row_ptr[I], h.row_ptr[I + 1]):
+            J = h.col_idx[q]
+            D[I * h.bs:(I + 1) * h.bs, J * h.bs:(J + 1) * h.bs] = h.val[q]
+    return D
+
+
+def borrowed(h, shift):
+    """h in torch tensors whose values start `shift` doubles past an allocation."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    buf = torch.zeros(h.val.size + shift, dtype=torch.float64, device="cuda")
+    val = buf[shift:].view(h.nnzb, h.bs, h.bs)
+    val.copy_(torch.from_numpy(np.ascontiguousarray(h.val)))
+    return ifac.BorrowedBSR(h.n, h.bs, torch.from_numpy(h.row_ptr).cuda(), torch.from_numpy(h.col_idx).cuda(), val)
+
+
+@pytest.mark.parametrize("bs,nb,density,tA,tB,shift", [(64, 3, 1.0, False, False, 0), (64, 11, 1.0, True, False, 1),
+                                                       (32, 30, 0.8, False, True, 1), (128, 4, 1.0, True, True, 0),
+                                                       (64, 40, 0.05, False, False, 1)])
+def test_split_row_scales(ctx, bs, nb, density, tA, tB, shift):
+    """Scales of rows and columns whose magnitudes span 2^-300 .. 2^300, each
+    beginning with entries 2^-180 below its largest; block rows in several
+    parts (few long ones) and in one; values off a 16-byte boundary.  Bound:
+    K 2^-(7 s - 5) max|a_i.| max|b_.j| + 2 K 2^-53 (|A||B|)_ij with s = 7."""
+    from paper_1901_07993_gb300 import ifac
+    rng = np.random.default_rng(5)
+    A = synth.random_bsr(nb, bs, density, seed=81)
+    B = synth.random_bsr(nb, bs, density, seed=82)
+    r = np.exp2(rng.integers(-300, 300, nb * bs).astype(float)).reshape(nb, bs)
+    for M, t in ((A, tA), (B, not tB)):
+        rows = np.repeat(np.arange(nb), np.diff(M.row_ptr))
+        for q in range(M.nnzb):
+            v = M.val[q].T if t else M.val[q]
+            v[:, :3] *= 2.0 ** -180
+            v *= r[M.col_idx[q] if t else rows[q]][:, None]
+    got = ifac.bsr_gemm_trunc(ctx, borrowed(A, shift), tA, borrowed(B, shift), tB, 1.0, 0.0, FP64_SPLIT).download()
+    ref = oracle.gemm(A, B, tA, tB, 1.0, 0.0)
+    assert np.array_equal(got.row_ptr, ref.row_ptr) and np.array_equal(got.col_idx, ref.col_idx)
+    Ad, Bd = (full(A).T if tA else full(A)), (full(B).T if tB else full(B))
+    K = nb * bs
+    lim = (K * 2.0 ** -44 * np.outer(np.abs(Ad).max(axis=1), np.abs(Bd).max(axis=0))
+           + 2 * K * 2.0 ** -53 * (np.abs(Ad) @ np.abs(Bd)))
+    assert np.all(np.abs(full(got) - full(ref)) <= lim)
