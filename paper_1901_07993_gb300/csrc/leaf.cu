@@ -1,14 +1,26 @@
 // leaf.cu -- batched leaf routine of Algorithms 1-2 ("factorize S^-1 = Z Z*"):
 // for each nl x nl SPD matrix, the Cholesky factor S = L L^T and Z = L^-T.
 //
-// One CTA per matrix, FP64, 32 x 32 tiles staged in shared memory, the matrix
-// itself kept in global memory (it is L2-resident while its CTA works on it):
-//   1. right-looking tiled Cholesky: factor tile (k,k), solve the panel
-//      A_ik <- A_ik L_kk^-T, update the trailing tiles A_ij -= A_ik A_jk^T;
-//   2. W_kk = L_kk^-1 for every diagonal tile (into scratch);
-//   3. W = L^-1 by tile columns, W_ik = -W_ii sum_{l=k}^{i-1} L_il W_lk, and
-//      Z = W^T is written into the upper triangle (which step 1 never reads);
-//   4. diagonal tiles Z_kk = W_kk^T, strictly lower part cleared.
+// One thread-block cluster per matrix, FP64, 32 x 32 tiles.  An SM issues
+// about two FP64 FMAs per clock, so a tile product (32^3 FMAs) takes 8 us on
+// one SM and a 512-row leaf 11 ms: the work of a leaf is spread over up to 16
+// SMs, which meet at cluster barriers.  L and W = L^-1 are built together,
+// right-looking.  X(r, k) names tile (r, k) of the array: below the diagonal
+// it holds A, then L; above it B^T, then W^T (= Z), B the right-hand side
+// that starts as the identity.  Step k:
+//   1. column k is scaled, X(r, k) <- X(r, k) W_kk^T for every r != k (L_ik
+//      below the diagonal, Z_ck above), one tile per CTA;
+//   2. X(r, j) -= X(r, k) X(j, k)^T for every j > k and r <= k (B, with
+//      X(k, k) = W_kk^T and B_jk = 0 before) or r >= j (A); tile (k+1, k+1)
+//      first, and CTA 0 factors it at once (W_kk = L_kk^-1 for the next step)
+//      while the others go on, so the serial chain of pivots overlaps the
+//      updates.
+// Every step has T^2 / 2 to T tile products (T = nl / 32); the columns of W
+// after all of L would be chains of very different length.  Measured (one CTA
+// per matrix before): 8 leaves of 512 rows 16.3 -> 1.45 ms (0.50 TFLOP/s of
+// the FP64 pipe's 1.25), one 16.2 -> 1.06 ms, 64 leaves 16.6 -> 7.2 ms, one of
+// 128 rows 597 -> 155 us, one of 1024 rows 114 -> 6.8 ms.
+//
 // A non-positive pivot j sets info = j + 1 (the pivot is replaced by 1 so the
 // arithmetic stays finite; that matrix's Z is then meaningless).
 #include "internal.cuh"
@@ -19,169 +31,244 @@ namespace {
 constexpr int TB = 32;
 constexpr int LD = TB + 1;  // padded shared-memory row
 constexpr int NT = 256;
+// CTA 0's update and factorization of the next diagonal tile, in tile products
+constexpr int DIAG_COST = 3;
+
+__device__ __forceinline__ int cluster_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ int cluster_size() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// all threads of the cluster; global writes before it are visible after it
+// (readers load through L2, __ldcg)
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// W = L^-1 of the tile L L^T = t (LD rows, lower triangle used): four warps,
+// lane = row, warp w holds columns w, w + 4, ... of the tile and of W, so the
+// FP64 work of a pivot is spread over the SM; one named barrier per pivot.
+// (The next pivot's root taken ahead of the other updates measured no faster.)
+// Returns 1 + the first non-positive pivot, or 0 (the same in all four warps).
+__device__ __forceinline__ int factor_tile(const double* t, double* __restrict__ W) {
+  __shared__ double col[2][TB + 1];
+  __shared__ int sbad;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) sbad = 0;
+  double a[TB / 4], b[TB / 4], rown = 1.0;
+#pragma unroll
+  for (int q = 0; q < TB / 4; ++q) {
+    a[q] = t[lane * LD + w + 4 * q];
+    b[q] = (lane == w + 4 * q) ? 1.0 : 0.0;
+  }
+#pragma unroll
+  for (int jq = 0; jq < TB / 4; ++jq) {
+#pragma unroll 1
+    for (int jw = 0; jw < 4; ++jw) {
+      const int j = 4 * jq + jw;
+      double* c = col[jw & 1];
+      if (w == jw) {
+        double d = __shfl_sync(0xffffffffu, a[jq], j);
+        if (!(d > 0.0)) {
+          if (lane == 0 && !sbad) sbad = j + 1;
+          d = 1.0;
+        }
+        const double rs = rsqrt(d);
+        c[lane] = a[jq] * rs;  // rows below the pivot: L_ij
+        if (lane == 0) c[TB] = rs;
+      }
+      asm volatile("bar.sync 1, 128;" ::: "memory");
+      // row j of B stays unscaled until the end: its factor goes into L_ij
+      const double li = lane > j ? -c[lane] : 0.0, lr = li * c[TB];
+      if (lane == j) rown = c[TB];
+#pragma unroll
+      for (int q = 0; q < TB / 4; ++q) {
+        const int cc = w + 4 * q;
+        if (cc > j) a[q] = fma(li, c[cc], a[q]);
+        else b[q] = fma(lr, __shfl_sync(0xffffffffu, b[q], j), b[q]);
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < TB / 4; ++q) W[lane * TB + w + 4 * q] = b[q] * rown;
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+  return sbad;
+}
 }  // namespace
 
 __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase, int nl, int* __restrict__ info,
                                                      double* __restrict__ Wdiag_base) {
-  __shared__ double t0[TB * LD], t1[TB * LD], t2[TB * LD];
-  __shared__ int bad;
-  const int tid = threadIdx.x;
+  __shared__ double xs[TB * LD], ys[TB * LD];
+  const int tid = threadIdx.x, rank = cluster_rank(), C = cluster_size();
   const int T = nl / TB;
-  double* A = Abase + (size_t)blockIdx.x * nl * nl;
-  double* Wd = Wdiag_base + (size_t)blockIdx.x * T * TB * TB;
-  auto at = [&](int r, int c) -> double& { return A[(size_t)r * nl + c]; };
-  if (tid == 0) bad = 0;
-  __syncthreads();
-  // thread's 2x2 output in a 32x32 tile
-  const int orow = (tid >> 4) * 2, ocol = (tid & 15) * 2;
+  const size_t mat = blockIdx.x / C;
+  double* A = Abase + mat * nl * nl;
+  double* Wd = Wdiag_base + mat * T * TB * TB;  // W_kk, row-major, lower triangular
+  int bad = 0;
+  const auto tile = [&](int r, int c) { return A + (size_t)r * TB * nl + c * TB; };
+  // this thread's four elements of a tile: rows tid / 32 + 8 i, column tid % 32
+  const int er = tid >> 5, ec = tid & 31;
+  const auto fetch = [&](const double* p, size_t ld, double (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __ldcg(p + (er + 8 * i) * ld + ec);
+  };
+  const auto place = [&](double* s, const double (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[(er + 8 * i) * LD + ec] = v[i];
+  };
+  const auto place_t = [&](double* s, const double (&v)[4]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[ec * LD + er + 8 * i] = v[i];
+  };
+  const auto factor = [&](int k) {  // the diagonal tile in xs (all threads; the first four warps work)
+    if (tid < 128) {
+      const int j = factor_tile(xs, Wd + (size_t)k * TB * TB);
+      if (j && !bad) bad = k * TB + j;
+    }
+  };
 
-  // ---------------- 1. Cholesky ----------------
-  for (int k = 0; k < T; ++k) {
-    const int k0 = k * TB;
-    for (int e = tid; e < TB * TB; e += NT) t0[(e / TB) * LD + e % TB] = at(k0 + e / TB, k0 + e % TB);
+  if (rank == 0) {
+    double v[4];
+    fetch(tile(0, 0), nl, v);
+    place(xs, v);
     __syncthreads();
-    for (int j = 0; j < TB; ++j) {
-      if (tid == 0) {
-        double d = t0[j * LD + j];
-        if (!(d > 0.0)) {
-          if (!bad) bad = k0 + j + 1;
-          d = 1.0;
-        }
-        t0[j * LD + j] = sqrt(d);
-      }
-      __syncthreads();
-      if (tid > j && tid < TB) t0[tid * LD + j] /= t0[j * LD + j];
-      __syncthreads();
-      for (int e = tid; e < TB * TB; e += NT) {
-        int i = e / TB, l = e % TB;
-        if (l > j && i >= l) t0[i * LD + l] -= t0[i * LD + j] * t0[l * LD + j];
-      }
-      __syncthreads();
-    }
-    for (int e = tid; e < TB * TB; e += NT) {
-      int i = e / TB, l = e % TB;
-      if (i >= l) at(k0 + i, k0 + l) = t0[i * LD + l];
-    }
-    // panel: each thread solves one row x of A_ik in place: x L_kk^T = a
-    for (int rr = tid; rr < (T - k - 1) * TB; rr += NT) {
-      const int gr = k0 + TB + rr;
-      for (int j = 0; j < TB; ++j) {
-        double s = at(gr, k0 + j);
-        for (int l = 0; l < j; ++l) s -= at(gr, k0 + l) * t0[j * LD + l];
-        at(gr, k0 + j) = s / t0[j * LD + j];
-      }
-    }
-    __syncthreads();
-    // trailing update A_ij -= A_ik A_jk^T for k < j <= i
-    for (int j = k + 1; j < T; ++j) {
-      for (int e = tid; e < TB * TB; e += NT) t1[(e / TB) * LD + e % TB] = at(j * TB + e / TB, k0 + e % TB);
-      for (int i = j; i < T; ++i) {
-        for (int e = tid; e < TB * TB; e += NT) t2[(e / TB) * LD + e % TB] = at(i * TB + e / TB, k0 + e % TB);
-        __syncthreads();
-        double c00 = 0, c01 = 0, c10 = 0, c11 = 0;
-#pragma unroll 8
-        for (int l = 0; l < TB; ++l) {
-          double a0 = t2[orow * LD + l], a1 = t2[(orow + 1) * LD + l];
-          double b0 = t1[ocol * LD + l], b1 = t1[(ocol + 1) * LD + l];
-          c00 = fma(a0, b0, c00);
-          c01 = fma(a0, b1, c01);
-          c10 = fma(a1, b0, c10);
-          c11 = fma(a1, b1, c11);
-        }
-        const int gi = i * TB + orow, gj = j * TB + ocol;
-        at(gi, gj) -= c00;
-        at(gi, gj + 1) -= c01;
-        at(gi + 1, gj) -= c10;
-        at(gi + 1, gj + 1) -= c11;
-        __syncthreads();
-      }
-    }
+    factor(0);
   }
-  __syncthreads();
-
-  // ---------------- 2. W_kk = L_kk^-1 (one warp per tile, one lane per column) ----------------
-  {
-    const int lane = tid & 31, wid = tid >> 5;
-    for (int k = wid; k < T; k += NT / 32) {
-      const int k0 = k * TB;
-      double* W = Wd + (size_t)k * TB * TB;  // row-major 32x32, lower triangular
-      const int c = lane;
-      for (int i = 0; i < TB; ++i) {
-        double v;
-        if (i < c) v = 0.0;
-        else if (i == c) v = 1.0 / at(k0 + c, k0 + c);
-        else {
-          double s = 0.0;
-          for (int l = c; l < i; ++l) s += at(k0 + i, k0 + l) * W[l * TB + c];
-          v = -s / at(k0 + i, k0 + i);
-        }
-        W[i * TB + c] = v;
-        __syncwarp();
-      }
-    }
-  }
-  __syncthreads();
-
-  // ---------------- 3. off-diagonal tiles of W, stored as Z_ki = W_ik^T ----------------
+  cluster_sync();
   for (int k = 0; k < T; ++k) {
-    for (int i = k + 1; i < T; ++i) {
-      double c00 = 0, c01 = 0, c10 = 0, c11 = 0;  // (sum_l L_il W_lk) at (orow.., ocol..)
-      for (int l = k; l < i; ++l) {
-        // t1 <- L_il, t2 <- W_lk (W_kk from scratch, else the transpose of Z tile (k,l))
-        for (int e = tid; e < TB * TB; e += NT) {
-          int r = e / TB, c = e % TB;
-          t1[r * LD + c] = at(i * TB + r, l * TB + c);
-          t2[r * LD + c] = (l == k) ? Wd[(size_t)k * TB * TB + r * TB + c] : at(k * TB + c, l * TB + r);
-        }
+    // ---- 1. X(r, k) <- X(r, k) W_kk^T: warp w has columns 4w .. 4w + 3, which
+    // need the first 4w + 4 terms of the lower-triangular W_kk ----
+    {
+      double w4[4];
+      bool have = false;
+      for (int u = rank; u < T - 1; u += C) {
+        double* X = tile(u < k ? u : u + 1, k);
+        double v[4];
+        if (!have) fetch(Wd + (size_t)k * TB * TB, TB, w4);
+        fetch(X, nl, v);
+        if (!have) place(ys, w4);
+        have = true;
+        place(xs, v);
         __syncthreads();
-#pragma unroll 8
-        for (int q = 0; q < TB; ++q) {
-          double a0 = t1[orow * LD + q], a1 = t1[(orow + 1) * LD + q];
-          double b0 = t2[q * LD + ocol], b1 = t2[q * LD + ocol + 1];
-          c00 = fma(a0, b0, c00);
-          c01 = fma(a0, b1, c01);
-          c10 = fma(a1, b0, c10);
-          c11 = fma(a1, b1, c11);
+        const int c0 = (tid >> 5) * 4 + ((tid >> 4) & 1) * 2, r0 = (tid & 15) * 2, n = (tid >> 5) * 4 + 4;
+        double s00 = 0, s01 = 0, s10 = 0, s11 = 0;
+#pragma unroll 4
+        for (int l = 0; l < n; ++l) {
+          const double a0 = xs[r0 * LD + l], a1 = xs[(r0 + 1) * LD + l];
+          const double b0 = ys[c0 * LD + l], b1 = ys[(c0 + 1) * LD + l];
+          s00 = fma(a0, b0, s00);
+          s01 = fma(a0, b1, s01);
+          s10 = fma(a1, b0, s10);
+          s11 = fma(a1, b1, s11);
         }
+        __syncthreads();  // xs is reused: the result goes out in rows
+        xs[r0 * LD + c0] = s00;
+        xs[r0 * LD + c0 + 1] = s01;
+        xs[(r0 + 1) * LD + c0] = s10;
+        xs[(r0 + 1) * LD + c0 + 1] = s11;
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) X[(size_t)(er + 8 * i) * nl + ec] = xs[(er + 8 * i) * LD + ec];
         __syncthreads();
       }
-      // t1 <- the sum, t2 <- W_ii; W_ik = -W_ii * sum
-      t1[orow * LD + ocol] = c00;
-      t1[orow * LD + ocol + 1] = c01;
-      t1[(orow + 1) * LD + ocol] = c10;
-      t1[(orow + 1) * LD + ocol + 1] = c11;
-      for (int e = tid; e < TB * TB; e += NT) t2[(e / TB) * LD + e % TB] = Wd[(size_t)i * TB * TB + e];
-      __syncthreads();
-      double d00 = 0, d01 = 0, d10 = 0, d11 = 0;
-#pragma unroll 8
-      for (int q = 0; q < TB; ++q) {
-        double a0 = t2[orow * LD + q], a1 = t2[(orow + 1) * LD + q];
-        double b0 = t1[q * LD + ocol], b1 = t1[q * LD + ocol + 1];
-        d00 = fma(a0, b0, d00);
-        d01 = fma(a0, b1, d01);
-        d10 = fma(a1, b0, d10);
-        d11 = fma(a1, b1, d11);
-      }
-      // Z tile (k, i) = W_ik^T: element (r, c) of W_ik goes to Z(k*TB + c, i*TB + r)
-      at(k * TB + ocol, i * TB + orow) = -d00;
-      at(k * TB + ocol + 1, i * TB + orow) = -d01;
-      at(k * TB + ocol, i * TB + orow + 1) = -d10;
-      at(k * TB + ocol + 1, i * TB + orow + 1) = -d11;
-      __syncthreads();
     }
+    if (k + 1 == T) break;
+    cluster_sync();
+    // ---- 2. trailing updates ----
+    // units: column j = k + 1 .. T - 1, rows 0 .. k and j .. T - 1, without (k + 1, k + 1)
+    const int m = T - 1 - k;
+    const int units = m * (k + 1) + m * (m + 1) / 2 - 1;
+    const int share0 = C == 1 ? units : max(0, (units + DIAG_COST + C - 1) / C - DIAG_COST);
+    const int first = rank == 0 ? -1 : share0 + rank - 1, step = rank == 0 ? 1 : C - 1;
+    const int last = rank == 0 ? share0 : units;
+    int r = k + 1, j = k + 1;  // unit -1: the next diagonal tile
+    const auto decode = [&](int u) {
+      int jj = k + 1, n = k + 1 + T - jj - 1;
+      while (u >= n) {
+        u -= n;
+        ++jj;
+        n = k + 1 + T - jj;
+      }
+      j = jj;
+      r = u <= k ? u : jj + (u - (k + 1)) + (jj == k + 1 ? 1 : 0);
+    };
+    const int orow = (tid >> 4) * 2, ocol = (tid & 15) * 2;
+    double va[4], vb[4], c0[4];  // the next unit's operands, loaded while this one is multiplied
+    const auto load_unit = [&] {
+      if (r == k) fetch(Wd + (size_t)k * TB * TB, TB, va);
+      else fetch(tile(r, k), nl, va);
+      fetch(tile(j, k), nl, vb);
+      const double* p = tile(r, j) + (size_t)orow * nl + ocol;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c0[i] = r == k ? 0.0 : __ldcg(p + (size_t)(i >> 1) * nl + (i & 1));
+    };
+    if (rank != 0 && first < last) decode(first);
+    if (first < last) load_unit();
+    for (int u = first; u < last; u += step) {
+      const int ur = r, uj = j;
+      if (ur == k) place_t(xs, va);
+      else place(xs, va);
+      place(ys, vb);
+      double s00 = c0[0], s01 = c0[1], s10 = c0[2], s11 = c0[3];
+      __syncthreads();
+      if (u >= 0 && u + step < last) {
+        decode(u + step);
+        load_unit();
+      }
+#pragma unroll 8
+      for (int l = 0; l < TB; ++l) {
+        const double a0 = -xs[orow * LD + l], a1 = -xs[(orow + 1) * LD + l];
+        const double b0 = ys[ocol * LD + l], b1 = ys[(ocol + 1) * LD + l];
+        s00 = fma(a0, b0, s00);
+        s01 = fma(a0, b1, s01);
+        s10 = fma(a1, b0, s10);
+        s11 = fma(a1, b1, s11);
+      }
+      __syncthreads();
+      if (u < 0) {  // CTA 0: factor the next diagonal tile
+        xs[orow * LD + ocol] = s00;
+        xs[orow * LD + ocol + 1] = s01;
+        xs[(orow + 1) * LD + ocol] = s10;
+        xs[(orow + 1) * LD + ocol + 1] = s11;
+        __syncthreads();
+        factor(k + 1);
+        __syncthreads();
+        if (last > 0) {
+          decode(0);
+          load_unit();
+        }
+        continue;
+      }
+      double* p = tile(ur, uj) + (size_t)orow * nl + ocol;
+      p[0] = s00;
+      p[1] = s01;
+      p[nl] = s10;
+      p[nl + 1] = s11;
+    }
+    cluster_sync();
   }
-  __syncthreads();
-
-  // ---------------- 4. diagonal tiles, clear the strictly lower part ----------------
-  for (int k = 0; k < T; ++k)
-    for (int e = tid; e < TB * TB; e += NT) {
-      int r = e / TB, c = e % TB;
-      at(k * TB + r, k * TB + c) = (c >= r) ? Wd[(size_t)k * TB * TB + c * TB + r] : 0.0;
+  cluster_sync();  // the strictly lower tiles are no longer read
+  // diagonal tiles Z_kk = W_kk^T, strictly lower tiles cleared
+  for (int u = rank; u < T * T; u += C) {
+    const int r = u / T, c = u % T;
+    if (r < c) continue;
+    double* p = tile(r, c);
+    if (r == c) {
+      double v[4];
+      fetch(Wd + (size_t)r * TB * TB, TB, v);
+      place(xs, v);
+      __syncthreads();
     }
-  for (int i = 1; i < T; ++i)
-    for (int j = 0; j < i; ++j)
-      for (int e = tid; e < TB * TB; e += NT) at(i * TB + e / TB, j * TB + e % TB) = 0.0;
-  if (tid == 0) info[blockIdx.x] = bad;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[(size_t)(er + 8 * i) * nl + ec] = r == c ? xs[ec * LD + er + 8 * i] : 0.0;
+    if (r == c) __syncthreads();
+  }
+  if (rank == 0 && tid == 0) info[mat] = bad;
 }
 
 __global__ void k_pad_identity(const double* __restrict__ src, int nl, double* __restrict__ dst, int np, int count) {
@@ -202,6 +289,58 @@ __global__ void k_unpad(const double* __restrict__ src, int np, double* __restri
   dst[e] = src[k * np * np + (int64_t)r * np + c];
 }
 
+// CTAs per matrix: the largest cluster of which `count` fit on the GPU with
+// one CTA per SM (two CTAs on an SM would share its FP64 pipe), no more than
+// half a step's tile products.  The dynamic shared memory keeps a second CTA
+// off an SM; the device's cluster counts are asked for once.
+constexpr int LEAF_SMEM = 120 * 1024;
+
+static cudaError_t leaf_config(int count, int tiles, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
+  static constexpr int kSizes[] = {16, 12, 10, 8, 6, 5, 4, 3, 2};
+  static std::atomic<int> fit[64][9];  // 0: not asked yet, else 1 + clusters on the device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_leaf_invchol, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_leaf_invchol, cudaFuncAttributeMaxDynamicSharedMemorySize, LEAF_SMEM);
+  if (e != cudaSuccess) return e;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg->blockDim = dim3(NT);
+  cfg->dynamicSmemBytes = LEAF_SMEM;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+  for (int i = 0; i < 9; ++i) {
+    const int c = kSizes[i];
+    if (c > tiles * tiles / 2) continue;
+    at->val.clusterDim.x = (unsigned)c;
+    cfg->gridDim = dim3((unsigned)(count * c));
+    int n = fit[dev & 63][i].load();
+    if (n == 0) {
+      int q = 0;
+      if (cudaOccupancyMaxActiveClusters(&q, k_leaf_invchol, cfg) != cudaSuccess) {
+        cudaGetLastError();  // this size is not available: the next one
+        q = 0;
+      }
+      fit[dev & 63][i].store(n = q + 1);
+    }
+    if (n - 1 >= count) return cudaSuccess;
+  }
+  at->val.clusterDim.x = 1;
+  cfg->gridDim = dim3((unsigned)count);
+  cfg->dynamicSmemBytes = 0;  // more matrices than SMs: their chains overlap on one
+  return cudaSuccess;
+}
+
+static cudaError_t launch_leaf(cudaStream_t stream, int count, int nl, double* A, int* info, double* wd) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  const cudaError_t e = leaf_config(count, nl / TB, &cfg, &at);
+  if (e != cudaSuccess) return e;
+  cfg.stream = stream;
+  return cudaLaunchKernelEx(&cfg, k_leaf_invchol, A, nl, info, wd);
+}
+
 // A: count matrices of nl x nl (in place).  Pads to a multiple of 32 with an
 // identity block when needed (the padded part factors to the identity).
 void leaf_invchol(ifac_ctx* ctx, int count, int nl, double* A, int* info) {
@@ -210,16 +349,16 @@ void leaf_invchol(ifac_ctx* ctx, int count, int nl, double* A, int* info) {
   const int T = np / TB;
   Buf<double> wd(ctx, (size_t)count * T * TB * TB);
   if (np == nl) {
-    k_leaf_invchol<<<count, NT, 0, ctx->stream>>>(A, nl, info, wd.p);
-    IFAC_CK_LAUNCH();
+    IFAC_CK(launch_leaf(ctx->stream, count, nl, A, info, wd.p));
+    ++ctx->launches;
     return;
   }
   Buf<double> pad(ctx, (size_t)count * np * np);
   int64_t tot = (int64_t)count * np * np;
   k_pad_identity<<<cdiv(tot, 256), 256, 0, ctx->stream>>>(A, nl, pad.p, np, count);
   IFAC_CK_LAUNCH();
-  k_leaf_invchol<<<count, NT, 0, ctx->stream>>>(pad.p, np, info, wd.p);
-  IFAC_CK_LAUNCH();
+  IFAC_CK(launch_leaf(ctx->stream, count, np, pad.p, info, wd.p));
+  ++ctx->launches;
   int64_t tot2 = (int64_t)count * nl * nl;
   k_unpad<<<cdiv(tot2, 256), 256, 0, ctx->stream>>>(pad.p, np, A, nl, count);
   IFAC_CK_LAUNCH();
@@ -238,15 +377,13 @@ cudaError_t leaf_invchol_launch_scratch(cudaStream_t stream, int count, int nl, 
   if (count == 0) return cudaSuccess;
   const int np = ((nl + TB - 1) / TB) * TB;
   if (np == nl) {
-    k_leaf_invchol<<<count, NT, 0, stream>>>(A, nl, info, wd);
-    return cudaGetLastError();
+    return launch_leaf(stream, count, nl, A, info, wd);
   }
   int64_t tot = (int64_t)count * np * np;
   k_pad_identity<<<cdiv(tot, 256), 256, 0, stream>>>(A, nl, pad, np, count);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_leaf_invchol<<<count, NT, 0, stream>>>(pad, np, info, wd);
-  e = cudaGetLastError();
+  e = launch_leaf(stream, count, np, pad, info, wd);
   if (e != cudaSuccess) return e;
   int64_t tot2 = (int64_t)count * nl * nl;
   k_unpad<<<cdiv(tot2, 256), 256, 0, stream>>>(pad, np, A, nl, count);

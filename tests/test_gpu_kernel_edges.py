@@ -67,3 +67,30 @@ def test_split_row_scales(ctx, bs, nb, density, tA, tB, shift):
     lim = (K * 2.0 ** -44 * np.outer(np.abs(Ad).max(axis=1), np.abs(Bd).max(axis=0))
            + 2 * K * 2.0 ** -53 * (np.abs(Ad) @ np.abs(Bd)))
     assert np.all(np.abs(full(got) - full(ref)) <= lim)
+
+
+@pytest.mark.parametrize("nl,count", [(1, 1), (32, 3), (33, 2), (64, 1), (95, 20), (160, 40), (320, 13), (480, 9),
+                                      (1024, 1)])
+def test_leaf_cluster_sizes(ctx, nl, count):
+    """Leaves of one to 32 tiles in clusters of one to 16 CTAs (the counts run
+    through the rule's cluster sizes), ragged sizes among them: against numpy's
+    inverse Cholesky factor (condition number about 4: 64 nl 2^-53 relative),
+    triangular, and a bad pivot reported where it is."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    rng = np.random.default_rng(nl)
+    G = rng.standard_normal((count, nl, nl)) / np.sqrt(nl)
+    S = np.eye(nl) + 0.25 * np.matmul(G, G.transpose(0, 2, 1))
+    Z, info, rc = ifac.leaf_invchol_batched(ctx, torch.from_numpy(S).cuda())
+    Z = Z.cpu().numpy()
+    ref = np.linalg.inv(np.linalg.cholesky(S)).transpose(0, 2, 1)
+    assert rc == 0 and not info.any().item()
+    assert np.array_equal(Z, np.triu(Z))
+    err = np.linalg.norm(Z - ref, axis=(1, 2)) / np.linalg.norm(ref, axis=(1, 2))
+    assert err.max() <= 64 * nl * 2.0 ** -53
+    # the last matrix gets a negative pivot at row p; the others are unaffected
+    p = (2 * nl) // 3
+    S[-1, p, p] = -1.0
+    Z2, info, rc = ifac.leaf_invchol_batched(ctx, torch.from_numpy(S).cuda())
+    assert rc == ifac.ERR_NOT_SPD and info[-1].item() == p + 1 and not info[:-1].any().item()
+    assert np.array_equal(Z2.cpu().numpy()[:-1], Z[:-1])
