@@ -1603,19 +1603,23 @@ __global__ void __launch_bounds__(256) k_split_finish(const int32_t* __restrict_
 // accumulator elements: 128 / bs block rows of C by 64 columns (two block
 // columns at bs 32, one at bs 64, half of one at bs 128, whose two halves the
 // same CTA takes one after the other).  Each K block is streamed in chunks of
-// at most 64 K elements; a chunk's slices are loaded once -- slice k of the
-// tile's op(A) rows and op(B) columns share one ring slot -- and, as soon as
-// slot k has landed, the MMAs of the slice pairs (a, b) with max(a, b) = k
-// are issued; a slot is released after the last pair that reads it.  Every
-// accumulation unit keeps its own FP32 accumulator in tensor memory (up to 8
-// units x 64 columns).  A window of K blocks is as long as every weight class
-// fits one unit; after each window the epilogue adds the units, scaled, into
+// at most 64 K elements; a chunk's op(B) slices are resident while its op(A)
+// slices stream through a ring.  Every weight class a + b has one FP32
+// accumulator in tensor memory (up to 8 classes x 64 columns), side by side,
+// as the op(B) slices lie one after the other in shared memory: op(A) slice a
+// meets op(B) slices b .. b + 3 in one instruction of 256 columns, whose
+// accumulators are the classes a + b .. a + b + 3.  (One instruction of 64
+// columns per pair read op(A) from shared memory for every pair: 36 pairs of
+// an 8-slice product 4.6 -> 2.9 ms a launch on a 4096-row 3D cluster factor,
+// 53% of the measured BF16 rate, and 0.95 ms a launch where it was 1.19 on
+// the 262,144-row chain.)  A window of K blocks is as long as every class
+// stays exact; after each window the epilogue adds the classes, scaled, into
 // 64-bit fixed-point sums held in registers, so a tile may span any number of
 // windows.  After the tile's last window the epilogue writes
 // S_ij 2^(ea + e_i + e_j) * am in FP64 and the block norms.
 // ---------------------------------------------------------------------------
 namespace band {
-constexpr int MAX_U = 8;                    // units live at once: 8 x 64 = 512 columns
+constexpr int MAX_U = 8;                    // weight classes (one unit each): 8 x 64 = 512 columns
 // 16 epilogue warps, four per tensor-memory lane quarter, each on 16 of the
 // tile's 64 columns: the epilogue's adds of the units into the fixed-point
 // sums stand between the MMAs of consecutive tiles (the accumulators hold
@@ -1624,8 +1628,9 @@ constexpr int MAX_U = 8;                    // units live at once: 8 x 64 = 512 
 constexpr int EPW = 16;
 constexpr int NTB = 32 * (2 + EPW);
 constexpr uint32_t TMEM_COLS = 512;
-// FP32 accumulate, A = B = BF16, both K-major, N = 64, M = 128
-constexpr uint32_t IDESC = idesc_of<2, 64, 128>();
+// FP32 accumulate, A = B = BF16, both K-major, M = 128; N is added per
+// instruction (64 to 256 columns)
+constexpr uint32_t IDESC0 = idesc_of<2, 0, 128>();
 
 template <int B>
 struct SB {
@@ -1687,7 +1692,6 @@ struct BandArgs {
   // on its own.
   int unit_step[band::MAX_U];
   uint32_t unit_first, unit_last;
-  int8_t unit_ab[band::SB<64>::MAXS * band::SB<64>::MAXS];  // unit of slice pair (a, b), a + b <= ns - 1
   int* err;
   int* ovf;
 };
@@ -1850,7 +1854,7 @@ __global__ void __launch_bounds__(band::NTB, 1)
               break;
             }
             tc_fence_after();
-            uint32_t started = 0;  // units whose accumulator holds this window's sum
+            uint32_t acc0 = 0;  // the window's first products overwrite the accumulators
             for (int j = w0; j < w1 && ok; ++j) {
               for (int c = 0; c < L::KCH && ok; ++c) {
                 if (!mbar_wait(smem_u32(&bfull[bb]), bphase, &abort_flag, args.err)) {
@@ -1869,16 +1873,20 @@ __global__ void __launch_bounds__(band::NTB, 1)
                   }
                   tc_fence_after();
                   const uint64_t da = smem_desc_sw(abase + (uint32_t)(slot * L::SLOT_A), L::SBO, L::SWZ);
-                  for (int b = 0; b < ns - a; ++b) {
-                    const int u = args.unit_ab[a * L::MAXS + b];
-                    const uint32_t tacc = tmem + (uint32_t)(u * N);
+                  // slice a of op(A) against slices b, b + 1, ... of op(B), up
+                  // to four in one instruction: the slices lie one after the
+                  // other in shared memory, and so do the accumulators of the
+                  // weight classes a + b, a + b + 1, ...
+                  for (int b = 0; b < ns - a; b += 4) {
+                    const int nn = min(4, ns - a - b);
+                    const uint32_t tacc = tmem + (uint32_t)((a + b) * N);
                     const uint64_t db = db0 + (uint64_t)(b * (L::SLOT_B >> 4));
-                    const uint32_t acc0 = (started >> u) & 1u;
+                    const uint32_t idesc = IDESC0 + (uint32_t)nn * ((uint32_t)(N >> 3) << 17);
 #pragma unroll
                     for (int kk = 0; kk < L::KSTEPS; ++kk)
-                      mma_kstep<2>(tacc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), IDESC, kk > 0 ? 1u : acc0);
-                    started |= 1u << u;
+                      mma_kstep<2>(tacc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, kk > 0 ? 1u : acc0);
                   }
+                  acc0 = 1u;  // slice 0 has started every class
                   mma_commit(smem_u32(&aempty[slot]));  // op(A) slice a is used up
                   if (++slot == RA) {
                     slot = 0;
@@ -2203,10 +2211,11 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
     bc->from_b = true;
   }
   // window of the narrow kernel: the K blocks (at most 1024 K elements) for
-  // which every unit stays exact, as long as at most band::MAX_U units
-  // result; the longest tile's K blocks when fewer
+  // which every weight class stays exact in one unit, so that unit u holds
+  // the slice pairs (a, b) with a + b = u; the longest tile's K blocks when
+  // fewer (one block always fits: 40,960 * 128 <= 2^24 at eight slices)
   int kwin = std::min(1024 / bs, std::max(kmax, 1));
-  while (kwin > 1 && unit_table(ns, kwin, bs).nunits > band::MAX_U) --kwin;
+  while (kwin > 1 && unit_table(ns, kwin, bs).nunits > ns) --kwin;
   // the windowed kernel adds into zeroed 64-bit sums that a second kernel
   // converts; the narrow kernel holds each tile's complete sums and writes FP64
   Buf<longlong2> part;
@@ -2262,7 +2271,7 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
     ba.slice_rows_a = (int)(A.nnzb + 1) * bs;
     ba.slice_rows_b = (int)(B.nnzb + 1) * bs;
     ba.nunits = ut.nunits;
-    if (ut.nunits > band::MAX_U) fail(IFAC_ERR_UNSUPPORTED, "split product: too many units for the narrow kernel");
+    if (ut.nunits != ns) fail(IFAC_ERR_UNSUPPORTED, "split product: a weight class needs two units");
     for (int u = 0; u < ut.nunits; ++u) ba.unit_sh[u] = fbits - SPLIT_BITS * ut.unit_g[u];
     // Horner groups: consecutive units with shifts >= 0 (descending, so each
     // step is 0 or 7 bits); a group's value is below ngroup 2^(24 + span),
@@ -2289,17 +2298,6 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
       }
       if (start >= 0) ba.unit_last |= 1u << (ut.nunits - 1);
     }
-    // the unit of each slice pair (a, b) with a + b <= ns - 1 (0-based)
-    for (int k = 0; k < band::SB<64>::MAXS * band::SB<64>::MAXS; ++k) ba.unit_ab[k] = -1;
-    for (int p = 0; p < ut.npairs; ++p) {
-      const int a = ut.si[p] - 1, b = ut.ti[p] - 1;
-      if (a < 0 || b < 0 || a + b > ns - 1) fail(IFAC_ERR_CUDA, "split product: slice pair outside the table");
-      ba.unit_ab[a * band::SB<64>::MAXS + b] = (int8_t)ut.pu[p];
-    }
-    for (int a = 0; a < ns; ++a)
-      for (int b = 0; b < ns - a; ++b)
-        if (ba.unit_ab[a * band::SB<64>::MAXS + b] < 0)
-          fail(IFAC_ERR_CUDA, "split product: inconsistent banded issue table");
     ba.err = ctx->dev_err;
     ba.ovf = ctx->dev_err;
     const int kc = bs < 64 ? bs : 64;  // K elements per chunk (band::SB<bs>::KC)
