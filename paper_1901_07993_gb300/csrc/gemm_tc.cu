@@ -1621,10 +1621,13 @@ __global__ void __launch_bounds__(256) k_split_finish(const int32_t* __restrict_
 namespace band {
 constexpr int MAX_U = 8;                    // weight classes (one unit each): 8 x 64 = 512 columns
 // 16 epilogue warps, four per tensor-memory lane quarter, each on 16 of the
-// tile's 64 columns: the epilogue's adds of the units into the fixed-point
-// sums stand between the MMAs of consecutive tiles (the accumulators hold
-// every unit, so they are not double-buffered), and twice the warps of the
-// other kernels halve that time
+// tile's 64 columns: the epilogue's reads of the classes stand between the
+// MMAs of consecutive windows (the accumulators fill tensor memory, so they
+// are not double-buffered).  Cycles a tile on the 262,144-row chain (two K
+// blocks a tile on average): classes into the sums 9.0k -> 4.8k, FP64 result
+// and norm 8.7k -> 7.0k, against 10.5k of MMAs; what is left between the MMAs
+// and the tensor rate is the op(A) and op(B) traffic from L2 (about 40 bytes
+// a clock and SM).
 constexpr int EPW = 16;
 constexpr int NTB = 32 * (2 + EPW);
 constexpr uint32_t TMEM_COLS = 512;
@@ -1662,6 +1665,17 @@ struct SB {
   static_assert(SLOT_A % 1024 == 0 && SLOT_B % 1024 == 0, "slots must keep the swizzle alignment");
   static_assert(RA >= 2, "op(A) ring too shallow");
 };
+
+// The 64-bit sums of a tile hold units of 2^-f: 2^d of the weight class that
+// lies in slot 6; `below` classes of lower weight round into it.
+struct FixedSum {
+  int below;         // classes below the one that holds the unit
+  int d;             // the unit is 2^d of that class, 0 <= d < 7
+  float m0, m1, m2;  // 2^-d, 2^(7 - d), 2^(14 - d)
+  int s1;            // 21 - d
+  int top;           // 2^(10 - d)
+  long long offset;  // what class_sums adds beside the classes
+};
 }  // namespace band
 
 struct BandArgs {
@@ -1682,19 +1696,132 @@ struct BandArgs {
   int kwin;                // K blocks per window (every weight class exact in one FP32 accumulator)
   int slice_rows_a;        // tensor-map rows between consecutive slices of op(A): (nnzb_A + 1) bs
   int slice_rows_b;
-  int nunits;
-  int unit_sh[band::MAX_U];
-  // Horner groups of units: unit u with unit_step[u] >= 0 enters its group's
-  // 64-bit accumulator as g = (g << unit_step[u]) + x_u (the first unit of a
-  // group, bit u of unit_first, starts it); at the group's last unit (bit u of
-  // unit_last) g is added into the sums at scale 2^unit_sh[u].  A unit with
-  // unit_step[u] < 0 (below the fixed-point scale) is rounded into the sums
-  // on its own.
-  int unit_step[band::MAX_U];
-  uint32_t unit_first, unit_last;
+  band::FixedSum fx;       // how the weight classes enter the 64-bit sums
+  bool wide;               // C's values start on a 32-byte boundary
   int* err;
   int* ovf;
 };
+
+// 32 lanes x 4 columns of tensor memory, without waiting for the values
+__device__ __forceinline__ void tmem_ld4_issue(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(taddr));
+}
+
+// the loads issued so far have arrived (the registers pass through the wait,
+// so that nothing that uses them moves before it)
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[8][4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0][0]), "+r"(r[0][1]), "+r"(r[0][2]), "+r"(r[0][3]), "+r"(r[1][0]), "+r"(r[1][1]),
+                 "+r"(r[1][2]), "+r"(r[1][3]), "+r"(r[2][0]), "+r"(r[2][1]), "+r"(r[2][2]), "+r"(r[2][3]),
+                 "+r"(r[3][0]), "+r"(r[3][1]), "+r"(r[3][2]), "+r"(r[3][3])::"memory");
+  asm volatile(""
+               : "+r"(r[4][0]), "+r"(r[4][1]), "+r"(r[4][2]), "+r"(r[4][3]), "+r"(r[5][0]), "+r"(r[5][1]),
+                 "+r"(r[5][2]), "+r"(r[5][3]), "+r"(r[6][0]), "+r"(r[6][1]), "+r"(r[6][2]), "+r"(r[6][3]),
+                 "+r"(r[7][0]), "+r"(r[7][1]), "+r"(r[7][2]), "+r"(r[7][3])::"memory");
+}
+
+// s[e] + the value of one window's classes x[0..7][e] (highest weight first, a
+// factor of 2^7 from slot to slot; integers of magnitude at most 2^24, as FP32
+// patterns) in units of slot 6 times 2^d, for four columns e side by side: the
+// steps of one column depend on each other.  The carries of the classes and
+// the digits that remain are formed in FP32, exactly: adding 1.5 2^23 rounds
+// to an integer and leaves it in the low bits, so neither the conversion
+// instructions (16 per clock and SM, against 125 FP32 operations and 63
+// integer ones) nor a 64-bit shift for every class is needed.  Three digits of
+// seven bits go into the 64-bit sum at once; the pattern of 1.5 2^23 that
+// comes with them is in fx.offset.
+__device__ __forceinline__ void class_sums(long long* s, uint32_t (&r)[8][4], const band::FixedSum& fx) {
+  constexpr float M = 12582912.0f;
+  const auto carry = [](float v) { return fmaf(v, 0.0078125f, 12582912.0f) - 12582912.0f; };  // round(v / 128)
+  float c[4] = {0.0f, 0.0f, 0.0f, 0.0f}, g0[4], g1[4];
+  if (fx.below) {
+    for (int k = 1; k < fx.below; ++k) {  // (more than one class below the unit: rare)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        r[6][e] = __float_as_uint(__uint_as_float(r[6][e]) + carry(__uint_as_float(r[7][e])));
+#pragma unroll
+        for (int u = 7; u > 0; --u) r[u][e] = r[u - 1][e];
+        r[0][e] = 0u;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) c[e] = carry(__uint_as_float(r[7][e]));
+  }
+  // slot u: the carry into the next slot in c, the digit returned
+  const auto digit = [&](int u, int e) -> float {
+    const float v = __uint_as_float(r[u][e]) + c[e];
+    c[e] = carry(v);
+    return fmaf(-128.0f, c[e], v);
+  };
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g0[e] = digit(6, e);
+  if (fx.d) {  // rounded to the unit
+#pragma unroll
+    for (int e = 0; e < 4; ++e) g0[e] = fmaf(g0[e], fx.m0, M) - M;
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g0[e] = fmaf(digit(5, e), fx.m1, g0[e] + M);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g0[e] = fmaf(digit(4, e), fx.m2, g0[e]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g1[e] = digit(3, e) + M;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g1[e] = fmaf(digit(2, e), 128.0f, g1[e]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) g1[e] = fmaf(digit(1, e), 16384.0f, g1[e]);
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const uint32_t top = (uint32_t)__float2int_rn(__uint_as_float(r[0][e]) + c[e]);
+    const uint32_t h = __float_as_uint(g1[e]);
+    unsigned long long t = (((unsigned long long)(h >> (32 - fx.s1))) << 32) | (h << fx.s1);
+    t += __float_as_uint(g0[e]);
+    t += (unsigned long long)(top * (uint32_t)fx.top) << 32;
+    s[e] = (long long)((unsigned long long)s[e] + t);
+  }
+}
+
+// v[e] = s[e] 2^E[e] rounded to nearest even from the integer's bits (results
+// outside the normal range: i64_ldexp); `bad` records |s| >= 2^62, which the
+// sums' scale rules out
+__device__ __forceinline__ void fixed_to_f64(const long long (&s)[4], const int (&E)[4], double (&v)[4], bool& bad) {
+  bool odd = false;
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const uint32_t sg = (uint32_t)(s[e] >> 63);  // 0 or all ones
+    const uint32_t xl = (uint32_t)s[e] ^ sg, xh = (uint32_t)(s[e] >> 32) ^ sg;
+    const unsigned long long u = (((unsigned long long)xh << 32) | xl) + (sg & 1u);
+    const uint32_t h = (uint32_t)(u >> 32), l = (uint32_t)u;
+    bad |= (h >> 30) != 0u;
+    const bool small = h == 0u;
+    const uint32_t a = small ? l : h, b = small ? 0u : l;
+    const int lz = __clz((int)a);
+    const uint32_t nh = __funnelshift_l(b, a, lz), nl = b << (lz & 31);
+    const uint32_t mh = nh >> 11, ml = __funnelshift_r(nl, nh, 11);
+    const uint32_t up = ((nl & 0x7ffu) + (ml & 1u)) > 0x400u ? 1u : 0u;
+    const int ex = E[e] + (small ? 1023 + 62 - 32 : 1023 + 62) - lz;  // exponent field - 1: mh holds the leading bit
+    odd |= (unsigned)ex > 2045u;
+    const unsigned long long m = (((unsigned long long)(((uint32_t)ex << 20) + mh)) << 32 | ml) + up;
+    const uint32_t zero = a == 0u ? 0u : 0xffffffffu;
+    v[e] = __hiloint2double((int)(((uint32_t)(m >> 32) | (sg & 0x80000000u)) & zero), (int)((uint32_t)m & zero));
+  }
+  if (odd) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = i64_ldexp(s[e], E[e]);
+  }
+}
+
+// four consecutive FP64 values, one 32-byte sector per lane when p is aligned
+__device__ __forceinline__ void store4(double* p, const double (&v)[4], bool wide) {
+  if (wide) {
+    // (no "memory": nothing here reads C, and the next columns' loads may move up)
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = v[i];
+  }
+}
 
 template <int B>
 __global__ void __launch_bounds__(band::NTB, 1)
@@ -1708,7 +1835,7 @@ __global__ void __launch_bounds__(band::NTB, 1)
   __shared__ __align__(8) uint64_t acc_full, acc_empty, drain_bar;
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile int abort_flag;
-  __shared__ double partial[4][EPW / 4];
+  __shared__ double partial[2][4][EPW / 4];
   __shared__ int32_t srec[32 * L::RECW];  // the producer's current chunk of plan records
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1727,7 +1854,7 @@ __global__ void __launch_bounds__(band::NTB, 1)
       mbar_init(smem_u32(&bempty[s]), 1);
     }
     mbar_init(smem_u32(&acc_full), 1);
-    mbar_init(smem_u32(&acc_empty), 1);
+    mbar_init(smem_u32(&acc_empty), EPW);  // one arrival per epilogue warp
     mbar_init(smem_u32(&drain_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1922,7 +2049,6 @@ __global__ void __launch_bounds__(band::NTB, 1)
     const int et = threadIdx.x - 64;
     uint32_t acc_phase = 0;
     const bool unit = (args.am == 1.0 || args.am == -1.0), neg = args.am < 0.0;
-    bool good = true;
     // the tile's K-step count, its block coordinates, and the C positions of
     // this warp's block and (threads et < TMB TNB) of the block whose norm it
     // writes, loaded a tile ahead
@@ -1936,7 +2062,9 @@ __global__ void __launch_bounds__(band::NTB, 1)
       if (et < CP) kn_n = args.cpos[(size_t)tn * CP + et];
     };
     if (mt > 0) load_next((int)blockIdx.x);
-    for (int it = 0; it < mt && good; ++it) {
+    const FixedSum fx = args.fx;
+    const int slot0 = MAX_U - ns - (fx.below ? 0 : 1);
+    for (int it = 0; it < mt; ++it) {
       const int t = (int)blockIdx.x + it * (int)gridDim.x;
       const int nk = nk_n;
       const int I0 = ti_n * TMB, J0 = tj_n * TNB;
@@ -1944,57 +2072,47 @@ __global__ void __launch_bounds__(band::NTB, 1)
       const int p = p_n;  // position of C_IJ in C (warp-uniform; -1: not in C)
       const int kn = kn_n;
       if (it + 1 < mt) load_next(t + (int)gridDim.x);
-      SqAcc sq;  // this thread's squares over the tile's column sub-tiles
-      for (int h = 0; h < L::NSUB && good; ++h) {
+      SqAcc4 sq;  // this thread's squares over the tile's column sub-tiles
+      bool got = true;
+      for (int h = 0; h < L::NSUB; ++h) {
         const int cin = (h * N + cg * CW) % B;  // first column of this warp within block J
+        // class_sums leaves its constants' offset in every window's sum
+        const long long s0 = -fx.offset * ((nk + args.kwin - 1) / args.kwin);
         long long s[CW];
 #pragma unroll
-        for (int e = 0; e < CW; ++e) s[e] = 0;
+        for (int e = 0; e < CW; ++e) s[e] = s0;
         bool bad = false;
         for (int w0 = 0; w0 < nk; w0 += args.kwin) {
-          const bool got = mbar_wait(smem_u32(&acc_full), acc_phase, &abort_flag, args.err);
+          // (a wait that failed is voted on after the tile: its reads of
+          // tensor memory are harmless and the call returns the error)
+          got = mbar_wait(smem_u32(&acc_full), acc_phase, &abort_flag, args.err) && got;
           acc_phase ^= 1u;
-          if (!epi_all<32 * EPW>(got)) {  // all epilogue warps go on, or all stop
-            good = false;
-            break;
-          }
+          __syncwarp();
           tc_fence_after();
-          // units of equal or adjacent weight combine in 64-bit Horner
-          // groups first, so a group costs one checked shift-and-add into
-          // the sums instead of one per unit (8 columns at a time)
+          // four columns at a time: every class's value is read behind one
+          // wait, in slots: the classes below the sums' unit end at slot 7,
+          // the others at slot 6
 #pragma unroll
-          for (int hf = 0; hf < CW / 8; ++hf) {
-            long long g[8];
-#pragma unroll 1
-            for (int u = 0; u < args.nunits; ++u) {
-              float v[8];
-              tmem_ld8(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(u * N + cg * CW + hf * 8), v);
-              const int sh = args.unit_sh[u], st = args.unit_step[u];
-              if (st < 0) {
+          for (int c4 = 0; c4 < CW / 4; ++c4) {
+            uint32_t r[MAX_U][4];
+            const uint32_t ta =
+                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(cg * CW + c4 * 4) - (uint32_t)(slot0 * N);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) s[hf * 8 + e] = fixed_add(s[hf * 8 + e], __float2int_rn(v[e]), sh, bad);
-              } else {
-                if ((args.unit_first >> u) & 1u) {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) g[e] = (long long)__float2int_rn(v[e]);
-                } else {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e)
-                    g[e] = (long long)((unsigned long long)g[e] << st) + (long long)__float2int_rn(v[e]);
-                }
-                if ((args.unit_last >> u) & 1u) {
-#pragma unroll
-                  for (int e = 0; e < 8; ++e) s[hf * 8 + e] = fixed_add64(s[hf * 8 + e], g[e], sh, bad);
-                }
-              }
+            for (int u = 0; u < MAX_U; ++u) {
+              if (u >= slot0 && u < slot0 + ns) tmem_ld4_issue(ta + (uint32_t)(u * N), r[u]);
+              else r[u][0] = r[u][1] = r[u][2] = r[u][3] = 0u;
             }
+            tmem_wait_ld(r);
+            if (c4 == CW / 4 - 1) {
+              // this warp has read its part of the accumulators: the next
+              // window's MMAs may overwrite them once every warp has
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&acc_empty));
+            }
+            class_sums(s + c4 * 4, r, fx);
           }
-          // the accumulators are read: the next window's MMAs may overwrite them
-          tc_fence_before();
-          epi_bar<32 * EPW>();
-          if (et == 0) mbar_arrive(smem_u32(&acc_empty));
         }
-        if (!good) break;
         // every K of the tile is in these sums: the FP64 result,
         // S_ij 2^(ea + e_i + e_j) * am rounded once, and its squares for the norm
         if (p >= 0) {
@@ -2002,24 +2120,29 @@ __global__ void __launch_bounds__(band::NTB, 1)
           const int* tj = args.taue + (size_t)J * B + cin;
           double* dst = args.cval + (size_t)p * B * B + (size_t)rin * B + cin;
 #pragma unroll
-          for (int e = 0; e < CW; e += 2) {
-            const long long x0 = (unit && neg) ? -s[e] : s[e], x1 = (unit && neg) ? -s[e + 1] : s[e + 1];
-            double v0 = i64_ldexp(x0, er + tj[e]), v1 = i64_ldexp(x1, er + tj[e + 1]);
+          for (int e = 0; e < CW; e += 4) {
+            const int4 tje = __ldg(reinterpret_cast<const int4*>(tj + e));
+            const int te[4] = {er + tje.x, er + tje.y, er + tje.z, er + tje.w};
+            long long x[4];
+            double v[4];
+#pragma unroll
+            for (int f = 0; f < 4; ++f) x[f] = (unit && neg) ? -s[e + f] : s[e + f];
+            fixed_to_f64(x, te, v, bad);
             if (!unit) {
-              v0 *= args.am;
-              v1 *= args.am;
+#pragma unroll
+              for (int f = 0; f < 4; ++f) v[f] *= args.am;
             }
-            sq.add_f64(v0);
-            sq.add_f64(v1);
-            *reinterpret_cast<double2*>(dst + e) = make_double2(v0, v1);
+            sq.add4(v);
+            store4(dst + e, v, args.wide);
           }
           if (bad) *args.ovf = 2;
         }
       }
-      if (!good) break;
-      const double ss = sq.warp_total();
-      if (lane == 0) partial[q][cg] = ss;
-      epi_bar<32 * EPW>();
+      const double ss = sq.total().warp_total();
+      if (lane == 0) partial[it & 1][q][cg] = ss;
+      // one barrier per tile (the partials alternate between two buffers):
+      // all epilogue warps go on, or all stop
+      if (!epi_all<32 * EPW>(got)) break;
       // norms: block (br, bc) of the tile sums the warps of its lane quarters
       // and column groups, in a fixed order
       if (et < CP && kn >= 0) {
@@ -2030,10 +2153,9 @@ __global__ void __launch_bounds__(band::NTB, 1)
         const int c1 = (bc + 1) * B / CW < EPW / 4 ? (bc + 1) * B / CW : EPW / 4;
         double sum = 0.0;
         for (int qq = br * B / 32; qq < q1; ++qq)
-          for (int cc = bc * B / CW; cc < c1; ++cc) sum += partial[qq][cc];
+          for (int cc = bc * B / CW; cc < c1; ++cc) sum += partial[it & 1][qq][cc];
         args.cnorm[kn] = sqrt(sum);
       }
-      epi_bar<32 * EPW>();
     }
   }
   tc_fence_before();
@@ -2088,6 +2210,16 @@ static UnitTable unit_table(int ns, int kw, int bs) {
     if (open) t.unit_end[t.nunits++] = t.npairs;
   }
   return t;
+}
+
+// whether a class of kw K blocks and the carry of the class below it (at most
+// 2^17) stay within 2^24, as class_sums adds them in FP32
+static bool class_carries_fit(int ns, int kw, int bs) {
+  for (int g = 2; g <= ns; ++g) {  // class g = s + t, 1-based slices; the last one takes no carry
+    const int64_t most = (int64_t)bs * kw * (g == 2 ? 128 * 128 : 2 * 128 * 64 + (int64_t)(g - 3) * 64 * 64);
+    if (most + (1 << 17) + 1 > (int64_t)1 << 24) return false;
+  }
+  return true;
 }
 
 template <int B>
@@ -2215,7 +2347,7 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   // the slice pairs (a, b) with a + b = u; the longest tile's K blocks when
   // fewer (one block always fits: 40,960 * 128 <= 2^24 at eight slices)
   int kwin = std::min(1024 / bs, std::max(kmax, 1));
-  while (kwin > 1 && unit_table(ns, kwin, bs).nunits > ns) --kwin;
+  while (kwin > 1 && (unit_table(ns, kwin, bs).nunits > ns || !class_carries_fit(ns, kwin, bs))) --kwin;
   // the windowed kernel adds into zeroed 64-bit sums that a second kernel
   // converts; the narrow kernel holds each tile's complete sums and writes FP64
   Buf<longlong2> part;
@@ -2263,41 +2395,27 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
     ba.cnorm = C.norms;
     ba.sige = sige_p;
     ba.taue = taue_p;
-    ba.ea = ea_alpha - 1 - fbits;
+    // (a unit below the last class's would hold zeros only)
+    const int fband = std::min(fbits, SPLIT_BITS * (ns + 1));
+    ba.ea = ea_alpha - 1 - fband;
     ba.am = am;
     ba.nb = nb;
     ba.ns = ns;
     ba.kwin = kwin;
     ba.slice_rows_a = (int)(A.nnzb + 1) * bs;
     ba.slice_rows_b = (int)(B.nnzb + 1) * bs;
-    ba.nunits = ut.nunits;
     if (ut.nunits != ns) fail(IFAC_ERR_UNSUPPORTED, "split product: a weight class needs two units");
-    for (int u = 0; u < ut.nunits; ++u) ba.unit_sh[u] = fbits - SPLIT_BITS * ut.unit_g[u];
-    // Horner groups: consecutive units with shifts >= 0 (descending, so each
-    // step is 0 or 7 bits); a group's value is below ngroup 2^(24 + span),
-    // kept within int64 by a span of at most 35 bits with at most 8 units
-    {
-      ba.unit_first = ba.unit_last = 0u;
-      int start = -1;
-      for (int u = 0; u < ut.nunits; ++u) {
-        const int sh = ba.unit_sh[u];
-        if (sh < 0) {
-          if (start >= 0) ba.unit_last |= 1u << (u - 1);
-          start = -1;
-          ba.unit_step[u] = -1;
-          continue;
-        }
-        if (start >= 0 && ba.unit_sh[start] - sh <= 35) {
-          ba.unit_step[u] = ba.unit_sh[u - 1] - sh;
-        } else {
-          if (start >= 0) ba.unit_last |= 1u << (u - 1);
-          start = u;
-          ba.unit_first |= 1u << u;
-          ba.unit_step[u] = 0;
-        }
-      }
-      if (start >= 0) ba.unit_last |= 1u << (ut.nunits - 1);
-    }
+    // the last class's weight is 2^-7(ns + 1): the unit 2^-f is 2^(7 below + d) of it
+    const int drop = SPLIT_BITS * (ns + 1) - fband;
+    ba.fx.below = drop / SPLIT_BITS;
+    ba.fx.d = drop % SPLIT_BITS;
+    ba.fx.m0 = std::ldexp(1.0f, -ba.fx.d);
+    ba.fx.m1 = std::ldexp(1.0f, 7 - ba.fx.d);
+    ba.fx.m2 = std::ldexp(1.0f, 14 - ba.fx.d);
+    ba.fx.s1 = 21 - ba.fx.d;
+    ba.fx.top = 1 << (10 - ba.fx.d);
+    ba.fx.offset = 0x4B400000ll * (1 + (1ll << ba.fx.s1));
+    ba.wide = (reinterpret_cast<uintptr_t>(C.val) & 31u) == 0;
     ba.err = ctx->dev_err;
     ba.ovf = ctx->dev_err;
     const int kc = bs < 64 ? bs : 64;  // K elements per chunk (band::SB<bs>::KC)

@@ -212,16 +212,6 @@ __device__ __forceinline__ long long fixed_add(long long d, int x, int sh, bool&
   return r;
 }
 
-// d + (x << sh) for a 64-bit x, sh >= 0, flagging a shift or sum that
-// overflows
-__device__ __forceinline__ long long fixed_add64(long long d, long long x, int sh, bool& bad) {
-  const long long t = (long long)((unsigned long long)x << sh);
-  bad |= (t >> sh) != x;
-  const long long r = (long long)((unsigned long long)d + (unsigned long long)t);
-  bad |= ((d ^ r) & (t ^ r)) < 0;
-  return r;
-}
-
 // Sum of squares of FP32 values for the block norms that truncation tests,
 // accurate to about 2^-42 relative without the FP64 pipe: each square of
 // x 2^32 is split exactly into p + e (FMA), p is added to the running sum with
@@ -312,6 +302,59 @@ struct SqAcc {
   }
   __device__ __forceinline__ double value() const {
     return (f32_to_f64_m64(hi) + f32_to_f64_m64(lo)) + big;  // (hi + lo) 2^-64 + big
+  }
+};
+
+// The same sums of squares for four FP64 values at a time, each with its own
+// running sum: the two-sums of one chain wait for each other, and a branch for
+// every value would keep the chains apart.
+struct SqAcc4 {
+  float hi[4] = {0.0f, 0.0f, 0.0f, 0.0f}, lo[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  double big = 0.0;
+  __device__ __forceinline__ void add4(const double (&v)[4]) {
+    bool large = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t bh = (uint32_t)__double2hiint(v[i]), bl = (uint32_t)__double2loint(v[i]);
+      const int f = (int)((bh >> 20) & 0x7ffu);
+      const bool far = f >= 1023 + 28;
+      large |= far;
+      // as SqAcc::add_f64: values below 2^-95 are left out, the low part of
+      // those below 2^-74 as well
+      const float y = (f < 1023 - 95 || far)
+                          ? 0.0f
+                          : __uint_as_float(((uint32_t)(f - 896 + 32) << 23) | (__funnelshift_l(bl, bh, 3) & 0x7fffffu));
+      const float z = (f < 949 || far) ? 0.0f
+                                       : __int2float_rn((int)(bl & 0x1fffffffu)) *
+                                             __uint_as_float((uint32_t)(f - 948 + 32) << 23);
+      const float p = y * y;
+      const float e = fmaf(y, y, -p);
+      const float c = 2.0f * y * z;
+      const float s = hi[i] + p;
+      const float bp = s - hi[i];
+      const float err = (hi[i] - (s - bp)) + (p - bp);
+      hi[i] = s;
+      lo[i] += err + (e + c);
+    }
+    if (large) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if ((int)(((uint32_t)__double2hiint(v[i]) >> 20) & 0x7ffu) >= 1023 + 28) big = fma(v[i], v[i], big);
+    }
+  }
+  __device__ __forceinline__ SqAcc total() const {
+    SqAcc t;
+    t.hi = hi[0];
+    t.lo = lo[0];
+    t.big = big;
+#pragma unroll
+    for (int i = 1; i < 4; ++i) {
+      const float s = t.hi + hi[i];
+      const float bp = s - t.hi;
+      t.lo += lo[i] + ((t.hi - (s - bp)) + (hi[i] - bp));
+      t.hi = s;
+    }
+    return t;
   }
 };
 

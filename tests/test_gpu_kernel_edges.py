@@ -94,3 +94,37 @@ def test_leaf_cluster_sizes(ctx, nl, count):
     Z2, info, rc = ifac.leaf_invchol_batched(ctx, torch.from_numpy(S).cuda())
     assert rc == ifac.ERR_NOT_SPD and info[-1].item() == p + 1 and not info[:-1].any().item()
     assert np.array_equal(Z2.cpu().numpy()[:-1], Z[:-1])
+
+
+@pytest.mark.parametrize("bs,nb,ns,kind", [(64, 3, 8, "normal"), (64, 7, 8, "normal"), (64, 23, 8, "ones"),
+                                           (64, 40, 8, "ones"), (64, 65, 8, "ones"), (64, 9, 3, "normal"),
+                                           (64, 15, 5, "normal"), (32, 30, 6, "ones"), (128, 4, 8, "normal"),
+                                           (64, 65, 7, "ones")])
+def test_split_class_sums(bs, nb, ns, kind):
+    """The weight classes in the 64-bit sums: one and several windows, odd and
+    even slice counts, and units that fall between two classes or below
+    several of them (entries of one magnitude: |sum| up to K, so the unit
+    2^-f grows with K).  Bound: K 2^-(7 s - 5) r_i c_j for the slices, half a
+    unit 2^-f for each window (at least three blocks of 64, or their share)
+    and K 2^-53 (|A||B|)_ij; f >= min(56, 62 - ceil(log2(1.125 K + 2)), 7 (s + 1))."""
+    from paper_1901_07993_gb300 import ifac
+    ctx = ifac.Context()
+    ctx.set_split_slices(ns)
+    rng = np.random.default_rng(7)
+    A, B = synth.random_bsr(nb, bs, 1.0, seed=91), synth.random_bsr(nb, bs, 1.0, seed=92)
+    if kind == "ones":
+        for M in (A, B):
+            M.val[:] = np.where(rng.random(M.val.shape) < 0.5, 1.0, 1.0 - 2.0 ** -9) - 2.0 ** -40 * rng.random(M.val.shape)
+    got = ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, A), False, ifac.upload(ctx, B), False, 1.0, 0.0,
+                              FP64_SPLIT).download()
+    Ad, Bd = full(A), full(B)
+    ref, K = Ad @ Bd, nb * bs
+    f = min(56, 62 - int(np.ceil(np.log2(1.125 * K + 2))), 7 * (ns + 1))
+    r, c = np.abs(Ad).max(axis=1), np.abs(Bd).max(axis=0)
+    windows = -(-K // 192)
+    lim = ((K * 2.0 ** -(7 * ns - 5) + windows * 4 * 2.0 ** -f) * np.outer(r, c)
+           + 2 * K * 2.0 ** -53 * (np.abs(Ad) @ np.abs(Bd)))
+    assert np.all(np.abs(full(got) - ref) <= lim)
+    norms = np.sqrt((got.val ** 2).sum(axis=(1, 2)))
+    dev = ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, A), False, ifac.upload(ctx, B), False, 1.0, 0.0, FP64_SPLIT)
+    assert abs(ifac.bsr_fro(ctx, dev) - np.sqrt((norms ** 2).sum())) <= 1e-12 * np.sqrt((norms ** 2).sum())
