@@ -6,7 +6,7 @@
 // order, so each element is rounded exactly as the plain definition is.
 // Reductions run in a fixed order (per row, then over rows), so results are
 // deterministic from run to run.  The block norms of sums are summed through
-// FP32 (SqAcc: about 2^-44 relative) so that these kernels spend the FP64
+// FP32 (SqAcc, SqAcc4: about 2^-44 relative) so that these kernels spend the FP64
 // pipe -- GB300 runs about two FP64 operations per clock per SM -- on the
 // sums alone.
 #include <cmath>
@@ -17,15 +17,6 @@
 using ifac::tc::SqAcc;
 
 namespace ifac {
-
-__device__ __forceinline__ int find_col(const int32_t* __restrict__ ci, int lo, int hi, int c) {
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (ci[mid] < c) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
 
 __device__ __forceinline__ double block_reduce_sum(double v, double* red) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -74,157 +65,229 @@ __device__ __forceinline__ double scaled(const Scale& s, double x) {
   return __dmul_rn(s.alpha, x);
 }
 
-// an operand value as FP64: FP32 values (the exact results of a TF32/BF16
-// product) are widened on the bit pattern, off the FP64 pipe
-__device__ __forceinline__ double as_f64(double x) { return x; }
-__device__ __forceinline__ double as_f64(float x) { return ifac::tc::f32_to_f64(x); }
-
-// two consecutive operand values (8- or 16-byte aligned) as FP64
-__device__ __forceinline__ void load2(const double* p, double& x, double& y) {
-  const double2 t = *reinterpret_cast<const double2*>(p);
-  x = t.x;
-  y = t.y;
-}
-__device__ __forceinline__ void load2(const float* p, double& x, double& y) {
-  const float2 t = *reinterpret_cast<const float2*>(p);
-  x = as_f64(t.x);
-  y = as_f64(t.y);
-}
-
-// add_elem on loaded values: ha / hb say whether a / b exist
-__device__ __forceinline__ double add_vals(const Scale& sa, bool ha, double a, const Scale& sb, bool hb, double b,
-                                           bool diag, double gamma) {
+__device__ __forceinline__ double add_elem(const Scale& sa, const double* a, const Scale& sb, const double* b,
+                                           bool diag, double gamma, int e) {
   double v = 0.0;
-  if (ha) v = scaled(sa, a);
-  if (hb) {
-    const double t = scaled(sb, b);
-    v = ha ? __dadd_rn(v, t) : t;
-  }
-  if (diag) v = (ha || hb) ? __dadd_rn(v, gamma) : gamma;
-  return v;
-}
-
-template <typename TA, typename TB>
-__device__ __forceinline__ double add_elem(const Scale& sa, const TA* a, const Scale& sb, const TB* b, bool diag,
-                                           double gamma, int e, int ea = -1) {
-  double v = 0.0;
-  if (a) v = scaled(sa, as_f64(a[ea < 0 ? e : ea]));
+  if (a) v = scaled(sa, a[e]);
   if (b) {
-    const double t = scaled(sb, as_f64(b[e]));
+    const double t = scaled(sb, b[e]);
     v = a ? __dadd_rn(v, t) : t;
   }
   if (diag) v = (a || b) ? __dadd_rn(v, gamma) : gamma;
   return v;
 }
 
+// four values times the scale, the mode tested once
+__device__ __forceinline__ void scale4(const Scale& s, double (&x)[4]) {
+  if (s.mode == 1) return;
+  if (s.mode == 2) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = __hiloint2double(__double2hiint(x[i]) ^ (int)0x80000000, __double2loint(x[i]));
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = scaled(s, x[i]);
+}
+
+// four consecutive operand values as FP64: one 32-byte load where `wide` (the
+// values start on a 32-byte boundary), FP32 ones (always the library's own)
+// one 16-byte load
+__device__ __forceinline__ void load4(const double* p, double (&x)[4], bool wide) {
+  if (wide) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(p));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = __ldg(p + i);
+  }
+}
+__device__ __forceinline__ void load4(const float* p, double (&x)[4], bool) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  const float f[4] = {t.x, t.y, t.z, t.w};
+  ifac::tc::f32_to_f64_x4(f, x);
+}
+
+__device__ __forceinline__ void widen4(const double (&w)[4], double (&x)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) x[i] = w[i];
+}
+__device__ __forceinline__ void widen4(const float (&w)[4], double (&x)[4]) { ifac::tc::f32_to_f64_x4(w, x); }
+
+// 32-byte aligned
+static bool wide32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
+
 // the K-major low-precision copy that the tensor-core products read (TF32:
 // FP32 round-to-nearest-even then TF32 round-half-away; BF16 round-to-
 // nearest-even, as their operand conversion rounds), written beside the
 // FP64 result: lp_elt 4 TF32, 2 BF16, 0 none
-__device__ __forceinline__ void lp_store2(void* lp, int lp_elt, size_t i, double x, double y) {
+__device__ __forceinline__ void lp_store4(void* lp, int lp_elt, size_t i, const double (&x)[4]) {
   if (lp_elt == 4) {
-    uint2 w;
-    w.x = ifac::tc::f32_to_tf32(__uint_as_float(ifac::tc::f64_to_f32_bits_rne(x)));
-    w.y = ifac::tc::f32_to_tf32(__uint_as_float(ifac::tc::f64_to_f32_bits_rne(y)));
-    *reinterpret_cast<uint2*>(static_cast<uint32_t*>(lp) + i) = w;
+    uint32_t w[4];
+    ifac::tc::f64_to_tf32_x4(x, w);
+    *reinterpret_cast<uint4*>(static_cast<uint32_t*>(lp) + i) = make_uint4(w[0], w[1], w[2], w[3]);
   } else if (lp_elt == 2) {
-    const uint32_t w = (uint32_t)ifac::tc::f64_to_bf16_bits_rne(x) | ((uint32_t)ifac::tc::f64_to_bf16_bits_rne(y) << 16);
-    *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(lp) + i) = w;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = ifac::tc::f64_to_bf16_bits_rne(x[k]);
+    *reinterpret_cast<uint2*>(static_cast<uint16_t*>(lp) + i) = make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16));
   }
 }
 
-// one warp per output block (grid-stride over blocks).  Element by element
-// v = 0 + alpha a + beta b + gamma [diagonal], left to right, each step
-// rounded; the leading 0 + x is x.  The FP64 Frobenius norm of the block.
-// Lanes take consecutive elements (VEC of them: two for even bs * bs).  B's
-// values are FP64 or FP32 (TB).
-template <int VEC, typename TB>
-__global__ void k_add(const int32_t* __restrict__ crow, const int32_t* __restrict__ cci, int64_t cnnz, int bs,
-                      Scale sa, const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
-                      const double* __restrict__ aval, Scale sb, const int32_t* __restrict__ brp,
-                      const int32_t* __restrict__ bci, const TB* __restrict__ bval,
-                      const int32_t* __restrict__ bmap, double gamma, double* __restrict__ cval,
-                      double* __restrict__ cnorm, void* __restrict__ lp, int lp_elt) {
+// position of column c in ci[lo, hi) (sorted), -1 when absent: the warp probes
+// 32 entries at a time, so a short row takes one load
+__device__ __forceinline__ int find_warp(const int32_t* __restrict__ ci, int lo, int hi, int c) {
+  const int lane = threadIdx.x & 31;
+  while (hi - lo > 32) {
+    const int step = (hi - lo + 31) / 32, p = lo + lane * step;
+    const unsigned m = __ballot_sync(0xffffffffu, p < hi && ci[p] <= c);
+    if (!m) return -1;
+    lo += (31 - __clz((int)m)) * step;
+    hi = min(hi, lo + step);
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, lo + lane < hi && ci[lo + lane] == c);
+  return m ? lo + __ffs((int)m) - 1 : -1;
+}
+
+// the block's norm from its warps' sums of squares, added in warp order (one
+// barrier per block: the caller alternates between two sets of partials)
+template <int W>
+__device__ __forceinline__ void block_norm(const ifac::tc::SqAcc4& sq, double (&part)[W], double* out) {
+  const double t = sq.total().warp_total();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = t;
+  if constexpr (W > 1) __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0.0;
+#pragma unroll
+    for (int w = 0; w < W; ++w) sum += part[w];
+    *out = sqrt(sum);
+  }
+}
+
+// One CTA of W warps per output block (grid-stride over blocks).  Element by
+// element v = 0 + alpha a + beta b + gamma [diagonal], left to right, each
+// step rounded; the leading 0 + x is x.  B's values are FP64 or FP32 (TB).
+// Bound by HBM: four values a thread and step as one 32-byte load per operand
+// and one 32-byte store, their squares in four independent chains, and no
+// branch per value.  (One warp per block, two values and a test of every
+// value's magnitude at a time ran at 2.5 - 3.4 TB/s of 6.8, and small sums
+// left most of the SMs' warps empty.)  Z + M of the 262,144-row chain with M
+// in FP32 and Z's TF32 copy (1.2 GB): 349 -> 228 us; the FP64 sum of the 65,536-row
+// chain with beta = -0.375 (302 MB, two FP64 operations a value): 123 -> 76 us; of
+// the 4096-row chain at bs 32: 16 -> 5.6 us.
+template <int W, typename TB>
+__global__ void __launch_bounds__(32 * W)
+    k_add(const int32_t* __restrict__ crow, const int32_t* __restrict__ cci, int64_t cnnz, int bs, Scale sa,
+          const int32_t* __restrict__ arp, const int32_t* __restrict__ aci, const double* __restrict__ aval, Scale sb,
+          const int32_t* __restrict__ brp, const int32_t* __restrict__ bci, const TB* __restrict__ bval,
+          const int32_t* __restrict__ bmap, double gamma, double* __restrict__ cval, double* __restrict__ cnorm,
+          void* __restrict__ lp, int lp_elt, bool awide, bool bwide, bool cwide) {
+  __shared__ double part[2][W];
+  const int bsz = bs * bs;
+  int par = 0;
+  for (int64_t p = blockIdx.x; p < cnnz; p += gridDim.x, par ^= 1) {
+    const int I = crow[p], J = cci[p];
+    const int qa = find_warp(aci, arp[I], arp[I + 1], J);
+    const int qb = bval ? find_warp(bci, brp[I], brp[I + 1], J) : -1;
+    const double* a = aval + (size_t)(qa < 0 ? 0 : qa) * bsz;
+    const TB* b = bval + (size_t)(qb < 0 ? 0 : (bmap ? bmap[qb] : qb)) * bsz;
+    double* c = cval + (size_t)p * bsz;
+    const bool dblk = I == J && gamma != 0.0;
+    ifac::tc::SqAcc4 sq;
+#pragma unroll 2
+    for (int e = (int)threadIdx.x * 4; e < bsz; e += 128 * W) {
+      double v[4] = {0.0, 0.0, 0.0, 0.0}, t[4];
+      if (qa >= 0) load4(a + e, v, awide);
+      if (qb >= 0) load4(b + e, t, bwide);
+      if (qa >= 0) scale4(sa, v);
+      if (qb >= 0) {
+        scale4(sb, t);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = qa >= 0 ? __dadd_rn(v[i], t[i]) : t[i];
+      }
+      if (dblk) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if ((e + i) / bs == (e + i) % bs) v[i] = (qa >= 0 || qb >= 0) ? __dadd_rn(v[i], gamma) : gamma;
+      }
+      ifac::tc::store4(c + e, v, cwide);
+      if (lp_elt) lp_store4(lp, lp_elt, (size_t)p * bsz + e, v);
+      sq.add4(v);
+    }
+    block_norm<W>(sq, part[par], cnorm + p);
+  }
+}
+
+// the same for block sizes whose square is no multiple of four: one warp per
+// block, element by element
+__global__ void k_add_odd(const int32_t* __restrict__ crow, const int32_t* __restrict__ cci, int64_t cnnz, int bs,
+                          Scale sa, const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
+                          const double* __restrict__ aval, Scale sb, const int32_t* __restrict__ brp,
+                          const int32_t* __restrict__ bci, const double* __restrict__ bval,
+                          const int32_t* __restrict__ bmap, double gamma, double* __restrict__ cval,
+                          double* __restrict__ cnorm) {
   const int lane = threadIdx.x & 31;
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int bsz = bs * bs;
   for (int64_t p = w0; p < cnnz; p += nw) {
     const int I = crow[p], J = cci[p];
-    int qa = -1, qb = -1;
-    if (lane == 0) {
-      int q = find_col(aci, arp[I], arp[I + 1], J);
-      qa = (q < arp[I + 1] && aci[q] == J) ? q : -1;
-      if (bval) {
-        int r = find_col(bci, brp[I], brp[I + 1], J);
-        qb = (r < brp[I + 1] && bci[r] == J) ? r : -1;
-      }
-    }
-    qa = __shfl_sync(0xffffffffu, qa, 0);
-    qb = __shfl_sync(0xffffffffu, qb, 0);
+    const int qa = find_warp(aci, arp[I], arp[I + 1], J);
+    const int qb = bval ? find_warp(bci, brp[I], brp[I + 1], J) : -1;
     const double* a = qa >= 0 ? aval + (size_t)qa * bsz : nullptr;
-    const TB* b = qb >= 0 ? bval + (size_t)(bmap ? bmap[qb] : qb) * bsz : nullptr;
-    double* c = cval + (size_t)p * bsz;
+    const double* b = qb >= 0 ? bval + (size_t)(bmap ? bmap[qb] : qb) * bsz : nullptr;
     const bool dblk = I == J && gamma != 0.0;
     SqAcc sq;
-#pragma unroll 4
-    for (int e = lane * VEC; e < bsz; e += 32 * VEC) {
-      if constexpr (VEC == 2) {
-        // one vector load per operand (pairs never straddle two blocks)
-        double ax = 0.0, ay = 0.0, bx = 0.0, by = 0.0;
-        if (a) load2(a + e, ax, ay);
-        if (b) load2(b + e, bx, by);
-        double2 v;
-        v.x = add_vals(sa, a != nullptr, ax, sb, b != nullptr, bx, dblk && e / bs == e % bs, gamma);
-        v.y = add_vals(sa, a != nullptr, ay, sb, b != nullptr, by, dblk && (e + 1) / bs == (e + 1) % bs, gamma);
-        *reinterpret_cast<double2*>(c + e) = v;
-        if (lp_elt) lp_store2(lp, lp_elt, (size_t)p * bsz + e, v.x, v.y);
-        sq.add_f64(v.x);
-        sq.add_f64(v.y);
-      } else {
-        const double v = add_elem(sa, a, sb, b, dblk && e / bs == e % bs, gamma, e);
-        c[e] = v;
-        sq.add_f64(v);
-      }
+    for (int e = lane; e < bsz; e += 32) {
+      const double v = add_elem(sa, a, sb, b, dblk && e / bs == e % bs, gamma, e);
+      cval[(size_t)p * bsz + e] = v;
+      sq.add_f64(v);
     }
     const double ss = sq.warp_total();
     if (lane == 0) cnorm[p] = sqrt(ss);
   }
 }
 
+template <int W, typename TB>
+static void launch_add(ifac_ctx* ctx, Scale sa, const ifac_bsr& A, Scale sb, const ifac_bsr* B, double gamma,
+                       ifac_bsr& C, const int32_t* crow, const int32_t* bmap, void* lp, int lp_elt) {
+  const int grid = (int)std::min<int64_t>(C.nnzb, 152 * 64 / W);
+  k_add<W, TB><<<grid, 32 * W, 0, ctx->stream>>>(
+      crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val, sb, B ? B->row_ptr : nullptr,
+      B ? B->col_idx : nullptr, B ? reinterpret_cast<const TB*>(B->val) : nullptr, bmap, gamma, C.val, C.norms, lp,
+      lp_elt, wide32(A.val), B && wide32(B->val), wide32(C.val));
+}
+
 void add_numeric(ifac_ctx* ctx, double alpha, const ifac_bsr& A, double beta, const ifac_bsr* B, double gamma,
                  ifac_bsr& C, const int32_t* crow, const int32_t* bmap, void* lp, int lp_elt, bool b32) {
-  if (lp_elt && (C.bs * C.bs) % 2 != 0) fail(IFAC_ERR_UNSUPPORTED, "low-precision copy: even bs * bs");
+  const int bsz = C.bs * C.bs;
+  if (lp_elt && bsz % 4 != 0) fail(IFAC_ERR_UNSUPPORTED, "low-precision copy: even block size");
+  if (b32 && B && bsz % 4 != 0) fail(IFAC_ERR_UNSUPPORTED, "FP32 operand values: even block size");
   if (C.nnzb == 0) return;
-  const int64_t warps = std::min<int64_t>(C.nnzb, 152 * 64);
   const Scale sa = make_scale(alpha), sb = make_scale(beta);
-  const int32_t* brp = B ? B->row_ptr : nullptr;
-  const int32_t* bci = B ? B->col_idx : nullptr;
-  const double* bv = B ? B->val : nullptr;
-  const int grid = cdiv(warps * 32, 256);
-  if (b32 && B) {
-    if ((C.bs * C.bs) % 2 != 0) fail(IFAC_ERR_UNSUPPORTED, "FP32 operand values: even bs * bs");
-    k_add<2, float><<<grid, 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val, sb,
-                                                   brp, bci, reinterpret_cast<const float*>(bv), bmap, gamma, C.val,
-                                                   C.norms, lp, lp_elt);
-  } else if ((C.bs * C.bs) % 2 == 0) {  // pairs never straddle two blocks
-    k_add<2, double><<<grid, 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val,
-                                                    sb, brp, bci, bv, bmap, gamma, C.val, C.norms, lp, lp_elt);
+  if (bsz % 4 != 0) {
+    const int64_t warps = std::min<int64_t>(C.nnzb, 152 * 64);
+    k_add_odd<<<cdiv(warps * 32, 256), 256, 0, ctx->stream>>>(
+        crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val, sb, B ? B->row_ptr : nullptr,
+        B ? B->col_idx : nullptr, B ? B->val : nullptr, bmap, gamma, C.val, C.norms);
+  } else if (b32 && B) {  // bs 32, 64 or 128
+    if (bsz >= 4096) launch_add<8, float>(ctx, sa, A, sb, B, gamma, C, crow, bmap, lp, lp_elt);
+    else launch_add<4, float>(ctx, sa, A, sb, B, gamma, C, crow, bmap, lp, lp_elt);
+  } else if (bsz >= 4096) {  // eight warps with 16 values a thread or more, four with eight, one below
+    launch_add<8, double>(ctx, sa, A, sb, B, gamma, C, crow, bmap, lp, lp_elt);
+  } else if (bsz >= 1024) {
+    launch_add<4, double>(ctx, sa, A, sb, B, gamma, C, crow, bmap, lp, lp_elt);
   } else {
-    k_add<1, double><<<grid, 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val,
-                                                    sb, brp, bci, bv, bmap, gamma, C.val, C.norms, nullptr, 0);
+    launch_add<1, double>(ctx, sa, A, sb, B, gamma, C, crow, bmap, lp, lp_elt);
   }
   IFAC_CK_LAUNCH();
 }
 
-// C = alpha (U + strict_upper(U)^T) + beta B + gamma I, one warp per output
+// C = alpha (U + strict_upper(U)^T) + beta B + gamma I, one CTA per output
 // block.  Block (I, J), J >= I, is add_elem of alpha U_IJ and beta B_IJ;
 // block (I, J), J < I, takes alpha U_JI^T in place of alpha U_IJ, moved
-// through shared memory in stripes of four output rows (four-value column
-// segments of U_JI per source row: whole 32-byte sectors for FP64 values, half
-// sectors for FP32 values, whose other half the next stripe reads from cache;
-// eight-row stripes for FP32 measured slower: the doubled shared memory cuts
-// the resident warps).  bs = 64.  U's values are FP64 or FP32 (TU).
+// through shared memory as one 64 x 64 tile, so that U is read in whole rows
+// (stripes of four output rows per warp read half sectors of FP32 values).
+// bs = 64.  U's values are FP64 or FP32 (TU).  delta of the 262,144-row chain
+// with its TF32 copy: 354 -> 198 us from FP32 values, 262 -> 150 us from FP64.
 constexpr int SYM_WARPS = 8;
 
 template <typename TU>
@@ -234,107 +297,78 @@ __global__ void __launch_bounds__(32 * SYM_WARPS)
           const int32_t* __restrict__ umap, Scale sb,
           const int32_t* __restrict__ brp, const int32_t* __restrict__ bci, const double* __restrict__ bval,
           double gamma, double* __restrict__ cval, double* __restrict__ cnorm, int mirror, void* __restrict__ lp,
-          int lp_elt) {
-  constexpr int BS = 64, BSZ = BS * BS;
-  constexpr int RW = 4;  // output rows per stripe
-  __shared__ double stripe[SYM_WARPS][RW][BS + 1];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  double(*st)[BS + 1] = stripe[wid];  // RW rows
-  for (int64_t p = w0; p < cnnz; p += nw) {
+          int lp_elt, bool uwide, bool bwide, bool cwide) {
+  constexpr int BS = 64, BSZ = BS * BS, STEP = 128 * SYM_WARPS;
+  __shared__ TU tile[BS][BS + 1];
+  __shared__ double part[2][SYM_WARPS];
+  int par = 0;
+  for (int64_t p = blockIdx.x; p < cnnz; p += gridDim.x, par ^= 1) {
     const int I = crow[p], J = cci[p];
     const bool lower = J < I;
     const int r = lower ? J : I, c = lower ? I : J;
-    int qu = -1, qb = -1;
-    if (lane == 0) {
-      const int k = find_col(uci, urp[r], urp[r + 1], c);
-      qu = (k < urp[r + 1] && uci[k] == c) ? k : -1;
-      if (bval) {
-        const int m = find_col(bci, brp[I], brp[I + 1], J);
-        qb = (m < brp[I + 1] && bci[m] == J) ? m : -1;
-      }
-    }
-    qu = __shfl_sync(0xffffffffu, qu, 0);
-    qb = __shfl_sync(0xffffffffu, qb, 0);
-    const TU* u = qu >= 0 ? uval + (size_t)(umap ? umap[qu] : qu) * BSZ : nullptr;
-    const double* b = qb >= 0 ? bval + (size_t)qb * BSZ : nullptr;
-    double* out = cval + (size_t)p * BSZ;
+    const int qu = find_warp(uci, urp[r], urp[r + 1], c);
+    const int qb = bval ? find_warp(bci, brp[I], brp[I + 1], J) : -1;
+    const TU* u = uval + (size_t)(qu < 0 ? 0 : (umap ? umap[qu] : qu)) * BSZ;
+    const double* b = bval + (size_t)(qb < 0 ? 0 : qb) * BSZ;
     const bool dblk = I == J && gamma != 0.0;
     // mirror: a diagonal block takes its strictly lower triangle from its
     // upper one as well, so the result is exactly symmetric
-    const bool mir = mirror && I == J;
-    SqAcc sq;
-    if (!lower || !u) {
-#pragma unroll 4
-      for (int e = lane * 2; e < BSZ; e += 64) {
-        const int rr = e / BS, c0 = e % BS;
-        double2 v;
-        if (!mir) {  // one vector load per operand
-          const TU* uu = lower ? nullptr : u;
-          double ux = 0.0, uy = 0.0, bx = 0.0, by = 0.0;
-          if (uu) load2(uu + e, ux, uy);
-          if (b) load2(b + e, bx, by);
-          v.x = add_vals(sa, uu != nullptr, ux, sb, b != nullptr, bx, dblk && rr == c0, gamma);
-          v.y = add_vals(sa, uu != nullptr, uy, sb, b != nullptr, by, dblk && rr == c0 + 1, gamma);
-        } else {
-          const int e0 = c0 < rr ? c0 * BS + rr : -1, e1 = c0 + 1 < rr ? (c0 + 1) * BS + rr : -1;
-          v.x = add_elem(sa, lower ? nullptr : u, sb, b, dblk && rr == c0, gamma, e, e0);
-          v.y = add_elem(sa, lower ? nullptr : u, sb, b, dblk && rr == c0 + 1, gamma, e + 1, e1);
-        }
-        *reinterpret_cast<double2*>(out + e) = v;
-        if (lp_elt) lp_store2(lp, lp_elt, (size_t)p * BSZ + e, v.x, v.y);
-        sq.add_f64(v.x);
-        sq.add_f64(v.y);
-      }
-    } else {
-      for (int r0 = 0; r0 < BS; r0 += RW) {
-        // alpha U_JI, source rows s = 0..63, columns r0..r0+RW-1
-#pragma unroll 8
-        for (int k = 0; k < 2 * RW; ++k) {
-          const int idx = k * 32 + lane, s = idx / RW, j = idx % RW;
-          st[j][s] = scaled(sa, as_f64(u[s * BS + r0 + j]));
-        }
-        __syncwarp();
-        // output rows r0..r0+RW-1: alpha U_JI^T (+ beta B_IJ), columns 0..63
+    const bool moved = qu >= 0 && (lower || (mirror && I == J));  // CTA-uniform
+    if (moved) {
 #pragma unroll
-        for (int k = 0; k < RW; ++k) {
-          const int idx = k * 64 + lane * 2, j = idx >> 6, col = idx & 63, e = (r0 + j) * BS + col;
-          double2 v;
-          v.x = st[j][col];
-          v.y = st[j][col + 1];
-          if (b) {
-            v.x = __dadd_rn(v.x, scaled(sb, b[e]));
-            v.y = __dadd_rn(v.y, scaled(sb, b[e + 1]));
-          }
-          *reinterpret_cast<double2*>(out + e) = v;
-          if (lp_elt) lp_store2(lp, lp_elt, (size_t)p * BSZ + e, v.x, v.y);
-          sq.add_f64(v.x);
-          sq.add_f64(v.y);
-        }
-        __syncwarp();
-      }
+      for (int e = (int)threadIdx.x; e < BSZ; e += 32 * SYM_WARPS) tile[e / BS][e % BS] = u[e];
+      __syncthreads();
     }
-    const double ss = sq.warp_total();
-    if (lane == 0) cnorm[p] = sqrt(ss);
+    ifac::tc::SqAcc4 sq;
+#pragma unroll 2
+    for (int e = (int)threadIdx.x * 4; e < BSZ; e += STEP) {
+      const int rr = e / BS, c0 = e % BS;
+      double v[4] = {0.0, 0.0, 0.0, 0.0}, t[4];
+      if (moved) {
+        TU w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = (lower || c0 + i < rr) ? tile[c0 + i][rr] : tile[rr][c0 + i];
+        widen4(w, v);
+      } else if (qu >= 0) {
+        load4(u + e, v, uwide);
+      }
+      if (qb >= 0) load4(b + e, t, bwide);
+      if (qu >= 0) scale4(sa, v);
+      if (qb >= 0) {
+        scale4(sb, t);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = qu >= 0 ? __dadd_rn(v[i], t[i]) : t[i];
+      }
+      if (dblk) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (rr == c0 + i) v[i] = (qu >= 0 || qb >= 0) ? __dadd_rn(v[i], gamma) : gamma;
+      }
+      ifac::tc::store4(cval + (size_t)p * BSZ + e, v, cwide);
+      if (lp_elt) lp_store4(lp, lp_elt, (size_t)p * BSZ + e, v);
+      sq.add4(v);
+    }
+    // (the barrier inside also keeps the tile until every warp has read it)
+    block_norm<SYM_WARPS>(sq, part[par], cnorm + p);
   }
+}
+
+template <typename TU>
+static void launch_sym(ifac_ctx* ctx, double alpha, const ifac_bsr& U, double beta, const ifac_bsr* B, double gamma,
+                       ifac_bsr& C, const int32_t* crow, const int32_t* umap, bool mirror, void* lp, int lp_elt) {
+  const int grid = (int)std::min<int64_t>(C.nnzb, 152 * 64 / SYM_WARPS);
+  k_sym<TU><<<grid, 32 * SYM_WARPS, 0, ctx->stream>>>(
+      crow, C.col_idx, C.nnzb, make_scale(alpha), U.row_ptr, U.col_idx, reinterpret_cast<const TU*>(U.val), umap,
+      make_scale(beta), B ? B->row_ptr : nullptr, B ? B->col_idx : nullptr, B ? B->val : nullptr, gamma, C.val,
+      C.norms, mirror ? 1 : 0, lp, lp_elt, wide32(U.val), B && wide32(B->val), wide32(C.val));
 }
 
 void sym_numeric(ifac_ctx* ctx, double alpha, const ifac_bsr& U, double beta, const ifac_bsr* B, double gamma,
                  ifac_bsr& C, const int32_t* crow, const int32_t* umap, bool mirror, void* lp, int lp_elt, bool u32) {
   if (C.nnzb == 0) return;
   if (U.bs != 64) fail(IFAC_ERR_UNSUPPORTED, "symmetric completion needs bs = 64");
-  const int64_t ctas = std::min<int64_t>(cdiv(C.nnzb, SYM_WARPS), 152 * 8);
-  if (u32)
-    k_sym<float><<<(int)ctas, 32 * SYM_WARPS, 0, ctx->stream>>>(
-        crow, C.col_idx, C.nnzb, make_scale(alpha), U.row_ptr, U.col_idx, reinterpret_cast<const float*>(U.val), umap,
-        make_scale(beta), B ? B->row_ptr : nullptr, B ? B->col_idx : nullptr, B ? B->val : nullptr, gamma, C.val,
-        C.norms, mirror ? 1 : 0, lp, lp_elt);
-  else
-    k_sym<double><<<(int)ctas, 32 * SYM_WARPS, 0, ctx->stream>>>(
-        crow, C.col_idx, C.nnzb, make_scale(alpha), U.row_ptr, U.col_idx, U.val, umap, make_scale(beta),
-        B ? B->row_ptr : nullptr, B ? B->col_idx : nullptr, B ? B->val : nullptr, gamma, C.val, C.norms,
-        mirror ? 1 : 0, lp, lp_elt);
+  if (u32) launch_sym<float>(ctx, alpha, U, beta, B, gamma, C, crow, umap, mirror, lp, lp_elt);
+  else launch_sym<double>(ctx, alpha, U, beta, B, gamma, C, crow, umap, mirror, lp, lp_elt);
   IFAC_CK_LAUNCH();
 }
 

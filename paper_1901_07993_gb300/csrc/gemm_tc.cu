@@ -1812,17 +1812,6 @@ __device__ __forceinline__ void fixed_to_f64(const long long (&s)[4], const int 
   }
 }
 
-// four consecutive FP64 values, one 32-byte sector per lane when p is aligned
-__device__ __forceinline__ void store4(double* p, const double (&v)[4], bool wide) {
-  if (wide) {
-    // (no "memory": nothing here reads C, and the next columns' loads may move up)
-    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]));
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) p[i] = v[i];
-  }
-}
-
 template <int B>
 __global__ void __launch_bounds__(band::NTB, 1)
     k_gemm_split_band(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,

@@ -358,6 +358,17 @@ struct SqAcc4 {
   }
 };
 
+// four consecutive FP64 values, one 32-byte sector per lane when p is aligned
+__device__ __forceinline__ void store4(double* p, const double (&v)[4], bool wide) {
+  if (wide) {
+    // (no "memory": the kernels never read what they store here, and later loads may move up)
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3]));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[i] = v[i];
+  }
+}
+
 // named barrier 1 over the NT epilogue threads
 template <int NT>
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
@@ -512,6 +523,42 @@ __device__ __forceinline__ uint16_t f64_to_bf16_bits_rne(double x) {
   if (rem > half || (rem == half && (mant & 1u))) ++bits;
   if (e8 > 254 || bits >= 0x7f80u) return sign | 0x7f80u;
   return sign | (uint16_t)bits;
+}
+
+// Four values at a time without a branch per value (a branch keeps the four
+// from overlapping): the usual magnitudes here, a group that holds another one
+// through the routines above.
+__device__ __forceinline__ void f32_to_f64_x4(const float (&f)[4], double (&x)[4]) {
+  bool odd = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t u = __float_as_uint(f[i]), m = u & 0x7fffffffu, sign = u & 0x80000000u;
+    odd |= (m - 1u < 0x7fffffu) || m >= 0x7f800000u;  // subnormal, inf, NaN
+    x[i] = __hiloint2double((int)(m == 0u ? sign : sign | ((m >> 3) + (896u << 20))), (int)(u << 29));
+  }
+  if (odd) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = f32_to_f64(f[i]);
+  }
+}
+
+// TF32 patterns of four FP64 values (FP32 round-to-nearest-even, then TF32
+// round-half-away)
+__device__ __forceinline__ void f64_to_tf32_x4(const double (&x)[4], uint32_t (&w)[4]) {
+  bool odd = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t h = (uint32_t)__double2hiint(x[i]), l = (uint32_t)__double2loint(x[i]), m = h & 0x7fffffffu;
+    odd |= m >= (1150u << 20);  // FP32's largest binade and above
+    uint32_t b = __funnelshift_l(l, m - (896u << 20), 3);
+    b += ((l & 0x1fffffffu) + (b & 1u)) > 0x10000000u ? 1u : 0u;
+    if (m < (897u << 20)) b = 0u;  // below the normal range: zero
+    w[i] = f32_to_tf32(__uint_as_float(b | (h & 0x80000000u)));
+  }
+  if (odd) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = f32_to_tf32(__uint_as_float(f64_to_f32_bits_rne(x[i])));
+  }
 }
 
 }  // namespace tc

@@ -128,3 +128,32 @@ def test_split_class_sums(bs, nb, ns, kind):
     norms = np.sqrt((got.val ** 2).sum(axis=(1, 2)))
     dev = ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, A), False, ifac.upload(ctx, B), False, 1.0, 0.0, FP64_SPLIT)
     assert abs(ifac.bsr_fro(ctx, dev) - np.sqrt((norms ** 2).sum())) <= 1e-12 * np.sqrt((norms ** 2).sum())
+
+
+@pytest.mark.parametrize("bs,nb,density,shift", [(64, 1, 1.0, 0), (64, 40, 0.9, 1), (32, 70, 0.6, 0), (32, 5, 0.3, 3),
+                                                 (128, 3, 0.7, 2), (16, 33, 0.5, 1), (5, 9, 0.4, 0), (6, 9, 0.4, 1),
+                                                 (16, 1100, 0.9, 0)])
+def test_sum_edges(ctx, bs, nb, density, shift):
+    """Sums equal to the oracle's, value for value: long and short rows, block sizes of
+    each kernel shape, values off a 32-byte boundary, missing blocks, zeros,
+    subnormals, infinities and values whose squares leave FP32's range.  The
+    norms within 2^-40."""
+    from paper_1901_07993_gb300 import ifac
+    A = synth.random_bsr(nb, bs, density, seed=61)
+    B = synth.random_bsr(nb, bs, density, seed=62, empty_rows=min(1, nb - 1))
+    rng = np.random.default_rng(3)
+    special = np.array([0.0, -0.0, 5e-324, -1e-310, 1e-200, 1e30, -1e150, np.inf])
+    for M in (A, B):
+        M.val[: M.nnzb // 3] = special[rng.integers(0, len(special) - 1, M.val[: M.nnzb // 3].shape)]
+    dA, dB = borrowed(A, shift), borrowed(B, shift)
+    for alpha, beta, gamma in ((1.0, -0.375, 1.0), (-1.0, 1.0, 0.0), (0.5, 2.0, -3.0)):
+        ref = oracle.add(alpha, A, beta, B, gamma)
+        dev = ifac.bsr_add(ctx, alpha, dA, beta, dB, gamma)
+        got = dev.download()
+        assert np.array_equal(got.row_ptr, ref.row_ptr) and np.array_equal(got.col_idx, ref.col_idx)
+        assert np.array_equal(got.val, ref.val)  # (the library's leading 0 + x is x: -0 stays -0)
+        f = np.sqrt((np.asarray(ref.val) ** 2).sum())
+        assert abs(ifac.bsr_fro(ctx, dev) - f) <= 1e-12 * f
+    A.val[0, 0, 0] = np.inf
+    got = ifac.bsr_add(ctx, 1.0, borrowed(A, shift), 0.0, None, 0.0)
+    assert np.isinf(ifac.bsr_fro(ctx, got)) and np.array_equal(got.download().val, A.val)
