@@ -134,6 +134,11 @@ void to_host(ifac_ctx* ctx, void* host, const void* dev, size_t bytes) {
   }
 }
 
+int32_t read_word(ifac_ctx* ctx, HostWord w) {
+  IFAC_CK(cudaStreamSynchronize(ctx->stream));
+  return *const_cast<volatile int32_t*>(host_word(ctx, w));
+}
+
 void to_host_many(ifac_ctx* ctx, std::initializer_list<HostRead> reads) {
   size_t off = 0;
   for (const HostRead& r : reads) {
@@ -297,12 +302,14 @@ int ifac_create(ifac_ctx** out, void* stream, const ifac_allocator* alloc) {
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
   }
-  if (cudaMallocHost(&c->pinned, 4096) != cudaSuccess) { delete c; return IFAC_ERR_CUDA; }
+  if (cudaHostAlloc(&c->pinned, 4096 + 256, cudaHostAllocMapped) != cudaSuccess) { delete c; return IFAC_ERR_CUDA; }
   void* words = nullptr;
   if (cudaMalloc(&words, 64) != cudaSuccess) { cudaFreeHost(c->pinned); delete c; return IFAC_ERR_CUDA; }
   cudaMemset(words, 0, 64);
   c->dev_err = static_cast<int*>(words);
   c->dev_pairs = reinterpret_cast<unsigned long long*>(static_cast<char*>(words) + 16);  // 4 counters
+  c->ticket = reinterpret_cast<unsigned*>(static_cast<char*>(words) + 48);
+  c->host_words = reinterpret_cast<int32_t*>(static_cast<char*>(c->pinned) + 4096);
   *out = c;
   return IFAC_OK;
 }

@@ -377,7 +377,7 @@ static Mat filter(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* seg, const in
                                                                           active, mode, keep.p);
     IFAC_CK_LAUNCH();
   }
-  return select_blocks(ctx, A, nullptr, keep.p);
+  return select_blocks(ctx, A, keep.p);
 }
 
 // explicit transpose: block q of A^T = (block src[q] of A)^T
@@ -544,7 +544,7 @@ static Mat leaf_factors(ifac_ctx* ctx, const ifac_bsr& S, const std::vector<Node
                                               Z.m.val, Z.m.norms);
   IFAC_CK_LAUNCH();
   IFAC_CK(cudaStreamSynchronize(ctx->stream));  // host vectors rp/ci go out of scope
-  return compact(ctx, std::move(Z), nullptr, tau);
+  return compact(ctx, std::move(Z), tau);
 }
 
 Mat leaf_factors_ranges(ifac_ctx* ctx, const ifac_bsr& S, const std::vector<std::pair<int, int>>& ranges,

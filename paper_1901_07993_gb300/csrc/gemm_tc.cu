@@ -38,6 +38,7 @@
 #include <cuda_bf16.h>
 
 #include "internal.cuh"
+#include "scan_tail.cuh"
 #include "tc_common.cuh"
 
 namespace ifac {
@@ -502,9 +503,13 @@ __global__ void __launch_bounds__(256) k_convert(const V* __restrict__ val, cons
     }
   };
   T* out = reinterpret_cast<T*>(dst);
-  for (int64_t qb = blockIdx.x; qb < nblk; qb += gridDim.x) {
-    const V* s = val + (size_t)(src ? src[qb] : qb) * BSZ;
+  for (int64_t qb = blockIdx.x; qb <= nblk; qb += gridDim.x) {
     T* d = out + (size_t)qb * BSZ;
+    if (qb == nblk) {  // the zero block
+      for (int e = threadIdx.x; e < BSZ; e += blockDim.x) d[e] = 0;
+      continue;
+    }
+    const V* s = val + (size_t)(src ? src[qb] : qb) * BSZ;
     if (!tr) {
       for (int e = threadIdx.x; e < BSZ; e += blockDim.x) d[e] = conv(s[e]);
       continue;
@@ -606,30 +611,26 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// flag[tile] = 1 for every tile holding a block of C's pattern
-__global__ void k_tile_flags(const int32_t* __restrict__ row, const int32_t* __restrict__ ci, int64_t nnz, int tm,
-                             int tn, int ntc, uint8_t* __restrict__ flag) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= nnz) return;
-  flag[(size_t)(row[p] / tm) * ntc + ci[p] / tn] = 1;
-}
-
 // Tiles of a sparse C in one pass over its blocks: block p owns its tile
 // (I / tm, J / tn) when the tile holds no earlier block, i.e. neither the block
 // before it in row I nor a block of the tile's earlier rows lies in the tile's
 // column range.  The owners, in C's order, list every tile once.
-__global__ void k_tile_owner(const int32_t* __restrict__ row, const int32_t* __restrict__ rp,
-                             const int32_t* __restrict__ ci, int64_t nnz, int tm, int tn, int32_t* __restrict__ own) {
+__global__ void __launch_bounds__(256)
+    k_tile_owner(const int32_t* __restrict__ row, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
+                 int64_t nnz, int tm, int tn, int32_t* __restrict__ own, int32_t* __restrict__ off,
+                 unsigned* __restrict__ ticket) {  // off null: scanned afterwards
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p >= nnz) return;
-  const int I = row[p], c0 = (ci[p] / tn) * tn;
-  int o = (p > rp[I] && ci[p - 1] >= c0) ? 0 : 1;
-  for (int I2 = (I / tm) * tm; o && I2 < I; ++I2) {
-    const int hi = rp[I2 + 1];
-    const int q = lower_bound_i32(ci, rp[I2], hi, c0);
-    if (q < hi && ci[q] < c0 + tn) o = 0;
+  if (p < nnz) {
+    const int I = row[p], c0 = (ci[p] / tn) * tn;
+    int o = (p > rp[I] && ci[p - 1] >= c0) ? 0 : 1;
+    for (int I2 = (I / tm) * tm; o && I2 < I; ++I2) {
+      const int hi = rp[I2 + 1];
+      const int q = lower_bound_i32(ci, rp[I2], hi, c0);
+      if (q < hi && ci[q] < c0 + tn) o = 0;
+    }
+    own[p] = o;
   }
-  own[p] = o;
+  if (off) scan_tail<256>(own, off, (int)nnz, ticket, nullptr);
 }
 
 __global__ void k_tile_owner_write(const int32_t* __restrict__ row, const int32_t* __restrict__ ci, int64_t nnz,
@@ -653,19 +654,27 @@ __device__ __forceinline__ int64_t grouped_to_rowmajor(int64_t li, int ntr, int 
   return (g * GROUP + off % rows) * ntc + off / rows;
 }
 
-__global__ void k_tile_count(const uint8_t* __restrict__ flag, int ntr, int ntc, int32_t* __restrict__ cnt) {
-  __shared__ int red[32];
+// flag[li] = 1 when tile li (grouped order) holds a block of C's pattern;
+// counts per chunk and their scan
+__global__ void __launch_bounds__(CHUNK)
+    k_tile_mark(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int nb, int tm, int tn, int ntr,
+                int ntc, uint8_t* __restrict__ flag, int32_t* __restrict__ cnt, int32_t* __restrict__ off,
+                unsigned* __restrict__ ticket) {
   const int64_t tot = (int64_t)ntr * ntc;
   const int64_t li = (int64_t)blockIdx.x * CHUNK + threadIdx.x;
-  const int f = (li < tot && flag[grouped_to_rowmajor(li, ntr, ntc)]) ? 1 : 0;
-  const unsigned m = __ballot_sync(0xffffffffu, f);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = __popc(m);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int t = 0;
-    for (int w = 0; w < CHUNK / 32; ++w) t += red[w];
-    cnt[blockIdx.x] = t;
+  int f = 0;
+  if (li < tot) {
+    const int64_t i = grouped_to_rowmajor(li, ntr, ntc);
+    const int I0 = (int)(i / ntc) * tm, c0 = (int)(i % ntc) * tn;
+    for (int I = I0; !f && I < min(I0 + tm, nb); ++I) {
+      const int hi = rp[I + 1], q = lower_bound_i32(ci, rp[I], hi, c0);
+      f = (q < hi && ci[q] < c0 + tn) ? 1 : 0;
+    }
+    flag[li] = (uint8_t)f;
   }
+  const int c = __syncthreads_count(f);
+  if (threadIdx.x == 0) cnt[blockIdx.x] = c;
+  scan_tail<CHUNK>(cnt, off, (int)gridDim.x, ticket, nullptr);
 }
 
 __global__ void k_tile_write(const uint8_t* __restrict__ flag, int ntr, int ntc, const int32_t* __restrict__ off,
@@ -674,7 +683,7 @@ __global__ void k_tile_write(const uint8_t* __restrict__ flag, int ntr, int ntc,
   const int64_t tot = (int64_t)ntr * ntc;
   const int64_t li = (int64_t)blockIdx.x * CHUNK + threadIdx.x;
   const int64_t i = li < tot ? grouped_to_rowmajor(li, ntr, ntc) : 0;
-  const bool f = li < tot && flag[i];
+  const bool f = li < tot && flag[li];
   const unsigned m = __ballot_sync(0xffffffffu, f);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   if (lane == 0) wbase[w] = __popc(m);
@@ -695,45 +704,92 @@ __global__ void k_tile_write(const uint8_t* __restrict__ flag, int ntr, int ntc,
   }
 }
 
-// dense block-index map of a CSR pattern: map[I*nb + J] = q for block q, else zero_idx
-__global__ void k_map_fill(int32_t* __restrict__ map, int64_t n, int32_t zero_idx) {
-  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < n) map[i] = zero_idx;
+// The same list for up to 65,536 tiles and blocks, in one CTA: flags in shared
+// memory from C's blocks, then one thread per tile.  (Two launches of searches
+// take 9 us on a few hundred block rows.)
+constexpr int SMALL_TILES = 65536;
+
+template <int TMB, int TNB>
+__global__ void __launch_bounds__(1024)
+    k_tiles_small(const int32_t* __restrict__ row, const int32_t* __restrict__ ci, int nnz, int ntr, int ntc,
+                  int32_t* __restrict__ out, int32_t* __restrict__ count) {
+  extern __shared__ uint32_t tbits[];  // [words] bit per tile, grouped order; [words] tiles before each word
+  __shared__ int wsum[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tot = ntr * ntc, words = (tot + 31) / 32, per = (words + 1023) / 1024;
+  int* before = reinterpret_cast<int*>(tbits + words);
+  for (int i = tid; i < words; i += 1024) tbits[i] = 0u;
+  __syncthreads();
+#pragma unroll 4
+  for (int p = tid; p < nnz; p += 1024) {
+    const int tr = row[p] / TMB, tc = ci[p] / TNB, g = tr / GROUP, rows = min(GROUP, ntr - g * GROUP);
+    const int li = g * GROUP * ntc + (tr - g * GROUP) + rows * tc;
+    const uint32_t bit = 1u << (li & 31);
+    if (!(tbits[li >> 5] & bit)) atomicOr(&tbits[li >> 5], bit);
+  }
+  __syncthreads();
+  const int w0 = min(tid * per, words), w1 = min(w0 + per, words);
+  int c = 0;
+  for (int w = w0; w < w1; ++w) c += __popc(tbits[w]);
+  int x = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[wid] = x;
+  __syncthreads();
+  int pos = x - c;
+  for (int w = 0; w < wid; ++w) pos += wsum[w];
+  if (tid == 1023) *count = pos + c;
+  for (int w = w0; w < w1; ++w) {
+    before[w] = pos;
+    pos += __popc(tbits[w]);
+  }
+  __syncthreads();
+  for (int li = tid; li < tot; li += 1024) {
+    const uint32_t u = tbits[li >> 5], bit = 1u << (li & 31);
+    if (!(u & bit)) continue;
+    const int q = before[li >> 5] + __popc(u & (bit - 1u));
+    const int g = li / (GROUP * ntc), rows = min(GROUP, ntr - g * GROUP), off = li - g * GROUP * ntc;
+    out[2 * q] = g * GROUP + off % rows;
+    out[2 * q + 1] = off / rows;
+  }
 }
 
-__global__ void k_map_scatter(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int nb,
-                              int32_t* __restrict__ map) {
+// What a tile plan reads, one warp per block row: the bitmap of op(A)'s row
+// (its K set) and, where they are kept, row I of the dense block-index maps,
+// map[I nb + J] = q for block q, else the zero block's index.
+//
+// Also the number of stored block pairs (op(A)_IK, op(B)_KJ) of the product,
+// i.e. |row K of op(B)| for every block (I, K): all of them, or with upper
+// only those with J >= I.  pairs (nullable) gets one per pair, wpairs
+// (nullable) w per pair.
+__global__ void __launch_bounds__(256)
+    k_plan_rows(const int32_t* __restrict__ arp, const int32_t* __restrict__ aci, const int32_t* __restrict__ brp,
+                const int32_t* __restrict__ bci, int nb, int W, uint32_t* __restrict__ bm, int32_t* __restrict__ mapA,
+                int32_t* __restrict__ mapB, int a_zero, int b_zero, int upper,
+                unsigned long long* __restrict__ pairs, unsigned long long* __restrict__ wpairs, int w) {
   const int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (row >= nb) return;
-  for (int p = rp[row] + lane; p < rp[row + 1]; p += 32) map[(size_t)row * nb + ci[p]] = p;
-}
-
-// pairs += |row K of op(B)| for every stored block (I, K) of op(A): the number
-// of (I, K, J) block triples, i.e. of stored-block products
-// stored block pairs (op(A)_IK, op(B)_KJ) of the product: all of them, or
-// with upper only those with J >= I (found by binary search in the sorted
-// op(B) row K).  wpairs (nullable) also gets w per pair.  Warp per row I.
-__global__ void k_count_pairs(const int32_t* __restrict__ arp, const int32_t* __restrict__ aci, int nb,
-                              const int32_t* __restrict__ brp, const int32_t* __restrict__ bci, int upper,
-                              unsigned long long* __restrict__ pairs, unsigned long long* __restrict__ wpairs,
-                              int w) {
-  const int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  unsigned long long c = 0;
-  if (row < nb)
-    for (int p = arp[row] + lane; p < arp[row + 1]; p += 32) {
-      const int K = aci[p];
-      int lo = brp[K];
-      const int hi = brp[K + 1];
-      if (upper) {
-        int h = hi;
-        while (lo < h) {
-          const int mid = (lo + h) >> 1;
-          if (bci[mid] < row) lo = mid + 1;
-          else h = mid;
-        }
-      }
-      c += (unsigned long long)(hi - lo);
+  uint32_t* bits = bm + (size_t)row * W;
+  for (int i = lane; i < W; i += 32) bits[i] = 0u;
+  if (mapA)
+    for (int c = lane; c < nb; c += 32) {
+      mapA[(size_t)row * nb + c] = a_zero;
+      mapB[(size_t)row * nb + c] = b_zero;
     }
+  __syncwarp();
+  unsigned long long c = 0;
+  for (int p = arp[row] + lane; p < arp[row + 1]; p += 32) {
+    const int K = aci[p];
+    atomicOr(bits + (K >> 5), 1u << (K & 31));
+    if (mapA) mapA[(size_t)row * nb + K] = p;
+    if (pairs) c += (unsigned long long)(brp[K + 1] - (upper ? lower_bound_i32(bci, brp[K], brp[K + 1], row) : brp[K]));
+  }
+  if (mapB)
+    for (int p = brp[row] + lane; p < brp[row + 1]; p += 32) mapB[(size_t)row * nb + bci[p]] = p;
+  if (!pairs) return;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (lane == 0 && c) {
@@ -769,13 +825,64 @@ static EncodeTiledFn encoder() {
 // op(A)_IK for each of its ROWS block rows and of op(B)_KJ for each of its
 // COLS block columns (the zero block when absent); K steps whose op(B) blocks
 // are all absent contribute nothing and are left out.  One warp per tile,
-// candidate K's 32 at a time, lane-parallel.  COUNT: the number of records
-// into nk[t] (and the largest into *kmax); else the records, from off[t] on,
-// and (cpos non-null) the position in C's pattern of each of the tile's
-// ROWS x COLS blocks (-1 where C holds none), so that a product's epilogue
-// finds its output blocks with one load instead of a search.
-template <int ROWS, int COLS, bool COUNT>
-__global__ void k_tile_plan(const int32_t* __restrict__ tiles, const int* __restrict__ ntiles,
+// candidate K's 32 at a time, lane-parallel.  PLAN_COUNT: the number of records
+// into nk[t], their offsets, and the total and the largest for the host;
+// PLAN_RECORDS: the records, from off[t] on; PLAN_BOTH: both in one pass, tile
+// t's records from t nb on.  With the records, the position in C's pattern of
+// each of the tile's ROWS x COLS blocks (-1 where C holds none), so that a
+// product's epilogue finds its output blocks with one load instead of a
+// search.
+// Exclusive scan for longer lists than scan_tail is good for (its one CTA of
+// 256 threads takes 31 us for 20,000 counts, one of 1024 threads 16 us).  CTA b
+// adds up everything before its 4096 counts by itself -- 80 KB from L2 at most
+// for those 20,000 -- so no CTA waits for another.  The total and the
+// longest tile (kmax, nullable) for the host.
+constexpr int TAIL_SCAN = 8192;
+constexpr int SCAN_CHUNK = 4096;
+
+__global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ out, int n,
+                                               int32_t* total, int* kmax, int32_t* host_kmax) {
+  __shared__ int wsum[2][32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, c0 = (int)blockIdx.x * SCAN_CHUNK;
+  int s = 0;
+#pragma unroll 8
+  for (int i = tid; i < c0; i += 1024) s += cnt[i];
+  s = (int)__reduce_add_sync(0xffffffffu, (unsigned)s);
+  if (lane == 0) wsum[0][wid] = s;
+  int v[4], t = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    v[k] = c0 + tid * 4 + k < n ? cnt[c0 + tid * 4 + k] : 0;
+    t += v[k];
+  }
+  int x = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[1][wid] = x;
+  __syncthreads();
+  const int own = wsum[1][lane], base = (int)__reduce_add_sync(0xffffffffu, (unsigned)wsum[0][lane]);
+  int run = base + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < wid ? own : 0)) + x - t;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int i = c0 + tid * 4 + k;
+    if (i < n) out[i] = run;
+    run += v[k];
+    if (i == n - 1) {
+      out[n] = run;
+      if (total) *total = run;
+      if (kmax) *host_kmax = atomicExch(kmax, 0);
+    }
+  }
+}
+
+enum PlanMode { PLAN_COUNT, PLAN_RECORDS, PLAN_BOTH };
+constexpr int PLAN_NT = 256;
+
+template <int ROWS, int COLS, int MODE>
+__global__ void __launch_bounds__(PLAN_NT) k_tile_plan(const int32_t* __restrict__ tiles, const int* __restrict__ ntiles,
                             const int32_t* __restrict__ off, const uint32_t* __restrict__ bm, int nb, int W,
                             const int32_t* __restrict__ mapA, const int32_t* __restrict__ mapB,
                             const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
@@ -783,14 +890,16 @@ __global__ void k_tile_plan(const int32_t* __restrict__ tiles, const int* __rest
                             const int32_t* __restrict__ amap, int32_t* __restrict__ rec, int32_t* __restrict__ nk_out,
                             int* __restrict__ kmax, const int32_t* __restrict__ crp = nullptr,
                             const int32_t* __restrict__ cci = nullptr, int32_t* __restrict__ cpos = nullptr,
-                            const int32_t* __restrict__ bmap = nullptr) {
+                            const int32_t* __restrict__ bmap = nullptr, int nt = 0, int32_t* off_out = nullptr,
+                            unsigned* ticket = nullptr, int32_t* host_kmax = nullptr) {
   static_assert(ROWS * COLS <= 32, "one lane per block of the tile");
   const int64_t t = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (t >= *ntiles) {  // the grid covers an upper bound of the tile count
-    if (COUNT && lane == 0) nk_out[t] = 0;
-    return;
-  }
+  constexpr bool COUNT = MODE == PLAN_COUNT;  // no records
+  // the grid covers an upper bound nt of the tile count
+  const int e0 = MODE == PLAN_COUNT ? 0 : MODE == PLAN_BOTH ? (int)t * nb : (t < *ntiles ? off[t] : 0);
+  int e = e0;
+  if (t < *ntiles) {
   const int I0 = tiles[2 * t] * ROWS, J0 = tiles[2 * t + 1] * COLS;
   if (!COUNT && cpos && lane < ROWS * COLS) {
     const int I = I0 + lane / COLS, J = J0 + lane % COLS;
@@ -802,7 +911,30 @@ __global__ void k_tile_plan(const int32_t* __restrict__ tiles, const int* __rest
     }
     cpos[(size_t)t * (ROWS * COLS) + lane] = pos;
   }
-  int e = COUNT ? 0 : off[t];
+  // op(B)'s copy indices of K, true when any block is stored
+  const auto b_blocks = [&](int K, int (&rb)[COLS]) -> bool {
+    bool any = false;
+    if (mapA) {
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) rb[c] = (J0 + c < nb) ? mapB[(size_t)K * nb + J0 + c] : b_zero;
+    } else {
+      const int hi = brp[K + 1];
+      int q = lower_bound_i32(bci, brp[K], hi, J0);
+#pragma unroll
+      for (int c = 0; c < COLS; ++c) {
+        int idx = b_zero;
+        if (q < hi && bci[q] == J0 + c) idx = q++;
+        rb[c] = idx;
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < COLS; ++c) any |= rb[c] != b_zero;
+    return any;
+  };
+  // 32 words of the K set at a time.  The lanes take the 32 K's of one word
+  // together (one K per word and lane left all but two lanes idle at 64 block
+  // rows).  The records are in the order of the products' K loops, which their
+  // FP32 sums depend on: the first K of every word, then the second, ...
   for (int wbase = 0; wbase < W; wbase += 32) {
     const int w = wbase + lane;
     uint32_t word = 0;
@@ -811,28 +943,41 @@ __global__ void k_tile_plan(const int32_t* __restrict__ tiles, const int* __rest
       for (int r = 0; r < ROWS; ++r)
         if (I0 + r < nb) word |= bm[(size_t)(I0 + r) * W + w];
     }
-    while (__any_sync(0xffffffffu, word != 0u)) {
-      int ra[ROWS], rb[COLS];
-      bool valid = false;
-      if (word != 0u) {
-        const int K = w * 32 + __ffs(word) - 1;
-        word &= word - 1u;
-        if (mapA) {
+    const unsigned nz = __ballot_sync(0xffffffffu, word != 0u);
+    if (!nz) continue;
+    uint32_t ranks = 0;  // this lane's word: bit j set when its j-th K has a record
+    for (unsigned z = nz; z; z &= z - 1u) {
+      const int src = __ffs((int)z) - 1;
+      const uint32_t wd = __shfl_sync(0xffffffffu, word, src);
+      int rb[COLS];
+      const bool rec_here = ((wd >> lane) & 1u) && b_blocks((wbase + src) * 32 + lane, rb);
+      const uint32_t m = __reduce_or_sync(0xffffffffu, rec_here ? 1u << __popc(wd & ((1u << lane) - 1u)) : 0u);
+      if (lane == src) ranks = m;
+    }
+    const int total = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(ranks));
+    if constexpr (!COUNT) {
+      // lane j: the words that have a j-th record, and the records before its j-th ones
+      uint32_t col = 0;
 #pragma unroll
-          for (int c = 0; c < COLS; ++c) rb[c] = (J0 + c < nb) ? mapB[(size_t)K * nb + J0 + c] : b_zero;
-        } else {
-          const int hi = brp[K + 1];
-          int q = lower_bound_i32(bci, brp[K], hi, J0);
+      for (int j = 0; j < 32; ++j) {
+        const uint32_t b = __ballot_sync(0xffffffffu, (ranks >> j) & 1u);
+        if (lane == j) col = b;
+      }
+      int before = __popc(col);
 #pragma unroll
-          for (int c = 0; c < COLS; ++c) {
-            int idx = b_zero;
-            if (q < hi && bci[q] == J0 + c) idx = q++;
-            rb[c] = idx;
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < COLS; ++c) valid |= rb[c] != b_zero;
-        if (!COUNT && valid) {
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, before, o);
+        if (lane >= o) before += y;
+      }
+      before -= __popc(col);
+      for (unsigned z = nz; z; z &= z - 1u) {
+        const int src = __ffs((int)z) - 1;
+        const uint32_t wd = __shfl_sync(0xffffffffu, word, src);
+        const int K = (wbase + src) * 32 + lane, j = __popc(wd & ((1u << lane) - 1u)) & 31;
+        const int pos = __shfl_sync(0xffffffffu, before, j) +
+                        __popc(__shfl_sync(0xffffffffu, col, j) & ((1u << src) - 1u));
+        int ra[ROWS], rb[COLS];
+        if (((wd >> lane) & 1u) && b_blocks(K, rb)) {
           if (mapA) {
 #pragma unroll
             for (int r = 0; r < ROWS; ++r) ra[r] = (I0 + r < nb) ? mapA[(size_t)(I0 + r) * nb + K] : a_zero;
@@ -848,22 +993,36 @@ __global__ void k_tile_plan(const int32_t* __restrict__ tiles, const int* __rest
               ra[r] = idx;
             }
           }
+          int32_t* out = rec + (size_t)(e + pos) * (ROWS + COLS);
+#pragma unroll
+          for (int r = 0; r < ROWS; ++r) out[r] = (amap && ra[r] != a_zero) ? amap[ra[r]] : ra[r];
+#pragma unroll
+          for (int c = 0; c < COLS; ++c) out[ROWS + c] = (bmap && rb[c] != b_zero) ? bmap[rb[c]] : rb[c];
         }
       }
-      const unsigned m = __ballot_sync(0xffffffffu, valid);
-      if (!COUNT && valid) {
-        int32_t* out = rec + (size_t)(e + __popc(m & ((1u << lane) - 1u))) * (ROWS + COLS);
-#pragma unroll
-        for (int r = 0; r < ROWS; ++r) out[r] = (amap && ra[r] != a_zero) ? amap[ra[r]] : ra[r];
-#pragma unroll
-        for (int c = 0; c < COLS; ++c) out[ROWS + c] = (bmap && rb[c] != b_zero) ? bmap[rb[c]] : rb[c];
-      }
-      e += __popc(m);
+    }
+    e += total;
+  }
+  }
+  if constexpr (MODE == PLAN_BOTH) {
+    if (lane == 0 && t < nt) {
+      nk_out[t] = e - e0;
+      off_out[t] = e0;
+      atomicMax(kmax, e - e0);
+    }
+    // the longest tile for the host
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(ticket, 1u) == gridDim.x - 1) {
+      *ticket = 0u;
+      *host_kmax = atomicExch(kmax, 0);
     }
   }
-  if (COUNT && lane == 0) {
-    nk_out[t] = e;
-    if (kmax) atomicMax(kmax, e);
+  if constexpr (COUNT) {
+    if (lane == 0 && t < nt) {
+      nk_out[t] = e;
+      atomicMax(kmax, e);
+    }
   }
 }
 
@@ -877,9 +1036,17 @@ struct Plan {
   int kmax = 0;
 };
 
+// the block pairs a plan counts on the way (once per product)
+struct PairCount {
+  bool upper = false;
+  unsigned long long* pairs = nullptr;
+  unsigned long long* wpairs = nullptr;
+  int w = 0;
+};
+
 template <int ROWS, int COLS>
-static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, bool tA, const View& brows,
-                      const ifac_bsr& B, const ifac_bsr& C, const int32_t* crow, bool want_kmax,
+static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const View& brows, const ifac_bsr& B,
+                      const ifac_bsr& C, const int32_t* crow, const PairCount& pc, bool want_kmax,
                       int kmax_limit = 0, const int32_t* amap = nullptr, const HostRead* extra = nullptr,
                       const int32_t* bmap = nullptr) {
   // amap (nullable): copy index of each op(A) view position, when op(A)'s
@@ -894,103 +1061,103 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, bool 
   Plan P;
   // K sets (bitmap rows of op(A)); dense block-index maps of op(A), op(B)
   // while they stay small, binary searches in the CSR patterns beyond that
-  Buf<uint32_t> bmA = pattern_bitmap(ctx, A, tA);
+  Buf<uint32_t> bmA(ctx, (size_t)nb * W);
   const int64_t nb2 = (int64_t)nb * nb;
   const bool dense_maps = nb2 <= (int64_t)4 << 20;
   Buf<int32_t> imA, imB;
   if (dense_maps) {
     imA = Buf<int32_t>(ctx, nb2);
     imB = Buf<int32_t>(ctx, nb2);
-    k_map_fill<<<cdiv(nb2, 256), 256, 0, ctx->stream>>>(imA.p, nb2, (int32_t)A.nnzb);
-    IFAC_CK_LAUNCH();
-    k_map_fill<<<cdiv(nb2, 256), 256, 0, ctx->stream>>>(imB.p, nb2, (int32_t)B.nnzb);
-    IFAC_CK_LAUNCH();
-    k_map_scatter<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(arows.rp, arows.ci, nb, imA.p);
-    IFAC_CK_LAUNCH();
-    k_map_scatter<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(brows.rp, brows.ci, nb, imB.p);
-    IFAC_CK_LAUNCH();
   }
+  k_plan_rows<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(
+      arows.rp, arows.ci, brows.rp, brows.ci, nb, W, bmA.p, imA.p, imB.p, (int)A.nnzb, (int)B.nnzb, pc.upper ? 1 : 0,
+      pc.pairs, pc.wpairs, pc.w);
+  IFAC_CK_LAUNCH();
   const int ntr = cdiv(nb, ROWS), ntc = cdiv(nb, COLS);
   P.ntot = (int64_t)ntr * ntc;
   if ((int64_t)C.nnzb * 16 < P.ntot) {
     // a sparse C (a banded product): its tiles from its blocks, in C's order
     P.nchunk = (int)C.nnzb;
-    P.tiles = Buf<int32_t>(ctx, (size_t)2 * std::max<int64_t>(C.nnzb, 1));
+    P.tiles = Buf<int32_t>(ctx, (size_t)2 * C.nnzb);
     P.coff = Buf<int32_t>(ctx, (size_t)C.nnzb + 1);
-    Buf<int32_t> own(ctx, (size_t)std::max<int64_t>(C.nnzb, 1));
-    if (C.nnzb) {
-      k_tile_owner<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.row_ptr, C.col_idx, C.nnzb, ROWS, COLS,
-                                                               own.p);
+    Buf<int32_t> own(ctx, (size_t)C.nnzb);
+    const bool tail = C.nnzb <= TAIL_SCAN;
+    k_tile_owner<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.row_ptr, C.col_idx, C.nnzb, ROWS, COLS, own.p,
+                                                             tail ? P.coff.p : nullptr, ctx->ticket);
+    IFAC_CK_LAUNCH();
+    if (!tail) {
+      k_scan<<<cdiv(C.nnzb, SCAN_CHUNK), 1024, 0, ctx->stream>>>(own.p, P.coff.p, (int)C.nnzb, nullptr, nullptr,
+                                                                 nullptr);
       IFAC_CK_LAUNCH();
     }
-    scan_counts(ctx, own.p, P.coff.p, (int)C.nnzb, false);
-    if (C.nnzb) {
-      k_tile_owner_write<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, ROWS, COLS,
-                                                                     P.coff.p, P.tiles.p);
-      IFAC_CK_LAUNCH();
-    }
+    k_tile_owner_write<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, ROWS, COLS, P.coff.p,
+                                                                   P.tiles.p);
+    IFAC_CK_LAUNCH();
+  } else if (P.ntot <= SMALL_TILES && C.nnzb <= SMALL_TILES) {
+    P.nchunk = 0;
+    P.tiles = Buf<int32_t>(ctx, (size_t)2 * P.ntot);
+    P.coff = Buf<int32_t>(ctx, 1);
+    k_tiles_small<ROWS, COLS><<<1, 1024, (size_t)cdiv(P.ntot, 32) * 8, ctx->stream>>>(
+        crow, C.col_idx, (int)C.nnzb, ntr, ntc, P.tiles.p, P.coff.p);
+    IFAC_CK_LAUNCH();
   } else {
     P.nchunk = cdiv(P.ntot, CHUNK);
     Buf<uint8_t> flags(ctx, (size_t)P.ntot);
     Buf<int32_t> ccnt(ctx, P.nchunk);
     P.tiles = Buf<int32_t>(ctx, (size_t)2 * P.ntot);
     P.coff = Buf<int32_t>(ctx, P.nchunk + 1);
-    IFAC_CK(cudaMemsetAsync(flags.p, 0, (size_t)P.ntot, ctx->stream));
-    k_tile_flags<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, ROWS, COLS, ntc, flags.p);
+    k_tile_mark<<<P.nchunk, CHUNK, 0, ctx->stream>>>(C.row_ptr, C.col_idx, nb, ROWS, COLS, ntr, ntc, flags.p, ccnt.p,
+                                                     P.coff.p, ctx->ticket);
     IFAC_CK_LAUNCH();
-    k_tile_count<<<P.nchunk, CHUNK, 0, ctx->stream>>>(flags.p, ntr, ntc, ccnt.p);
-    IFAC_CK_LAUNCH();
-    scan_counts(ctx, ccnt.p, P.coff.p, P.nchunk, false);
     k_tile_write<<<P.nchunk, CHUNK, 0, ctx->stream>>>(flags.p, ntr, ntc, P.coff.p, P.tiles.p);
     IFAC_CK_LAUNCH();
   }
   const int* ntiles = P.coff.p + P.nchunk;
   // the per-tile kernels and arrays are sized by a bound of the tile count
-  // (every tile holds a block of C), not by all ntr x ntc positions
+  // (every tile holds a block of C, which is not empty), not by all ntr x ntc
+  // positions
   const int nt = (int)std::min<int64_t>(P.ntot, C.nnzb);
   P.ntiles = nt;
-  P.tnk = Buf<int32_t>(ctx, (size_t)std::max(nt, 1));
+  P.tnk = Buf<int32_t>(ctx, (size_t)nt);
   P.off = Buf<int32_t>(ctx, (size_t)nt + 1);
-  Buf<int> dk(ctx, 1);
-  IFAC_CK(cudaMemsetAsync(dk.p, 0, sizeof(int), ctx->stream));
-  int64_t total = 0;
-  if (nt > 0) {
-    k_tile_plan<ROWS, COLS, true><<<cdiv((int64_t)nt * 32, 256), 256, 0, ctx->stream>>>(
-        P.tiles.p, ntiles, nullptr, bmA.p, nb, W, dense_maps ? imA.p : nullptr, dense_maps ? imB.p : nullptr,
-        arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb, (int)B.nnzb, nullptr, nullptr, P.tnk.p,
-        want_kmax ? dk.p : nullptr);
+  P.cpos = Buf<int32_t>(ctx, (size_t)nt * (ROWS * COLS));
+  const int pgrid = cdiv((int64_t)nt * 32, PLAN_NT);
+  int* const kmax_dev = reinterpret_cast<int*>(ctx->ticket + 1);
+  // While every tile could have nb K steps within 128 MB, the records are
+  // written in one pass at a fixed stride, and only the longest tile is read
+  // back; a longer list is counted first.
+  if ((int64_t)nt * nb * (ROWS + COLS) <= (int64_t)32 << 20) {
+    P.rec = Buf<int32_t>(ctx, (size_t)nt * nb * (ROWS + COLS));
+    k_tile_plan<ROWS, COLS, PLAN_BOTH><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
+        P.tiles.p, ntiles, nullptr, bmA.p, nb, W, imA.p, imB.p, arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb,
+        (int)B.nnzb, amap, P.rec.p, P.tnk.p, kmax_dev, C.row_ptr, C.col_idx, P.cpos.p, bmap, nt, P.off.p,
+        ctx->ticket, host_word(ctx, HW_KMAX));
     IFAC_CK_LAUNCH();
-    scan_counts(ctx, P.tnk.p, P.off.p, nt, false);
+    if (extra) to_host_many(ctx, {*extra});
+    if (extra || want_kmax) P.kmax = read_word(ctx, HW_KMAX);
+    return P;
   }
-  {
-    // the record count, the longest tile and the caller's extra read-back
-    // behind one synchronisation
-    int32_t tot32 = 0;
-    const HostRead none{nullptr, nullptr, 0};
-    const HostRead ex = extra ? *extra : none;
-    if (ex.bytes) {
-      to_host_many(ctx, {{&tot32, nt > 0 ? (const void*)(P.off.p + nt) : (const void*)dk.p, sizeof(int32_t)},
-                         {&P.kmax, dk.p, sizeof(int)},
-                         ex});
-    } else {
-      to_host_many(ctx, {{&tot32, nt > 0 ? (const void*)(P.off.p + nt) : (const void*)dk.p, sizeof(int32_t)},
-                         {&P.kmax, dk.p, sizeof(int)}});
-    }
-    total = nt > 0 ? tot32 : 0;
-    if (!want_kmax) P.kmax = 0;
-  }
+  k_tile_plan<ROWS, COLS, PLAN_COUNT><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
+      P.tiles.p, ntiles, nullptr, bmA.p, nb, W, imA.p, imB.p, arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb,
+      (int)B.nnzb, nullptr, nullptr, P.tnk.p, kmax_dev, nullptr, nullptr, nullptr, nullptr, nt, nullptr, nullptr,
+      nullptr);
+  IFAC_CK_LAUNCH();
+  k_scan<<<cdiv(nt, SCAN_CHUNK), 1024, 0, ctx->stream>>>(P.tnk.p, P.off.p, nt, host_word(ctx, HW_PLAN), kmax_dev,
+                                                         host_word(ctx, HW_KMAX));
+  IFAC_CK_LAUNCH();
+  // the record count, the longest tile and the caller's extra read-back
+  // behind one synchronisation
+  if (extra) to_host_many(ctx, {*extra});
+  const int64_t total = extra ? *const_cast<volatile int32_t*>(host_word(ctx, HW_PLAN)) : read_word(ctx, HW_PLAN);
+  P.kmax = *const_cast<volatile int32_t*>(host_word(ctx, HW_KMAX));
   if (total > (int64_t)0x7fffffff / (ROWS + COLS))
     fail(IFAC_ERR_TOO_LARGE, "tensor-core product: tile plan exceeds 2^31 entries");
-  if (want_kmax && kmax_limit > 0 && P.kmax > kmax_limit) return P;
+  if (kmax_limit > 0 && P.kmax > kmax_limit) return P;
   P.rec = Buf<int32_t>(ctx, (size_t)std::max<int64_t>(total, 1) * (ROWS + COLS));
-  P.cpos = Buf<int32_t>(ctx, (size_t)std::max(nt, 1) * (ROWS * COLS));
-  if (nt > 0) {
-    k_tile_plan<ROWS, COLS, false><<<cdiv((int64_t)nt * 32, 256), 256, 0, ctx->stream>>>(
-        P.tiles.p, ntiles, P.off.p, bmA.p, nb, W, dense_maps ? imA.p : nullptr, dense_maps ? imB.p : nullptr,
-        arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb, (int)B.nnzb, amap, P.rec.p, nullptr, nullptr,
-        C.row_ptr, C.col_idx, P.cpos.p, bmap);
-    IFAC_CK_LAUNCH();
-  }
+  k_tile_plan<ROWS, COLS, PLAN_RECORDS><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
+      P.tiles.p, ntiles, P.off.p, bmA.p, nb, W, imA.p, imB.p, arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb,
+      (int)B.nnzb, amap, P.rec.p, nullptr, nullptr, C.row_ptr, C.col_idx, P.cpos.p, bmap);
+  IFAC_CK_LAUNCH();
   // the plan kernel has read the maps and the bitmap before they are freed
   // (stream-ordered frees)
   return P;
@@ -1046,7 +1213,7 @@ static CUtensorMap make_map_box(int bs, void* base, int64_t nblk, int inner, int
 template <int ELT, typename V = double>
 static void convert_blocks(ifac_ctx* ctx, int bs, const V* val, const int32_t* src, int64_t nblk, bool tr,
                            void* dst) {
-  const int grid = (int)std::min<int64_t>(nblk, 152 * 16);
+  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
   if (bs == 32) k_convert<ELT, 32, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
   else if (bs == 64) k_convert<ELT, 64, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
   else k_convert<ELT, 128, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
@@ -1054,12 +1221,12 @@ static void convert_blocks(ifac_ctx* ctx, int bs, const V* val, const int32_t* s
 }
 
 // the narrow-tile plan of a block size (tile of 128 / bs x max(64, bs) / bs blocks)
-static Plan band_plan(ifac_ctx* ctx, int bs, const View& arows, const ifac_bsr& A, bool tA, const View& brows,
-                      const ifac_bsr& B, const ifac_bsr& C, const int32_t* crow, int kmax_limit,
-                      const int32_t* amap, const HostRead* extra = nullptr, const int32_t* bmap = nullptr) {
-  if (bs == 32) return make_plan<4, 2>(ctx, arows, A, tA, brows, B, C, crow, true, kmax_limit, amap, extra, bmap);
-  if (bs == 64) return make_plan<2, 1>(ctx, arows, A, tA, brows, B, C, crow, true, kmax_limit, amap, extra, bmap);
-  return make_plan<1, 1>(ctx, arows, A, tA, brows, B, C, crow, true, kmax_limit, amap, extra, bmap);
+static Plan band_plan(ifac_ctx* ctx, int bs, const View& arows, const ifac_bsr& A, const View& brows,
+                      const ifac_bsr& B, const ifac_bsr& C, const int32_t* crow, const PairCount& pc, bool want_kmax,
+                      int kmax_limit, const int32_t* amap, const HostRead* extra = nullptr, const int32_t* bmap = nullptr) {
+  if (bs == 32) return make_plan<4, 2>(ctx, arows, A, brows, B, C, crow, pc, want_kmax, kmax_limit, amap, extra, bmap);
+  if (bs == 64) return make_plan<2, 1>(ctx, arows, A, brows, B, C, crow, pc, want_kmax, kmax_limit, amap, extra, bmap);
+  return make_plan<1, 1>(ctx, arows, A, brows, B, C, crow, pc, want_kmax, kmax_limit, amap, extra, bmap);
 }
 
 // out32: C's values are written as FP32 (C.val holds floats); b32: B's values
@@ -1089,9 +1256,8 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
   const bool hit = ac && ac->conv_elt == ELT;
   if (!hit) {
     la = Buf<uint8_t>(ctx, (size_t)(A.nnzb + 1) * bbytes);
-    IFAC_CK(cudaMemsetAsync(la.p + (size_t)A.nnzb * bbytes, 0, bbytes, ctx->stream));
     Buf<int32_t> asrc;
-    if (A.nnzb) convert_blocks<ELT>(ctx, bs, A.val, value_src(ctx, arows.src, avmap, A.nnzb, asrc), A.nnzb, tA, la.p);
+    convert_blocks<ELT>(ctx, bs, A.val, value_src(ctx, arows.src, avmap, A.nnzb, asrc), A.nnzb, tA, la.p);
     if (ac) {
       ac->conv = std::move(la);
       ac->conv_elt = ELT;
@@ -1100,13 +1266,10 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
   uint8_t* const la_p = ac ? ac->conv.p : la.p;
   if (!bhit && !bsym) {
     lb = Buf<uint8_t>(ctx, (size_t)(B.nnzb + 1) * bbytes);
-    IFAC_CK(cudaMemsetAsync(lb.p + (size_t)B.nnzb * bbytes, 0, bbytes, ctx->stream));
     Buf<int32_t> bsrc;
-    if (B.nnzb) {
-      const int32_t* vs = value_src(ctx, brows.src, bvmap, B.nnzb, bsrc);
-      if (b32) convert_blocks<ELT, float>(ctx, bs, reinterpret_cast<const float*>(B.val), vs, B.nnzb, !tB, lb.p);
-      else convert_blocks<ELT>(ctx, bs, B.val, vs, B.nnzb, !tB, lb.p);
-    }
+    const int32_t* vs = value_src(ctx, brows.src, bvmap, B.nnzb, bsrc);
+    if (b32) convert_blocks<ELT, float>(ctx, bs, reinterpret_cast<const float*>(B.val), vs, B.nnzb, !tB, lb.p);
+    else convert_blocks<ELT>(ctx, bs, B.val, vs, B.nnzb, !tB, lb.p);
   }
   uint8_t* const lb_p = (bhit || bsym) ? bpre->conv.p : lb.p;
   if (bc && !tB && !bhit && !bsym) {  // op(B) = B in its stored order: keep the copy for a later op(A) = B^T
@@ -1115,18 +1278,25 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
     bc->conv_elt = ELT;
     bc->from_b = true;
   }
-  k_count_pairs<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(arows.rp, arows.ci, nb, brows.rp, brows.ci,
-                                                                      upper ? 1 : 0, pairs, nullptr, 0);
-  IFAC_CK_LAUNCH();
+  PairCount pc;
+  pc.upper = upper;
+  pc.pairs = pairs;
   // narrow tiles (gemm_band.cu) for every product at bs 32 and 128, and for
   // the banded ones at bs 64 (no 128 x 64 tile with more than KW K steps);
   // the super-tiles below for the other bs-64 products
   // (the context's schedule can ask for super-tiles only, or narrow tiles up
   // to another K length)
   const int nk_lim = ctx->narrow_kmax < 0 ? KW : ctx->narrow_kmax;
-  if (bs != 64 || nk_lim > 0) {
+  // (no plan is made to find out where a full operand tells: every tile's K
+  // set is then as long as a row of the other, which holds more than nk_lim
+  // blocks on average)
+  const int64_t full = (int64_t)nb * nb;
+  const bool wide = (B.nnzb == full && A.nnzb > (int64_t)nk_lim * nb) ||
+                    (A.nnzb == full && B.nnzb > (int64_t)nk_lim * nb);
+  if (bs != 64 || (nk_lim > 0 && !wide)) {
     const BandShape sh = band_lp_shape(ELT, bs);
-    Plan Pb = band_plan(ctx, bs, arows, A, tA, brows, B, C, crow, bs == 64 ? nk_lim : 0, amap, nullptr, bmap);
+    Plan Pb = band_plan(ctx, bs, arows, A, brows, B, C, crow, pc, bs == 64, bs == 64 ? nk_lim : 0, amap, nullptr, bmap);
+    pc.pairs = nullptr;  // counted
     if (bs != 64 || (Pb.kmax >= 1 && Pb.kmax <= nk_lim)) {
       const CUtensorMap mapA = make_map_bs(ELT, bs, la_p, A.nnzb + 1, sh);
       const CUtensorMap mapB = make_map_bs(ELT, bs, lb_p, B.nnzb + 1, sh);
@@ -1140,7 +1310,7 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
   }
   const CUtensorMap mapA = make_map<ELT>(la_p, A.nnzb + 1);
   const CUtensorMap mapB = make_map<ELT>(lb_p, B.nnzb + 1);
-  Plan P = make_plan<PAIR * TM, Cf::TN>(ctx, arows, A, tA, brows, B, C, crow, false, 0, amap, nullptr, bmap);
+  Plan P = make_plan<PAIR * TM, Cf::TN>(ctx, arows, A, brows, B, C, crow, pc, false, 0, amap, nullptr, bmap);
   static std::atomic<unsigned long long> attr{0};
   if (first_on_device(attr, ctx->device))
     IFAC_CK(cudaFuncSetAttribute(k_gemm_tc<ELT>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM_BYTES));
@@ -1478,10 +1648,16 @@ __global__ void __launch_bounds__(256) k_split(const double* __restrict__ val, c
   constexpr int BSZ = B * B;
   __shared__ double tile[32][33];  // transposed views: 32 x 32 sub-blocks
   const size_t slice_stride = (size_t)(nblk + 1) * BSZ;
-  for (int64_t qb = blockIdx.x; qb < nblk; qb += gridDim.x) {
+  for (int64_t qb = blockIdx.x; qb <= nblk; qb += gridDim.x) {
+    __nv_bfloat16* d = dst + (size_t)qb * BSZ;
+    if (qb == nblk) {  // the zero block of every slice
+      for (int k = 0; k < ns; ++k)
+        for (int e = threadIdx.x; e < BSZ / 2; e += blockDim.x)
+          *reinterpret_cast<uint32_t*>(d + (size_t)k * slice_stride + 2 * e) = 0u;
+      continue;
+    }
     const double* s = val + (size_t)(src ? src[qb] : qb) * BSZ;
     const int* se = sexp + (size_t)sblk[qb] * B;
-    __nv_bfloat16* d = dst + (size_t)qb * BSZ;
     if (!tr) {
       for (int e2 = threadIdx.x; e2 < BSZ / 2; e2 += blockDim.x) {
         const int e = 2 * e2, r = e / B;
@@ -1510,7 +1686,7 @@ __global__ void __launch_bounds__(256) k_split(const double* __restrict__ val, c
 
 static void split_blocks(ifac_ctx* ctx, int bs, const double* val, const int32_t* src, int64_t nblk, bool tr,
                          const int32_t* sblk, const int* sexp, int ns, void* dst) {
-  const int grid = (int)std::min<int64_t>(nblk, 152 * 16);
+  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
   __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(dst);
   if (bs == 32) k_split<32><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, sblk, sexp, ns, d);
   else if (bs == 64) k_split<64><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, sblk, sexp, ns, d);
@@ -2259,24 +2435,17 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   // slices: row scale block of an op(A) entry is its CSR row; of an op(B) entry its CSR column
   const size_t bbytes = (size_t)bs * bs * 2;
   Buf<uint8_t> la, lb(ctx, (size_t)ns * (B.nnzb + 1) * bbytes);
-  for (int k = 0; k < ns; ++k)
-    IFAC_CK(cudaMemsetAsync(lb.p + ((size_t)k * (B.nnzb + 1) + B.nnzb) * bbytes, 0, bbytes, ctx->stream));
   if (!hit) {
     la = Buf<uint8_t>(ctx, (size_t)nsa * (A.nnzb + 1) * bbytes);
-    for (int k = 0; k < nsa; ++k)
-      IFAC_CK(cudaMemsetAsync(la.p + ((size_t)k * (A.nnzb + 1) + A.nnzb) * bbytes, 0, bbytes, ctx->stream));
-    if (A.nnzb) {
-      Buf<int32_t> arow(ctx, A.nnzb);
-      expand_rows(ctx, arows.rp, nb, arow.p);
-      split_blocks(ctx, bs, A.val, value_src(ctx, arows.src, avmap, A.nnzb, asrc), A.nnzb, tA, arow.p, sige.p, nsa,
-                   la.p);
-    }
+    Buf<int32_t> arow(ctx, A.nnzb);
+    expand_rows(ctx, arows.rp, nb, arow.p);
+    split_blocks(ctx, bs, A.val, value_src(ctx, arows.src, avmap, A.nnzb, asrc), A.nnzb, tA, arow.p, sige.p, nsa,
+                 la.p);
   }
   uint8_t* const la_p = hit ? ac->split.p : la.p;
   const int* const sige_p = hit ? ac->sexp.p : sige.p;
   const int* const taue_p = taue.p;
-  if (B.nnzb)
-    split_blocks(ctx, bs, B.val, value_src(ctx, brows.src, bvmap, B.nnzb, bsrc), B.nnzb, !tB, brows.ci, taue.p, ns,
+  split_blocks(ctx, bs, B.val, value_src(ctx, brows.src, bvmap, B.nnzb, bsrc), B.nnzb, !tB, brows.ci, taue.p, ns,
                  lb.p);
   // one tensor map over all slices of each operand (slice s at row s (nnzb + 1) bs)
   if ((int64_t)ns * (std::max(A.nnzb, B.nnzb) + 1) * bs > (int64_t)0x7fffffff)
@@ -2296,20 +2465,22 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   const int nk_lim = ctx->narrow_kmax_split < 0 ? INT_MAX : ctx->narrow_kmax_split;
   Plan Pb;
   bool banded = bs != 64;
+  // block pairs, and block pairs times the ns (ns + 1) / 2 slice pairs
+  PairCount pc;
+  pc.upper = upper;
+  pc.pairs = pairs;
+  pc.wpairs = pairs + 1;
+  pc.w = ns * (ns + 1) / 2;
   if (bs != 64 || nk_lim > 0) {
-    Pb = band_plan(ctx, bs, arows, A, tA, brows, B, C, crow, bs == 64 && nk_lim < INT_MAX ? nk_lim : 0, amap,
+    Pb = band_plan(ctx, bs, arows, A, brows, B, C, crow, pc, true, bs == 64 && nk_lim < INT_MAX ? nk_lim : 0, amap,
                    &l1read);
+    pc.pairs = pc.wpairs = nullptr;  // counted
     if (bs == 64) banded = Pb.kmax >= 1 && Pb.kmax <= nk_lim;
   } else {
     to_host(ctx, l1h, l1.p, sizeof(l1h));
   }
   Plan P;
-  if (!banded) P = make_plan<PAIR * TM, Cf::TN>(ctx, arows, A, tA, brows, B, C, crow, true, 0, amap);
-  // block pairs, and block pairs times the ns (ns + 1) / 2 slice pairs
-  k_count_pairs<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(arows.rp, arows.ci, nb, brows.rp, brows.ci,
-                                                                      upper ? 1 : 0, pairs, pairs + 1,
-                                                                      ns * (ns + 1) / 2);
-  IFAC_CK_LAUNCH();
+  if (!banded) P = make_plan<PAIR * TM, Cf::TN>(ctx, arows, A, brows, B, C, crow, pc, true, 0, amap);
   const int kmax = banded ? Pb.kmax : P.kmax;
   if (hit) {
     l1h[0] = ac->l1;

@@ -37,8 +37,11 @@ struct ifac_ctx {
   bool profile = false;
   std::vector<cudaEvent_t> events;
   size_t events_used = 0;
-  // small pinned host buffer for scalar read-backs
+  // small pinned host buffer for scalar read-backs, and behind it the words
+  // that kernels write for the host (host_word)
   void* pinned = nullptr;
+  int32_t* host_words = nullptr;
+  unsigned* ticket = nullptr;  // device word of scan_tail, zero between launches
   // device words: [0] error flag set by bounded waits that expired;
   // counters [1] FP64 and [2] tensor-core block pairs of the current call
   int* dev_err = nullptr;
@@ -153,10 +156,14 @@ struct HostRead {
 };
 void to_host_many(ifac_ctx* ctx, std::initializer_list<HostRead> reads);
 
+// Words a kernel writes for the host (mapped pinned memory), read after the
+// stream is synchronised.
+enum HostWord { HW_NNZ = 0, HW_KEPT, HW_PLAN, HW_KMAX, HW_COUNT };
+inline int32_t* host_word(ifac_ctx* ctx, HostWord w) { return ctx->host_words + w; }
+int32_t read_word(ifac_ctx* ctx, HostWord w);  // synchronises the stream
+
 // ---- pattern utilities (pattern.cu) ----
 int words_per_row(int nb);
-// exclusive scan of in[0..n) into out[0..n], out[n] = total; returns total (syncs)
-int64_t scan_counts(ifac_ctx* ctx, const int32_t* in, int32_t* out, int n, bool want_total);
 // CSR view of op(X): rows of X^T with the index of the source block of X.
 struct View {
   const int32_t* rp = nullptr;
@@ -165,19 +172,15 @@ struct View {
   Buf<int32_t> own_rp, own_ci, own_src;
 };
 View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans);
-// Bitmap (nb x W words) of the pattern of op(A): bit (r, c) set when op(A)_rc is stored.
-Buf<uint32_t> pattern_bitmap(ifac_ctx* ctx, const ifac_bsr& A, bool trans);
 // Row pattern from a bitmap: allocates and fills rp[nb+1], ci[nnzb].
 struct Pattern {
   Buf<int32_t> rp, ci, row;
   int64_t nnzb = 0;
 };
-// known_nnzb >= 0: the number of set bits is known (e.g. a transposed
-// pattern), so it is not read back from the device
-Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb, int64_t known_nnzb = -1);
+Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb);
 // Symbolic product pattern of op(A) op(B); upper: only the blocks (I, J)
 // with J >= I.
-Pattern product_pattern(ifac_ctx* ctx, const View& arows, const ifac_bsr& B, bool transB, int nb,
+Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const ifac_bsr& B, bool transB, int nb,
                         bool upper = false);
 // Union pattern of A, B (nullable) and the diagonal (if diag).
 Pattern union_pattern(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr* B, bool diag);
@@ -187,9 +190,11 @@ Pattern sym_pattern(ifac_ctx* ctx, const ifac_bsr& U, const ifac_bsr* B, bool di
 void expand_rows(ifac_ctx* ctx, const int32_t* rp, int nb, int32_t* row);
 // Keep blocks with !(norm < tau) of an (uncompacted) matrix; returns the compacted one.
 // nocopy: the kept blocks stay where they are (the result's vmap points to them).
-Mat compact(ifac_ctx* ctx, Mat&& full, const int32_t* row, double tau, bool nocopy = false);
-// Keep blocks selected by a per-block mask (1 keep / 0 drop).
-Mat select_blocks(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* row, const uint8_t* keep);
+Mat compact(ifac_ctx* ctx, Mat&& full, double tau, bool nocopy = false);
+// Keep blocks selected by a per-block mask (1 keep / 0 drop), or by the same
+// test of their norms.
+Mat select_blocks(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep);
+Mat select_norms(ifac_ctx* ctx, const ifac_bsr& A, double tau);
 
 // ---- numeric kernels ----
 // FP64 numeric block product into the pattern (rp/ci/row) of C; writes

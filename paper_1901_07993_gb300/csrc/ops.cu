@@ -30,7 +30,7 @@ Mat gemm(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, 
   if (b32 && !lowp) fail(IFAC_ERR_INVALID, "FP32 operand values: TF32/BF16 products only");
   out32 = out32 && lowp && nocopy;  // compaction copies would move FP64 values
   View arows = view_rows(ctx, A, tA);
-  Pattern P = product_pattern(ctx, arows, B, tB, nb, upper);
+  Pattern P = product_pattern(ctx, arows, A.nnzb, B, tB, nb, upper);
   Mat C(ctx);
   C.m.n = A.n;
   C.m.bs = A.bs;
@@ -61,7 +61,7 @@ Mat gemm(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, 
                     ctx->dev_pairs + (prec == IFAC_FP64_SPLIT ? 2 : 1), acache, bcache, bpre, avmap, bvmap, out32,
                     b32);
   }
-  Mat R = compact(ctx, std::move(C), P.row.p, tau, nocopy);
+  Mat R = compact(ctx, std::move(C), tau, nocopy);
   R.f32 = out32;
   ctx->products += 1;
   return R;
@@ -139,11 +139,6 @@ Mat add(ifac_ctx* ctx, double alpha, const ifac_bsr& A, double beta, const ifac_
   return C;
 }
 
-__global__ void k_keep_norm(const double* __restrict__ norms, int64_t n, double tau, uint8_t* __restrict__ keep) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p < n) keep[p] = (norms[p] < tau) ? 0 : 1;
-}
-
 Mat truncate(ifac_ctx* ctx, const ifac_bsr& A, double tau) {
   Buf<double> tmp;
   const double* norms = A.norms;
@@ -154,12 +149,7 @@ Mat truncate(ifac_ctx* ctx, const ifac_bsr& A, double tau) {
   }
   ifac_bsr a = A;
   a.norms = const_cast<double*>(norms);
-  Buf<uint8_t> keep(ctx, A.nnzb);
-  if (A.nnzb) {
-    k_keep_norm<<<cdiv(A.nnzb, 256), 256, 0, ctx->stream>>>(norms, A.nnzb, tau, keep.p);
-    IFAC_CK_LAUNCH();
-  }
-  return select_blocks(ctx, a, nullptr, keep.p);
+  return select_norms(ctx, a, tau);
 }
 
 Mat copy_mat(ifac_ctx* ctx, const ifac_bsr& A) {

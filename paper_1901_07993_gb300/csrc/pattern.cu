@@ -7,157 +7,310 @@
 // blocks are stored); the pattern of a sum is the OR of the operands' bitmaps.
 // Enumerating set bits in word order yields sorted column lists directly, so
 // no sort is needed.  Row pointers come from an exclusive scan of popcounts.
+//
+// What bounds it is launches: at a few thousand rows each of these kernels
+// runs for 2 us.  So a small pattern (rule_small) is one CTA from the bitmaps
+// in shared memory to the column lists, and a larger one is a bitmap kernel, a
+// count kernel whose last CTA scans (scan_tail) and a fill kernel; totals
+// reach the host through mapped memory.  Before, each was up to nine launches
+// (clear, scatter, OR, count, scan, copy to the host, fill).  FP64 product of
+// the 1000-row chain 171 -> 119 us; refinement of the 4096-row chain 5.0 -> 3.5
+// ms (500 launches -> 162).
 #include "internal.cuh"
+#include "scan_tail.cuh"
 
 namespace ifac {
 
 int words_per_row(int nb) { return (nb + 31) / 32; }
 
-// ---------------------------------------------------------------------------
-// exclusive scan of n int32 (single CTA): each thread takes 16 consecutive
-// entries (loads issued together), the CTA scans the thread totals, carries
-// between chunks of 16 blockDim entries; out[n] = the total
-// ---------------------------------------------------------------------------
-__global__ void k_scan_excl(const int32_t* __restrict__ in, int32_t* __restrict__ out, int n) {
-  constexpr int K = 16;
+namespace {
+
+constexpr int NT = 256;         // threads of the row kernels (one warp per block row)
+constexpr int SMALL_NB = 512;   // block rows of a one-CTA pattern: two bitmaps of 32 KB
+constexpr int SMALL_IN = 16384;  // and blocks of an operand: 64 KB of staged lists
+
+// one operand's pattern as a bitmap source, transposed or not
+struct Source {
+  const int32_t* rp;
+  const int32_t* ci;
+  int trans;
+};
+
+struct Job {
+  Source s[3];
+  int nsrc;
+  int diag;             // the diagonal blocks as well
+  int nb, W;
+  const int32_t* arp;   // a product: rows of op(A) (the sources are op(B)); null: the union of the sources
+  const int32_t* aci;
+  int upper;            // only columns >= the row
+  int32_t* rp;
+  int32_t* ci;
+  int32_t* row;
+  // a transposed view: the position of each entry's block in the source matrix
+  const int32_t* frp;
+  const int32_t* fci;
+  int32_t* src;
+  int32_t* total;       // host word, or null
+};
+
+__device__ __forceinline__ uint32_t upper_bits(uint32_t v, int row, int w) {
+  if (w < (row >> 5)) return 0u;
+  return w == (row >> 5) ? v & ~((1u << (row & 31)) - 1u) : v;
+}
+
+// entry (r, c) of A^T: the position of block (c, r) in A's sorted row c
+__device__ __forceinline__ int find_src(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int r, int c) {
+  int lo = rp[c], hi = rp[c + 1];
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (ci[mid] < r) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// the set bits of word w of row r at positions pos, pos + 1, ...
+__device__ __forceinline__ void emit(const Job& j, uint32_t word, int r, int w, int pos) {
+  while (word) {
+    const int c = w * 32 + __ffs((int)word) - 1;
+    j.ci[pos] = c;
+    if (j.row) j.row[pos] = r;
+    ++pos;
+    word &= word - 1;
+  }
+}
+
+// A whole small pattern in one CTA.  Every phase takes all rows at once (a
+// group of 1024 / nb threads each), and a product's op(A) lists are staged in
+// shared memory first: a loop over rows would pay the latency of global memory
+// for each (nb = 512: 20 us that way).
+__global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
+  extern __shared__ uint32_t sh[];
   __shared__ int32_t wsum[32];
-  __shared__ int32_t carry;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if (threadIdx.x == 0) carry = 0;
+  const int nw = j.nb * j.W;
+  uint32_t* bm = sh;                                // [nb * W] the sources
+  int32_t* off = reinterpret_cast<int32_t*>(bm + nw);  // [nb + 1]
+  uint32_t* out = j.arp ? reinterpret_cast<uint32_t*>(off + j.nb + 1) : bm;  // [nb * W] the pattern
+  int32_t* arp = reinterpret_cast<int32_t*>(out + nw);  // product: [nb + 1], [nnza]
+  int32_t* aci = arp + j.nb + 1;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int lg = 5;  // log2 of the threads that share a row
+  while ((j.nb << lg) > 1024 && lg > 0) --lg;
+  const int G = 1 << lg, grow = tid >> lg, glane = tid & (G - 1);
+  for (int i = tid; i < nw; i += 1024) bm[i] = 0u;
+  if (j.arp) {
+    for (int i = tid; i <= j.nb; i += 1024) arp[i] = j.arp[i];
+    for (int i = tid; i < nnza; i += 1024) aci[i] = j.aci[i];
+  }
   __syncthreads();
-  for (int base = 0; base < n; base += blockDim.x * K) {
-    const int i0 = base + threadIdx.x * K;
-    int v[K];
-    int t = 0;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      v[k] = (i0 + k < n) ? in[i0 + k] : 0;
-      t += v[k];
+  if (grow < j.nb) {
+    for (int k = 0; k < j.nsrc; ++k) {
+      const int p1 = j.s[k].rp[grow + 1];
+      for (int p = j.s[k].rp[grow] + glane; p < p1; p += G) {
+        const int c = j.s[k].ci[p], br = j.s[k].trans ? c : grow, bc = j.s[k].trans ? grow : c;
+        atomicOr(&bm[br * j.W + (bc >> 5)], 1u << (bc & 31));
+      }
     }
-    int x = t;
+    if (j.diag && glane == 0) atomicOr(&bm[grow * j.W + (grow >> 5)], 1u << (grow & 31));
+  }
+  __syncthreads();
+  if (j.arp) {
+    for (int i = tid; i < nw; i += 1024) {
+      const int r = i / j.W, w = i % j.W;
+      uint32_t acc = 0;
+      for (int p = arp[r]; p < arp[r + 1]; ++p) acc |= bm[aci[p] * j.W + w];
+      out[i] = j.upper ? upper_bits(acc, r, w) : acc;
+    }
+    __syncthreads();
+  }
+  int c = 0;
+  if (tid < j.nb)
+    for (int w = 0; w < j.W; ++w) c += __popc(out[tid * j.W + w]);
+  int x = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) wsum[wid] = x;
+  __syncthreads();
+  int run = x - c;
+  for (int w = 0; w < wid; ++w) run += wsum[w];
+  if (tid < j.nb) {
+    off[tid] = run;
+    j.rp[tid] = run;
+    if (tid == j.nb - 1) {
+      j.rp[j.nb] = run + c;
+      if (j.total) *j.total = run + c;
+    }
+  }
+  __syncthreads();
+  const auto before = [&](int r, int w) {  // set bits of row r in the words before w
+    int n = off[r];
+    for (int v = 0; v < w; ++v) n += __popc(out[r * j.W + v]);
+    return n;
+  };
+  for (int i = tid; i < nw; i += 1024) {
+    const uint32_t word = out[i];
+    if (word) emit(j, word, i / j.W, i % j.W, before(i / j.W, i % j.W));
+  }
+  if (j.src && grow < j.nb) {  // (a transposed view: each stored block finds its own place)
+    const int p1 = j.frp[grow + 1];
+    for (int p = j.frp[grow] + glane; p < p1; p += G) {
+      const int r = j.fci[p], w = grow >> 5;
+      j.src[before(r, w) + __popc(out[r * j.W + w] & ((1u << (grow & 31)) - 1u))] = p;
+    }
+  }
+}
+
+// the sources' bits in a cleared bitmap (one warp per block row)
+__global__ void __launch_bounds__(NT) k_scatter(Job j, uint32_t* __restrict__ bm) {
+  const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row >= j.nb) return;
+  for (int k = 0; k < j.nsrc; ++k)
+    for (int p = j.s[k].rp[row] + lane; p < j.s[k].rp[row + 1]; p += 32) {
+      const int c = j.s[k].ci[p], r = j.s[k].trans ? c : row, col = j.s[k].trans ? row : c;
+      atomicOr(&bm[(size_t)r * j.W + (col >> 5)], 1u << (col & 31));
+    }
+  if (j.diag && lane == 0) atomicOr(&bm[(size_t)row * j.W + (row >> 5)], 1u << (row & 31));
+}
+
+// the product's rows, out[I] = OR over K in row I of op(A) of bm[K] (or bm
+// itself), their counts and the row pointers
+__global__ void __launch_bounds__(NT) k_rows_scan(Job j, const uint32_t* __restrict__ bm, uint32_t* __restrict__ out,
+                                                  int32_t* __restrict__ cnt, unsigned* __restrict__ ticket) {
+  const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row < j.nb) {
+    int c = 0;
+    const int p0 = j.arp ? j.arp[row] : 0, p1 = j.arp ? j.arp[row + 1] : 0;
+    for (int w = lane; w < j.W; w += 32) {
+      uint32_t acc = 0;
+      if (j.arp) {
+        for (int p = p0; p < p1; ++p) acc |= bm[(size_t)j.aci[p] * j.W + w];
+        if (j.upper) acc = upper_bits(acc, row, w);
+        out[(size_t)row * j.W + w] = acc;
+      } else {
+        acc = bm[(size_t)row * j.W + w];
+      }
+      c += __popc(acc);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) cnt[row] = c;
+  }
+  scan_tail<NT>(cnt, j.rp, j.nb, ticket, j.total);
+}
+
+// enumerate the set bits of each row in increasing column (warp per row)
+__global__ void __launch_bounds__(NT) k_row_fill(Job j, const uint32_t* __restrict__ bm) {
+  const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row >= j.nb) return;
+  int pos = j.rp[row];
+  for (int base = 0; base < j.W; base += 32) {
+    const int w = base + lane;
+    const uint32_t word = w < j.W ? bm[(size_t)row * j.W + w] : 0u;
+    const int c = __popc(word);
+    int x = c;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, x, o);
       if (lane >= o) x += y;
     }
-    if (lane == 31) wsum[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-      int sw = (lane < nw) ? wsum[lane] : 0;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, sw, o);
-        if (lane >= o) sw += y;
-      }
-      wsum[lane] = sw;
-    }
-    __syncthreads();
-    int run = carry + (wid > 0 ? wsum[wid - 1] : 0) + x - t;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      if (i0 + k < n) out[i0 + k] = run;
-      run += v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = run;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[n] = carry;
-}
-
-int64_t scan_counts(ifac_ctx* ctx, const int32_t* in, int32_t* out, int n, bool want_total) {
-  k_scan_excl<<<1, 1024, 0, ctx->stream>>>(in, out, n);
-  IFAC_CK_LAUNCH();
-  if (!want_total) return -1;
-  int32_t tot = 0;
-  to_host(ctx, &tot, out + n, sizeof(int32_t));
-  return tot;
-}
-
-// ---------------------------------------------------------------------------
-// bitmaps
-// ---------------------------------------------------------------------------
-// one warp per block row of A; sets bit (r, c) of op(A)
-__global__ void k_bitmap(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int nb, int W,
-                         int trans, uint32_t* __restrict__ bm) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= nb) return;
-  for (int p = rp[row] + lane; p < rp[row + 1]; p += 32) {
-    int c = ci[p];
-    int r = trans ? c : row, col = trans ? row : c;
-    atomicOr(&bm[(size_t)r * W + (col >> 5)], 1u << (col & 31));
-  }
-}
-
-__global__ void k_bitmap_diag(int nb, int W, uint32_t* __restrict__ bm) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < nb) bm[(size_t)i * W + (i >> 5)] |= 1u << (i & 31);
-}
-
-Buf<uint32_t> pattern_bitmap(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
-  int W = words_per_row(A.nb);
-  Buf<uint32_t> bm(ctx, (size_t)A.nb * W);
-  IFAC_CK(cudaMemsetAsync(bm.p, 0, sizeof(uint32_t) * (size_t)A.nb * W, ctx->stream));
-  if (A.nnzb > 0) {
-    k_bitmap<<<cdiv((int64_t)A.nb * 32, 256), 256, 0, ctx->stream>>>(A.row_ptr, A.col_idx, A.nb, W, trans ? 1 : 0, bm.p);
-    IFAC_CK_LAUNCH();
-  }
-  return bm;
-}
-
-// per-row popcount (warp per row)
-__global__ void k_row_popc(const uint32_t* __restrict__ bm, int nb, int W, int32_t* __restrict__ cnt) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= nb) return;
-  int c = 0;
-  for (int w = lane; w < W; w += 32) c += __popc(bm[(size_t)row * W + w]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) cnt[row] = c;
-}
-
-// enumerate set bits of each row in increasing column (warp per row)
-__global__ void k_row_fill(const uint32_t* __restrict__ bm, int nb, int W, const int32_t* __restrict__ rp,
-                           int32_t* __restrict__ ci, int32_t* __restrict__ row_of) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= nb) return;
-  int pos = rp[row];
-  for (int base = 0; base < W; base += 32) {
-    int w = base + lane;
-    uint32_t word = (w < W) ? bm[(size_t)row * W + w] : 0u;
-    int c = __popc(word);
-    int x = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    int off = pos + x - c;
-    while (word) {
-      int b = __ffs(word) - 1;
-      ci[off] = w * 32 + b;
-      if (row_of) row_of[off] = row;
-      ++off;
-      word &= word - 1;
-    }
+    emit(j, word, row, w, pos + x - c);
+    if (j.src)
+      for (uint32_t u = word, q = (uint32_t)(pos + x - c); u; u &= u - 1u, ++q)
+        j.src[q] = find_src(j.frp, j.fci, row, w * 32 + __ffs((int)u) - 1);
     pos += __shfl_sync(0xffffffffu, x, 31);
   }
 }
 
-Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb, int64_t known_nnzb) {
-  int W = words_per_row(nb);
+int row_grid(int nb) { return cdiv((int64_t)nb * 32, NT); }
+
+// One CTA does a pattern of up to SMALL_NB block rows whose operands hold up
+// to 16,384 blocks and whose result at most 32,768 (about 10 us there: what
+// three kernels with all their warps take); beyond that the rows go over the
+// whole GPU.
+bool rule_small(int nb, int64_t in_blocks, int64_t out_bound) {
+  return nb <= SMALL_NB && in_blocks <= SMALL_IN && out_bound <= 32768;
+}
+
+void launch_small(ifac_ctx* ctx, const Job& j, int64_t nnza) {
+  const size_t nw = (size_t)j.nb * j.W, smem = 4 * (nw + j.nb + 1 + (j.arp ? nw + j.nb + 1 + (size_t)nnza : 0));
+  if (smem > 48 * 1024)  // set at every such launch, so that no other thread can launch before it
+    IFAC_CK(cudaFuncSetAttribute(k_pattern_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 4 * (2 * (SMALL_NB * (SMALL_NB / 32) + SMALL_NB + 1) + SMALL_IN)));
+  k_pattern_small<<<1, 1024, smem, ctx->stream>>>(j, (int)nnza);
+  IFAC_CK_LAUNCH();
+}
+
+// The pattern of a job: known >= 0 the number of its blocks where the host
+// knows it (a transposed view), so nothing is read back; guess what it will
+// be about, cap its bound.
+Pattern run_job(ifac_ctx* ctx, Job j, int64_t in_blocks, int64_t guess, int64_t cap, int64_t known,
+                Buf<int32_t>* src, int64_t nnza = 0) {
+  Pattern P;
+  j.W = words_per_row(j.nb);
+  P.rp = Buf<int32_t>(ctx, j.nb + 1);
+  j.rp = P.rp.p;
+  j.total = known < 0 ? host_word(ctx, HW_NNZ) : nullptr;
+  const auto alloc = [&](int64_t n) {
+    P.ci = Buf<int32_t>(ctx, n);
+    P.row = Buf<int32_t>(ctx, n);
+    j.ci = P.ci.p;
+    j.row = P.row.p;
+    if (src) {
+      *src = Buf<int32_t>(ctx, n);
+      j.src = src->p;
+    }
+  };
+  if (rule_small(j.nb, in_blocks, guess)) {
+    alloc(cap);
+    launch_small(ctx, j, nnza);
+    P.nnzb = known >= 0 ? known : read_word(ctx, HW_NNZ);
+    return P;
+  }
+  const size_t words = (size_t)j.nb * j.W;
+  Buf<uint32_t> bm(ctx, words), rows(ctx, j.arp ? words : 1);
+  Buf<int32_t> cnt(ctx, j.nb);
+  IFAC_CK(cudaMemsetAsync(bm.p, 0, sizeof(uint32_t) * words, ctx->stream));
+  k_scatter<<<row_grid(j.nb), NT, 0, ctx->stream>>>(j, bm.p);
+  IFAC_CK_LAUNCH();
+  k_rows_scan<<<row_grid(j.nb), NT, 0, ctx->stream>>>(j, bm.p, rows.p, cnt.p, ctx->ticket);
+  IFAC_CK_LAUNCH();
+  P.nnzb = known >= 0 ? known : read_word(ctx, HW_NNZ);
+  alloc(P.nnzb);
+  if (P.nnzb > 0) {
+    k_row_fill<<<row_grid(j.nb), NT, 0, ctx->stream>>>(j, j.arp ? rows.p : bm.p);
+    IFAC_CK_LAUNCH();
+  }
+  return P;
+}
+
+void add_source(Job& j, const int32_t* rp, const int32_t* ci, int64_t nnzb, bool trans) {
+  if (nnzb > 0) j.s[j.nsrc++] = Source{rp, ci, trans ? 1 : 0};
+}
+
+}  // namespace
+
+Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb) {
+  Job j{};
+  j.nb = nb;
+  j.W = words_per_row(nb);
   Pattern P;
   P.rp = Buf<int32_t>(ctx, nb + 1);
+  j.rp = P.rp.p;
+  j.total = host_word(ctx, HW_NNZ);
   Buf<int32_t> cnt(ctx, nb);
-  int grid = cdiv((int64_t)nb * 32, 256);
-  k_row_popc<<<grid, 256, 0, ctx->stream>>>(bm, nb, W, cnt.p);
+  k_rows_scan<<<row_grid(nb), NT, 0, ctx->stream>>>(j, bm, nullptr, cnt.p, ctx->ticket);
   IFAC_CK_LAUNCH();
-  P.nnzb = scan_counts(ctx, cnt.p, P.rp.p, nb, known_nnzb < 0);
-  if (known_nnzb >= 0) P.nnzb = known_nnzb;
+  P.nnzb = read_word(ctx, HW_NNZ);
   P.ci = Buf<int32_t>(ctx, P.nnzb);
   P.row = Buf<int32_t>(ctx, P.nnzb);
+  j.ci = P.ci.p;
+  j.row = P.row.p;
   if (P.nnzb > 0) {
-    k_row_fill<<<grid, 256, 0, ctx->stream>>>(bm, nb, W, P.rp.p, P.ci.p, P.row.p);
+    k_row_fill<<<row_grid(nb), NT, 0, ctx->stream>>>(j, bm);
     IFAC_CK_LAUNCH();
   }
   return P;
@@ -166,26 +319,16 @@ Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb, int64_t k
 // ---------------------------------------------------------------------------
 // transposed views
 // ---------------------------------------------------------------------------
-// entry q of A^T (row c = row_t[q], column r = ci_t[q]) comes from block (r, c)
-// of A, found by binary search in A's sorted row r.
+// out[q] for block q = (row[q], ci[q]) of A: the position of its transpose
 __global__ void k_find_src(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci, int64_t nnz,
-                           const int32_t* __restrict__ row_t, const int32_t* __restrict__ ci_t,
-                           int32_t* __restrict__ src) {
-  int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (q >= nnz) return;
-  int r = ci_t[q], c = row_t[q];
-  int lo = rp[r], hi = rp[r + 1];
-  while (lo < hi) {
-    int mid = (lo + hi) >> 1;
-    if (ci[mid] < c) lo = mid + 1;
-    else hi = mid;
-  }
-  src[q] = lo;
+                           const int32_t* __restrict__ row, int32_t* __restrict__ out) {
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (q < nnz) out[q] = find_src(rp, ci, row[q], ci[q]);
 }
 
 void transposed_positions(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* row, int32_t* out) {
   if (A.nnzb == 0) return;
-  k_find_src<<<cdiv(A.nnzb, 256), 256, 0, ctx->stream>>>(A.row_ptr, A.col_idx, A.nnzb, row, A.col_idx, out);
+  k_find_src<<<cdiv(A.nnzb, 256), 256, 0, ctx->stream>>>(A.row_ptr, A.col_idx, A.nnzb, row, out);
   IFAC_CK_LAUNCH();
 }
 
@@ -197,13 +340,12 @@ View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
     v.src = nullptr;
     return v;
   }
-  Buf<uint32_t> bm = pattern_bitmap(ctx, A, true);
-  Pattern P = pattern_from_bitmap(ctx, bm.p, A.nb, A.nnzb);  // A^T has A's blocks
-  v.own_src = Buf<int32_t>(ctx, P.nnzb);
-  if (P.nnzb > 0) {
-    k_find_src<<<cdiv(P.nnzb, 256), 256, 0, ctx->stream>>>(A.row_ptr, A.col_idx, P.nnzb, P.row.p, P.ci.p, v.own_src.p);
-    IFAC_CK_LAUNCH();
-  }
+  Job j{};
+  j.nb = A.nb;
+  add_source(j, A.row_ptr, A.col_idx, A.nnzb, true);
+  j.frp = A.row_ptr;
+  j.fci = A.col_idx;
+  Pattern P = run_job(ctx, j, A.nnzb, A.nnzb, A.nnzb, A.nnzb, &v.own_src);  // A^T has A's blocks
   v.own_rp = std::move(P.rp);
   v.own_ci = std::move(P.ci);
   v.rp = v.own_rp.p;
@@ -215,78 +357,41 @@ View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
 // ---------------------------------------------------------------------------
 // product and union patterns
 // ---------------------------------------------------------------------------
-// bmC[I] = OR over K in row I of op(A) of bmB[K]   (warp per row)
-__global__ void k_product_rows(const int32_t* __restrict__ arp, const int32_t* __restrict__ aci, int nb, int W,
-                               const uint32_t* __restrict__ bmB, uint32_t* __restrict__ bmC) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= nb) return;
-  int p0 = arp[row], p1 = arp[row + 1];
-  for (int w = lane; w < W; w += 32) {
-    uint32_t acc = 0;
-    for (int p = p0; p < p1; ++p) acc |= bmB[(size_t)aci[p] * W + w];
-    bmC[(size_t)row * W + w] = acc;
-  }
-}
-
-// keep the bits of row i at columns j >= i (the upper block triangle)
-__global__ void k_bitmap_upper(int nb, int W, uint32_t* __restrict__ bm) {
-  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= (int64_t)nb * W) return;
-  const int i = (int)(e / W), w = (int)(e % W);
-  if (w < (i >> 5)) bm[e] = 0u;
-  else if (w == (i >> 5)) bm[e] &= ~((1u << (i & 31)) - 1u);
-}
-
-Pattern product_pattern(ifac_ctx* ctx, const View& arows, const ifac_bsr& B, bool transB, int nb, bool upper) {
-  int W = words_per_row(nb);
-  Buf<uint32_t> bmB = pattern_bitmap(ctx, B, transB);
-  Buf<uint32_t> bmC(ctx, (size_t)nb * W);
-  k_product_rows<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(arows.rp, arows.ci, nb, W, bmB.p, bmC.p);
-  IFAC_CK_LAUNCH();
-  if (upper) {
-    k_bitmap_upper<<<cdiv((int64_t)nb * W, 256), 256, 0, ctx->stream>>>(nb, W, bmC.p);
-    IFAC_CK_LAUNCH();
-  }
-  return pattern_from_bitmap(ctx, bmC.p, nb);
-}
-
-__global__ void k_or_into(uint32_t* __restrict__ dst, const uint32_t* __restrict__ src, size_t n) {
-  size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (i < n) dst[i] |= src[i];
+Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const ifac_bsr& B, bool transB, int nb,
+                        bool upper) {
+  Job j{};
+  j.nb = nb;
+  add_source(j, B.row_ptr, B.col_idx, B.nnzb, transB);
+  j.arp = arows.rp;
+  j.aci = arows.ci;
+  j.upper = upper ? 1 : 0;
+  // a row of op(A) with k blocks meets about k nnz(B) / nb of op(B); what the
+  // lists may hold is nb^2 (at most 1 MB where one CTA writes them)
+  const int64_t full = (int64_t)nb * nb, guess = std::min(full, nnza * std::max<int64_t>(1, B.nnzb / nb));
+  return run_job(ctx, j, std::max(nnza, B.nnzb), guess, full, -1, nullptr, nnza);
 }
 
 Pattern union_pattern(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr* B, bool diag) {
-  int nb = A.nb, W = words_per_row(nb);
-  Buf<uint32_t> bm = pattern_bitmap(ctx, A, false);
-  if (B) {
-    Buf<uint32_t> bb = pattern_bitmap(ctx, *B, false);
-    size_t n = (size_t)nb * W;
-    k_or_into<<<cdiv(n, 256), 256, 0, ctx->stream>>>(bm.p, bb.p, n);
-    IFAC_CK_LAUNCH();
-  }
-  if (diag) {
-    k_bitmap_diag<<<cdiv(nb, 256), 256, 0, ctx->stream>>>(nb, W, bm.p);
-    IFAC_CK_LAUNCH();
-  }
-  return pattern_from_bitmap(ctx, bm.p, nb);
+  Job j{};
+  j.nb = A.nb;
+  add_source(j, A.row_ptr, A.col_idx, A.nnzb, false);
+  if (B) add_source(j, B->row_ptr, B->col_idx, B->nnzb, false);
+  j.diag = diag ? 1 : 0;
+  const int64_t in = A.nnzb + (B ? B->nnzb : 0);
+  const int64_t cap = std::min<int64_t>(in + (diag ? A.nb : 0), (int64_t)A.nb * A.nb);
+  return run_job(ctx, j, in, cap, cap, -1, nullptr);
 }
 
 Pattern sym_pattern(ifac_ctx* ctx, const ifac_bsr& U, const ifac_bsr* B, bool diag) {
-  int nb = U.nb, W = words_per_row(nb);
-  Buf<uint32_t> bm = pattern_bitmap(ctx, U, false);
-  if (U.nnzb > 0) {
-    k_bitmap<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(U.row_ptr, U.col_idx, nb, W, 1, bm.p);
-    IFAC_CK_LAUNCH();
-  }
-  if (B && B->nnzb > 0) {
-    k_bitmap<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(B->row_ptr, B->col_idx, nb, W, 0, bm.p);
-    IFAC_CK_LAUNCH();
-  }
-  if (diag) {
-    k_bitmap_diag<<<cdiv(nb, 256), 256, 0, ctx->stream>>>(nb, W, bm.p);
-    IFAC_CK_LAUNCH();
-  }
-  return pattern_from_bitmap(ctx, bm.p, nb);
+  Job j{};
+  j.nb = U.nb;
+  add_source(j, U.row_ptr, U.col_idx, U.nnzb, false);
+  add_source(j, U.row_ptr, U.col_idx, U.nnzb, true);
+  if (B) add_source(j, B->row_ptr, B->col_idx, B->nnzb, false);
+  j.diag = diag ? 1 : 0;
+  const int64_t in = 2 * U.nnzb + (B ? B->nnzb : 0);
+  const int64_t cap = std::min<int64_t>(in + (diag ? U.nb : 0), (int64_t)U.nb * U.nb);
+  return run_job(ctx, j, in, cap, cap, -1, nullptr);
 }
 
 __global__ void k_expand_rows(const int32_t* __restrict__ rp, int nb, int32_t* __restrict__ row) {
@@ -303,55 +408,107 @@ void expand_rows(ifac_ctx* ctx, const int32_t* rp, int nb, int32_t* row) {
 // ---------------------------------------------------------------------------
 // block selection / truncation with order-preserving compaction
 // ---------------------------------------------------------------------------
-__global__ void k_keep_from_norms(const double* __restrict__ norms, int64_t n, double tau, uint8_t* __restrict__ keep) {
-  int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (p < n) keep[p] = (norms[p] < tau) ? 0 : 1;  // NaN norms are kept, as in the oracle
+// whether block p stays: by mask, or (keep null) by !(norm < tau) -- NaN norms
+// are kept, as in the oracle
+__device__ __forceinline__ bool stays(const uint8_t* __restrict__ keep, const double* __restrict__ norms, double tau,
+                                      int p) {
+  return keep ? keep[p] != 0 : !(norms[p] < tau);
 }
 
-__global__ void k_row_keep_count(const int32_t* __restrict__ rp, int nb, const uint8_t* __restrict__ keep,
-                                 int32_t* __restrict__ cnt) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (row >= nb) return;
-  int c = 0;
-  for (int p = rp[row] + lane; p < rp[row + 1]; p += 32) c += keep[p];
+// kept blocks per block row, and their row pointers
+__global__ void __launch_bounds__(NT)
+    k_keep_scan(const int32_t* __restrict__ rp, int nb, const uint8_t* __restrict__ keep,
+                const double* __restrict__ norms, double tau, int32_t* __restrict__ cnt, int32_t* __restrict__ rp_new,
+                unsigned* __restrict__ ticket, int32_t* __restrict__ total) {
+  const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (row < nb) {
+    int c = 0;
+    for (int p = rp[row] + lane; p < rp[row + 1]; p += 32) c += stays(keep, norms, tau, p) ? 1 : 0;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) cnt[row] = c;
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if (lane == 0) cnt[row] = c;
+  }
+  scan_tail<NT>(cnt, rp_new, nb, ticket, total);
 }
 
-// dest[p]: the new position of block p (-1: dropped); vmap (optional):
-// vmap[new position] = p
-__global__ void k_row_keep_dest(const int32_t* __restrict__ rp, int nb, const uint8_t* __restrict__ keep,
-                                const int32_t* __restrict__ rp_new, const int32_t* __restrict__ ci,
-                                const double* __restrict__ norms, int32_t* __restrict__ ci_new,
-                                double* __restrict__ norms_new, int32_t* __restrict__ dest,
-                                int32_t* __restrict__ vmap = nullptr) {
-  int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+// dest[p]: the new position of block p (-1: dropped), if dest; vmap[new
+// position] = p, if vmap
+__global__ void __launch_bounds__(NT)
+    k_keep_dest(const int32_t* __restrict__ rp, int nb, const uint8_t* __restrict__ keep,
+                const double* __restrict__ norms, double tau, const int32_t* __restrict__ rp_new,
+                const int32_t* __restrict__ ci, int32_t* __restrict__ ci_new, double* __restrict__ norms_new,
+                int32_t* __restrict__ dest, int32_t* __restrict__ vmap) {
+  const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (row >= nb) return;
   int pos = rp_new[row];
   for (int base = rp[row]; base < rp[row + 1]; base += 32) {
-    int p = base + lane;
-    bool k = (p < rp[row + 1]) && keep[p];
-    unsigned m = __ballot_sync(0xffffffffu, k);
-    if (p < rp[row + 1]) {
-      int d = k ? pos + __popc(m & ((1u << lane) - 1u)) : -1;
-      if (dest) dest[p] = d;
-      if (k) {
-        ci_new[d] = ci[p];
-        norms_new[d] = norms[p];
-        if (vmap) vmap[d] = p;
-      }
+    const int p = base + lane;
+    const bool in = p < rp[row + 1], k = in && stays(keep, norms, tau, p);
+    const unsigned m = __ballot_sync(0xffffffffu, k);
+    const int d = k ? pos + __popc(m & ((1u << lane) - 1u)) : -1;
+    if (in && dest) dest[p] = d;
+    if (k) {
+      ci_new[d] = ci[p];
+      norms_new[d] = norms[p];
+      if (vmap) vmap[d] = p;
     }
     pos += __popc(m);
   }
 }
 
+// The same for up to SMALL_KEEP blocks, in one CTA (1024 blocks take 1.5 us; at
+// 12,000 the two kernels above, 10 us, are faster): kept blocks stay in CSR
+// order, so a block's new position is the number of kept ones before it.
+constexpr int SMALL_KEEP = 4096;
+
+__global__ void __launch_bounds__(1024)
+    k_keep_small(const int32_t* __restrict__ rp, int nb, int nnz, const uint8_t* __restrict__ keep,
+                 const double* __restrict__ norms, double tau, const int32_t* __restrict__ ci,
+                 int32_t* __restrict__ rp_new, int32_t* __restrict__ ci_new, double* __restrict__ norms_new,
+                 int32_t* __restrict__ dest, int32_t* __restrict__ vmap, int32_t* __restrict__ total) {
+  extern __shared__ int32_t before[];  // [nnz + 1] kept blocks before block p
+  __shared__ int wsum[2][32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  int carry = 0;
+  for (int base = 0, par = 0; base < nnz; base += 1024, par ^= 1) {
+    const int p = base + tid;
+    const bool k = p < nnz && stays(keep, norms, tau, p);
+    const unsigned m = __ballot_sync(0xffffffffu, k);
+    if (lane == 0) wsum[par][wid] = __popc(m);
+    __syncthreads();
+    const int c = wsum[par][lane];  // every warp adds up the warps' counts
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    const int d = carry + __shfl_sync(0xffffffffu, x - c, wid) + __popc(m & ((1u << lane) - 1u));
+    if (p < nnz) {
+      before[p] = d;
+      if (dest) dest[p] = k ? d : -1;
+    }
+    if (k) {
+      ci_new[d] = ci[p];
+      norms_new[d] = norms[p];
+      if (vmap) vmap[d] = p;
+    }
+    carry += __shfl_sync(0xffffffffu, x, 31);
+  }
+  if (tid == 0) {
+    before[nnz] = carry;
+    *total = carry;
+  }
+  __syncthreads();
+  for (int r = tid; r <= nb; r += 1024) rp_new[r] = before[rp[r]];
+}
+
 __global__ void k_copy_blocks(const double* __restrict__ src, const int32_t* __restrict__ dest, int64_t nblk,
-                              int bsz, double* __restrict__ dst) {
+                              int bsz, bool wide, double* __restrict__ dst) {
   for (int64_t p = blockIdx.x; p < nblk; p += gridDim.x) {
     int d = dest[p];
     if (d < 0) continue;
-    if ((bsz & 1) == 0) {  // even block size: every block starts 16-byte aligned
+    if (wide && (bsz & 1) == 0) {  // aligned values and even block size: every block starts 16-byte aligned
       const double2* s = reinterpret_cast<const double2*>(src + (size_t)p * bsz);
       double2* t = reinterpret_cast<double2*>(dst + (size_t)d * bsz);
       for (int e = threadIdx.x; e < bsz / 2; e += blockDim.x) t[e] = s[e];
@@ -361,79 +518,90 @@ __global__ void k_copy_blocks(const double* __restrict__ src, const int32_t* __r
   }
 }
 
-// row pointers of the kept blocks (keep[p] = 1), returns their number
-static int64_t count_kept(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep, Buf<int32_t>& rp_new) {
+// The kept blocks' pattern and norms, in A's order, with their values left
+// out; dest / vmap as in k_keep_dest.  The lists are sized for every block, so
+// that both kernels go out before the count is read.
+struct Kept {
+  Buf<int32_t> rp, ci, map;
+  Buf<double> norms;
+  int64_t n = 0;
+};
+
+static Kept keep_pattern(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep, double tau, bool want_vmap) {
+  Kept k;
   const int nb = A.nb;
-  Buf<int32_t> cnt(ctx, nb);
-  if (A.nnzb > 0) {
-    k_row_keep_count<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(A.row_ptr, nb, keep, cnt.p);
-    IFAC_CK_LAUNCH();
-  } else {
-    IFAC_CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * nb, ctx->stream));
+  k.rp = Buf<int32_t>(ctx, nb + 1);
+  if (A.nnzb == 0) {
+    IFAC_CK(cudaMemsetAsync(k.rp.p, 0, sizeof(int32_t) * (nb + 1), ctx->stream));
+    k.ci = Buf<int32_t>(ctx, 1);
+    k.norms = Buf<double>(ctx, 1);
+    return k;
   }
-  rp_new = Buf<int32_t>(ctx, nb + 1);
-  return scan_counts(ctx, cnt.p, rp_new.p, nb, true);
+  k.ci = Buf<int32_t>(ctx, A.nnzb);
+  k.norms = Buf<double>(ctx, A.nnzb);
+  k.map = Buf<int32_t>(ctx, A.nnzb);
+  if (A.nnzb <= SMALL_KEEP) {
+    k_keep_small<<<1, 1024, 4 * ((size_t)A.nnzb + 1), ctx->stream>>>(A.row_ptr, nb, (int)A.nnzb, keep, A.norms, tau, A.col_idx, k.rp.p,
+                                                 k.ci.p, k.norms.p, want_vmap ? nullptr : k.map.p,
+                                                 want_vmap ? k.map.p : nullptr, host_word(ctx, HW_KEPT));
+    IFAC_CK_LAUNCH();
+    k.n = read_word(ctx, HW_KEPT);
+    return k;
+  }
+  Buf<int32_t> cnt(ctx, nb);
+  k_keep_scan<<<row_grid(nb), NT, 0, ctx->stream>>>(A.row_ptr, nb, keep, A.norms, tau, cnt.p, k.rp.p, ctx->ticket,
+                                                    host_word(ctx, HW_KEPT));
+  IFAC_CK_LAUNCH();
+  k_keep_dest<<<row_grid(nb), NT, 0, ctx->stream>>>(A.row_ptr, nb, keep, A.norms, tau, k.rp.p, A.col_idx, k.ci.p,
+                                                    k.norms.p, want_vmap ? nullptr : k.map.p,
+                                                    want_vmap ? k.map.p : nullptr);
+  IFAC_CK_LAUNCH();
+  k.n = read_word(ctx, HW_KEPT);
+  return k;
 }
 
-// a new matrix of the kept blocks of A, in order
-static Mat gather_kept(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep, Buf<int32_t>&& rp_new, int64_t tot) {
-  const int nb = A.nb;
+// a new matrix of the kept blocks, in order
+static Mat gather_kept(ifac_ctx* ctx, const ifac_bsr& A, Kept&& k) {
   Mat R(ctx);
   R.m.n = A.n;
   R.m.bs = A.bs;
-  R.m.nb = nb;
-  R.m.nnzb = tot;
-  R.m.row_ptr = rp_new.release();
-  R.m.col_idx = static_cast<int32_t*>(dalloc(ctx, sizeof(int32_t) * (tot ? tot : 1)));
-  R.m.norms = static_cast<double*>(dalloc(ctx, sizeof(double) * (tot ? tot : 1)));
-  R.m.val = static_cast<double*>(dalloc(ctx, sizeof(double) * (size_t)(tot ? tot : 1) * A.bs * A.bs));
-  if (A.nnzb > 0 && tot > 0) {
-    const int grid = cdiv((int64_t)nb * 32, 256);
-    Buf<int32_t> dest(ctx, A.nnzb);
-    k_row_keep_dest<<<grid, 256, 0, ctx->stream>>>(A.row_ptr, nb, keep, R.m.row_ptr, A.col_idx, A.norms,
-                                                   R.m.col_idx, R.m.norms, dest.p);
-    IFAC_CK_LAUNCH();
-    int blocks = (int)std::min<int64_t>(A.nnzb, 152 * 16);
-    k_copy_blocks<<<blocks, 256, 0, ctx->stream>>>(A.val, dest.p, A.nnzb, A.bs * A.bs, R.m.val);
+  R.m.nb = A.nb;
+  R.m.nnzb = k.n;
+  R.m.row_ptr = k.rp.release();
+  R.m.col_idx = k.ci.release();
+  R.m.norms = k.norms.release();
+  R.m.val = static_cast<double*>(dalloc(ctx, sizeof(double) * (size_t)(k.n ? k.n : 1) * A.bs * A.bs));
+  if (k.n > 0) {
+    const int blocks = (int)std::min<int64_t>(A.nnzb, 152 * 16);
+    k_copy_blocks<<<blocks, 256, 0, ctx->stream>>>(A.val, k.map.p, A.nnzb, A.bs * A.bs, aligned16(A.val), R.m.val);
     IFAC_CK_LAUNCH();
   }
   return R;
 }
 
-Mat select_blocks(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* row, const uint8_t* keep) {
-  (void)row;
-  Buf<int32_t> rp_new;
-  const int64_t tot = count_kept(ctx, A, keep, rp_new);
-  return gather_kept(ctx, A, keep, std::move(rp_new), tot);
+Mat select_blocks(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep) {
+  return gather_kept(ctx, A, keep_pattern(ctx, A, keep, 0.0, false));
 }
 
-Mat compact(ifac_ctx* ctx, Mat&& full, const int32_t* row, double tau, bool nocopy) {
-  (void)row;
+Mat select_norms(ifac_ctx* ctx, const ifac_bsr& A, double tau) {
+  return gather_kept(ctx, A, keep_pattern(ctx, A, nullptr, tau, false));
+}
+
+Mat compact(ifac_ctx* ctx, Mat&& full, double tau, bool nocopy) {
   if (full.m.nnzb == 0 || !(tau > 0)) return std::move(full);
-  Buf<uint8_t> keep(ctx, full.m.nnzb);
-  k_keep_from_norms<<<cdiv(full.m.nnzb, 256), 256, 0, ctx->stream>>>(full.m.norms, full.m.nnzb, tau, keep.p);
-  IFAC_CK_LAUNCH();
-  Buf<int32_t> rp_new;
-  const int64_t tot = count_kept(ctx, full.m, keep.p, rp_new);
-  if (tot == full.m.nnzb) return std::move(full);  // nothing dropped: no copy
-  if (!nocopy) return gather_kept(ctx, full.m, keep.p, std::move(rp_new), tot);
+  Kept k = keep_pattern(ctx, full.m, nullptr, tau, nocopy);
+  if (k.n == full.m.nnzb) return std::move(full);  // nothing dropped: no copy
+  if (!nocopy) return gather_kept(ctx, full.m, std::move(k));
   // the kept blocks stay in full's value array, which the result takes over
-  const int nb = full.m.nb;
   Mat R(ctx);
   R.m.n = full.m.n;
   R.m.bs = full.m.bs;
-  R.m.nb = nb;
-  R.m.nnzb = tot;
-  R.m.row_ptr = rp_new.release();
-  R.m.col_idx = static_cast<int32_t*>(dalloc(ctx, sizeof(int32_t) * (tot ? tot : 1)));
-  R.m.norms = static_cast<double*>(dalloc(ctx, sizeof(double) * (tot ? tot : 1)));
-  R.vmap = Buf<int32_t>(ctx, (size_t)(tot ? tot : 1));
-  if (tot > 0) {
-    k_row_keep_dest<<<cdiv((int64_t)nb * 32, 256), 256, 0, ctx->stream>>>(
-        full.m.row_ptr, nb, keep.p, R.m.row_ptr, full.m.col_idx, full.m.norms, R.m.col_idx, R.m.norms, nullptr,
-        R.vmap.p);
-    IFAC_CK_LAUNCH();
-  }
+  R.m.nb = full.m.nb;
+  R.m.nnzb = k.n;
+  R.m.row_ptr = k.rp.release();
+  R.m.col_idx = k.ci.release();
+  R.m.norms = k.norms.release();
+  R.vmap = std::move(k.map);
   R.m.val = full.m.val;
   full.m.val = nullptr;
   return R;

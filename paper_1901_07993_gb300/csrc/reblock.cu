@@ -132,7 +132,7 @@ Mat reblock(ifac_ctx* ctx, const ifac_bsr& A, int bs_b) {
         keep.p);
     IFAC_CK_LAUNCH();
   }
-  return select_blocks(ctx, F.m, nullptr, keep.p);
+  return select_blocks(ctx, F.m, keep.p);
 }
 
 // ---------------------------------------------------------------------------

@@ -49,7 +49,7 @@ Mat quadrant(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* seg, const int32_t
                                                                             qr, qc, keep.p);
     IFAC_CK_LAUNCH();
   }
-  return select_blocks(ctx, A, nullptr, keep.p);
+  return select_blocks(ctx, A, keep.p);
 }
 
 // Z for the ranges of S (S holds blocks inside those ranges only)

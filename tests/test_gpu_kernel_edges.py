@@ -157,3 +157,68 @@ def test_sum_edges(ctx, bs, nb, density, shift):
     A.val[0, 0, 0] = np.inf
     got = ifac.bsr_add(ctx, 1.0, borrowed(A, shift), 0.0, None, 0.0)
     assert np.isinf(ifac.bsr_fro(ctx, got)) and np.array_equal(got.download().val, A.val)
+
+
+def _pattern_ref(A, B, tA, tB, upper):
+    """Stored blocks of op(A) op(B) before truncation."""
+    ma, mb = np.zeros((A.nb, A.nb), int), np.zeros((A.nb, A.nb), int)
+    for m, h in ((ma, A), (mb, B)):
+        m[np.repeat(np.arange(h.nb), np.diff(h.row_ptr)), h.col_idx] = 1
+    m = (ma.T if tA else ma) @ (mb.T if tB else mb) > 0
+    return np.triu(m) if upper else m
+
+
+@pytest.mark.parametrize("nb,density", [(1, 1.0), (31, 0.1), (33, 0.9), (64, 1.0), (255, 0.02), (512, 0.006),
+                                        (512, 0.2), (513, 0.006), (1100, 0.002), (1500, 0.0003)])
+@pytest.mark.parametrize("tA,tB", [(False, False), (True, False), (False, True), (True, True)])
+def test_patterns(ctx, nb, density, tA, tB):
+    """Patterns of products and sums on both sides of the one-CTA limits (block
+    rows, stored blocks, expected result), empty rows included, against
+    numpy's: every block once, rows sorted, and the values of a product and of
+    a truncation in the right place."""
+    from paper_1901_07993_gb300 import ifac
+    A = synth.random_bsr(nb, 16, density, seed=nb, empty_rows=nb // 7)
+    B = synth.random_bsr(nb, 16, density, seed=nb + 1, empty_rows=nb // 9)
+    if A.nnzb == 0 or B.nnzb == 0:
+        pytest.skip("an operand without blocks")
+    dA, dB = ifac.upload(ctx, A), ifac.upload(ctx, B)
+    ref = _pattern_ref(A, B, tA, tB, False)
+    for tau in (0.0, 60.0):
+        got = ifac.bsr_gemm_trunc(ctx, dA, tA, dB, tB, 1.0, tau).download()
+        want = oracle.gemm(A, B, tA, tB, 1.0, tau)
+        if tau == 0.0:
+            assert np.array_equal(got.row_ptr, np.concatenate([[0], np.cumsum(ref.sum(axis=1))]))
+            assert np.array_equal(got.col_idx, np.nonzero(ref)[1])
+        assert np.array_equal(got.row_ptr, want.row_ptr) and np.array_equal(got.col_idx, want.col_idx)
+        assert got.nnzb == 0 or np.abs(got.val - want.val).max() <= 1e-12 * np.abs(want.val).max()
+    s, ws = ifac.bsr_add(ctx, 1.0, dA, 2.0, dB, 0.5).download(), oracle.add(1.0, A, 2.0, B, 0.5)
+    assert np.array_equal(s.row_ptr, ws.row_ptr) and np.array_equal(s.col_idx, ws.col_idx)
+    assert np.array_equal(s.val, ws.val)
+    t, wt = ifac.bsr_truncate(ctx, dA, 16.0).download(), oracle.truncate(A, 16.0)
+    assert np.array_equal(t.row_ptr, wt.row_ptr) and np.array_equal(t.col_idx, wt.col_idx)
+    assert np.array_equal(t.val, wt.val)
+
+
+@pytest.mark.parametrize("bs,nb,density", [(64, 5, 1.0), (64, 40, 0.4), (64, 64, 1.0), (64, 130, 0.05), (64, 300, 0.012),
+                                           (32, 100, 0.3), (32, 520, 0.004), (128, 20, 0.6), (64, 1500, 0.0012)])
+@pytest.mark.parametrize("prec", [TF32, BF16])
+def test_tile_plans(ctx, bs, nb, density, prec):
+    """Tile lists and plans of every kind (one CTA or several, records in one
+    pass or counted first, tiles from C's blocks, both tile shapes at bs 64):
+    small integers, so that every product is exact."""
+    from paper_1901_07993_gb300 import ifac
+    rng = np.random.default_rng(nb)
+    A = synth.random_bsr(nb, bs, density, seed=nb)
+    B = synth.random_bsr(nb, bs, density, seed=nb + 1, empty_rows=1)
+    A.val[:] = rng.integers(-1, 2, A.val.shape)
+    B.val[:] = rng.integers(-1, 2, B.val.shape)
+    dA, dB = ifac.upload(ctx, A), ifac.upload(ctx, B)
+    for tA in (False, True):
+        want = oracle.gemm(A, B, tA, False, 1.0, 0.0)
+        got = ifac.bsr_gemm_trunc(ctx, dA, tA, dB, False, 1.0, 0.0, prec).download()
+        assert np.array_equal(got.row_ptr, want.row_ptr) and np.array_equal(got.col_idx, want.col_idx)
+        assert np.array_equal(got.val, want.val)
+        if bs == 64:
+            up = ifac.bsr_gemm_sym_trunc(ctx, dA, True, dA, False, 1.0, 0.0, prec).download()
+            ref = oracle.gemm(A, A, True, False, 1.0, 0.0)
+            assert np.array_equal(up.col_idx, ref.col_idx) and np.array_equal(up.val, ref.val)
