@@ -222,3 +222,28 @@ def test_tile_plans(ctx, bs, nb, density, prec):
             up = ifac.bsr_gemm_sym_trunc(ctx, dA, True, dA, False, 1.0, 0.0, prec).download()
             ref = oracle.gemm(A, A, True, False, 1.0, 0.0)
             assert np.array_equal(up.col_idx, ref.col_idx) and np.array_equal(up.val, ref.val)
+
+
+@pytest.mark.parametrize("bs,nb,density", [(32, 1, 1.0), (32, 50, 1.0), (32, 52, 1.0), (64, 3, 0.7), (64, 51, 0.9),
+                                           (64, 53, 1.0), (16, 40, 0.5)])
+@pytest.mark.parametrize("tA,tB", [(False, False), (True, False), (False, True), (True, True)])
+def test_fp64_product_block_counts(ctx, bs, nb, density, tA, tB):
+    """FP64 products on both sides of the limit on output blocks at which a
+    block stops being split over four CTAs (2584 blocks on 152 SMs): values
+    within 2 K 2^-53 (|A||B|)_ij, norms within 1e-13, pairs counted once."""
+    from paper_1901_07993_gb300 import ifac
+    A = synth.random_bsr(nb, bs, density, seed=71)
+    B = synth.random_bsr(nb, bs, density, seed=72)
+    if A.nnzb == 0 or B.nnzb == 0:
+        pytest.skip("an operand without blocks")
+    dev = ifac.bsr_gemm_trunc(ctx, borrowed(A, 1), tA, borrowed(B, 1), tB, -0.75, 0.0)
+    got, ref = dev.download(), oracle.gemm(A, B, tA, tB, -0.75, 0.0)
+    assert np.array_equal(got.row_ptr, ref.row_ptr) and np.array_equal(got.col_idx, ref.col_idx)
+    Ad, Bd = (full(A).T if tA else full(A)), (full(B).T if tB else full(B))
+    lim = 2 * nb * bs * 2.0 ** -53 * (np.abs(Ad) @ np.abs(Bd))
+    assert np.all(np.abs(full(got) - full(ref)) <= lim + 1e-300)
+    norms = np.sqrt((np.asarray(ref.val) ** 2).sum(axis=(1, 2)))
+    tau = float(np.median(norms)) * (1 + 1e-9)
+    cut = ifac.bsr_gemm_trunc(ctx, borrowed(A, 1), tA, borrowed(B, 1), tB, -0.75, tau)
+    assert cut.nnzb == int((norms >= tau).sum())
+    assert abs(ifac.bsr_fro(ctx, dev) - np.sqrt((norms ** 2).sum())) <= 1e-13 * np.sqrt((norms ** 2).sum())
