@@ -134,9 +134,30 @@ void to_host(ifac_ctx* ctx, void* host, const void* dev, size_t bytes) {
   }
 }
 
+constexpr int32_t kNotWritten = -1;  // (every word is a count)
+
+int32_t* host_word(ifac_ctx* ctx, HostWord w) {
+  *const_cast<volatile int32_t*>(ctx->host_words + w) = kNotWritten;
+  return ctx->host_words + w;
+}
+
 int32_t read_word(ifac_ctx* ctx, HostWord w) {
-  IFAC_CK(cudaStreamSynchronize(ctx->stream));
-  return *const_cast<volatile int32_t*>(host_word(ctx, w));
+  const volatile int32_t* p = ctx->host_words + w;
+  for (int spin = 1;; ++spin) {
+    int32_t v = *p;
+    if (v == kNotWritten && spin % 4096 == 0) {
+      // a failed kernel never writes: ask the stream now and then
+      const cudaError_t e = cudaStreamQuery(ctx->stream);
+      if (e == cudaErrorNotReady) continue;
+      IFAC_CK(e);
+      v = *p;
+      if (v == kNotWritten) fail(IFAC_ERR_CUDA, "a kernel did not report its count");
+    }
+    if (v != kNotWritten) {
+      std::atomic_thread_fence(std::memory_order_acquire);
+      return v;
+    }
+  }
 }
 
 void to_host_many(ifac_ctx* ctx, std::initializer_list<HostRead> reads) {

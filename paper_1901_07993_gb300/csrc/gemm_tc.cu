@@ -1015,7 +1015,8 @@ __global__ void __launch_bounds__(PLAN_NT) k_tile_plan(const int32_t* __restrict
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(ticket, 1u) == gridDim.x - 1) {
       *ticket = 0u;
-      *host_kmax = atomicExch(kmax, 0);
+      const int longest = atomicExch(kmax, 0);
+      if (host_kmax) *host_kmax = longest;
     }
   }
   if constexpr (COUNT) {
@@ -1131,10 +1132,10 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
     k_tile_plan<ROWS, COLS, PLAN_BOTH><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
         P.tiles.p, ntiles, nullptr, bmA.p, nb, W, imA.p, imB.p, arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb,
         (int)B.nnzb, amap, P.rec.p, P.tnk.p, kmax_dev, C.row_ptr, C.col_idx, P.cpos.p, bmap, nt, P.off.p,
-        ctx->ticket, host_word(ctx, HW_KMAX));
+        ctx->ticket, want_kmax ? host_word(ctx, HW_KMAX) : nullptr);  // (a word nobody reads is not written)
     IFAC_CK_LAUNCH();
     if (extra) to_host_many(ctx, {*extra});
-    if (extra || want_kmax) P.kmax = read_word(ctx, HW_KMAX);
+    if (want_kmax) P.kmax = read_word(ctx, HW_KMAX);
     return P;
   }
   k_tile_plan<ROWS, COLS, PLAN_COUNT><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
@@ -1148,8 +1149,8 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
   // the record count, the longest tile and the caller's extra read-back
   // behind one synchronisation
   if (extra) to_host_many(ctx, {*extra});
-  const int64_t total = extra ? *const_cast<volatile int32_t*>(host_word(ctx, HW_PLAN)) : read_word(ctx, HW_PLAN);
-  P.kmax = *const_cast<volatile int32_t*>(host_word(ctx, HW_KMAX));
+  const int64_t total = read_word(ctx, HW_PLAN);
+  P.kmax = read_word(ctx, HW_KMAX);
   if (total > (int64_t)0x7fffffff / (ROWS + COLS))
     fail(IFAC_ERR_TOO_LARGE, "tensor-core product: tile plan exceeds 2^31 entries");
   if (kmax_limit > 0 && P.kmax > kmax_limit) return P;

@@ -156,11 +156,14 @@ struct HostRead {
 };
 void to_host_many(ifac_ctx* ctx, std::initializer_list<HostRead> reads);
 
-// Words a kernel writes for the host (mapped pinned memory), read after the
-// stream is synchronised.
+// Words a kernel writes for the host (mapped pinned memory).  host_word marks
+// the word as not written and gives its address for a launch; read_word waits
+// for the value itself, not for the stream: the host goes on to the next
+// launches while the kernel that wrote it drains, where a synchronisation
+// costs 10 us between two kernels.
 enum HostWord { HW_NNZ = 0, HW_KEPT, HW_PLAN, HW_KMAX, HW_COUNT };
-inline int32_t* host_word(ifac_ctx* ctx, HostWord w) { return ctx->host_words + w; }
-int32_t read_word(ifac_ctx* ctx, HostWord w);  // synchronises the stream
+int32_t* host_word(ifac_ctx* ctx, HostWord w);
+int32_t read_word(ifac_ctx* ctx, HostWord w);
 
 // ---- pattern utilities (pattern.cu) ----
 int words_per_row(int nb);
