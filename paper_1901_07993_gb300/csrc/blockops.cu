@@ -14,6 +14,7 @@
 #include "internal.cuh"
 #include "tc_common.cuh"
 
+using ifac::tc::load4;
 using ifac::tc::SqAcc;
 
 namespace ifac {
@@ -89,31 +90,11 @@ __device__ __forceinline__ void scale4(const Scale& s, double (&x)[4]) {
   for (int i = 0; i < 4; ++i) x[i] = scaled(s, x[i]);
 }
 
-// four consecutive operand values as FP64: one 32-byte load where `wide` (the
-// values start on a 32-byte boundary), FP32 ones (always the library's own)
-// one 16-byte load
-__device__ __forceinline__ void load4(const double* p, double (&x)[4], bool wide) {
-  if (wide) {
-    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(p));
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) x[i] = __ldg(p + i);
-  }
-}
-__device__ __forceinline__ void load4(const float* p, double (&x)[4], bool) {
-  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
-  const float f[4] = {t.x, t.y, t.z, t.w};
-  ifac::tc::f32_to_f64_x4(f, x);
-}
-
 __device__ __forceinline__ void widen4(const double (&w)[4], double (&x)[4]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i) x[i] = w[i];
 }
 __device__ __forceinline__ void widen4(const float (&w)[4], double (&x)[4]) { ifac::tc::f32_to_f64_x4(w, x); }
-
-// 32-byte aligned
-static bool wide32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 
 // the K-major low-precision copy that the tensor-core products read (TF32:
 // FP32 round-to-nearest-even then TF32 round-half-away; BF16 round-to-
@@ -253,7 +234,7 @@ static void launch_add(ifac_ctx* ctx, Scale sa, const ifac_bsr& A, Scale sb, con
   k_add<W, TB><<<grid, 32 * W, 0, ctx->stream>>>(
       crow, C.col_idx, C.nnzb, C.bs, sa, A.row_ptr, A.col_idx, A.val, sb, B ? B->row_ptr : nullptr,
       B ? B->col_idx : nullptr, B ? reinterpret_cast<const TB*>(B->val) : nullptr, bmap, gamma, C.val, C.norms, lp,
-      lp_elt, wide32(A.val), B && wide32(B->val), wide32(C.val));
+      lp_elt, aligned32(A.val), B && aligned32(B->val), aligned32(C.val));
 }
 
 void add_numeric(ifac_ctx* ctx, double alpha, const ifac_bsr& A, double beta, const ifac_bsr* B, double gamma,
@@ -360,7 +341,7 @@ static void launch_sym(ifac_ctx* ctx, double alpha, const ifac_bsr& U, double be
   k_sym<TU><<<grid, 32 * SYM_WARPS, 0, ctx->stream>>>(
       crow, C.col_idx, C.nnzb, make_scale(alpha), U.row_ptr, U.col_idx, reinterpret_cast<const TU*>(U.val), umap,
       make_scale(beta), B ? B->row_ptr : nullptr, B ? B->col_idx : nullptr, B ? B->val : nullptr, gamma, C.val,
-      C.norms, mirror ? 1 : 0, lp, lp_elt, wide32(U.val), B && wide32(B->val), wide32(C.val));
+      C.norms, mirror ? 1 : 0, lp, lp_elt, aligned32(U.val), B && aligned32(B->val), aligned32(C.val));
 }
 
 void sym_numeric(ifac_ctx* ctx, double alpha, const ifac_bsr& U, double beta, const ifac_bsr* B, double gamma,

@@ -1470,15 +1470,16 @@ struct RowPart {
 };
 
 template <int B, bool TR>
-__global__ void __launch_bounds__(256) k_row_scale(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
-                                                   int splits, const double* __restrict__ val, bool wide,
-                                                   int* __restrict__ eout, unsigned int* __restrict__ l1max,
-                                                   unsigned int* __restrict__ l2max, RowPart* __restrict__ part) {
+constexpr int row_scale_smem() { return (TR ? 512 / B : 8) * B * (int)sizeof(RowScale); }
+
+// the sums of op() row threadIdx.x (< B; the others' result is meaningless)
+// over the view's blocks qa .. qe - 1, by the whole CTA
+template <int B, bool TR>
+__device__ __forceinline__ RowPart row_scale_part(const int32_t* __restrict__ src, int qa, int qe,
+                                                  const double* __restrict__ val, bool wide, uint8_t* smem) {
   constexpr int RG = TR ? 512 / B : 8;  // threads that share a row of op(X)
-  __shared__ RowScale sh[RG][B];
-  const int I = (int)blockIdx.x / splits, sp = (int)blockIdx.x % splits, tid = threadIdx.x;
-  const int q0 = rp[I], cnt = rp[I + 1] - q0, per = (cnt + splits - 1) / splits;
-  const int qa = min(q0 + sp * per, q0 + cnt), qe = min(qa + per, q0 + cnt);
+  RowScale(*sh)[B] = reinterpret_cast<RowScale(*)[B]>(smem);
+  const int tid = threadIdx.x;
   if constexpr (TR) {
     const int c = (tid % (B / 2)) * 2, r0 = tid / (B / 2);
     RowScale a0, a1;
@@ -1514,20 +1515,36 @@ __global__ void __launch_bounds__(256) k_row_scale(const int32_t* __restrict__ r
     for (int g = 0; g < RS; ++g) sh[lane & 7][(wid * RS + g) * 4 + (lane >> 3)] = a[g];
   }
   __syncthreads();
-  if (tid >= B) return;
   RowPart t{0u, 0u, 0, 0.0f, 0.0f};
+  if (tid < B) {
 #pragma unroll
-  for (int g = 0; g < RG; ++g) {
-    t.hi = max(t.hi, sh[g][tid].hi);
-    t.lo |= sh[g][tid].lo;
-  }
-  t.e = row_exponent(t.hi, t.lo);
+    for (int g = 0; g < RG; ++g) {
+      t.hi = max(t.hi, sh[g][tid].hi);
+      t.lo |= sh[g][tid].lo;
+    }
+    t.e = row_exponent(t.hi, t.lo);
 #pragma unroll
-  for (int g = 0; g < RG; ++g) {  // a sum's unit is 2^(ref + 127 - 1023)
-    const int k = sh[g][tid].ref - 896 - t.e;
-    t.l1 += scale_f32(sh[g][tid].l1, k);
-    t.sq += scale_f32(sh[g][tid].sq, 2 * k);
+    for (int g = 0; g < RG; ++g) {  // a sum's unit is 2^(ref + 127 - 1023)
+      const int k = sh[g][tid].ref - 896 - t.e;
+      t.l1 += scale_f32(sh[g][tid].l1, k);
+      t.sq += scale_f32(sh[g][tid].sq, 2 * k);
+    }
   }
+  __syncthreads();  // (the caller may use smem again)
+  return t;
+}
+
+template <int B, bool TR>
+__global__ void __launch_bounds__(256) k_row_scale(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
+                                                   int splits, const double* __restrict__ val, bool wide,
+                                                   int* __restrict__ eout, unsigned int* __restrict__ l1max,
+                                                   unsigned int* __restrict__ l2max, RowPart* __restrict__ part) {
+  __shared__ __align__(16) uint8_t sh[row_scale_smem<B, TR>()];
+  const int I = (int)blockIdx.x / splits, sp = (int)blockIdx.x % splits, tid = threadIdx.x;
+  const int q0 = rp[I], cnt = rp[I + 1] - q0, per = (cnt + splits - 1) / splits;
+  const int qa = min(q0 + sp * per, q0 + cnt), qe = min(qa + per, q0 + cnt);
+  const RowPart t = row_scale_part<B, TR>(src, qa, qe, val, wide, sh);
+  if (tid >= B) return;
   const size_t row = (size_t)I * B + tid;
   if (splits == 1) {
     uint32_t n1, n2;
@@ -1592,107 +1609,222 @@ static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* 
   }
 }
 
-// NS BF16 slice copies (K-major, op() CSR order) of a view; row r of block qb
-// has scale exponent sexp[sblk[qb] * B + r].  With Y = x 2^(62 - e) held as a
-// 64-bit integer (|Y| < 2^62; bits below 2^-62 of sigma dropped by rounding),
-// digit k is q_k = round(Y_k / 2^(62 - 7k)) (ties up), Y_{k+1} = Y_k - q_k 2^(62 - 7k).
-__device__ __forceinline__ void split_digits(double x, int e, int ns, int (&q)[8]) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int ea = (int)((u >> 52) & 0x7ff);
-  unsigned long long mant = u & 0xfffffffffffffull;
-  int eb = ea;
-  if (ea) mant |= 1ull << 52;
-  else eb = 1;
-  // |x| = mant 2^(eb - 1075);  |Y| = mant 2^(eb - 1013 - e)
-  const int sh = eb - 1013 - e;
-  unsigned long long Y = 0;
-  if (sh >= 0) Y = mant << sh;  // sh <= 9 since |x| < sigma
-  else if (sh > -63) Y = (mant + (1ull << (-sh - 1))) >> (-sh);
-  const long long y = (u >> 63) ? -(long long)Y : (long long)Y;
-  // the digits in closed form: with R_k = floor((y + 2^(d_k - 1)) / 2^d_k),
-  // y rounded (half up) to a multiple of 2^d_k, the digits so far sum to
-  // R_k 2^d_k, so q_1 = R_1 and q_k = R_k - 2^7 R_(k-1).  Each q_k is small,
-  // so 32-bit arithmetic on the low words of the R_k suffices.
-  int rprev = 0;
+// NS BF16 slice copies (K-major, op() CSR order) of a view; row r of a block
+// has a scale exponent e (|x| < 2^e).  With Y = x 2^(62 - e) held as a 64-bit
+// integer (|Y| < 2^62; bits below 2^-62 of sigma dropped by rounding) and
+// R_k = Y rounded (half up) to a multiple of 2^(62 - 7k), the digits up to k
+// sum to R_k.  Three digits at a time, c = R_(k+3) - 2^21 R_k is a 22-bit
+// integer (32-bit arithmetic on the low words suffices), whose digits q
+// (|q| <= 64, the first 128) FP32 arithmetic separates exactly: an integer
+// unit result is half the rate of an FP32 one, and digit by digit the integers
+// were what bounded this kernel (60 operations a value).
+//
+// Four values of one row, slices k0 .. k0 + N - 1 from the digits in c.
+template <int N>
+__device__ __forceinline__ void put_digits(const int (&c)[4], int k0, __nv_bfloat16* dst, size_t slice_stride) {
+  constexpr float M = 12582912.0f;  // 1.5 2^23: adding it rounds to an integer
+  float q[3][4];
 #pragma unroll
-  for (int k = 1; k <= 8; ++k) {
-    if (k > ns) break;
-    const int d = 62 - SPLIT_BITS * k;
-    const unsigned long long t = (unsigned long long)y + (1ull << (d - 1));
-    const uint32_t lo = (uint32_t)t, hi = (uint32_t)(t >> 32);
-    const int r = d >= 32 ? ((int)hi >> (d - 32)) : (int)__funnelshift_r(lo, hi, d);
-    q[k - 1] = k == 1 ? r : (int)((uint32_t)r - ((uint32_t)rprev << 7));
-    rprev = r;
+  for (int i = 0; i < 4; ++i) {
+    float f = __int_as_float(0x4B400000 + c[i]) - M;
+    if (N == 3) {
+      q[0][i] = fmaf(f, 0x1p-14f, M) - M;
+      f = fmaf(-0x1p14f, q[0][i], f);
+    }
+    if (N >= 2) {
+      q[N - 2][i] = fmaf(f, 0x1p-7f, M) - M;
+      f = fmaf(-0x1p7f, q[N - 2][i], f);
+    }
+    q[N - 1][i] = f;
+  }
+#pragma unroll
+  for (int k = 0; k < N; ++k) {  // integers up to 128: the upper half of their FP32 pattern is exact
+    uint2 w;
+    w.x = __byte_perm(__float_as_uint(q[k][0]), __float_as_uint(q[k][1]), 0x7632);
+    w.y = __byte_perm(__float_as_uint(q[k][2]), __float_as_uint(q[k][3]), 0x7632);
+    *reinterpret_cast<uint2*>(dst + (size_t)(k0 + k) * slice_stride) = w;
   }
 }
 
-// digits of elements (r, c) and (r, c + 1) of op(X)'s block into the slices
-__device__ __forceinline__ void split_pair(double x0, double x1, int e, int ns, __nv_bfloat16* dst,
-                                           size_t slice_stride) {
-  int q0[8], q1[8];
-  split_digits(x0, e, ns, q0);
-  split_digits(x1, e, ns, q1);
-  // |q| <= 128 is exact in BF16: the upper half of its FP32 pattern, formed
-  // with one integer and one FP32 add (2^23 + 2^22 + q, minus that offset)
-  const auto bf = [](int q) -> uint32_t {
-    return __float_as_uint(__int_as_float(0x4B400000 + q) - 12582912.0f) >> 16;
-  };
-  for (int k = 0; k < ns; ++k)
-    *reinterpret_cast<uint32_t*>(dst + (size_t)k * slice_stride) = bf(q0[k]) | (bf(q1[k]) << 16);
+__device__ __forceinline__ void split4(const double (&x)[4], int e, int ns, __nv_bfloat16* dst, size_t slice_stride) {
+  long long y[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t h = (uint32_t)__double2hiint(x[i]), l = (uint32_t)__double2loint(x[i]);
+    const int ea = (int)((h >> 20) & 0x7ffu);
+    const uint32_t m = (h & 0xfffffu) | (ea ? 0x100000u : 0u);
+    // |x| = mant 2^(max(ea, 1) - 1075), |Y| = mant 2^9 2^-t, t >= 0 since |x| < 2^e
+    const int t = 1022 + e - max(ea, 1);
+    const unsigned long long v = ((unsigned long long)__funnelshift_l(l, m, 9) << 32) | (l << 9);
+    const unsigned long long half = t > 0 ? 1ull << ((t - 1) & 63) : 0ull;
+    const unsigned long long Y = t > 62 ? 0ull : (v + half) >> (t & 63);
+    y[i] = (h >> 31) ? -(long long)Y : (long long)Y;
+  }
+  int r3[4], c[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) c[i] = r3[i] = (int)((y[i] + (1ll << 40)) >> 41);  // (ns >= 3)
+  put_digits<3>(c, 0, dst, slice_stride);
+  if (ns == 3) return;
+  // digits 4 .. k2, k2 = min(ns, 6)
+  const int n2 = min(ns, 6) - 3, d2 = 41 - 7 * n2;
+  int r6[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r6[i] = (int)((y[i] + (1ll << (d2 - 1))) >> d2);
+    c[i] = (int)((uint32_t)r6[i] - ((uint32_t)r3[i] << (7 * n2)));
+  }
+  if (n2 == 3) put_digits<3>(c, 3, dst, slice_stride);
+  else if (n2 == 2) put_digits<2>(c, 3, dst, slice_stride);
+  else put_digits<1>(c, 3, dst, slice_stride);
+  if (ns <= 6) return;
+  const int n3 = ns - 6, d3 = 20 - 7 * n3;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    c[i] = (int)((uint32_t)((y[i] + (1ll << (d3 - 1))) >> d3) - ((uint32_t)r6[i] << (7 * n3)));
+  if (n3 == 2) put_digits<2>(c, 6, dst, slice_stride);
+  else put_digits<1>(c, 6, dst, slice_stride);
 }
 
-template <int B>
-__global__ void __launch_bounds__(256) k_split(const double* __restrict__ val, const int32_t* __restrict__ src,
-                                               int64_t nblk, int tr, const int32_t* __restrict__ sblk,
-                                               const int* __restrict__ sexp, int ns,
+// the slices of one stored block s (the whole CTA, 256 threads); se: the scale
+// exponents of its op() rows.  TR: op() row r is column r of the stored block,
+// moved through shared memory in tiles of 64 x 64, whose columns are permuted
+// by their row so that neither side meets bank conflicts.
+template <int B, bool TR>
+__device__ __forceinline__ void split_block(const double* __restrict__ s, bool wide, const int* se, int ns,
+                                            __nv_bfloat16* __restrict__ d, size_t slice_stride, double* tile) {
+  double x[4];
+  if constexpr (!TR) {
+#pragma unroll 2
+    for (int e = (int)threadIdx.x * 4; e < B * B; e += 1024) {
+      load4(s + e, x, wide);
+      split4(x, se[e / B], ns, d + e, slice_stride);
+    }
+  } else {
+    constexpr int TS = B < 64 ? B : 64;
+    const auto at = [](int r, int c) { return r * TS + (c ^ ((r >> 2) & 15)); };
+    for (int ti = 0; ti < B / TS; ++ti)
+      for (int tj = 0; tj < B / TS; ++tj) {
+#pragma unroll
+        for (int e = (int)threadIdx.x * 4; e < TS * TS; e += 1024) {
+          const int r = e / TS, c = e % TS;
+          load4(s + (size_t)(ti * TS + r) * B + tj * TS + c, x, wide);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) tile[at(r, c + i)] = x[i];
+        }
+        __syncthreads();
+#pragma unroll 2
+        for (int e = (int)threadIdx.x * 4; e < TS * TS; e += 1024) {
+          const int r = e / TS, c = e % TS;  // op() row tj TS + r, columns ti TS + c ..
+#pragma unroll
+          for (int i = 0; i < 4; ++i) x[i] = tile[at(c + i, r)];
+          split4(x, se[tj * TS + r], ns, d + (size_t)(tj * TS + r) * B + ti * TS + c, slice_stride);
+        }
+        __syncthreads();
+      }
+  }
+}
+
+// the zero block of every slice
+__device__ __forceinline__ void split_zero(int bsz, int ns, __nv_bfloat16* __restrict__ d, size_t slice_stride) {
+  for (int k = 0; k < ns; ++k)
+    for (int e = threadIdx.x; e < bsz / 2; e += blockDim.x)
+      *reinterpret_cast<uint32_t*>(d + (size_t)k * slice_stride + 2 * e) = 0u;
+}
+
+// Slices with the scales at hand; the block qb of the view has the exponents
+// sexp[sblk[qb] * B ..].
+template <int B, bool TR>
+__global__ void __launch_bounds__(256) k_split(const double* __restrict__ val, bool wide,
+                                               const int32_t* __restrict__ src, int64_t nblk,
+                                               const int32_t* __restrict__ sblk, const int* __restrict__ sexp, int ns,
                                                __nv_bfloat16* __restrict__ dst) {
-  constexpr int BSZ = B * B;
-  __shared__ double tile[32][33];  // transposed views: 32 x 32 sub-blocks
+  constexpr int BSZ = B * B, TS = B < 64 ? B : 64;
+  __shared__ double tile[TR ? TS * TS : 1];
   const size_t slice_stride = (size_t)(nblk + 1) * BSZ;
   for (int64_t qb = blockIdx.x; qb <= nblk; qb += gridDim.x) {
     __nv_bfloat16* d = dst + (size_t)qb * BSZ;
-    if (qb == nblk) {  // the zero block of every slice
-      for (int k = 0; k < ns; ++k)
-        for (int e = threadIdx.x; e < BSZ / 2; e += blockDim.x)
-          *reinterpret_cast<uint32_t*>(d + (size_t)k * slice_stride + 2 * e) = 0u;
-      continue;
-    }
-    const double* s = val + (size_t)(src ? src[qb] : qb) * BSZ;
-    const int* se = sexp + (size_t)sblk[qb] * B;
-    if (!tr) {
-      for (int e2 = threadIdx.x; e2 < BSZ / 2; e2 += blockDim.x) {
-        const int e = 2 * e2, r = e / B;
-        split_pair(s[e], s[e + 1], se[r], ns, d + e, slice_stride);
-      }
-      continue;
-    }
-    // op(X) row r = stored column r: stored rows 32 ti.., columns 32 tj.. give
-    // op rows 32 tj.., columns 32 ti.. (coalesced reads through shared memory)
-    for (int ti = 0; ti < B / 32; ++ti)
-      for (int tj = 0; tj < B / 32; ++tj) {
-        for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-          const int r = e >> 5, c = e & 31;
-          tile[r][c] = s[(size_t)(ti * 32 + r) * B + tj * 32 + c];
-        }
-        __syncthreads();
-        for (int e2 = threadIdx.x; e2 < 512; e2 += blockDim.x) {
-          const int r = (2 * e2) >> 5, c = (2 * e2) & 31;  // op sub-block element (r, c), (r, c + 1)
-          const int orow = tj * 32 + r, ocol = ti * 32 + c;
-          split_pair(tile[c][r], tile[c + 1][r], se[orow], ns, d + (size_t)orow * B + ocol, slice_stride);
-        }
-        __syncthreads();
-      }
+    if (qb == nblk) split_zero(BSZ, ns, d, slice_stride);
+    else
+      split_block<B, TR>(val + (size_t)(src ? src[qb] : qb) * BSZ, wide, sexp + (size_t)sblk[qb] * B, ns, d,
+                         slice_stride, tile);
   }
+}
+
+// Scales and slices in one kernel for short block rows (a banded operand): CTA
+// I finds the scales of the op() rows of view row I, then reads the row's
+// blocks again, from L2, for their slices, so that HBM sees the values once.
+// out (nullable): the copy index of each view entry, else its position.
+template <int B, bool TR>
+__global__ void __launch_bounds__(256) k_split_rows(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
+                                                    const int32_t* __restrict__ out, int nb, int64_t nblk,
+                                                    const double* __restrict__ val, bool wide, int ns,
+                                                    int* __restrict__ eout, unsigned int* __restrict__ l1max,
+                                                    unsigned int* __restrict__ l2max,
+                                                    __nv_bfloat16* __restrict__ dst) {
+  constexpr int BSZ = B * B, TS = B < 64 ? B : 64;
+  constexpr int SH = row_scale_smem<B, TR>();
+  constexpr int TILE = TR ? TS * TS * (int)sizeof(double) : 8;
+  __shared__ __align__(16) uint8_t sh[SH > TILE ? SH : TILE];
+  __shared__ int se[B];
+  const size_t slice_stride = (size_t)(nblk + 1) * BSZ;
+  const int I = blockIdx.x;
+  if (I == nb) {
+    split_zero(BSZ, ns, dst + (size_t)nblk * BSZ, slice_stride);
+    return;
+  }
+  const int q0 = rp[I], q1 = rp[I + 1];
+  const RowPart t = row_scale_part<B, TR>(src, q0, q1, val, wide, sh);
+  if (threadIdx.x < B) {
+    uint32_t n1, n2;
+    se[threadIdx.x] = t.e;
+    eout[(size_t)I * B + threadIdx.x] = t.e;
+    row_bounds((t.hi | t.lo) != 0u, t.e, t.l1, t.sq, (q1 - q0) * B, n1, n2);
+    row_scale_max(n1, n2, l1max, l2max);
+  }
+  __syncthreads();
+  for (int q = q0; q < q1; ++q) {
+    const int sb = src ? src[q] : q;
+    split_block<B, TR>(val + (size_t)sb * BSZ, wide, se, ns, dst + (size_t)(out ? out[q] : q) * BSZ, slice_stride,
+                       reinterpret_cast<double*>(sh));
+  }
+}
+
+template <int B, bool TR>
+static void launch_split(ifac_ctx* ctx, const double* val, const int32_t* src, int64_t nblk, const int32_t* sblk,
+                         const int* sexp, int ns, void* dst) {
+  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
+  k_split<B, TR><<<grid, 256, 0, ctx->stream>>>(val, aligned32(val), src, nblk, sblk, sexp, ns,
+                                                reinterpret_cast<__nv_bfloat16*>(dst));
+  IFAC_CK_LAUNCH();
 }
 
 static void split_blocks(ifac_ctx* ctx, int bs, const double* val, const int32_t* src, int64_t nblk, bool tr,
                          const int32_t* sblk, const int* sexp, int ns, void* dst) {
-  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
+  if (bs == 32) tr ? launch_split<32, true>(ctx, val, src, nblk, sblk, sexp, ns, dst)
+                   : launch_split<32, false>(ctx, val, src, nblk, sblk, sexp, ns, dst);
+  else if (bs == 64) tr ? launch_split<64, true>(ctx, val, src, nblk, sblk, sexp, ns, dst)
+                        : launch_split<64, false>(ctx, val, src, nblk, sblk, sexp, ns, dst);
+  else tr ? launch_split<128, true>(ctx, val, src, nblk, sblk, sexp, ns, dst)
+          : launch_split<128, false>(ctx, val, src, nblk, sblk, sexp, ns, dst);
+}
+
+// Scales and slices of a view (rows rp, blocks src of nblk) in one launch, when
+// its block rows are short and many enough for one CTA each; false where the
+// two kernels are to be used.
+static bool split_rows(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, const int32_t* out, int nb,
+                       int64_t nblk, bool tr, const double* val, int ns, int* eout, unsigned int* l1max,
+                       unsigned int* l2max, void* dst) {
+  if (nb < 2 * 152 || nblk > 8 * (int64_t)nb) return false;
   __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(dst);
-  if (bs == 32) k_split<32><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, sblk, sexp, ns, d);
-  else if (bs == 64) k_split<64><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, sblk, sexp, ns, d);
-  else k_split<128><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, sblk, sexp, ns, d);
-  IFAC_CK_LAUNCH();
+  const bool wide = aligned32(val);
+  const auto go = [&](auto kernel) {
+    kernel<<<nb + 1, 256, 0, ctx->stream>>>(rp, src, out, nb, nblk, val, wide, ns, eout, l1max, l2max, d);
+    IFAC_CK_LAUNCH();
+  };
+  if (bs == 32) tr ? go(k_split_rows<32, true>) : go(k_split_rows<32, false>);
+  else if (bs == 64) tr ? go(k_split_rows<64, true>) : go(k_split_rows<64, false>);
+  else tr ? go(k_split_rows<128, true>) : go(k_split_rows<128, false>);
+  return true;
 }
 
 // x 2^E rounded to nearest (ties to even), built from the integer's bits;
@@ -2408,7 +2540,7 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   using Cf = Cfg<2>;
   const int nb = A.nb, bs = A.bs;
   const int64_t rows = (int64_t)nb * bs;
-  if (ns < 1 || ns > 8) fail(IFAC_ERR_UNSUPPORTED, "split product: 1 to 8 slices");
+  if (ns < 3 || ns > 8) fail(IFAC_ERR_UNSUPPORTED, "split product: 3 to 8 slices");
   // a cache filled by an earlier product's op(B) (transposed blocks in the
   // stored order, with that operand's column scales) serves op(A) = that
   // matrix transposed, through the view's source indices, and nothing else
@@ -2422,32 +2554,36 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   // [0] / [1]: scaled 1-norm bounds of op(A) rows / op(B) columns, [2] / [3]: 2-norm bounds
   Buf<unsigned int> l1(ctx, 4);
   IFAC_CK(cudaMemsetAsync(l1.p, 0, 4 * sizeof(unsigned int), ctx->stream));
-  if (!hit) {
-    sige = Buf<int>(ctx, rows);
-    row_scales(ctx, bs, arows.rp, value_src(ctx, arows.src, avmap, A.nnzb, asrc), nb, A.nnzb, tA, A.val, sige.p, l1.p,
-               l1.p + 2);
-  }
-  {
-    View bt = view_rows(ctx, B, !tB);
-    Buf<int32_t> btsrc;
-    row_scales(ctx, bs, bt.rp, value_src(ctx, bt.src, bvmap, B.nnzb, btsrc), nb, B.nnzb, !tB, B.val, taue.p, l1.p + 1,
-               l1.p + 3);
-  }
   // slices: row scale block of an op(A) entry is its CSR row; of an op(B) entry its CSR column
   const size_t bbytes = (size_t)bs * bs * 2;
   Buf<uint8_t> la, lb(ctx, (size_t)ns * (B.nnzb + 1) * bbytes);
   if (!hit) {
+    sige = Buf<int>(ctx, rows);
     la = Buf<uint8_t>(ctx, (size_t)nsa * (A.nnzb + 1) * bbytes);
-    Buf<int32_t> arow(ctx, A.nnzb);
-    expand_rows(ctx, arows.rp, nb, arow.p);
-    split_blocks(ctx, bs, A.val, value_src(ctx, arows.src, avmap, A.nnzb, asrc), A.nnzb, tA, arow.p, sige.p, nsa,
-                 la.p);
+    const int32_t* as = value_src(ctx, arows.src, avmap, A.nnzb, asrc);
+    if (!split_rows(ctx, bs, arows.rp, as, nullptr, nb, A.nnzb, tA, A.val, nsa, sige.p, l1.p, l1.p + 2, la.p)) {
+      row_scales(ctx, bs, arows.rp, as, nb, A.nnzb, tA, A.val, sige.p, l1.p, l1.p + 2);
+      Buf<int32_t> arow(ctx, A.nnzb);
+      expand_rows(ctx, arows.rp, nb, arow.p);
+      split_blocks(ctx, bs, A.val, as, A.nnzb, tA, arow.p, sige.p, nsa, la.p);
+    }
+  }
+  {
+    // (the columns of op(B) are the rows of the other view; with op(B) = B its
+    // entries' copies lie in B's stored order)
+    View bt = view_rows(ctx, B, !tB);
+    Buf<int32_t> btsrc;
+    const int32_t* bs_ = value_src(ctx, bt.src, bvmap, B.nnzb, btsrc);
+    if (tB || !split_rows(ctx, bs, bt.rp, bs_, bt.src, nb, B.nnzb, true, B.val, ns, taue.p, l1.p + 1, l1.p + 3,
+                          lb.p)) {
+      row_scales(ctx, bs, bt.rp, bs_, nb, B.nnzb, !tB, B.val, taue.p, l1.p + 1, l1.p + 3);
+      split_blocks(ctx, bs, B.val, value_src(ctx, brows.src, bvmap, B.nnzb, bsrc), B.nnzb, !tB, brows.ci, taue.p, ns,
+                   lb.p);
+    }
   }
   uint8_t* const la_p = hit ? ac->split.p : la.p;
   const int* const sige_p = hit ? ac->sexp.p : sige.p;
   const int* const taue_p = taue.p;
-  split_blocks(ctx, bs, B.val, value_src(ctx, brows.src, bvmap, B.nnzb, bsrc), B.nnzb, !tB, brows.ci, taue.p, ns,
-                 lb.p);
   // one tensor map over all slices of each operand (slice s at row s (nnzb + 1) bs)
   if ((int64_t)ns * (std::max(A.nnzb, B.nnzb) + 1) * bs > (int64_t)0x7fffffff)
     fail(IFAC_ERR_TOO_LARGE, "split product: slice copies exceed the 2^31-row tensor-map range");

@@ -418,6 +418,7 @@ void check_device_error(ifac_ctx* ctx);
 // whether 16-byte loads may read p (matrices a caller lends may start on any
 // multiple of eight bytes)
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+inline bool aligned32(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0; }
 inline int cdiv(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 
 }  // namespace ifac

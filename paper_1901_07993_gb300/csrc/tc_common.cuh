@@ -542,6 +542,23 @@ __device__ __forceinline__ void f32_to_f64_x4(const float (&f)[4], double (&x)[4
   }
 }
 
+// four consecutive operand values as FP64: one 32-byte load where `wide` (the
+// values start on a 32-byte boundary), FP32 ones (always the library's own)
+// one 16-byte load
+__device__ __forceinline__ void load4(const double* p, double (&x)[4], bool wide) {
+  if (wide) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x[0]), "=d"(x[1]), "=d"(x[2]), "=d"(x[3]) : "l"(p));
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = __ldg(p + i);
+  }
+}
+__device__ __forceinline__ void load4(const float* p, double (&x)[4], bool) {
+  const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+  const float f[4] = {t.x, t.y, t.z, t.w};
+  f32_to_f64_x4(f, x);
+}
+
 // TF32 patterns of four FP64 values (FP32 round-to-nearest-even, then TF32
 // round-half-away)
 __device__ __forceinline__ void f64_to_tf32_x4(const double (&x)[4], uint32_t (&w)[4]) {

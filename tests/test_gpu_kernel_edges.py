@@ -247,3 +247,51 @@ def test_fp64_product_block_counts(ctx, bs, nb, density, tA, tB):
     cut = ifac.bsr_gemm_trunc(ctx, borrowed(A, 1), tA, borrowed(B, 1), tB, -0.75, tau)
     assert cut.nnzb == int((norms >= tau).sum())
     assert abs(ifac.bsr_fro(ctx, dev) - np.sqrt((norms ** 2).sum())) <= 1e-13 * np.sqrt((norms ** 2).sum())
+
+
+@pytest.mark.parametrize("bs", [32, 64, 128])
+@pytest.mark.parametrize("tA,tB,shift", [(False, False, 0), (True, False, 1), (False, True, 0), (True, True, 2)])
+@pytest.mark.parametrize("ns", [3, 5, 8])
+def test_split_banded_operands(bs, tA, tB, shift, ns):
+    """Operands of many short block rows (scales and slices in one kernel) with
+    empty rows and values off a 32-byte boundary, magnitudes over 2^+-40 with
+    zeros and exact powers of two among them (ties of the digits): the bound of
+    the row-scale test for s slices."""
+    from paper_1901_07993_gb300 import ifac
+    ctx = ifac.Context()
+    ctx.set_split_slices(ns)
+    nb = 330
+    rng = np.random.default_rng(11)
+
+    def banded(seed):
+        mask = np.abs(np.subtract.outer(np.arange(nb), np.arange(nb))) <= 1
+        mask[rng.choice(nb, 5, replace=False)] = False
+        rows, cols = np.nonzero(mask)
+        v = rng.standard_normal((len(rows), bs, bs)) * np.exp2(rng.integers(-40, 41, (len(rows), 1, 1)))
+        v[::3] = np.exp2(rng.integers(-12, 13, v[::3].shape)) * rng.integers(-1, 2, v[::3].shape)
+        rp = np.concatenate([[0], np.cumsum(mask.sum(axis=1))]).astype(np.int32)
+        return synth.HostBSR(nb * bs, bs, rp, cols.astype(np.int32), v)
+
+    A, B = banded(1), banded(2)
+    got = ifac.bsr_gemm_trunc(ctx, borrowed(A, shift), tA, borrowed(B, shift), tB, 1.0, 0.0, FP64_SPLIT).download()
+    ref = oracle.gemm(A, B, tA, tB, 1.0, 0.0)
+    assert np.array_equal(got.row_ptr, ref.row_ptr) and np.array_equal(got.col_idx, ref.col_idx)
+
+    def maxima(M, t):  # largest magnitude of every scalar row of op(M), by block row
+        out = np.zeros((nb, bs))
+        rows = np.repeat(np.arange(nb), np.diff(M.row_ptr))
+        for q in range(M.nnzb):
+            v = np.abs(M.val[q].T if t else M.val[q]).max(axis=1)
+            I = M.col_idx[q] if t else rows[q]
+            out[I] = np.maximum(out[I], v)
+        return out
+
+    r, c = maxima(A, tA), maxima(B, not tB)
+    absA = synth.HostBSR(A.n, bs, A.row_ptr, A.col_idx, np.abs(A.val))
+    absB = synth.HostBSR(B.n, bs, B.row_ptr, B.col_idx, np.abs(B.val))
+    aref = oracle.gemm(absA, absB, tA, tB, 1.0, 0.0)
+    K = 3 * bs
+    rows = np.repeat(np.arange(nb), np.diff(ref.row_ptr))
+    lim = (K * 2.0 ** -(7 * ns - 5) * r[rows][:, :, None] * c[ref.col_idx][:, None, :]
+           + 2 * K * 2.0 ** -53 * np.asarray(aref.val))
+    assert np.all(np.abs(got.val - ref.val) <= lim)
