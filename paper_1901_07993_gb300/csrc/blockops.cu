@@ -107,8 +107,7 @@ __device__ __forceinline__ void lp_store4(void* lp, int lp_elt, size_t i, const 
     *reinterpret_cast<uint4*>(static_cast<uint32_t*>(lp) + i) = make_uint4(w[0], w[1], w[2], w[3]);
   } else if (lp_elt == 2) {
     uint32_t w[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) w[k] = ifac::tc::f64_to_bf16_bits_rne(x[k]);
+    ifac::tc::f64_to_bf16_x4(x, w);
     *reinterpret_cast<uint2*>(static_cast<uint16_t*>(lp) + i) = make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16));
   }
 }

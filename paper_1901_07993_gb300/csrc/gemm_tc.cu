@@ -484,50 +484,82 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 // operand conversion and tile list
 // ---------------------------------------------------------------------------
 // dst[q] = low-precision copy of block src[q] of X (B x B blocks; K-major:
-// transposed when tr).  Reads are coalesced; a transposed copy goes through
-// shared memory in 32 x 32 sub-blocks.  X's values are FP64 (V = double) or
-// the FP32 results of a TF32/BF16 product (V = float), rounded alike.
-template <int ELT, int B, typename V>
-__global__ void __launch_bounds__(256) k_convert(const V* __restrict__ val, const int32_t* __restrict__ src,
-                                                 int64_t nblk, int tr, void* __restrict__ dst) {
-  constexpr int BSZ = B * B;
+// transposed when TR), one zero block appended.  X's values are FP64 (V =
+// double) or the FP32 results of a TF32/BF16 product (V = float), rounded
+// alike.  Bound by HBM: four values a thread and step, one vector load and one
+// vector store; a transposed copy goes through shared memory in tiles of 64 x
+// 64 whose columns are permuted by their row, so that neither side meets bank
+// conflicts.  One value at a time and 32 x 32 tiles before: BF16 copies of the
+// dense 8192 x 8192 matrix 165 -> 101 us as stored, 165 -> 121 us transposed (640
+// MB each, 5.3 - 6.3 TB/s); TF32 copies of the 262,144-row chain 115 -> 94 us
+// from FP64, 123 -> 64 us from FP32.
+template <int ELT, typename V>
+__device__ __forceinline__ void convert4(const V* __restrict__ p, bool wide, uint32_t (&w)[4]) {
+  if constexpr (std::is_same<V, float>::value) {
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    const float f[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = ELT == 2 ? f32_to_bf16_bits_rne(f[i]) : f32_to_tf32(f32_flush(f[i]));
+  } else {
+    double x[4];
+    load4(p, x, wide);
+    if constexpr (ELT == 4) f64_to_tf32_x4(x, w);
+    else f64_to_bf16_x4(x, w);
+  }
+}
+
+template <int ELT>
+__device__ __forceinline__ void put4(void* dst, size_t i, const uint32_t (&w)[4]) {
+  if constexpr (ELT == 4)
+    *reinterpret_cast<uint4*>(static_cast<uint32_t*>(dst) + i) = make_uint4(w[0], w[1], w[2], w[3]);
+  else
+    *reinterpret_cast<uint2*>(static_cast<uint16_t*>(dst) + i) = make_uint2(w[0] | (w[1] << 16), w[2] | (w[3] << 16));
+}
+
+template <int ELT, int B, bool TR, typename V>
+__global__ void __launch_bounds__(256) k_convert(const V* __restrict__ val, bool wide, const int32_t* __restrict__ src,
+                                                 int64_t nblk, void* __restrict__ dst) {
+  constexpr int BSZ = B * B, TS = B < 64 ? B : 64;
   using T = typename std::conditional<ELT == 2, uint16_t, uint32_t>::type;
-  __shared__ T tile[32][33];
-  auto conv = [](V x) -> T {
-    if constexpr (std::is_same<V, float>::value) {
-      if constexpr (ELT == 2) return f32_to_bf16_bits_rne(x);
-      else return f32_to_tf32(f32_flush(x));
-    } else {
-      if constexpr (ELT == 2) return f64_to_bf16_bits_rne(x);
-      else return f32_to_tf32(__uint_as_float(f64_to_f32_bits_rne(x)));
-    }
-  };
-  T* out = reinterpret_cast<T*>(dst);
+  __shared__ T tile[TR ? TS * TS : 1];
+  // element (r, c) of a tile: rows of four permute the groups' places
+  const auto at = [](int r, int c) { return r * TS + (c ^ ((r >> 2) & 15)); };
   for (int64_t qb = blockIdx.x; qb <= nblk; qb += gridDim.x) {
-    T* d = out + (size_t)qb * BSZ;
+    const size_t d = (size_t)qb * BSZ;
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
     if (qb == nblk) {  // the zero block
-      for (int e = threadIdx.x; e < BSZ; e += blockDim.x) d[e] = 0;
+      for (int e = (int)threadIdx.x * 4; e < BSZ; e += 1024) put4<ELT>(dst, d + e, w);
       continue;
     }
     const V* s = val + (size_t)(src ? src[qb] : qb) * BSZ;
-    if (!tr) {
-      for (int e = threadIdx.x; e < BSZ; e += blockDim.x) d[e] = conv(s[e]);
-      continue;
-    }
-    for (int ti = 0; ti < B / 32; ++ti)
-      for (int tj = 0; tj < B / 32; ++tj) {
-        // stored rows 32 ti.., columns 32 tj.. -> copy rows 32 tj.., columns 32 ti..
-        for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-          const int r = e >> 5, c = e & 31;
-          tile[r][c] = conv(s[(size_t)(ti * 32 + r) * B + tj * 32 + c]);
-        }
-        __syncthreads();
-        for (int e = threadIdx.x; e < 1024; e += blockDim.x) {
-          const int r = e >> 5, c = e & 31;
-          d[(size_t)(tj * 32 + r) * B + ti * 32 + c] = tile[c][r];
-        }
-        __syncthreads();
+    if constexpr (!TR) {
+#pragma unroll 4
+      for (int e = (int)threadIdx.x * 4; e < BSZ; e += 1024) {
+        convert4<ELT>(s + e, wide, w);
+        put4<ELT>(dst, d + e, w);
       }
+    } else {
+      for (int ti = 0; ti < B / TS; ++ti)
+        for (int tj = 0; tj < B / TS; ++tj) {
+          // stored rows ti TS.., columns tj TS.. -> copy rows tj TS.., columns ti TS..
+#pragma unroll
+          for (int e = (int)threadIdx.x * 4; e < TS * TS; e += 1024) {
+            const int r = e / TS, c = e % TS;
+            convert4<ELT>(s + (size_t)(ti * TS + r) * B + tj * TS + c, wide, w);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) tile[at(r, c + i)] = (T)w[i];
+          }
+          __syncthreads();
+#pragma unroll
+          for (int e = (int)threadIdx.x * 4; e < TS * TS; e += 1024) {
+            const int r = e / TS, c = e % TS;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = tile[at(c + i, r)];
+            put4<ELT>(dst, d + (size_t)(tj * TS + r) * B + ti * TS + c, w);
+          }
+          __syncthreads();
+        }
+    }
   }
 }
 
@@ -1211,14 +1243,21 @@ static CUtensorMap make_map_box(int bs, void* base, int64_t nblk, int inner, int
   return m;
 }
 
+template <int ELT, bool TR, typename V>
+static void launch_convert(ifac_ctx* ctx, int bs, const V* val, const int32_t* src, int64_t nblk, void* dst) {
+  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
+  const bool wide = aligned32(val);
+  if (bs == 32) k_convert<ELT, 32, TR, V><<<grid, 256, 0, ctx->stream>>>(val, wide, src, nblk, dst);
+  else if (bs == 64) k_convert<ELT, 64, TR, V><<<grid, 256, 0, ctx->stream>>>(val, wide, src, nblk, dst);
+  else k_convert<ELT, 128, TR, V><<<grid, 256, 0, ctx->stream>>>(val, wide, src, nblk, dst);
+  IFAC_CK_LAUNCH();
+}
+
 template <int ELT, typename V = double>
 static void convert_blocks(ifac_ctx* ctx, int bs, const V* val, const int32_t* src, int64_t nblk, bool tr,
                            void* dst) {
-  const int grid = (int)std::min<int64_t>(nblk + 1, 152 * 16);
-  if (bs == 32) k_convert<ELT, 32, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
-  else if (bs == 64) k_convert<ELT, 64, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
-  else k_convert<ELT, 128, V><<<grid, 256, 0, ctx->stream>>>(val, src, nblk, tr ? 1 : 0, dst);
-  IFAC_CK_LAUNCH();
+  if (tr) launch_convert<ELT, true>(ctx, bs, val, src, nblk, dst);
+  else launch_convert<ELT, false>(ctx, bs, val, src, nblk, dst);
 }
 
 // the narrow-tile plan of a block size (tile of 128 / bs x max(64, bs) / bs blocks)
@@ -1626,7 +1665,8 @@ __device__ __forceinline__ void put_digits(const int (&c)[4], int k0, __nv_bfloa
   float q[3][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    float f = __int_as_float(0x4B400000 + c[i]) - M;
+    // (half a unit more, so that ties round up, as the R_k do)
+    float f = (__int_as_float(0x4B400000 + c[i]) - M) + 0.5f;
     if (N == 3) {
       q[0][i] = fmaf(f, 0x1p-14f, M) - M;
       f = fmaf(-0x1p14f, q[0][i], f);
@@ -1635,7 +1675,7 @@ __device__ __forceinline__ void put_digits(const int (&c)[4], int k0, __nv_bfloa
       q[N - 2][i] = fmaf(f, 0x1p-7f, M) - M;
       f = fmaf(-0x1p7f, q[N - 2][i], f);
     }
-    q[N - 1][i] = f;
+    q[N - 1][i] = f - 0.5f;
   }
 #pragma unroll
   for (int k = 0; k < N; ++k) {  // integers up to 128: the upper half of their FP32 pattern is exact
@@ -1752,7 +1792,9 @@ __global__ void __launch_bounds__(256) k_split(const double* __restrict__ val, b
 
 // Scales and slices in one kernel for short block rows (a banded operand): CTA
 // I finds the scales of the op() rows of view row I, then reads the row's
-// blocks again, from L2, for their slices, so that HBM sees the values once.
+// blocks again, from L2, for their slices, so that HBM sees the values once:
+// 280 us for the 262,144-row chain with 5 to 7 slices (1.0 - 1.1 GB), 485 us in
+// two kernels before.
 // out (nullable): the copy index of each view entry, else its position.
 template <int B, bool TR>
 __global__ void __launch_bounds__(256) k_split_rows(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,

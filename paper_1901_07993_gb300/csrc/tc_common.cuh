@@ -578,5 +578,25 @@ __device__ __forceinline__ void f64_to_tf32_x4(const double (&x)[4], uint32_t (&
   }
 }
 
+// BF16 patterns of four FP64 values (round to nearest even)
+__device__ __forceinline__ void f64_to_bf16_x4(const double (&x)[4], uint32_t (&w)[4]) {
+  bool odd = false;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t h = (uint32_t)__double2hiint(x[i]), l = (uint32_t)__double2loint(x[i]), m = h & 0x7fffffffu;
+    odd |= m >= (1150u << 20);  // BF16's largest binade and above
+    // exponent field moved, 7 of the fraction's bits; the 45 below decide
+    uint32_t b = (m - (896u << 20)) >> 13;
+    const uint32_t rest = ((m & 0x1fffu) << 1) | (l != 0u ? 1u : 0u);  // half is 0x2000
+    b += rest + (b & 1u) > 0x2000u ? 1u : 0u;
+    if (m < (897u << 20)) b = 0u;  // below the normal range: zero
+    w[i] = b | (h >> 31 << 15);
+  }
+  if (odd) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = f64_to_bf16_bits_rne(x[i]);
+  }
+}
+
 }  // namespace tc
 }  // namespace ifac
