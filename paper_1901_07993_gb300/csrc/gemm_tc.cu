@@ -1350,6 +1350,17 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
   }
   const CUtensorMap mapA = make_map<ELT>(la_p, A.nnzb + 1);
   const CUtensorMap mapB = make_map<ELT>(lb_p, B.nnzb + 1);
+  // C's blocks fill more tiles of 4 x 4 than half the SMs: 256 x 256 elements a
+  // CTA (gemm_wide.cu); a smaller product spreads over CTA pairs
+  if (C.nnzb > 16 * 76) {
+    Plan Pw = make_plan<4, 4>(ctx, arows, A, brows, B, C, crow, pc, false, 0, amap, nullptr, bmap);
+    prof_begin(ctx, 1);
+    wide_product(ctx, ELT, &mapA, &mapB, Pw.tiles.p, Pw.coff.p + Pw.nchunk, Pw.tnk.p, Pw.rec.p, Pw.off.p, Pw.cpos.p,
+                 Pw.ntiles, alpha, C, out32);
+    prof_end(ctx);
+    ++ctx->tc_launches;
+    return;
+  }
   Plan P = make_plan<PAIR * TM, Cf::TN>(ctx, arows, A, brows, B, C, crow, pc, false, 0, amap, nullptr, bmap);
   static std::atomic<unsigned long long> attr{0};
   if (first_on_device(attr, ctx->device))

@@ -276,6 +276,12 @@ BandShape band_lp_shape(int elt, int bs);
 void band_lp_product(ifac_ctx* ctx, int elt, int bs, const void* mapA, const void* mapB, const int32_t* tiles,
                      const int* ntiles, const int32_t* tile_nk, const int32_t* rec, const int32_t* rec_off,
                      const int32_t* cpos, int tiles_bound, double alpha, ifac_bsr& C, bool out32 = false);
+// TF32 / BF16 product at bs 64 on tiles of 4 x 4 blocks, one CTA each
+// (gemm_wide.cu): maps with boxes of one 128-byte atom by 64 rows, the plan for
+// 4 x 4 blocks
+void wide_product(ifac_ctx* ctx, int elt, const void* mapA, const void* mapB, const int32_t* tiles, const int* ntiles,
+                  const int32_t* tile_nk, const int32_t* rec, const int32_t* rec_off, const int32_t* cpos,
+                  int tiles_bound, double alpha, ifac_bsr& C, bool out32);
 // the same matrix with block size bs (32, 64, 128), exact (reblock.cu)
 Mat reblock(ifac_ctx* ctx, const ifac_bsr& A, int bs);
 // block size and bs-64 tile schedule of a batch from timed probe products

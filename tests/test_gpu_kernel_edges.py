@@ -295,3 +295,32 @@ def test_split_banded_operands(bs, tA, tB, shift, ns):
     lim = (K * 2.0 ** -(7 * ns - 5) * r[rows][:, :, None] * c[ref.col_idx][:, None, :]
            + 2 * K * 2.0 ** -53 * np.asarray(aref.val))
     assert np.all(np.abs(got.val - ref.val) <= lim)
+
+
+@pytest.mark.parametrize("nb,density", [(34, 1.0), (35, 1.0), (36, 0.9), (37, 1.0), (39, 0.7), (70, 0.6), (131, 0.3)])
+@pytest.mark.parametrize("prec", [TF32, BF16])
+def test_wide_tiles(ctx, nb, density, prec):
+    """Dense low-precision products around the block count from which a CTA
+    takes 256 x 256 elements (1216 blocks of C), with every remainder of the
+    block rows modulo four: small integers, so that values, norms and the
+    truncation at a median norm are exact; full and upper-triangle products."""
+    from paper_1901_07993_gb300 import ifac
+    rng = np.random.default_rng(nb)
+    A = synth.random_bsr(nb, 64, density, seed=nb, n=nb * 64 - 5)
+    B = synth.random_bsr(nb, 64, density, seed=nb + 1, n=nb * 64 - 5)
+    A.val[:] = rng.integers(-2, 3, A.val.shape)
+    B.val[:] = rng.integers(-2, 3, B.val.shape)
+    dA, dB = ifac.upload(ctx, A), ifac.upload(ctx, B)
+    for tA, tB in ((False, False), (True, False), (False, True)):
+        want = oracle.gemm(A, B, tA, tB, -0.5, 0.0)
+        dev = ifac.bsr_gemm_trunc(ctx, dA, tA, dB, tB, -0.5, 0.0, prec)
+        got = dev.download()
+        assert np.array_equal(got.row_ptr, want.row_ptr) and np.array_equal(got.col_idx, want.col_idx)
+        assert np.array_equal(got.val, want.val)
+        norms = np.sqrt((np.asarray(want.val) ** 2).sum(axis=(1, 2)))
+        total = np.sqrt((norms ** 2).sum())
+        assert abs(ifac.bsr_fro(ctx, dev) - total) <= 1e-11 * total
+        tau = float(np.median(norms)) * (1 + 1e-9)
+        assert ifac.bsr_gemm_trunc(ctx, dA, tA, dB, tB, -0.5, tau, prec).nnzb == int((norms >= tau).sum())
+    up, ref = ifac.bsr_gemm_sym_trunc(ctx, dA, True, dA, False, 1.0, 0.0, prec).download(), oracle.gemm(A, A, True)
+    assert np.array_equal(up.col_idx, ref.col_idx) and np.array_equal(up.val, ref.val)
