@@ -14,7 +14,8 @@
 //   Yh = -Pi_Y(deltah), Zh += Pi_Z(X Yh^T), Xh = Pi_X(Z Yh), Zh += Pi_Z(S^T Xh),
 //   Sh += Pi_S(Xh Z^T),
 // from Zh_K = Pi_{Z_K}((F + F^T) Z_K).  The recording run keeps every
-// intermediate of every sweep (checkpoints), so nothing is recomputed.
+// product of every sweep (checkpoints) and the patterns of delta and P, whose
+// values are formed again.
 #include <cmath>
 #include <vector>
 
@@ -22,16 +23,24 @@
 
 namespace ifac {
 
-// alpha op(A) op(B) computed on exactly the block pattern of P
-static Mat gemm_masked(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, double alpha,
-                       const ifac_bsr& P) {
-  Mat C = mat_alloc(ctx, A.n, A.bs, A.nb, P.nnzb);
+// a matrix of P's block pattern (values to be written) and its blocks' rows
+static Mat like(ifac_ctx* ctx, const ifac_bsr& P, Buf<int32_t>* row) {
+  Mat C = mat_alloc(ctx, P.n, P.bs, P.nb, P.nnzb);
   IFAC_CK(cudaMemcpyAsync(C.m.row_ptr, P.row_ptr, sizeof(int32_t) * (P.nb + 1), cudaMemcpyDeviceToDevice,
                           ctx->stream));
   if (P.nnzb == 0) return C;
   IFAC_CK(cudaMemcpyAsync(C.m.col_idx, P.col_idx, sizeof(int32_t) * P.nnzb, cudaMemcpyDeviceToDevice, ctx->stream));
-  Buf<int32_t> row(ctx, P.nnzb);
-  expand_rows(ctx, C.m.row_ptr, C.m.nb, row.p);
+  *row = Buf<int32_t>(ctx, P.nnzb);
+  expand_rows(ctx, C.m.row_ptr, C.m.nb, row->p);
+  return C;
+}
+
+// alpha op(A) op(B) computed on exactly the block pattern of P
+static Mat gemm_masked(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, double alpha,
+                       const ifac_bsr& P) {
+  Buf<int32_t> row;
+  Mat C = like(ctx, P, &row);
+  if (P.nnzb == 0) return C;
   View arows = view_rows(ctx, A, tA);
   View bcols = view_rows(ctx, B, !tB);
   Buf<unsigned long long> pairs(ctx, 1);
@@ -41,17 +50,24 @@ static Mat gemm_masked(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr
   return C;
 }
 
-// Pi_P(A): A's blocks on the pattern of P, zero blocks where A has none
-static Mat project(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr& P) {
-  Mat C = mat_alloc(ctx, A.n, A.bs, A.nb, P.nnzb);
-  IFAC_CK(cudaMemcpyAsync(C.m.row_ptr, P.row_ptr, sizeof(int32_t) * (P.nb + 1), cudaMemcpyDeviceToDevice,
-                          ctx->stream));
-  if (P.nnzb == 0) return C;
-  IFAC_CK(cudaMemcpyAsync(C.m.col_idx, P.col_idx, sizeof(int32_t) * P.nnzb, cudaMemcpyDeviceToDevice, ctx->stream));
-  Buf<int32_t> row(ctx, P.nnzb);
-  expand_rows(ctx, C.m.row_ptr, C.m.nb, row.p);
-  add_numeric(ctx, 1.0, A, 0.0, nullptr, 0.0, C.m, row.p);
+// Pi_P(alpha A + beta B + gamma I), B nullable: zero blocks where none has
+// one.  The pattern is at hand, so a sum of the reverse sweep is one pass, where
+// projecting its terms and adding them on the union of their patterns was
+// three and a read-back.
+static Mat sum_on(ifac_ctx* ctx, const ifac_bsr& P, double alpha, const ifac_bsr& A, double beta = 0.0,
+                  const ifac_bsr* B = nullptr, double gamma = 0.0) {
+  Buf<int32_t> row;
+  Mat C = like(ctx, P, &row);
+  if (P.nnzb) add_numeric(ctx, alpha, A, beta, B, gamma, C.m, row.p);
   return C;
+}
+
+// keeps a matrix's pattern only: delta and P are formed again in the reverse
+// sweep, so that the checkpoints take no more memory for them
+static void drop_values(Mat& A) {
+  dfree(A.ctx, A.m.val);
+  dfree(A.ctx, A.m.norms);
+  A.m.val = A.m.norms = nullptr;
 }
 
 // per-CTA partial sums of a[i] * b[i], then a fixed-order total
@@ -82,7 +98,7 @@ __global__ void k_sum_parts(const double* __restrict__ part, int n, double* __re
 
 // <A, B> over the pattern of A (B restricted to it)
 static double dot_on(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr& B) {
-  Mat Bp = project(ctx, B, A);
+  Mat Bp = sum_on(ctx, A, 1.0, B);
   const int64_t n = A.nnzb * (int64_t)A.bs * A.bs;
   const int grid = 152 * 4;
   Buf<double> part(ctx, grid), out(ctx, 1);
@@ -109,59 +125,54 @@ int refine_adjoint(ifac_ctx* ctx, const ifac_bsr& S_in, const ifac_bsr& F, int K
   Mat S = truncate(ctx, S_in, tau);
   const double beta = gershgorin_host(ctx, S.m);
   const double c = 1.0 / std::sqrt(beta);
-  std::vector<Mat> X(K), Y(K), D(K), M(K), Z(K + 1);
+  std::vector<Mat> X(K), Y(K), del(K), D(K), P(K), M(K), Z(K + 1);
   Z[0] = scaled_identity(ctx, S.m.n, S.m.bs, S.m.nb, c);
   for (int k = 0; k < K; ++k) {  // recording run: truncation fixes the patterns
     X[k] = gemm(ctx, S.m, false, Z[k].m, false, 1.0, tau);
     Y[k] = gemm(ctx, Z[k].m, true, X[k].m, false, 1.0, tau);
-    Mat delta = add(ctx, -1.0, Y[k].m, 0.0, nullptr, 1.0);
-    D[k] = gemm(ctx, delta.m, false, delta.m, false, 1.0, tau);
-    Mat P = add(ctx, 0.5, delta.m, 0.375, &D[k].m, 0.0);
-    M[k] = gemm(ctx, Z[k].m, false, P.m, false, 1.0, tau);
+    del[k] = add(ctx, -1.0, Y[k].m, 0.0, nullptr, 1.0);
+    D[k] = gemm(ctx, del[k].m, false, del[k].m, false, 1.0, tau);
+    P[k] = add(ctx, 0.5, del[k].m, 0.375, &D[k].m, 0.0);
+    M[k] = gemm(ctx, Z[k].m, false, P[k].m, false, 1.0, tau);
+    drop_values(del[k]);
+    drop_values(P[k]);
     Z[k + 1] = add(ctx, 1.0, Z[k].m, 1.0, &M[k].m, 0.0);
   }
   const ifac_bsr& ZK = Z[K].m;
-  {
-    Mat FZ = gemm_masked(ctx, F, false, ZK, false, 1.0, ZK);
-    *L_out = dot_on(ctx, ZK, FZ.m);
-  }
   Mat Zh;
   {
     Mat FZ = gemm_masked(ctx, F, false, ZK, false, 1.0, ZK);
+    *L_out = dot_on(ctx, ZK, FZ.m);
     Mat FtZ = gemm_masked(ctx, F, true, ZK, false, 1.0, ZK);
-    Zh = add(ctx, 1.0, FZ.m, 1.0, &FtZ.m, 0.0);
+    Zh = sum_on(ctx, ZK, 1.0, FZ.m, 1.0, &FtZ.m);
   }
-  Mat Sh = project(ctx, S.m, S.m);
+  Mat Sh = sum_on(ctx, S.m, 1.0, S.m);
   zero_values(ctx, Sh.m);
   for (int k = K - 1; k >= 0; --k) {
     const ifac_bsr& Zk = Z[k].m;
-    const ifac_bsr& Xk = X[k].m;
-    Mat delta = add(ctx, -1.0, Y[k].m, 0.0, nullptr, 1.0);
-    Mat P = add(ctx, 0.5, delta.m, 0.375, &D[k].m, 0.0);
-    Mat Mh = project(ctx, Zh.m, M[k].m);
-    Mat Zn = project(ctx, Zh.m, Zk);
-    Mat t1 = gemm_masked(ctx, Mh.m, false, P.m, true, 1.0, Zk);       // Pi_Z(Mh P^T)
-    Mat Zacc = add(ctx, 1.0, Zn.m, 1.0, &t1.m, 0.0);
-    Mat Ph = gemm_masked(ctx, Zk, true, Mh.m, false, 1.0, P.m);       // Pi_P(Z^T Mh)
-    Mat Dh = project(ctx, Ph.m, D[k].m);
-    Mat Dh38 = add(ctx, 0.375, Dh.m, 0.0, nullptr, 0.0);
-    Mat a1 = gemm_masked(ctx, Dh38.m, false, delta.m, true, 1.0, delta.m);  // Pi_delta(Dh delta^T)
-    Mat a2 = gemm_masked(ctx, delta.m, true, Dh38.m, false, 1.0, delta.m);  // Pi_delta(delta^T Dh)
-    Mat Phd = project(ctx, Ph.m, delta.m);
-    Mat s1 = add(ctx, 0.5, Phd.m, 1.0, &a1.m, 0.0);
-    Mat deltah = add(ctx, 1.0, s1.m, 1.0, &a2.m, 0.0);
-    Mat Yh0 = project(ctx, deltah.m, Y[k].m);
-    Mat Yh = add(ctx, -1.0, Yh0.m, 0.0, nullptr, 0.0);
-    Mat t2 = gemm_masked(ctx, Xk, false, Yh.m, true, 1.0, Zk);         // Pi_Z(X Yh^T)
-    Mat Zacc2 = add(ctx, 1.0, Zacc.m, 1.0, &t2.m, 0.0);
-    Mat Xh = gemm_masked(ctx, Zk, false, Yh.m, false, 1.0, Xk);        // Pi_X(Z Yh)
-    Mat t3 = gemm_masked(ctx, S.m, true, Xh.m, false, 1.0, Zk);        // Pi_Z(S^T Xh)
-    Mat t4 = gemm_masked(ctx, Xh.m, false, Zk, true, 1.0, S.m);        // Pi_S(Xh Z^T)
-    Sh = add(ctx, 1.0, Sh.m, 1.0, &t4.m, 0.0);
-    Zh = add(ctx, 1.0, Zacc2.m, 1.0, &t3.m, 0.0);
+    const Mat dk = sum_on(ctx, del[k].m, -1.0, Y[k].m, 0.0, nullptr, 1.0);
+    const Mat pk = sum_on(ctx, P[k].m, 0.5, dk.m, 0.375, &D[k].m);
+    const ifac_bsr& delta = dk.m;
+    Mat Mh = sum_on(ctx, M[k].m, 1.0, Zh.m);
+    Mat t1 = gemm_masked(ctx, Mh.m, false, pk.m, true, 1.0, Zk);        // Pi_Z(Mh P^T)
+    Mat Zacc = sum_on(ctx, Zk, 1.0, Zh.m, 1.0, &t1.m);
+    Mat Ph = gemm_masked(ctx, Zk, true, Mh.m, false, 1.0, pk.m);         // Pi_P(Z^T Mh)
+    Mat Dh38 = sum_on(ctx, D[k].m, 0.375, Ph.m);
+    Mat a1 = gemm_masked(ctx, Dh38.m, false, delta, true, 1.0, delta);   // Pi_delta(Dh delta^T)
+    Mat a2 = gemm_masked(ctx, delta, true, Dh38.m, false, 1.0, delta);   // Pi_delta(delta^T Dh)
+    Mat s1 = sum_on(ctx, delta, 0.5, Ph.m, 1.0, &a1.m);
+    Mat deltah = sum_on(ctx, delta, 1.0, s1.m, 1.0, &a2.m);
+    Mat Yh = sum_on(ctx, Y[k].m, -1.0, deltah.m);
+    Mat t2 = gemm_masked(ctx, X[k].m, false, Yh.m, true, 1.0, Zk);       // Pi_Z(X Yh^T)
+    Mat Zacc2 = sum_on(ctx, Zk, 1.0, Zacc.m, 1.0, &t2.m);
+    Mat Xh = gemm_masked(ctx, Zk, false, Yh.m, false, 1.0, X[k].m);      // Pi_X(Z Yh)
+    Mat t3 = gemm_masked(ctx, S.m, true, Xh.m, false, 1.0, Zk);          // Pi_Z(S^T Xh)
+    Mat t4 = gemm_masked(ctx, Xh.m, false, Zk, true, 1.0, S.m);          // Pi_S(Xh Z^T)
+    Sh = sum_on(ctx, S.m, 1.0, Sh.m, 1.0, &t4.m);
+    Zh = sum_on(ctx, Zk, 1.0, Zacc2.m, 1.0, &t3.m);
   }
   // the gradient on the pattern of the caller's S (zero on truncated blocks)
-  Mat G = project(ctx, Sh.m, S_in);
+  Mat G = sum_on(ctx, S_in, 1.0, Sh.m);
   IFAC_CK(cudaStreamSynchronize(ctx->stream));
   *Sbar_out = G.release();
   return IFAC_OK;

@@ -88,45 +88,47 @@ __device__ __forceinline__ void emit(const Job& j, uint32_t word, int r, int w, 
 __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
   extern __shared__ uint32_t sh[];
   __shared__ int32_t wsum[32];
-  const int nw = j.nb * j.W;
-  uint32_t* bm = sh;                                // [nb * W] the sources
+  const int WP = j.W | 1, nw = j.nb * WP;           // odd row stride: no bank conflicts across rows
+  uint32_t* bm = sh;                                // [nb * WP] the sources
   int32_t* off = reinterpret_cast<int32_t*>(bm + nw);  // [nb + 1]
-  uint32_t* out = j.arp ? reinterpret_cast<uint32_t*>(off + j.nb + 1) : bm;  // [nb * W] the pattern
+  uint32_t* out = j.arp ? reinterpret_cast<uint32_t*>(off + j.nb + 1) : bm;  // [nb * WP] the pattern
   int32_t* arp = reinterpret_cast<int32_t*>(out + nw);  // product: [nb + 1], [nnza]
   int32_t* aci = arp + j.nb + 1;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   int lg = 5;  // log2 of the threads that share a row
   while ((j.nb << lg) > 1024 && lg > 0) --lg;
   const int G = 1 << lg, grow = tid >> lg, glane = tid & (G - 1);
+  const bool live = grow < j.nb;
   for (int i = tid; i < nw; i += 1024) bm[i] = 0u;
   if (j.arp) {
     for (int i = tid; i <= j.nb; i += 1024) arp[i] = j.arp[i];
     for (int i = tid; i < nnza; i += 1024) aci[i] = j.aci[i];
   }
   __syncthreads();
-  if (grow < j.nb) {
+  if (live) {
     for (int k = 0; k < j.nsrc; ++k) {
       const int p1 = j.s[k].rp[grow + 1];
+#pragma unroll 4
       for (int p = j.s[k].rp[grow] + glane; p < p1; p += G) {
         const int c = j.s[k].ci[p], br = j.s[k].trans ? c : grow, bc = j.s[k].trans ? grow : c;
-        atomicOr(&bm[br * j.W + (bc >> 5)], 1u << (bc & 31));
+        atomicOr(&bm[br * WP + (bc >> 5)], 1u << (bc & 31));
       }
     }
-    if (j.diag && glane == 0) atomicOr(&bm[grow * j.W + (grow >> 5)], 1u << (grow & 31));
+    if (j.diag && glane == 0) atomicOr(&bm[grow * WP + (grow >> 5)], 1u << (grow & 31));
   }
   __syncthreads();
   if (j.arp) {
-    for (int i = tid; i < nw; i += 1024) {
-      const int r = i / j.W, w = i % j.W;
-      uint32_t acc = 0;
-      for (int p = arp[r]; p < arp[r + 1]; ++p) acc |= bm[aci[p] * j.W + w];
-      out[i] = j.upper ? upper_bits(acc, r, w) : acc;
-    }
+    if (live)
+      for (int w = glane; w < j.W; w += G) {
+        uint32_t acc = 0;
+        for (int p = arp[grow]; p < arp[grow + 1]; ++p) acc |= bm[aci[p] * WP + w];
+        out[grow * WP + w] = j.upper ? upper_bits(acc, grow, w) : acc;
+      }
     __syncthreads();
   }
   int c = 0;
   if (tid < j.nb)
-    for (int w = 0; w < j.W; ++w) c += __popc(out[tid * j.W + w]);
+    for (int w = 0; w < j.W; ++w) c += __popc(out[tid * WP + w]);
   int x = c;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -135,8 +137,7 @@ __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
   }
   if (lane == 31) wsum[wid] = x;
   __syncthreads();
-  int run = x - c;
-  for (int w = 0; w < wid; ++w) run += wsum[w];
+  const int run = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < wid ? wsum[lane] : 0)) + x - c;
   if (tid < j.nb) {
     off[tid] = run;
     j.rp[tid] = run;
@@ -146,20 +147,21 @@ __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
     }
   }
   __syncthreads();
+  if (!live) return;
   const auto before = [&](int r, int w) {  // set bits of row r in the words before w
     int n = off[r];
-    for (int v = 0; v < w; ++v) n += __popc(out[r * j.W + v]);
+    for (int v = 0; v < w; ++v) n += __popc(out[r * WP + v]);
     return n;
   };
-  for (int i = tid; i < nw; i += 1024) {
-    const uint32_t word = out[i];
-    if (word) emit(j, word, i / j.W, i % j.W, before(i / j.W, i % j.W));
+  for (int w = glane; w < j.W; w += G) {
+    const uint32_t word = out[grow * WP + w];
+    if (word) emit(j, word, grow, w, before(grow, w));
   }
-  if (j.src && grow < j.nb) {  // (a transposed view: each stored block finds its own place)
+  if (j.src) {  // (a transposed view: each stored block finds its own place)
     const int p1 = j.frp[grow + 1];
     for (int p = j.frp[grow] + glane; p < p1; p += G) {
       const int r = j.fci[p], w = grow >> 5;
-      j.src[before(r, w) + __popc(out[r * j.W + w] & ((1u << (grow & 31)) - 1u))] = p;
+      j.src[before(r, w) + __popc(out[r * WP + w] & ((1u << (grow & 31)) - 1u))] = p;
     }
   }
 }
@@ -236,10 +238,10 @@ bool rule_small(int nb, int64_t in_blocks, int64_t out_bound) {
 }
 
 void launch_small(ifac_ctx* ctx, const Job& j, int64_t nnza) {
-  const size_t nw = (size_t)j.nb * j.W, smem = 4 * (nw + j.nb + 1 + (j.arp ? nw + j.nb + 1 + (size_t)nnza : 0));
+  const size_t nw = (size_t)j.nb * (j.W | 1), smem = 4 * (nw + j.nb + 1 + (j.arp ? nw + j.nb + 1 + (size_t)nnza : 0));
   if (smem > 48 * 1024)  // set at every such launch, so that no other thread can launch before it
     IFAC_CK(cudaFuncSetAttribute(k_pattern_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 4 * (2 * (SMALL_NB * (SMALL_NB / 32) + SMALL_NB + 1) + SMALL_IN)));
+                                 4 * (2 * (SMALL_NB * (SMALL_NB / 32 + 1) + SMALL_NB + 1) + SMALL_IN)));
   k_pattern_small<<<1, 1024, smem, ctx->stream>>>(j, (int)nnza);
   IFAC_CK_LAUNCH();
 }
