@@ -20,6 +20,9 @@
 // from L2 by the second CTA.  Each CTA loads its own copy of every tile it
 // contracts (no cluster, no cross-CTA signalling).
 //
+// Products with enough 256 x 256 tiles for half the SMs run in gemm_wide.cu
+// instead, banded ones in gemm_band.cu; run() decides.
+//
 // Roles (320 threads, one CTA per SM):
 //   warp 0      : TMA producer -- one 64-row box per block and 128-byte
 //                 atom, 128-byte swizzle, into a STAGES-deep ring;
