@@ -146,6 +146,10 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256) k_gemm_fp64_qua
   __shared__ double Bs[BS * LDB];  // its columns, [k][j]
   __shared__ int pa[32], pb[32], npairs;
   __shared__ double red[8], quad[4];
+  // the first CTA's shared memory may be written only once that CTA is known
+  // to run: arrive here, wait before the store (the products lie between, so
+  // the wait costs nothing)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, lane = tid & 31, wid = tid >> 5;
   const int rank = (int)(blockIdx.x & 3), r0 = (rank >> 1) * H, c0 = (rank & 1) * H;
   const int64_t p = blockIdx.x >> 2;
@@ -234,6 +238,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256) k_gemm_fp64_qua
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if (lane == 0) red[wid] = ss;
   __syncthreads();
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
   if (tid == 0) {
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += red[w];
@@ -242,6 +247,7 @@ __global__ void __cluster_dims__(4, 1, 1) __launch_bounds__(256) k_gemm_fp64_qua
     asm volatile("mapa.shared::cluster.u32 %0, %0, 0;" : "+r"(at));
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(at), "d"(t) : "memory");
   }
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (rank == 0 && tid == 0) {
     cnorm[p] = sqrt((quad[0] + quad[1]) + (quad[2] + quad[3]));

@@ -1,0 +1,59 @@
+"""Calls that once went wrong: each test names what it guards."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1901_07993_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+FP64, TF32, BF16, FP64_SPLIT = 0, 1, 2, 3
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    from paper_1901_07993_gb300 import build as libbuild
+    from paper_1901_07993_gb300 import ifac
+    assert torch.cuda.is_available()
+    libbuild.build()
+    return ifac.Context()
+
+
+@pytest.mark.parametrize("bs", [32, 64])
+def test_split_block_norms(ctx, bs):
+    """Norms of FP64 output blocks that a cluster of four CTAs forms (their sums
+    of squares meet in one CTA): products of one block pair each, whose CTAs
+    end soonest; the same norms every time, within 1e-13 of the values'."""
+    from paper_1901_07993_gb300 import ifac
+    nb = 500
+    v = np.random.default_rng(1).standard_normal((nb, bs, bs))
+    A = synth.HostBSR(nb * bs, bs, np.arange(nb + 1, dtype=np.int32), np.arange(nb, dtype=np.int32), v)
+    dA = ifac.upload(ctx, A)
+    first = None
+    for _ in range(20):
+        C = ifac.bsr_gemm_trunc(ctx, dA, False, dA, True, 1.0, 0.0)
+        fro = ifac.bsr_fro(ctx, C)
+        val = C.download().val
+        want = np.sqrt((val ** 2).sum())
+        assert abs(fro - want) <= 1e-13 * want
+        first = fro if first is None else first
+        assert fro == first
+
+
+def test_adjoint_blocks_without_pairs(ctx):
+    """Masked products whose output blocks have no block pair (an F of one
+    block): L and the gradient as the oracle's."""
+    from paper_1901_07993_gb300 import ifac
+    K, tau = 3, 1e-10
+    S = synth.chain_overlap(512, 32, seed=0)
+    F = synth.HostBSR(S.n, 32, np.concatenate([[0], np.ones(S.nb)]).astype(np.int32), np.zeros(1, np.int32),
+                      np.random.default_rng(2).standard_normal((1, 32, 32)))
+    c = 1.0 / np.sqrt(oracle.gershgorin(oracle.truncate(S, tau)))
+    tape, Fo = oracle.Tape(S, c, K, tau), oracle.Mat(F.n, F.bs, F.row_ptr, F.col_idx, F.val)
+    L_ref, blocks = tape.loss(Fo), tape.adjoint(Fo).blocks()
+    L, G = ifac.inv_factor_refine_adjoint(ctx, ifac.upload(ctx, S), ifac.upload(ctx, F), K, tau)
+    assert abs(L - L_ref) <= 1e-12 * abs(L_ref)
+    g = G.download()
+    rows = np.repeat(np.arange(S.nb), np.diff(S.row_ptr))
+    want = np.array([blocks.get((int(i), int(j)), np.zeros((32, 32))) for i, j in zip(rows, S.col_idx)])
+    assert np.linalg.norm(g.val - want) <= 1e-10 * np.linalg.norm(want)
