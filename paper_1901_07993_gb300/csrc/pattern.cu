@@ -239,7 +239,9 @@ bool rule_small(int nb, int64_t in_blocks, int64_t out_bound) {
 
 void launch_small(ifac_ctx* ctx, const Job& j, int64_t nnza) {
   const size_t nw = (size_t)j.nb * (j.W | 1), smem = 4 * (nw + j.nb + 1 + (j.arp ? nw + j.nb + 1 + (size_t)nnza : 0));
-  if (smem > 48 * 1024)  // set at every such launch, so that no other thread can launch before it
+  // (a kernel has 48 KB without asking, its static shared memory included; set
+  // at every launch above 32 KB, so that no other thread can launch before it)
+  if (smem > 32 * 1024)
     IFAC_CK(cudaFuncSetAttribute(k_pattern_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  4 * (2 * (SMALL_NB * (SMALL_NB / 32 + 1) + SMALL_NB + 1) + SMALL_IN)));
   k_pattern_small<<<1, 1024, smem, ctx->stream>>>(j, (int)nnza);
