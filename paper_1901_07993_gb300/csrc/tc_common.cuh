@@ -216,13 +216,15 @@ __device__ __forceinline__ long long fixed_add(long long d, int x, int sh, bool&
 // accurate to about 2^-42 relative without the FP64 pipe: each square of
 // x 2^32 is split exactly into p + e (FMA), p is added to the running sum with
 // an error-free two-sum, and the errors are collected in a second FP32 word.
-// The scale 2^32 keeps squares of |x| in [2^-95, 2^28) normal, and 64 of
-// them finite; larger magnitudes (rare) are squared in FP64, smaller ones
-// contribute below 2^-190 each.
+// The scale 2^32 keeps the squares of |x| in [2^-95, 2^20) normal and each of
+// them below 2^104, so that the sums of a whole warp stay finite up to 2^23
+// values (a block of 2896 rows; 2^11 are the most a product's epilogue adds);
+// larger magnitudes (rare) are squared in FP64, smaller ones contribute below
+// 2^-190 each.
 struct SqAcc {
   float hi = 0.0f, lo = 0.0f;
   double big = 0.0;
-  // |x| < 2^28 (the caller checks a whole chunk first)
+  // |x| < 2^20 (the caller checks a whole chunk first)
   __device__ __forceinline__ void add_small(float x) {
     const float y = x * 4294967296.0f;
     const float p = y * y;
@@ -233,14 +235,14 @@ struct SqAcc {
     hi = s;
     lo += err + e;
   }
-  // K values: the FP32 path when all are below 2^28 (the usual case), else
+  // K values: the FP32 path when all are below 2^20 (the usual case), else
   // FP64 squares (a separate branch of K FP64 FMAs)
   template <int K>
   __device__ __forceinline__ void add(const float (&v)[K]) {
     float mx = 0.0f;
 #pragma unroll
     for (int i = 0; i < K; ++i) mx = fmaxf(mx, fabsf(v[i]));
-    if (mx < 268435456.0f) {
+    if (mx < 1048576.0f) {
 #pragma unroll
       for (int i = 0; i < K; ++i) add_small(v[i]);
     } else {
@@ -252,12 +254,12 @@ struct SqAcc {
   // an FP64 value, squared through FP32 without the FP64 pipe: its top 24
   // significand bits hi and the next 29 bits lo (rounded to 24) give
   // v^2 = hi^2 + 2 hi lo + lo^2 with lo^2 < 2^-46 v^2 left out.  |v| in
-  // [2^-95, 2^28): FP32 path (lo dropped below 2^-74); larger: FP64; smaller:
+  // [2^-95, 2^20): FP32 path (lo dropped below 2^-74); larger: FP64; smaller:
   // below 2^-190 each, left out.
   __device__ __forceinline__ void add_f64(double v) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
     const int f = (int)((b >> 52) & 0x7ffu);
-    if (f >= 1023 - 95 && f < 1023 + 28) {
+    if (f >= 1023 - 95 && f < 1023 + 20) {
       // hi 2^32 and lo 2^32 (exponent fields offset by +32)
       const float y = __uint_as_float(((uint32_t)(f - 896 + 32) << 23) | (uint32_t)((b >> 29) & 0x7fffffu));
       const float z = f >= 949 ? __int2float_rn((int)(b & 0x1fffffffu)) *
@@ -271,7 +273,7 @@ struct SqAcc {
       const float err = (hi - (s - bp)) + (p - bp);
       hi = s;
       lo += err + (e + c);
-    } else if (f >= 1023 + 28) {
+    } else if (f >= 1023 + 20) {
       big = fma(v, v, big);
     }
   }
@@ -317,7 +319,7 @@ struct SqAcc4 {
     for (int i = 0; i < 4; ++i) {
       const uint32_t bh = (uint32_t)__double2hiint(v[i]), bl = (uint32_t)__double2loint(v[i]);
       const int f = (int)((bh >> 20) & 0x7ffu);
-      const bool far = f >= 1023 + 28;
+      const bool far = f >= 1023 + 20;
       large |= far;
       // as SqAcc::add_f64: values below 2^-95 are left out, the low part of
       // those below 2^-74 as well
@@ -339,7 +341,7 @@ struct SqAcc4 {
     if (large) {
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if ((int)(((uint32_t)__double2hiint(v[i]) >> 20) & 0x7ffu) >= 1023 + 28) big = fma(v[i], v[i], big);
+        if ((int)(((uint32_t)__double2hiint(v[i]) >> 20) & 0x7ffu) >= 1023 + 20) big = fma(v[i], v[i], big);
     }
   }
   __device__ __forceinline__ SqAcc total() const {

@@ -94,3 +94,49 @@ def test_first_product_of_a_process(nb, per_row):
         assert q.get(timeout=180) == "ok"
     finally:
         p.join(30)
+
+
+@pytest.mark.parametrize("bs", [32, 64, 128])
+@pytest.mark.parametrize("v", [2.0 ** 19, 2.0 ** 20, 1.5 * 2.0 ** 26, 1.875 * 2.0 ** 27, 2.0 ** 28, 2.0 ** 40])
+def test_norms_of_large_values(ctx, bs, v):
+    """Block norms of blocks filled with one magnitude: the FP32 sums of squares
+    of a whole warp (up to 2^11 values) stay in range or the values are squared
+    in FP64.  Sums, products in every precision by the identity (exact), narrow
+    tiles, tiles of CTA pairs and of 256 x 256 elements: norms within 2^-36."""
+    from paper_1901_07993_gb300 import ifac
+    sign = np.random.default_rng(4).integers(0, 2, (40 * 40, bs, bs)) * 2.0 - 1.0
+
+    def full_bsr(nb):
+        rp = (np.arange(nb + 1) * nb).astype(np.int32)
+        return synth.HostBSR(nb * bs, bs, rp, np.tile(np.arange(nb), nb).astype(np.int32), v * sign[:nb * nb])
+
+    def eye(nb, filled):  # the identity, stored on every block or on the diagonal
+        if filled:
+            val = np.zeros((nb * nb, bs, bs))
+            val[::nb + 1] = np.eye(bs)
+            return synth.HostBSR(nb * bs, bs, (np.arange(nb + 1) * nb).astype(np.int32),
+                                 np.tile(np.arange(nb), nb).astype(np.int32), val)
+        return synth.HostBSR(nb * bs, bs, np.arange(nb + 1, dtype=np.int32), np.arange(nb, dtype=np.int32),
+                             np.tile(np.eye(bs), (nb, 1, 1)))
+
+    def check(M, nb):
+        want = v * nb * bs
+        assert abs(ifac.bsr_fro(ctx, M) - want) <= 2.0 ** -36 * want
+
+    for nb in (2, 36) if bs == 64 else (2,):
+        V = ifac.upload(ctx, full_bsr(nb))
+        check(ifac.bsr_add(ctx, 1.0, V, 0.0, None, 0.0), nb)
+        check(ifac.bsr_add(ctx, 0.5, V, 0.5, V, 0.0), nb)
+        for prec in (TF32, BF16, FP64_SPLIT):
+            check(ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, eye(nb, False)), False, V, False, 1.0, 0.0, prec), nb)
+    check(ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, eye(2, False)), False, ifac.upload(ctx, full_bsr(2)), False, 1.0, 0.0)
+          if bs < 128 else ifac.bsr_add(ctx, 1.0, ifac.upload(ctx, full_bsr(2)), 0.0, None, 0.0), 2)
+    if bs != 64:
+        return
+    for nb in (20, 36):  # pairs, 256 x 256
+        V, E = ifac.upload(ctx, full_bsr(nb)), ifac.upload(ctx, eye(nb, True))
+        for prec in (TF32, BF16):
+            check(ifac.bsr_gemm_trunc(ctx, E, False, V, False, 1.0, 0.0, prec), nb)
+    U = ifac.upload(ctx, full_bsr(2))
+    for prec in (FP64, TF32, BF16, FP64_SPLIT):
+        check(ifac.bsr_gemm_sym_trunc(ctx, ifac.upload(ctx, eye(2, False)), False, U, False, 1.0, 0.0, prec), 2)
