@@ -1507,15 +1507,18 @@ __device__ __forceinline__ void row_scale_max(uint32_t n1, uint32_t n2, unsigned
   }
 }
 
-// Row scales of a view.  CTA (I, sp) reads part sp of `splits` of block row
-// I's blocks with 16-byte loads; TR: op(X) row r is column r of the stored
-// blocks, a thread takes two columns and every (512 / B)-th row; else eight
-// lanes share a row in segments of 128 bytes.  With splits > 1 -- a matrix of
-// few, long block rows, which would leave most SMs without a CTA -- each
-// part's sums go to `part` and k_row_scale_join adds them in order.  Measured:
-// 3D cluster factor of 4096 rows (64 block rows of 64 blocks) 896 -> 39 us
-// (one CTA of 64 threads per block row before), 262,144-row chain (4096 block
-// rows of three, 400 MB) 212 -> 101 us, rows stored as rows 486 -> 92 us.
+// Row scales of a view.  While its block rows are short, CTA I reads block row I
+// (k_row_scale); else CTA c the view's blocks [c L, (c + 1) L), row by row
+// (k_row_parts).  16-byte loads; TR: op(X) row r is column r of the stored blocks, a
+// thread takes two columns and every (512 / B)-th row; else eight lanes share a
+// row in segments of 128 bytes.  The sums of each block row it meets go to
+// `part`, and k_row_scale_join adds a row's parts in order, so no long row is one
+// CTA's alone.  Measured: 3D cluster factor of 4096 rows (64 block rows of 64
+// blocks) 896 -> 39 us (one CTA of 64 threads per block row before), 262,144-row
+// chain (4096 block rows of three, 400 MB) 212 -> 101 us, rows stored as rows
+// 486 -> 92 us; a product A^T B, bs 64, of 2000 block rows of three and one full
+// block column of A 17.9 -> 1.5 ms in all (one CTA of 256 threads per block row
+// before).
 struct RowPart {
   uint32_t hi, lo;
   int e;  // l1 and sq relative to 2^e and 2^2e
@@ -1589,77 +1592,106 @@ __device__ __forceinline__ RowPart row_scale_part(const int32_t* __restrict__ sr
 
 template <int B, bool TR>
 __global__ void __launch_bounds__(256) k_row_scale(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
-                                                   int splits, const double* __restrict__ val, bool wide,
-                                                   int* __restrict__ eout, unsigned int* __restrict__ l1max,
-                                                   unsigned int* __restrict__ l2max, RowPart* __restrict__ part) {
+                                                   const double* __restrict__ val, bool wide, int* __restrict__ eout,
+                                                   unsigned int* __restrict__ l1max, unsigned int* __restrict__ l2max) {
   __shared__ __align__(16) uint8_t sh[row_scale_smem<B, TR>()];
-  const int I = (int)blockIdx.x / splits, sp = (int)blockIdx.x % splits, tid = threadIdx.x;
-  const int q0 = rp[I], cnt = rp[I + 1] - q0, per = (cnt + splits - 1) / splits;
-  const int qa = min(q0 + sp * per, q0 + cnt), qe = min(qa + per, q0 + cnt);
-  const RowPart t = row_scale_part<B, TR>(src, qa, qe, val, wide, sh);
+  const int I = (int)blockIdx.x, tid = threadIdx.x, q0 = rp[I], q1 = rp[I + 1];
+  const RowPart t = row_scale_part<B, TR>(src, q0, q1, val, wide, sh);
   if (tid >= B) return;
-  const size_t row = (size_t)I * B + tid;
-  if (splits == 1) {
-    uint32_t n1, n2;
-    eout[row] = t.e;
-    row_bounds((t.hi | t.lo) != 0u, t.e, t.l1, t.sq, cnt * B, n1, n2);
-    row_scale_max(n1, n2, l1max, l2max);
-  } else {
-    part[(size_t)sp * (gridDim.x / splits) * B + row] = t;
+  uint32_t n1, n2;
+  eout[(size_t)I * B + tid] = t.e;
+  row_bounds((t.hi | t.lo) != 0u, t.e, t.l1, t.sq, (q1 - q0) * B, n1, n2);
+  row_scale_max(n1, n2, l1max, l2max);
+}
+
+// part[(c + I) B + r]: CTA c's sums of row r of block row I (c + I grows from
+// each segment to the next, so no two share a place)
+template <int B, bool TR>
+__global__ void __launch_bounds__(256) k_row_parts(const int32_t* __restrict__ rp, const int32_t* __restrict__ src,
+                                                   int nb, int nblk, int L, const double* __restrict__ val, bool wide,
+                                                   RowPart* __restrict__ part) {
+  __shared__ __align__(16) uint8_t sh[row_scale_smem<B, TR>()];
+  const int c = (int)blockIdx.x, qe = min((c + 1) * L, nblk), lane = threadIdx.x & 31;
+  int I = 0, end = nb;  // the row that holds block c L: the last with rp[I] <= c L
+  while (end - I > 1) {  // (every warp by itself, 32 probes at a time)
+    const int step = (end - I + 31) / 32, p = I + lane * step;
+    const unsigned m = __ballot_sync(0xffffffffu, p < end && rp[p] <= c * L);
+    I += (31 - __clz((int)m)) * step;  // (probe 0 holds)
+    end = min(end, I + step);
+  }
+  for (int q = c * L; q < qe; ++I) {
+    const int q1 = min(rp[I + 1], qe);
+    if (q1 <= q) continue;  // an empty row
+    const RowPart t = row_scale_part<B, TR>(src, q, q1, val, wide, sh);
+    if (threadIdx.x < B) part[(size_t)(c + I) * B + threadIdx.x] = t;
+    q = q1;
   }
 }
 
 // the parts of every row joined, in order (nrows is a multiple of 32)
-__global__ void k_row_scale_join(const int32_t* __restrict__ rp, int bs, int64_t nrows, int splits,
+__global__ void k_row_scale_join(const int32_t* __restrict__ rp, int bs, int64_t nrows, int L,
                                  const RowPart* __restrict__ part, int* __restrict__ eout,
                                  unsigned int* __restrict__ l1max, unsigned int* __restrict__ l2max) {
   const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (r >= nrows) return;
+  const int I = (int)(r / bs), q0 = rp[I], q1 = rp[I + 1];
+  const int c0 = q0 / L, n = q1 > q0 ? (q1 - 1) / L - c0 + 1 : 0;
+  const RowPart* p = part + (size_t)(c0 + I) * bs + r % bs;
   uint32_t hi = 0, lo = 0;
-  for (int s = 0; s < splits; ++s) {
-    hi = max(hi, part[s * nrows + r].hi);
-    lo |= part[s * nrows + r].lo;
+#pragma unroll 8
+  for (int s = 0; s < n; ++s) {
+    hi = max(hi, p[(size_t)s * bs].hi);
+    lo |= p[(size_t)s * bs].lo;
   }
   const int e = row_exponent(hi, lo);
   float l1 = 0.0f, sq = 0.0f;
-  for (int s = 0; s < splits; ++s) {
-    const RowPart p = part[s * nrows + r];
-    l1 += scale_f32(p.l1, p.e - e);
-    sq += scale_f32(p.sq, 2 * (p.e - e));
+#pragma unroll 4
+  for (int s = 0; s < n; ++s) {
+    const RowPart t = p[(size_t)s * bs];
+    l1 += scale_f32(t.l1, t.e - e);
+    sq += scale_f32(t.sq, 2 * (t.e - e));
   }
-  const int I = (int)(r / bs);
   uint32_t n1, n2;
   eout[r] = e;
-  row_bounds((hi | lo) != 0u, e, l1, sq, (rp[I + 1] - rp[I]) * bs, n1, n2);
+  row_bounds((hi | lo) != 0u, e, l1, sq, (q1 - q0) * bs, n1, n2);
   row_scale_max(n1, n2, l1max, l2max);
 }
 
-template <int B>
-static void launch_row_scale(ifac_ctx* ctx, const int32_t* rp, const int32_t* src, int nb, int splits, bool tr,
-                             const double* val, int* eout, unsigned int* l1max, unsigned int* l2max,
-                             RowPart* part) {
-  const int grid = nb * splits;
-  const bool wide = aligned16(val);
-  if (tr) k_row_scale<B, true><<<grid, 256, 0, ctx->stream>>>(rp, src, splits, val, wide, eout, l1max, l2max, part);
-  else k_row_scale<B, false><<<grid, 256, 0, ctx->stream>>>(rp, src, splits, val, wide, eout, l1max, l2max, part);
-  IFAC_CK_LAUNCH();
+// Whether one CTA for each block row will do: the longest row (-1: not known)
+// holds no more blocks than a quarter of an SM's share of them all, or 16.
+static bool rows_short(int nb, int64_t nnzb, int longest) {
+  return (longest < 0 ? nb : longest) <= std::max<int64_t>(16, nnzb / (4 * 152));
 }
 
 // sigma exponents (and the scaled norm bounds) of the rows of a row view of nnzb blocks
-static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, int nb, int64_t nnzb, bool tr,
-                       const double* val, int* eout, unsigned int* l1max, unsigned int* l2max) {
-  const int64_t rows = (int64_t)nb * bs;
-  // about four CTAs per SM, each with at least two blocks of its row
-  const int splits = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(4 * 152, nb), nnzb / (2 * (int64_t)nb)));
-  Buf<RowPart> part;
-  if (splits > 1) part = Buf<RowPart>(ctx, rows * splits);
-  if (bs == 32) launch_row_scale<32>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
-  else if (bs == 64) launch_row_scale<64>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
-  else launch_row_scale<128>(ctx, rp, src, nb, splits, tr, val, eout, l1max, l2max, part.p);
-  if (splits > 1) {
-    k_row_scale_join<<<cdiv(rows, 128), 128, 0, ctx->stream>>>(rp, bs, rows, splits, part.p, eout, l1max, l2max);
-    IFAC_CK_LAUNCH();
+static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, int nb, int64_t nnzb, int longest,
+                       bool tr, const double* val, int* eout, unsigned int* l1max, unsigned int* l2max) {
+  const bool wide = aligned16(val);
+  const auto pick = [&](auto k32t, auto k32, auto k64t, auto k64, auto k128t, auto k128, auto go) {
+    if (bs == 32) tr ? go(k32t) : go(k32);
+    else if (bs == 64) tr ? go(k64t) : go(k64);
+    else tr ? go(k128t) : go(k128);
+  };
+  if (rows_short(nb, nnzb, longest)) {
+    pick(k_row_scale<32, true>, k_row_scale<32, false>, k_row_scale<64, true>, k_row_scale<64, false>,
+         k_row_scale<128, true>, k_row_scale<128, false>, [&](auto kernel) {
+           kernel<<<nb, 256, 0, ctx->stream>>>(rp, src, val, wide, eout, l1max, l2max);
+           IFAC_CK_LAUNCH();
+         });
+    return;
   }
+  // about four CTAs per SM, each with 2 to 32 blocks
+  const int64_t rows = (int64_t)nb * bs;
+  const int L = (int)std::max<int64_t>(2, std::min<int64_t>(32, nnzb / (4 * 152)));
+  const int grid = cdiv(std::max<int64_t>(nnzb, 1), L);
+  Buf<RowPart> part(ctx, (size_t)(grid + nb) * bs);
+  pick(k_row_parts<32, true>, k_row_parts<32, false>, k_row_parts<64, true>, k_row_parts<64, false>,
+       k_row_parts<128, true>, k_row_parts<128, false>, [&](auto kernel) {
+         kernel<<<grid, 256, 0, ctx->stream>>>(rp, src, nb, (int)nnzb, L, val, wide, part.p);
+         IFAC_CK_LAUNCH();
+       });
+  k_row_scale_join<<<cdiv(rows, 128), 128, 0, ctx->stream>>>(rp, bs, rows, L, part.p, eout, l1max, l2max);
+  IFAC_CK_LAUNCH();
 }
 
 // NS BF16 slice copies (K-major, op() CSR order) of a view; row r of a block
@@ -1866,11 +1898,15 @@ static void split_blocks(ifac_ctx* ctx, int bs, const double* val, const int32_t
 
 // Scales and slices of a view (rows rp, blocks src of nblk) in one launch, when
 // its block rows are short and many enough for one CTA each; false where the
-// two kernels are to be used.
+// two kernels are to be used.  A CTA takes 4 to 6 us for a block of 64, so none
+// may get a long row (rows_short): S S with one full block row among 2000 of
+// three blocks took 16.0 ms in one kernel and takes 1.5 ms in two.
+static bool split_rows_sizes(int nb, int64_t nblk) { return nb >= 2 * 152 && nblk <= 8 * (int64_t)nb; }
+
 static bool split_rows(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* src, const int32_t* out, int nb,
-                       int64_t nblk, bool tr, const double* val, int ns, int* eout, unsigned int* l1max,
+                       int64_t nblk, int longest, bool tr, const double* val, int ns, int* eout, unsigned int* l1max,
                        unsigned int* l2max, void* dst) {
-  if (nb < 2 * 152 || nblk > 8 * (int64_t)nb) return false;
+  if (!split_rows_sizes(nb, nblk) || !rows_short(nb, nblk, longest)) return false;
   __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(dst);
   const bool wide = aligned32(val);
   const auto go = [&](auto kernel) {
@@ -2611,28 +2647,32 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   Buf<unsigned int> l1(ctx, 4);
   IFAC_CK(cudaMemsetAsync(l1.p, 0, 4 * sizeof(unsigned int), ctx->stream));
   // slices: row scale block of an op(A) entry is its CSR row; of an op(B) entry its CSR column
+  // (the columns of op(B) are the rows of the other view, made first so that
+  // the host has its longest row when op(A)'s slices are under way)
+  View bt = view_rows(ctx, B, !tB, nb > 16);
+  if (tB) bt.longest = brows.longest_col;
   const size_t bbytes = (size_t)bs * bs * 2;
   Buf<uint8_t> la, lb(ctx, (size_t)ns * (B.nnzb + 1) * bbytes);
   if (!hit) {
     sige = Buf<int>(ctx, rows);
     la = Buf<uint8_t>(ctx, (size_t)nsa * (A.nnzb + 1) * bbytes);
     const int32_t* as = value_src(ctx, arows.src, avmap, A.nnzb, asrc);
-    if (!split_rows(ctx, bs, arows.rp, as, nullptr, nb, A.nnzb, tA, A.val, nsa, sige.p, l1.p, l1.p + 2, la.p)) {
-      row_scales(ctx, bs, arows.rp, as, nb, A.nnzb, tA, A.val, sige.p, l1.p, l1.p + 2);
+    if (!split_rows(ctx, bs, arows.rp, as, nullptr, nb, A.nnzb, arows.longest, tA, A.val, nsa, sige.p, l1.p, l1.p + 2,
+                    la.p)) {
+      row_scales(ctx, bs, arows.rp, as, nb, A.nnzb, arows.longest, tA, A.val, sige.p, l1.p, l1.p + 2);
       Buf<int32_t> arow(ctx, A.nnzb);
       expand_rows(ctx, arows.rp, nb, arow.p);
       split_blocks(ctx, bs, A.val, as, A.nnzb, tA, arow.p, sige.p, nsa, la.p);
     }
   }
   {
-    // (the columns of op(B) are the rows of the other view; with op(B) = B its
-    // entries' copies lie in B's stored order)
-    View bt = view_rows(ctx, B, !tB);
+    // (with op(B) = B the view's entries' copies lie in B's stored order)
+    if (!tB && nb > 16) bt.longest = read_word(ctx, HW_LONGEST_B);
     Buf<int32_t> btsrc;
     const int32_t* bs_ = value_src(ctx, bt.src, bvmap, B.nnzb, btsrc);
-    if (tB || !split_rows(ctx, bs, bt.rp, bs_, bt.src, nb, B.nnzb, true, B.val, ns, taue.p, l1.p + 1, l1.p + 3,
-                          lb.p)) {
-      row_scales(ctx, bs, bt.rp, bs_, nb, B.nnzb, !tB, B.val, taue.p, l1.p + 1, l1.p + 3);
+    if (tB || !split_rows(ctx, bs, bt.rp, bs_, bt.src, nb, B.nnzb, bt.longest, true, B.val, ns, taue.p,
+                               l1.p + 1, l1.p + 3, lb.p)) {
+      row_scales(ctx, bs, bt.rp, bs_, nb, B.nnzb, bt.longest, !tB, B.val, taue.p, l1.p + 1, l1.p + 3);
       split_blocks(ctx, bs, B.val, value_src(ctx, brows.src, bvmap, B.nnzb, bsrc), B.nnzb, !tB, brows.ci, taue.p, ns,
                    lb.p);
     }

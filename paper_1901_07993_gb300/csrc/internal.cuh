@@ -161,7 +161,7 @@ void to_host_many(ifac_ctx* ctx, std::initializer_list<HostRead> reads);
 // for the value itself, not for the stream: the host goes on to the next
 // launches while the kernel that wrote it drains, where a synchronisation
 // costs 10 us between two kernels.
-enum HostWord { HW_NNZ = 0, HW_KEPT, HW_PLAN, HW_KMAX, HW_COUNT };
+enum HostWord { HW_NNZ = 0, HW_KEPT, HW_PLAN, HW_KMAX, HW_LONGEST_A, HW_LONGEST_B, HW_COUNT };
 int32_t* host_word(ifac_ctx* ctx, HostWord w);
 int32_t read_word(ifac_ctx* ctx, HostWord w);
 
@@ -173,18 +173,25 @@ struct View {
   const int32_t* ci = nullptr;
   const int32_t* src = nullptr;  // nullptr = identity
   Buf<int32_t> own_rp, own_ci, own_src;
+  // blocks of the longest row, and of the longest column, where asked for (else -1)
+  int longest = -1, longest_col = -1;
 };
-View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans);
+// want_longest (a transposed view): the blocks of its longest row go to
+// HW_LONGEST_B, for the caller to read
+View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans, bool want_longest = false);
 // Row pattern from a bitmap: allocates and fills rp[nb+1], ci[nnzb].
 struct Pattern {
   Buf<int32_t> rp, ci, row;
   int64_t nnzb = 0;
+  // a product, where asked for: blocks of op(A)'s longest row, and, for op(B) =
+  // B^T, of op(B)'s longest column
+  int longest_a = -1, longest_b = -1;
 };
 Pattern pattern_from_bitmap(ifac_ctx* ctx, const uint32_t* bm, int nb);
 // Symbolic product pattern of op(A) op(B); upper: only the blocks (I, J)
 // with J >= I.
 Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const ifac_bsr& B, bool transB, int nb,
-                        bool upper = false);
+                        bool upper = false, bool want_longest = false);
 // Union pattern of A, B (nullable) and the diagonal (if diag).
 Pattern union_pattern(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr* B, bool diag);
 // Pattern of U + U^T, B (nullable) and the diagonal (if diag).

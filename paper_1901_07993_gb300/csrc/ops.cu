@@ -30,7 +30,8 @@ Mat gemm(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, 
   if (b32 && !lowp) fail(IFAC_ERR_INVALID, "FP32 operand values: TF32/BF16 products only");
   out32 = out32 && lowp && nocopy;  // compaction copies would move FP64 values
   View arows = view_rows(ctx, A, tA);
-  Pattern P = product_pattern(ctx, arows, A.nnzb, B, tB, nb, upper);
+  Pattern P = product_pattern(ctx, arows, A.nnzb, B, tB, nb, upper, prec == IFAC_FP64_SPLIT);
+  arows.longest = P.longest_a;
   Mat C(ctx);
   C.m.n = A.n;
   C.m.bs = A.bs;
@@ -57,6 +58,7 @@ Mat gemm(ifac_ctx* ctx, const ifac_bsr& A, bool tA, const ifac_bsr& B, bool tB, 
     gemm_numeric_fp64(ctx, arows, tA, A, bcols, tB, B, alpha, C.m, P.row.p, ctx->dev_pairs);
   } else {
     View brows = view_rows(ctx, B, tB);
+    brows.longest_col = P.longest_b;
     gemm_numeric_tc(ctx, prec, arows, tA, A, brows, tB, B, alpha, C.m, P.row.p, upper,
                     ctx->dev_pairs + (prec == IFAC_FP64_SPLIT ? 2 : 1), acache, bcache, bpre, avmap, bvmap, out32,
                     b32);

@@ -52,6 +52,10 @@ struct Job {
   const int32_t* fci;
   int32_t* src;
   int32_t* total;       // host word, or null
+  // host words (or null) for the blocks of the longest row of lrp, or of the
+  // pattern itself (lrp null)
+  const int32_t* lrp[2];
+  int32_t* longest[2];
 };
 
 __device__ __forceinline__ uint32_t upper_bits(uint32_t v, int row, int w) {
@@ -87,7 +91,7 @@ __device__ __forceinline__ void emit(const Job& j, uint32_t word, int r, int w, 
 // for each (nb = 512: 20 us that way).
 __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
   extern __shared__ uint32_t sh[];
-  __shared__ int32_t wsum[32];
+  __shared__ int32_t wsum[32], wlen[2][32];
   const int WP = j.W | 1, nw = j.nb * WP;           // odd row stride: no bank conflicts across rows
   uint32_t* bm = sh;                                // [nb * WP] the sources
   int32_t* off = reinterpret_cast<int32_t*>(bm + nw);  // [nb + 1]
@@ -136,7 +140,18 @@ __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
     if (lane >= o) x += y;
   }
   if (lane == 31) wsum[wid] = x;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (j.longest[i]) {
+      const int len = tid >= j.nb ? 0 : j.lrp[i] ? j.lrp[i][tid + 1] - j.lrp[i][tid] : c;
+      const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)len);
+      if (lane == 0) wlen[i][wid] = m;
+    }
   __syncthreads();
+  if (wid < 2 && j.longest[wid]) {
+    const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)wlen[wid][lane]);
+    if (lane == 0) *j.longest[wid] = m;
+  }
   const int run = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < wid ? wsum[lane] : 0)) + x - c;
   if (tid < j.nb) {
     off[tid] = run;
@@ -179,12 +194,13 @@ __global__ void __launch_bounds__(NT) k_scatter(Job j, uint32_t* __restrict__ bm
 }
 
 // the product's rows, out[I] = OR over K in row I of op(A) of bm[K] (or bm
-// itself), their counts and the row pointers
+// itself), their counts and the row pointers; ticket[1] and [2] are zero between launches
 __global__ void __launch_bounds__(NT) k_rows_scan(Job j, const uint32_t* __restrict__ bm, uint32_t* __restrict__ out,
                                                   int32_t* __restrict__ cnt, unsigned* __restrict__ ticket) {
+  __shared__ int32_t wlen[2][NT / 32];
   const int row = (int)((blockIdx.x * (size_t)NT + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  int c = 0;
   if (row < j.nb) {
-    int c = 0;
     const int p0 = j.arp ? j.arp[row] : 0, p1 = j.arp ? j.arp[row + 1] : 0;
     for (int w = lane; w < j.W; w += 32) {
       uint32_t acc = 0;
@@ -201,7 +217,20 @@ __global__ void __launch_bounds__(NT) k_rows_scan(Job j, const uint32_t* __restr
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if (lane == 0) cnt[row] = c;
   }
-  scan_tail<NT>(cnt, j.rp, j.nb, ticket, j.total);
+  int* const lmax = reinterpret_cast<int*>(ticket + 1);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (j.longest[i] && lane == 0)
+      wlen[i][threadIdx.x >> 5] = row >= j.nb ? 0 : j.lrp[i] ? j.lrp[i][row + 1] - j.lrp[i][row] : c;
+  if (j.longest[0] || j.longest[1]) __syncthreads();
+  if (threadIdx.x < 2 && j.longest[threadIdx.x]) {  // one atomic for each CTA
+    int len = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) len = max(len, wlen[threadIdx.x][w]);
+    atomicMax(lmax + threadIdx.x, len);
+  }
+  if (scan_tail<NT>(cnt, j.rp, j.nb, ticket, j.total) && threadIdx.x < 2 && j.longest[threadIdx.x])
+    *j.longest[threadIdx.x] = atomicExch(lmax + threadIdx.x, 0);
 }
 
 // enumerate the set bits of each row in increasing column (warp per row)
@@ -251,6 +280,7 @@ void launch_small(ifac_ctx* ctx, const Job& j, int64_t nnza) {
 // The pattern of a job: known >= 0 the number of its blocks where the host
 // knows it (a transposed view), so nothing is read back; guess what it will
 // be about, cap its bound.
+// j's longest[] are set by the caller.
 Pattern run_job(ifac_ctx* ctx, Job j, int64_t in_blocks, int64_t guess, int64_t cap, int64_t known,
                 Buf<int32_t>* src, int64_t nnza = 0) {
   Pattern P;
@@ -336,7 +366,7 @@ void transposed_positions(ifac_ctx* ctx, const ifac_bsr& A, const int32_t* row, 
   IFAC_CK_LAUNCH();
 }
 
-View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
+View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans, bool want_longest) {
   View v;
   if (!trans) {
     v.rp = A.row_ptr;
@@ -349,6 +379,7 @@ View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
   add_source(j, A.row_ptr, A.col_idx, A.nnzb, true);
   j.frp = A.row_ptr;
   j.fci = A.col_idx;
+  if (want_longest) j.longest[0] = host_word(ctx, HW_LONGEST_B);
   Pattern P = run_job(ctx, j, A.nnzb, A.nnzb, A.nnzb, A.nnzb, &v.own_src);  // A^T has A's blocks
   v.own_rp = std::move(P.rp);
   v.own_ci = std::move(P.ci);
@@ -362,7 +393,7 @@ View view_rows(ifac_ctx* ctx, const ifac_bsr& A, bool trans) {
 // product and union patterns
 // ---------------------------------------------------------------------------
 Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const ifac_bsr& B, bool transB, int nb,
-                        bool upper) {
+                        bool upper, bool want_longest) {
   Job j{};
   j.nb = nb;
   add_source(j, B.row_ptr, B.col_idx, B.nnzb, transB);
@@ -372,7 +403,19 @@ Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const if
   // a row of op(A) with k blocks meets about k nnz(B) / nb of op(B); what the
   // lists may hold is nb^2 (at most 1 MB where one CTA writes them)
   const int64_t full = (int64_t)nb * nb, guess = std::min(full, nnza * std::max<int64_t>(1, B.nnzb / nb));
-  return run_job(ctx, j, std::max(nnza, B.nnzb), guess, full, -1, nullptr, nnza);
+  const bool want_a = want_longest, want_b = want_longest && transB;
+  if (want_a) {
+    j.lrp[0] = arows.rp;
+    j.longest[0] = host_word(ctx, HW_LONGEST_A);
+  }
+  if (want_b) {
+    j.lrp[1] = B.row_ptr;
+    j.longest[1] = host_word(ctx, HW_LONGEST_B);
+  }
+  Pattern P = run_job(ctx, j, std::max(nnza, B.nnzb), guess, full, -1, nullptr, nnza);
+  if (want_a) P.longest_a = read_word(ctx, HW_LONGEST_A);  // (written with the total)
+  if (want_b) P.longest_b = read_word(ctx, HW_LONGEST_B);
+  return P;
 }
 
 Pattern union_pattern(ifac_ctx* ctx, const ifac_bsr& A, const ifac_bsr* B, bool diag) {

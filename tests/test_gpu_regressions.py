@@ -140,3 +140,47 @@ def test_norms_of_large_values(ctx, bs, v):
     U = ifac.upload(ctx, full_bsr(2))
     for prec in (FP64, TF32, BF16, FP64_SPLIT):
         check(ifac.bsr_gemm_sym_trunc(ctx, ifac.upload(ctx, eye(2, False)), False, U, False, 1.0, 0.0, prec), 2)
+
+
+@pytest.mark.parametrize("bs,nb", [(64, 400), (32, 700)])
+@pytest.mark.parametrize("tA,tB", [(False, False), (True, False), (False, True), (True, True)])
+def test_split_operand_with_one_long_row(ctx, bs, nb, tA, tB):
+    """Split products of an operand with one full block row among short ones:
+    values within K 2^-(7 s - 5) r_i c_j + 2 K 2^-53 (|A||B|)_ij (K scalar
+    terms, s = 7), and no more than six times the time of the same number of
+    blocks in short rows (one CTA for every block of the long row: 20 times and
+    more)."""
+    import time
+
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    band = np.abs(np.subtract.outer(np.arange(nb), np.arange(nb)))
+    long_row = band <= 1
+    long_row[nb // 2] = True
+
+    def make(mask, seed):
+        rows, cols = np.nonzero(mask)
+        rp = np.concatenate([[0], np.cumsum(mask.sum(axis=1))]).astype(np.int32)
+        v = np.random.default_rng(seed).standard_normal((len(rows), bs, bs))
+        return synth.HostBSR(nb * bs, bs, rp, cols.astype(np.int32), v)
+
+    A, B, even = make(long_row, 1), make(band <= 1, 2), make(band <= 1, 3)
+    dA, dB, dE = ifac.upload(ctx, A), ifac.upload(ctx, B), ifac.upload(ctx, even)
+    prod = lambda X: ifac.bsr_gemm_trunc(ctx, X, tA, dB, tB, 1.0, 0.0, FP64_SPLIT)
+    got, ref = prod(dA).download(), oracle.gemm(A, B, tA, tB, 1.0, 0.0)
+    assert np.array_equal(got.row_ptr, ref.row_ptr) and np.array_equal(got.col_idx, ref.col_idx)
+    K = nb * bs
+    mx = [np.abs(M.val).max() for M in (A, B)]
+    assert np.abs(got.val - ref.val).max() <= (K * 2.0 ** -44 + 2 * K * 2.0 ** -53 * K) * mx[0] * mx[1]
+
+    def best(X):
+        t = []
+        for _ in range(6):
+            torch.cuda.synchronize()
+            a = time.perf_counter()
+            prod(X)
+            torch.cuda.synchronize()
+            t.append(time.perf_counter() - a)
+        return min(t)
+
+    assert best(dA) <= 6 * best(dE)
