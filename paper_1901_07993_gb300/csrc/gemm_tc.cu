@@ -1437,6 +1437,9 @@ __device__ __forceinline__ double2 load_pair(const double* p, bool wide) {
   return make_double2(p[0], p[1]);
 }
 
+// blocks whose values one thread may add up in FP32 (row_bounds)
+constexpr int ROW_BLOCKS = 32;
+
 // x 2^k in FP32, k of any size (sums are non-negative; too large: infinity)
 __device__ __forceinline__ float scale_f32(float x, int k) {
   return x == 0.0f ? 0.0f : ldexpf(x, max(-2000, min(2000, k)));
@@ -1489,11 +1492,15 @@ __device__ __forceinline__ void row_bounds(bool any, int e, float l1, float sq, 
     n1 = n2 = __float_as_uint(3.0e38f);
     return;
   }
-  // magnitudes are truncated to 24 bits and the FP32 sums rounded: 1e-3 covers
-  // both; values left out of a sum are below 2^-126 (2^-63 for the squares) of
-  // a value of the row
-  n1 = __float_as_uint(fminf(l1 * 1.001f + (float)nscalars * 1.2e-38f, 3.0e38f));
-  n2 = __float_as_uint(fminf(sqrtf(sq + (float)nscalars * 1.2e-38f) * 1.001f + 1e-30f, 3.0e38f));
+  // The sums decide how many bits the fixed-point sums of a product keep, so
+  // the bounds are tight: magnitudes are truncated to 24 bits (1.2e-7), a thread
+  // adds at most ROW_BLOCKS blocks (1024 values: 6.1e-5 of the squares' sum,
+  // 3.1e-5 of its root), and the few partial sums that follow add 1e-6; 5e-5
+  // covers them.  (The 1-norm's like share is within the margin its user adds.)
+  // Values left out of a sum are below 2^-126 (2^-63 for the squares) of a
+  // value of the row.
+  n1 = __float_as_uint(fminf(l1 + (float)nscalars * 1.2e-38f, 3.0e38f));
+  n2 = __float_as_uint(fminf(sqrtf(sq + (float)nscalars * 1.2e-38f) * 1.00005f + 1e-30f, 3.0e38f));
 }
 
 // the warp's largest norm bounds, one atomic each (32 rows' atomics on one
@@ -1644,12 +1651,14 @@ __global__ void k_row_scale_join(const int32_t* __restrict__ rp, int bs, int64_t
     lo |= p[(size_t)s * bs].lo;
   }
   const int e = row_exponent(hi, lo);
-  float l1 = 0.0f, sq = 0.0f;
+  float l1 = 0.0f, sq = 0.0f, rest = 0.0f;  // (a row may have thousands of parts: what each add of squares loses is kept)
 #pragma unroll 4
   for (int s = 0; s < n; ++s) {
     const RowPart t = p[(size_t)s * bs];
     l1 += scale_f32(t.l1, t.e - e);
-    sq += scale_f32(t.sq, 2 * (t.e - e));
+    const float y = scale_f32(t.sq, 2 * (t.e - e)) - rest, z = sq + y;
+    rest = (z - sq) - y;
+    sq = z;
   }
   uint32_t n1, n2;
   eout[r] = e;
@@ -1658,9 +1667,10 @@ __global__ void k_row_scale_join(const int32_t* __restrict__ rp, int bs, int64_t
 }
 
 // Whether one CTA for each block row will do: the longest row (-1: not known)
-// holds no more blocks than a quarter of an SM's share of them all, or 16.
+// holds no more blocks than a quarter of an SM's share of them all, or 16, and
+// no more than a thread may add up.
 static bool rows_short(int nb, int64_t nnzb, int longest) {
-  return (longest < 0 ? nb : longest) <= std::max<int64_t>(16, nnzb / (4 * 152));
+  return (longest < 0 ? nb : longest) <= std::min<int64_t>(ROW_BLOCKS, std::max<int64_t>(16, nnzb / (4 * 152)));
 }
 
 // sigma exponents (and the scaled norm bounds) of the rows of a row view of nnzb blocks
@@ -1680,9 +1690,9 @@ static void row_scales(ifac_ctx* ctx, int bs, const int32_t* rp, const int32_t* 
          });
     return;
   }
-  // about four CTAs per SM, each with 2 to 32 blocks
+  // about four CTAs per SM, each with 2 to ROW_BLOCKS blocks
   const int64_t rows = (int64_t)nb * bs;
-  const int L = (int)std::max<int64_t>(2, std::min<int64_t>(32, nnzb / (4 * 152)));
+  const int L = (int)std::max<int64_t>(2, std::min<int64_t>(ROW_BLOCKS, nnzb / (4 * 152)));
   const int grid = cdiv(std::max<int64_t>(nnzb, 1), L);
   Buf<RowPart> part(ctx, (size_t)(grid + nb) * bs);
   pick(k_row_parts<32, true>, k_row_parts<32, false>, k_row_parts<64, true>, k_row_parts<64, false>,

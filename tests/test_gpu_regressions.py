@@ -184,3 +184,54 @@ def test_split_operand_with_one_long_row(ctx, bs, nb, tA, tB):
         return min(t)
 
     assert best(dA) <= 6 * best(dE)
+
+
+def test_split_fixed_point_bits():
+    """The fixed-point sums keep f = 62 - ceil(log2(1.125 b + 2)) bits, b the
+    product of the largest scaled row and column 2-norms, each widened by 0.0125
+    sqrt(K) and rounded up by no more than 1e-4.  Here 1.125 b + 2 = 128 (1 -
+    1e-4) for norms rounded up by 1e-4, so f = 55: the entries (sums that cancel
+    to v 2^-28, v an odd multiple of 2^-27) are multiples of 2^-55 and come out
+    exactly; one bit less and each is off by 2^-55."""
+    from paper_1901_07993_gb300 import ifac
+    ctx = ifac.Context()
+    ctx.set_split_slices(8)
+    nb, bs = 3, 64
+    K = nb * bs
+    rk = 0.0125 * np.sqrt(K)
+    v = (np.sqrt((128 * (1 - 1e-4) - 2) / 1.125) - rk) / (np.sqrt(K) * 1.0001)
+    v = (round(v * 2 ** 27) | 1) / 2.0 ** 27
+    j = np.arange(K)
+    Ad = np.full((K, K), v)
+    Bd = np.where((j[:, None] + j[None, :]) % 2 == 1, v, -v)
+    Bd[j, j] += 2.0 ** -28
+    rp, ci = (np.arange(nb + 1) * nb).astype(np.int32), np.tile(np.arange(nb), nb).astype(np.int32)
+    blocks = lambda D: D.reshape(nb, bs, nb, bs).transpose(0, 2, 1, 3).reshape(nb * nb, bs, bs).copy()
+    A, B = (ifac.upload(ctx, synth.HostBSR(K, bs, rp, ci, blocks(D))) for D in (Ad, Bd))
+    for X, tX, Y, tY in ((A, False, B, False), (A, True, B, False), (A, False, B, True)):
+        got = ifac.bsr_gemm_trunc(ctx, X, tX, Y, tY, 1.0, 0.0, FP64_SPLIT).download()
+        assert np.array_equal(got.val, np.full((nb * nb, bs, bs), v * 2.0 ** -28))
+
+
+@pytest.mark.parametrize("bs,nb", [(32, 2), (64, 700), (128, 40)])
+def test_split_norm_bounds_hold(bs, nb):
+    """The bounds of rows with many values are bounds: all-equal rows, long
+    enough that FP32 sums of their squares round the same way again and again,
+    and rows whose largest value comes last; no overflow of the fixed-point sums
+    and values within the slices' bound."""
+    from paper_1901_07993_gb300 import ifac
+    ctx = ifac.Context()
+    rng = np.random.default_rng(9)
+    rows = np.concatenate([np.zeros(nb, int), np.arange(1, nb)])  # block row 0 full, the others one block
+    cols = np.concatenate([np.arange(nb), np.zeros(nb - 1, int)])
+    order = np.lexsort((cols, rows))
+    rows, cols = rows[order], cols[order]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=nb))]).astype(np.int32)
+    val = np.full((len(rows), bs, bs), 1.0 - 2.0 ** -24)
+    val[rows > 0] = rng.standard_normal((int((rows > 0).sum()), bs, bs)) * np.exp2(np.linspace(-60, 0, bs))
+    A = synth.HostBSR(nb * bs, bs, rp, cols.astype(np.int32), val)
+    dA = ifac.upload(ctx, A)
+    got, ref = ifac.bsr_gemm_trunc(ctx, dA, False, dA, True, 1.0, 0.0, FP64_SPLIT).download(), oracle.gemm(A, A, False, True)
+    K = nb * bs
+    top = np.abs(A.val).max()
+    assert np.abs(got.val - ref.val).max() <= (K * 2.0 ** -44 + 2 * K * 2.0 ** -53 * K) * top ** 2
