@@ -8,18 +8,23 @@
 // right-looking.  X(r, k) names tile (r, k) of the array: below the diagonal
 // it holds A, then L; above it B^T, then W^T (= Z), B the right-hand side
 // that starts as the identity.  Step k:
-//   1. column k is scaled, X(r, k) <- X(r, k) W_kk^T for every r != k (L_ik
-//      below the diagonal, Z_ck above), one tile per CTA;
+//   1. column k: below the diagonal Y L_kk^T = X(r, k) is solved by substitution
+//      (Y = L_rk), above it X(r, k) <- X(r, k) W_kk^T (Z_rk), one tile per CTA;
 //   2. X(r, j) -= X(r, k) X(j, k)^T for every j > k and r <= k (B, with
 //      X(k, k) = W_kk^T and B_jk = 0 before) or r >= j (A); tile (k+1, k+1)
-//      first, and CTA 0 factors it at once (W_kk = L_kk^-1 for the next step)
-//      while the others go on, so the serial chain of pivots overlaps the
-//      updates.
+//      first, and CTA 0 factors it at once (L_kk and W_kk = L_kk^-1 for the
+//      next step) while the others go on, so the serial chain of pivots overlaps
+//      the updates.
+// For accuracy a tile product is summed by itself and subtracted once (one chain
+// of FMAs through all of a tile's products loses a factor of three on 3D
+// leaves), and neither the panel nor the pivots go through a reciprocal: the
+// panel times W_kk^T loses up to a factor of 15 in Z on chains of condition
+// 1e6 and more.
 // Every step has T^2 / 2 to T tile products (T = nl / 32); the columns of W
-// after all of L would be chains of very different length.  Measured (one CTA
-// per matrix before): 8 leaves of 512 rows 16.3 -> 1.45 ms (0.50 TFLOP/s of
-// the FP64 pipe's 1.25), one 16.2 -> 1.06 ms, 64 leaves 16.6 -> 7.2 ms, one of
-// 128 rows 597 -> 155 us, one of 1024 rows 114 -> 6.8 ms.
+// after all of L would be chains of very different length.  Call times against
+// one CTA per matrix: 8 leaves of 512 rows 15.9 -> 1.65 ms (0.43 TFLOP/s of the
+// FP64 pipe's 1.25), one 15.9 -> 1.30 ms, 32 leaves 16.0 -> 4.1 ms, one of 128
+// rows 572 -> 224 us, one of 1024 rows 113 -> 7.3 ms, 1000 of 32 rows 227 -> 202 us.
 //
 // A non-positive pivot j sets info = j + 1 (the pivot is replaced by 1 so the
 // arithmetic stays finite; that matrix's Z is then meaningless).
@@ -50,17 +55,32 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// x / d from r ~ 1 / d: one Newton step on the residual, which leaves the
+// quotient as accurate as a division (r up to an ulp off) in three dependent
+// FP64 operations.  With a division and a root for every pivot a leaf of 32 rows
+// took 77 us, eight of 512 rows 2.2 ms.
+__device__ __forceinline__ double quotient(double x, double d, double r) {
+  const double q = x * r;
+  return fma(fma(-q, d, x), r, q);
+}
+// positive, of a magnitude whose root, reciprocal and residuals stay normal (on
+// the exponent field: a comparison would wait for the FP64 pipe)
+__device__ __forceinline__ bool usual(double x) {
+  return (uint32_t)__double2hiint(x) - ((1023u - 800u) << 20) < (1600u << 20);
+}
+
 // W = L^-1 of the tile L L^T = t (LD rows, lower triangle used): four warps,
 // lane = row, warp w holds columns w, w + 4, ... of the tile and of W, so the
 // FP64 work of a pivot is spread over the SM; one named barrier per pivot.
 // (The next pivot's root taken ahead of the other updates measured no faster.)
-// Returns 1 + the first non-positive pivot, or 0 (the same in all four warps).
-__device__ __forceinline__ int factor_tile(const double* t, double* __restrict__ W) {
+// L takes the tile's place.  Returns 1 + the first non-positive pivot, or 0 (the
+// same in all four warps).
+__device__ __forceinline__ int factor_tile(double* t, double* __restrict__ W) {
   __shared__ double col[2][TB + 1];
   __shared__ int sbad;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) sbad = 0;
-  double a[TB / 4], b[TB / 4], rown = 1.0;
+  double a[TB / 4], b[TB / 4], rown = 1.0, rinv = 1.0;
 #pragma unroll
   for (int q = 0; q < TB / 4; ++q) {
     a[q] = t[lane * LD + w + 4 * q];
@@ -74,18 +94,32 @@ __device__ __forceinline__ int factor_tile(const double* t, double* __restrict__
       double* c = col[jw & 1];
       if (w == jw) {
         double d = __shfl_sync(0xffffffffu, a[jq], j);
-        if (!(d > 0.0)) {
+        if (!usual(d) && !(d > 0.0)) {
           if (lane == 0 && !sbad) sbad = j + 1;
           d = 1.0;
         }
-        const double rs = rsqrt(d);
-        c[lane] = a[jq] * rs;  // rows below the pivot: L_ij
-        if (lane == 0) c[TB] = rs;
+        // rows below the pivot: L_ij; row j: 1 / L_jj
+        const double x = lane == j ? 1.0 : a[jq];
+        double r, q;
+        if (usual(d)) {  // the root by a Newton step from rsqrt
+          const double rs = rsqrt(d), r0 = d * rs;
+          r = fma(fma(-r0, r0, d), 0.5 * rs, r0);
+          q = quotient(x, r, rs);
+        } else {
+          r = sqrt(d);
+          q = x / r;
+        }
+        c[lane] = q;
+        if (lane == 0) c[TB] = r;
+        if (lane >= j) t[lane * LD + j] = lane == j ? r : q;
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");
       // row j of B stays unscaled until the end: its factor goes into L_ij
-      const double li = lane > j ? -c[lane] : 0.0, lr = li * c[TB];
-      if (lane == j) rown = c[TB];
+      const double li = lane > j ? -c[lane] : 0.0, lr = li * c[j];
+      if (lane == j) {
+        rown = c[TB];
+        rinv = c[j];
+      }
 #pragma unroll
       for (int q = 0; q < TB / 4; ++q) {
         const int cc = w + 4 * q;
@@ -94,16 +128,48 @@ __device__ __forceinline__ int factor_tile(const double* t, double* __restrict__
       }
     }
   }
+  const bool quick = usual(rown);
 #pragma unroll
-  for (int q = 0; q < TB / 4; ++q) W[lane * TB + w + 4 * q] = b[q] * rown;
+  for (int q = 0; q < TB / 4; ++q) W[lane * TB + w + 4 * q] = quick ? quotient(b[q], rown, rinv) : b[q] / rown;
   asm volatile("bar.sync 1, 128;" ::: "memory");
   return sbad;
+}
+
+// Y L^T = X for the tile X in x (LD rows) by substitution, L lower triangular
+// in l (LD rows), rd[j] = 1 / L_jj, Y in x's place: lane = row, warp w holds columns w, w + 8, ...,
+// one barrier per column (256 threads; callers have synchronised).
+__device__ __forceinline__ void solve_tile(double* x, const double* l, const double* rd) {
+  __shared__ double col[2][TB];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double a[TB / 8];
+#pragma unroll
+  for (int q = 0; q < TB / 8; ++q) a[q] = x[lane * LD + w + 8 * q];
+#pragma unroll
+  for (int jq = 0; jq < TB / 8; ++jq) {
+#pragma unroll 1
+    for (int jw = 0; jw < 8; ++jw) {
+      const int j = 8 * jq + jw;
+      double* c = col[jw & 1];
+      if (w == jw) {
+        const double d = l[j * LD + j], y = usual(d) ? quotient(a[jq], d, rd[j]) : a[jq] / d;
+        c[lane] = y;
+        a[jq] = y;
+      }
+      __syncthreads();
+      const double y = -c[lane];
+#pragma unroll
+      for (int q = jq; q < TB / 8; ++q)
+        if (w + 8 * q > j) a[q] = fma(y, l[(w + 8 * q) * LD + j], a[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < TB / 8; ++q) x[lane * LD + w + 8 * q] = a[q];
 }
 }  // namespace
 
 __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase, int nl, int* __restrict__ info,
                                                      double* __restrict__ Wdiag_base) {
-  __shared__ double xs[TB * LD], ys[TB * LD];
+  __shared__ double xs[TB * LD], ys[TB * LD], zs[TB * LD], rd[TB];
   const int tid = threadIdx.x, rank = cluster_rank(), C = cluster_size();
   const int T = nl / TB;
   const size_t mat = blockIdx.x / C;
@@ -130,6 +196,10 @@ __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase,
       const int j = factor_tile(xs, Wd + (size_t)k * TB * TB);
       if (j && !bad) bad = k * TB + j;
     }
+    __syncthreads();
+    double* p = tile(k, k);  // L_kk, below and on the diagonal
+#pragma unroll
+    for (int i = 0; i < 4; ++i) p[(size_t)(er + 8 * i) * nl + ec] = xs[(er + 8 * i) * LD + ec];
   };
 
   if (rank == 0) {
@@ -141,36 +211,46 @@ __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase,
   }
   cluster_sync();
   for (int k = 0; k < T; ++k) {
-    // ---- 1. X(r, k) <- X(r, k) W_kk^T: warp w has columns 4w .. 4w + 3, which
-    // need the first 4w + 4 terms of the lower-triangular W_kk ----
+    // ---- 1. column k: tiles u < k above the diagonal times W_kk^T, the others solved ----
     {
-      double w4[4];
-      bool have = false;
+      bool have_w = false, have_l = false;  // W_kk in ys; L_kk in zs, 1 / its diagonal in rd
       for (int u = rank; u < T - 1; u += C) {
-        double* X = tile(u < k ? u : u + 1, k);
-        double v[4];
-        if (!have) fetch(Wd + (size_t)k * TB * TB, TB, w4);
+        const bool above = u < k;
+        double* X = tile(above ? u : u + 1, k);
+        double v[4], d4[4];
+        const bool need = above ? !have_w : !have_l;
+        if (need) {
+          if (above) fetch(Wd + (size_t)k * TB * TB, TB, d4);
+          else fetch(tile(k, k), nl, d4);
+        }
+        if (!above && need && tid < TB) rd[tid] = __ldcg(Wd + (size_t)k * TB * TB + tid * (TB + 1));
         fetch(X, nl, v);
-        if (!have) place(ys, w4);
-        have = true;
+        if (need) place(above ? ys : zs, d4);
+        (above ? have_w : have_l) = true;
         place(xs, v);
         __syncthreads();
-        const int c0 = (tid >> 5) * 4 + ((tid >> 4) & 1) * 2, r0 = (tid & 15) * 2, n = (tid >> 5) * 4 + 4;
-        double s00 = 0, s01 = 0, s10 = 0, s11 = 0;
+        if (above) {
+          // warp w has columns 4w .. 4w + 3, which need the first 4w + 4 terms
+          // of the lower-triangular W_kk
+          const int c0 = (tid >> 5) * 4 + ((tid >> 4) & 1) * 2, r0 = (tid & 15) * 2, n = (tid >> 5) * 4 + 4;
+          double s00 = 0, s01 = 0, s10 = 0, s11 = 0;
 #pragma unroll 4
-        for (int l = 0; l < n; ++l) {
-          const double a0 = xs[r0 * LD + l], a1 = xs[(r0 + 1) * LD + l];
-          const double b0 = ys[c0 * LD + l], b1 = ys[(c0 + 1) * LD + l];
-          s00 = fma(a0, b0, s00);
-          s01 = fma(a0, b1, s01);
-          s10 = fma(a1, b0, s10);
-          s11 = fma(a1, b1, s11);
+          for (int l = 0; l < n; ++l) {
+            const double a0 = xs[r0 * LD + l], a1 = xs[(r0 + 1) * LD + l];
+            const double b0 = ys[c0 * LD + l], b1 = ys[(c0 + 1) * LD + l];
+            s00 = fma(a0, b0, s00);
+            s01 = fma(a0, b1, s01);
+            s10 = fma(a1, b0, s10);
+            s11 = fma(a1, b1, s11);
+          }
+          __syncthreads();  // xs is reused: the result goes out in rows
+          xs[r0 * LD + c0] = s00;
+          xs[r0 * LD + c0 + 1] = s01;
+          xs[(r0 + 1) * LD + c0] = s10;
+          xs[(r0 + 1) * LD + c0 + 1] = s11;
+        } else {
+          solve_tile(xs, zs, rd);
         }
-        __syncthreads();  // xs is reused: the result goes out in rows
-        xs[r0 * LD + c0] = s00;
-        xs[r0 * LD + c0 + 1] = s01;
-        xs[(r0 + 1) * LD + c0] = s10;
-        xs[(r0 + 1) * LD + c0 + 1] = s11;
         __syncthreads();
 #pragma unroll
         for (int i = 0; i < 4; ++i) X[(size_t)(er + 8 * i) * nl + ec] = xs[(er + 8 * i) * LD + ec];
@@ -214,7 +294,8 @@ __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase,
       if (ur == k) place_t(xs, va);
       else place(xs, va);
       place(ys, vb);
-      double s00 = c0[0], s01 = c0[1], s10 = c0[2], s11 = c0[3];
+      const double x00 = c0[0], x01 = c0[1], x10 = c0[2], x11 = c0[3];
+      double s00 = 0.0, s01 = 0.0, s10 = 0.0, s11 = 0.0;
       __syncthreads();
       if (u >= 0 && u + step < last) {
         decode(u + step);
@@ -222,13 +303,17 @@ __global__ void __launch_bounds__(NT) k_leaf_invchol(double* __restrict__ Abase,
       }
 #pragma unroll 8
       for (int l = 0; l < TB; ++l) {
-        const double a0 = -xs[orow * LD + l], a1 = -xs[(orow + 1) * LD + l];
+        const double a0 = xs[orow * LD + l], a1 = xs[(orow + 1) * LD + l];
         const double b0 = ys[ocol * LD + l], b1 = ys[(ocol + 1) * LD + l];
         s00 = fma(a0, b0, s00);
         s01 = fma(a0, b1, s01);
         s10 = fma(a1, b0, s10);
         s11 = fma(a1, b1, s11);
       }
+      s00 = x00 - s00;
+      s01 = x01 - s01;
+      s10 = x10 - s10;
+      s11 = x11 - s11;
       __syncthreads();
       if (u < 0) {  // CTA 0: factor the next diagonal tile
         xs[orow * LD + ocol] = s00;

@@ -235,3 +235,68 @@ def test_split_norm_bounds_hold(bs, nb):
     K = nb * bs
     top = np.abs(A.val).max()
     assert np.abs(got.val - ref.val).max() <= (K * 2.0 ** -44 + 2 * K * 2.0 ** -53 * K) * top ** 2
+
+
+def _inverse_cholesky(S, dtype, tile=32):
+    """Z = L^-T by tiles in dtype: pivots by root and division, panels by
+    substitution, a tile's product subtracted whole; W = L^-1 alike."""
+    n = S.shape[0]
+    A, W = S.astype(dtype), np.zeros((n, n), dtype)
+    for k in range(0, n, tile):
+        e = min(k + tile, n)
+        for j in range(k, e):
+            A[j, j] = np.sqrt(A[j, j])
+            A[j + 1:, j] /= A[j, j]
+            for i in range(j + 1, e):
+                A[i:, i] -= A[i:, j] * A[i, j]
+        if e < n:
+            A[e:, e:] -= np.tril(A[e:, k:e] @ A[e:, k:e].T)
+    L = np.tril(A)
+    for k in range(0, n, tile):
+        e = min(k + tile, n)
+        for i in range(k, e):  # the tile's own inverse
+            W[i, k:i] = -(L[i, k:i] @ W[k:i, k:i]) / L[i, i]
+            W[i, i] = 1 / L[i, i]
+        rhs = np.zeros((e - k, k), dtype)
+        for m in range(0, k, tile):
+            rhs -= L[k:e, m:m + tile] @ W[m:m + tile, :k]
+        W[k:e, :k] = W[k:e, k:e] @ rhs
+    return W.T
+
+
+LEAVES = [("cluster", 0), ("cluster", 1), ("cluster", 2), ("chain", 0), ("spd", 2), ("spd", 5), ("points", 18),
+          ("points", 10), ("points", 15)]
+
+
+def _leaf_matrix(kind, k):
+    if kind == "cluster":
+        return synth.cluster_overlap(512, 32, seed=k).to_dense()[:256, :256]
+    if kind == "chain":
+        return synth.chain_overlap(512, 32, seed=k).to_dense()[:256, :256]
+    r = np.random.default_rng(100 + k)
+    n = 256
+    if kind == "spd":  # condition 10^k
+        Q, _ = np.linalg.qr(r.standard_normal((n, n)))
+        S = (Q * np.logspace(0, -k, n)) @ Q.T
+        return (S + S.T) / 2
+    x = np.sort(r.uniform(0, 1, n) * n * r.uniform(0.45, 0.9))  # condition 8.6e5, 2.7e10, 3.8e10
+    return np.exp(-(x[:, None] - x[None]) ** 2) + 10 ** r.uniform(-10.5, -5) * np.eye(n)
+
+
+@pytest.mark.parametrize("kind,k", LEAVES)
+def test_leaf_accuracy(ctx, kind, k):
+    """Leaf factors of well and badly conditioned matrices: no more than twice
+    as far from the factor in extended precision as the plain tiled algorithm in
+    FP64 (with tiles of 16, 32 or 64, whichever is farthest)."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    S = _leaf_matrix(kind, k)
+    exact = _inverse_cholesky(S, np.longdouble)
+    dist = lambda Z: float(np.linalg.norm((Z - exact).astype(float)) / np.linalg.norm(exact.astype(float)))
+    plain = max(dist(_inverse_cholesky(S, np.float64, tile)) for tile in (16, 32, 64))
+    for count in (1, 20):  # clusters of different sizes
+        Z, info, rc = ifac.leaf_invchol_batched(ctx, torch.from_numpy(np.ascontiguousarray(np.tile(S, (count, 1, 1)))).cuda())
+        assert rc == 0
+        Z = Z.cpu().numpy()
+        assert np.array_equal(Z[0], Z[-1])
+        assert dist(Z[0]) <= 2 * plain
