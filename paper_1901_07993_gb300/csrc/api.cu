@@ -3,6 +3,7 @@
 // internal errors into status codes.
 #include <cstdio>
 #include <cstring>
+#include <thread>
 
 #include "internal.cuh"
 
@@ -143,12 +144,16 @@ int32_t* host_word(ifac_ctx* ctx, HostWord w) {
 
 int32_t read_word(ifac_ctx* ctx, HostWord w) {
   const volatile int32_t* p = ctx->host_words + w;
-  for (int spin = 1;; ++spin) {
+  for (unsigned spin = 1;; ++spin) {  // (seconds of work queued ahead are billions of polls)
     int32_t v = *p;
     if (v == kNotWritten && spin % 4096 == 0) {
-      // a failed kernel never writes: ask the stream now and then
+      // a failed kernel never writes: ask the stream now and then; after 0.1 ms
+      // or so let other threads have the core
       const cudaError_t e = cudaStreamQuery(ctx->stream);
-      if (e == cudaErrorNotReady) continue;
+      if (e == cudaErrorNotReady) {
+        if (spin >= 1u << 16) std::this_thread::yield();
+        continue;
+      }
       IFAC_CK(e);
       v = *p;
       if (v == kNotWritten) fail(IFAC_ERR_CUDA, "a kernel did not report its count");

@@ -1,10 +1,9 @@
 // scan_tail.cuh -- the exclusive scan of the counts that a kernel's CTAs have
 // just written, done by whichever CTA finishes last, with the total also
-// written where the host reads it (pinned memory) after its next
-// synchronisation.  One launch in place of a count kernel, a single-CTA scan
-// and a device-to-host copy: each costs about 2 us on the device and 3 us of
-// host time, and a block-sparse product at a few thousand rows is made of
-// little else.
+// written to a word of mapped memory that the host polls.  One launch in place
+// of a count kernel, a single-CTA scan and a device-to-host copy: each costs
+// about 2 us on the device and 3 us of host time, and a block-sparse product at
+// a few thousand rows is made of little else.
 #pragma once
 
 #include <cstdint>

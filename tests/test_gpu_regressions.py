@@ -300,3 +300,27 @@ def test_leaf_accuracy(ctx, kind, k):
         Z = Z.cpu().numpy()
         assert np.array_equal(Z[0], Z[-1])
         assert dist(Z[0]) <= 2 * plain
+
+
+def test_streams_with_work_ahead():
+    """Counts that kernels write for the host: right with work of the caller's
+    queued ahead on the stream, and when the context moves to another stream
+    between calls (small and large patterns, truncation, plans)."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    ctx = ifac.Context(stream=streams[0].cuda_stream)
+    mats = [synth.random_bsr(nb, 32, d, seed=nb) for nb, d in ((40, 0.3), (700, 0.004))]
+    refs = [(oracle.gemm(M, M, True, False, 1.0, 30.0), oracle.add(1.0, M, 2.0, M, 1.0)) for M in mats]
+    for i in range(6):
+        st = streams[i % 2]
+        ctx.set_stream(st.cuda_stream)
+        M, (prod, total) = mats[(i // 2) % 2], refs[(i // 2) % 2]
+        dM = ifac.upload(ctx, M)
+        with torch.cuda.stream(st):
+            torch.cuda._sleep(100_000_000)  # about 50 ms
+        got = ifac.bsr_gemm_trunc(ctx, dM, True, dM, False, 1.0, 30.0, FP64_SPLIT if i % 3 == 2 else FP64).download()
+        assert np.array_equal(got.row_ptr, prod.row_ptr) and np.array_equal(got.col_idx, prod.col_idx)
+        assert np.abs(got.val - prod.val).max() <= 1e-11 * np.abs(prod.val).max()
+        s = ifac.bsr_add(ctx, 1.0, dM, 2.0, dM, 1.0).download()
+        assert np.array_equal(s.col_idx, total.col_idx) and np.array_equal(s.val, total.val)
