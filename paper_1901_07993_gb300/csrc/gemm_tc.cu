@@ -852,42 +852,56 @@ static EncodeTiledFn encoder() {
   return fn;
 }
 
-// 2D view of a low-precision block array: rows = (nblk) * 64, 64 elements per
-// row; boxes of one 128-byte atom x 64 rows, 128-byte swizzle
-
-// Plan records of every super-tile: for each K of the union of its rows'
-// bitmaps at which some op(B)_KJ of its columns is stored, the copy index of
-// op(A)_IK for each of its ROWS block rows and of op(B)_KJ for each of its
-// COLS block columns (the zero block when absent); K steps whose op(B) blocks
-// are all absent contribute nothing and are left out.  One warp per tile,
-// candidate K's 32 at a time, lane-parallel.  PLAN_COUNT: the number of records
-// into nk[t], their offsets, and the total and the largest for the host;
-// PLAN_RECORDS: the records, from off[t] on; PLAN_BOTH: both in one pass, tile
-// t's records from t nb on.  With the records, the position in C's pattern of
-// each of the tile's ROWS x COLS blocks (-1 where C holds none), so that a
-// product's epilogue finds its output blocks with one load instead of a
-// search.
 // Exclusive scan for longer lists than scan_tail is good for (its one CTA of
 // 256 threads takes 31 us for 20,000 counts, one of 1024 threads 16 us).  CTA b
-// adds up everything before its 4096 counts by itself -- 80 KB from L2 at most
-// for those 20,000 -- so no CTA waits for another.  The total and the
-// longest tile (kmax, nullable) for the host.
+// adds up everything before its 4096 counts by itself, so no CTA waits for
+// another: 80 KB from L2 at most for those 20,000, but reads grow with the
+// square (0.5 GB at 10^6 counts), so from SCAN_LONG counts on (1 MB a CTA)
+// k_chunk_sums leaves each chunk's sum first and a CTA adds up those before its
+// own: a TF32 product of 10^6 blocks, two scans, 8.87 -> 8.81 ms.  The total and
+// the longest tile (kmax, nullable) for the host.
 constexpr int TAIL_SCAN = 8192;
 constexpr int SCAN_CHUNK = 4096;
+constexpr int SCAN_LONG = 1 << 18;
 
-__global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ cnt, int32_t* __restrict__ out, int n,
-                                               int32_t* total, int* kmax, int32_t* host_kmax) {
+// sum of a thread's values over a CTA of 1024 threads, in every thread
+__device__ __forceinline__ int cta_sum(int s, int* wsum) {
+  s = (int)__reduce_add_sync(0xffffffffu, (unsigned)s);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
+  __syncthreads();
+  return (int)__reduce_add_sync(0xffffffffu, (unsigned)wsum[threadIdx.x & 31]);
+}
+
+__global__ void __launch_bounds__(1024) k_chunk_sums(const int32_t* __restrict__ cnt, int n, int32_t* __restrict__ sums) {
+  __shared__ int wsum[32];
+  int s = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_CHUNK / 1024; ++k) {
+    const int64_t i = (int64_t)blockIdx.x * SCAN_CHUNK + k * 1024 + threadIdx.x;
+    s += i < n ? cnt[i] : 0;
+  }
+  s = cta_sum(s, wsum);
+  if (threadIdx.x == 0) sums[blockIdx.x] = s;
+}
+
+// sums: the chunks' sums, or null
+__global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ cnt, const int32_t* __restrict__ sums,
+                                               int32_t* __restrict__ out, int n, int32_t* total, int* kmax,
+                                               int32_t* host_kmax) {
   __shared__ int wsum[2][32];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, c0 = (int)blockIdx.x * SCAN_CHUNK;
   int s = 0;
+  if (sums) {
+    for (int i = tid; i < (int)blockIdx.x; i += 1024) s += sums[i];
+  } else {
 #pragma unroll 8
-  for (int i = tid; i < c0; i += 1024) s += cnt[i];
-  s = (int)__reduce_add_sync(0xffffffffu, (unsigned)s);
-  if (lane == 0) wsum[0][wid] = s;
+    for (int i = tid; i < c0; i += 1024) s += cnt[i];
+  }
+  const int base = cta_sum(s, wsum[0]);
   int v[4], t = 0;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    v[k] = c0 + tid * 4 + k < n ? cnt[c0 + tid * 4 + k] : 0;
+    v[k] = n - c0 > tid * 4 + k ? cnt[c0 + tid * 4 + k] : 0;
     t += v[k];
   }
   int x = t;
@@ -898,7 +912,7 @@ __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ cnt, 
   }
   if (lane == 31) wsum[1][wid] = x;
   __syncthreads();
-  const int own = wsum[1][lane], base = (int)__reduce_add_sync(0xffffffffu, (unsigned)wsum[0][lane]);
+  const int own = wsum[1][lane];
   int run = base + (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < wid ? own : 0)) + x - t;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
@@ -913,6 +927,31 @@ __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ cnt, 
   }
 }
 
+static void scan_counts(ifac_ctx* ctx, const int32_t* cnt, int32_t* out, int64_t n, int32_t* total, int* kmax,
+                        int32_t* host_kmax) {
+  const int chunks = cdiv(n, SCAN_CHUNK);
+  Buf<int32_t> sums;
+  if (n >= SCAN_LONG) {
+    sums = Buf<int32_t>(ctx, chunks);
+    k_chunk_sums<<<chunks, 1024, 0, ctx->stream>>>(cnt, (int)n, sums.p);
+    IFAC_CK_LAUNCH();
+  }
+  k_scan<<<chunks, 1024, 0, ctx->stream>>>(cnt, sums.p, out, (int)n, total, kmax, host_kmax);
+  IFAC_CK_LAUNCH();
+}
+
+// Plan records of every super-tile: for each K of the union of its rows'
+// bitmaps at which some op(B)_KJ of its columns is stored, the copy index of
+// op(A)_IK for each of its ROWS block rows and of op(B)_KJ for each of its
+// COLS block columns (the zero block when absent); K steps whose op(B) blocks
+// are all absent contribute nothing and are left out.  One warp per tile,
+// candidate K's 32 at a time, lane-parallel.  PLAN_COUNT: the number of records
+// into nk[t], their offsets, and the total and the largest for the host;
+// PLAN_RECORDS: the records, from off[t] on; PLAN_BOTH: both in one pass, tile
+// t's records from t nb on.  With the records, the position in C's pattern of
+// each of the tile's ROWS x COLS blocks (-1 where C holds none), so that a
+// product's epilogue finds its output blocks with one load instead of a
+// search.
 enum PlanMode { PLAN_COUNT, PLAN_RECORDS, PLAN_BOTH };
 constexpr int PLAN_NT = 256;
 
@@ -1088,9 +1127,8 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
   // amap (nullable): copy index of each op(A) view position, when op(A)'s
   // low-precision copy is not in view order (a shared copy of a transposed
   // operand, held in the stored order).  bmap (nullable): the same for
-  // op(B) (a symmetric op(B) read from its op(A) copy).  extra (nullable): one more small
-  // read-back the caller needs, taken with the plan's sizes in one
-  // synchronisation.
+  // op(B) (a symmetric op(B) read from its op(A) copy).  extra (nullable): one
+  // more small read-back the caller needs, taken behind the plan's kernels.
   // kmax_limit > 0: a plan whose longest tile has more K steps is not wanted;
   // it returns after the count pass with kmax set and no records
   const int nb = A.nb, W = words_per_row(nb);
@@ -1122,9 +1160,7 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
                                                              tail ? P.coff.p : nullptr, ctx->ticket);
     IFAC_CK_LAUNCH();
     if (!tail) {
-      k_scan<<<cdiv(C.nnzb, SCAN_CHUNK), 1024, 0, ctx->stream>>>(own.p, P.coff.p, (int)C.nnzb, nullptr, nullptr,
-                                                                 nullptr);
-      IFAC_CK_LAUNCH();
+      scan_counts(ctx, own.p, P.coff.p, C.nnzb, nullptr, nullptr, nullptr);
     }
     k_tile_owner_write<<<cdiv(C.nnzb, 256), 256, 0, ctx->stream>>>(crow, C.col_idx, C.nnzb, ROWS, COLS, P.coff.p,
                                                                    P.tiles.p);
@@ -1178,11 +1214,9 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
       (int)B.nnzb, nullptr, nullptr, P.tnk.p, kmax_dev, nullptr, nullptr, nullptr, nullptr, nt, nullptr, nullptr,
       nullptr);
   IFAC_CK_LAUNCH();
-  k_scan<<<cdiv(nt, SCAN_CHUNK), 1024, 0, ctx->stream>>>(P.tnk.p, P.off.p, nt, host_word(ctx, HW_PLAN), kmax_dev,
-                                                         host_word(ctx, HW_KMAX));
-  IFAC_CK_LAUNCH();
-  // the record count, the longest tile and the caller's extra read-back
-  // behind one synchronisation
+  scan_counts(ctx, P.tnk.p, P.off.p, nt, host_word(ctx, HW_PLAN), kmax_dev, host_word(ctx, HW_KMAX));
+  // the caller's extra read-back waits for the stream; the record count and
+  // the longest tile are there then, or polled
   if (extra) to_host_many(ctx, {*extra});
   const int64_t total = read_word(ctx, HW_PLAN);
   P.kmax = read_word(ctx, HW_KMAX);
@@ -1199,6 +1233,8 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
   return P;
 }
 
+// 2D view of a low-precision block array: rows = (nblk) * 64, 64 elements per
+// row; boxes of one 128-byte atom x 64 rows, 128-byte swizzle
 template <int ELT>
 static CUtensorMap make_map(void* base, int64_t nblk) {
   CUtensorMap m;

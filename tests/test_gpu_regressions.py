@@ -324,3 +324,33 @@ def test_streams_with_work_ahead():
         assert np.abs(got.val - prod.val).max() <= 1e-11 * np.abs(prod.val).max()
         s = ifac.bsr_add(ctx, 1.0, dM, 2.0, dM, 1.0).download()
         assert np.array_equal(s.col_idx, total.col_idx) and np.array_equal(s.val, total.val)
+
+
+def _on_device(nb, bs, rows, cols, val):
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    rp = torch.from_numpy(np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=nb))]).astype(np.int32)).cuda()
+    return ifac.BorrowedBSR(nb * bs, bs, rp, torch.from_numpy(cols.astype(np.int32)).cuda(), val)
+
+
+@pytest.mark.parametrize("prec", [TF32, FP64_SPLIT])
+def test_scan_of_many_counts(ctx, prec):
+    """Tile lists and plans of more than 2^18 blocks and tiles, whose scans go
+    through the chunks' sums: the identity times a band of small integers is
+    that band."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    nb, bs, w = 30000, 32, 4
+    rows = np.repeat(np.arange(nb), 2 * w + 1)
+    cols = (np.arange(nb)[:, None] + np.arange(-w, w + 1)[None]).ravel()
+    ok = (cols >= 0) & (cols < nb)
+    rows, cols = rows[ok], cols[ok]
+    assert len(rows) > 1 << 18
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    val = torch.randint(-3, 4, (len(rows), bs, bs), device="cuda", generator=g).double()
+    eye = torch.eye(bs, dtype=torch.float64, device="cuda").expand(nb, bs, bs).contiguous()
+    E, A = _on_device(nb, bs, np.arange(nb), np.arange(nb), eye), _on_device(nb, bs, rows, cols, val)
+    C = ifac.bsr_gemm_trunc(ctx, E, False, A, False, 1.0, 0.0, prec)
+    rp, ci, v = ifac.device_tensors(C)
+    assert torch.equal(rp, A.keep[0]) and torch.equal(ci, A.keep[1]) and torch.equal(v, val)
