@@ -354,3 +354,45 @@ def test_scan_of_many_counts(ctx, prec):
     C = ifac.bsr_gemm_trunc(ctx, E, False, A, False, 1.0, 0.0, prec)
     rp, ci, v = ifac.device_tensors(C)
     assert torch.equal(rp, A.keep[0]) and torch.equal(ci, A.keep[1]) and torch.equal(v, val)
+
+
+@pytest.mark.parametrize("bs", [32, 64, 128])
+@pytest.mark.parametrize("prec", [TF32, BF16, FP64_SPLIT])
+def test_plans_counted_first(ctx, bs, prec):
+    """Tile plans whose records are counted before they are written (more than
+    2^25 words if every tile had all K steps), their tile lists scanned by
+    several CTAs: small integers, so that every product is exact."""
+    from paper_1901_07993_gb300 import ifac
+    nb = 4400 if bs == 128 else 2600
+    rng = np.random.default_rng(nb)
+    A = synth.random_bsr(nb, bs, 2.0 / nb, seed=1, empty_rows=3)
+    B = synth.random_bsr(nb, bs, 2.0 / nb, seed=2)
+    A.val[:] = rng.integers(-1, 2, A.val.shape)
+    B.val[:] = rng.integers(-1, 2, B.val.shape)
+    dA, dB = ifac.upload(ctx, A), ifac.upload(ctx, B)
+    for tA in (False, True):
+        want = oracle.gemm(A, B, tA, False, 1.0, 0.0)
+        assert want.nnzb > 8192 and want.nnzb * nb * {32: 6, 64: 3, 128: 2}[bs] > 1 << 25
+        got = ifac.bsr_gemm_trunc(ctx, dA, tA, dB, False, 1.0, 0.0, prec).download()
+        assert np.array_equal(got.row_ptr, want.row_ptr) and np.array_equal(got.col_idx, want.col_idx)
+        assert np.array_equal(got.val, want.val)
+
+
+@pytest.mark.parametrize("prec", [TF32, BF16])
+def test_wide_plan_counted_first(ctx, prec):
+    """The same for tiles of 256 x 256: full operands of 410 block rows against
+    FP32 products of the same small integers (exact: |sums| < 2^24)."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    nb, bs = 410, 64
+    n = nb * bs
+    g = torch.Generator(device="cuda")
+    g.manual_seed(2)
+    D = [torch.randint(-1, 2, (n, n), device="cuda", generator=g).float() for _ in range(2)]
+    rows, cols = np.repeat(np.arange(nb), nb), np.tile(np.arange(nb), nb)
+    block = lambda X: X.view(nb, bs, nb, bs).transpose(1, 2).reshape(nb * nb, bs, bs)
+    dA, dB = (_on_device(nb, bs, rows, cols, block(X).double().contiguous()) for X in D)
+    C = ifac.bsr_gemm_trunc(ctx, dA, False, dB, False, 1.0, 0.0, prec)
+    assert not torch.backends.cuda.matmul.allow_tf32
+    want = block(D[0] @ D[1])
+    assert C.nnzb == nb * nb and torch.equal(ifac.device_tensors(C)[2], want.double())
