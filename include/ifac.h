@@ -81,7 +81,12 @@ typedef struct {
 
 /* Device memory provider.  alloc returns NULL on failure; both are called
  * with the context's stream.  Pass NULL to ifac_create to use the device's
- * stream-ordered pool (cudaMallocAsync / cudaFreeAsync). */
+ * stream-ordered pool (cudaMallocAsync / cudaFreeAsync).  With the
+ * pool the lists of a result may be sized by a bound (col_idx and norms: the
+ * blocks before truncation), and a product's tile plan by one of up to 128 MB
+ * while it runs; from a caller's memory a result's list is at most 64 KB longer
+ * than it needs, and a plan is counted first where its bound exceeds an eighth
+ * of C's values. */
 typedef struct {
   void* (*alloc)(void* user, size_t bytes, void* stream);
   void (*free)(void* user, void* ptr, void* stream);

@@ -1195,10 +1195,12 @@ static Plan make_plan(ifac_ctx* ctx, const View& arows, const ifac_bsr& A, const
   P.cpos = Buf<int32_t>(ctx, (size_t)nt * (ROWS * COLS));
   const int pgrid = cdiv((int64_t)nt * 32, PLAN_NT);
   int* const kmax_dev = reinterpret_cast<int*>(ctx->ticket + 1);
-  // While every tile could have nb K steps within 128 MB, the records are
-  // written in one pass at a fixed stride, and only the longest tile is read
-  // back; a longer list is counted first.
-  if ((int64_t)nt * nb * (ROWS + COLS) <= (int64_t)32 << 20) {
+  // While every tile could have nb K steps within 128 MB (in a caller's memory:
+  // within an eighth of C's values), the records are written in one pass at a
+  // fixed stride, and only the longest tile is read back; a longer list is
+  // counted first.
+  const int64_t most = (int64_t)nt * nb * (ROWS + COLS), fits = (int64_t)32 << 20;
+  if (most <= (ctx->custom_alloc ? std::min(fits, C.nnzb * C.bs * C.bs / 8) : fits)) {
     P.rec = Buf<int32_t>(ctx, (size_t)nt * nb * (ROWS + COLS));
     k_tile_plan<ROWS, COLS, PLAN_BOTH><<<pgrid, PLAN_NT, 0, ctx->stream>>>(
         P.tiles.p, ntiles, nullptr, bmA.p, nb, W, imA.p, imB.p, arows.rp, arows.ci, brows.rp, brows.ci, (int)A.nnzb,

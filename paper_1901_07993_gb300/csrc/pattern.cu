@@ -41,6 +41,7 @@ struct Job {
   int nsrc;
   int diag;             // the diagonal blocks as well
   int nb, W;
+  int cap;              // one-CTA kernel: what the lists hold; a longer pattern is only counted
   const int32_t* arp;   // a product: rows of op(A) (the sources are op(B)); null: the union of the sources
   const int32_t* aci;
   int upper;            // only columns >= the row
@@ -157,12 +158,12 @@ __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
     off[tid] = run;
     j.rp[tid] = run;
     if (tid == j.nb - 1) {
-      j.rp[j.nb] = run + c;
+      off[j.nb] = j.rp[j.nb] = run + c;
       if (j.total) *j.total = run + c;
     }
   }
   __syncthreads();
-  if (!live) return;
+  if (!live || off[j.nb] > j.cap) return;
   const auto before = [&](int r, int w) {  // set bits of row r in the words before w
     int n = off[r];
     for (int v = 0; v < w; ++v) n += __popc(out[r * WP + v]);
@@ -277,11 +278,21 @@ void launch_small(ifac_ctx* ctx, const Job& j, int64_t nnza) {
   IFAC_CK_LAUNCH();
 }
 
+// A list that a result keeps, in a caller's memory: one of the exact size in
+// place of one taken by a bound, where that saves more than 64 KB.
+template <typename T>
+void shrink(ifac_ctx* ctx, Buf<T>& b, int64_t n) {
+  if (!ctx->custom_alloc || (b.n - (size_t)n) * sizeof(T) <= 65536) return;
+  Buf<T> c(ctx, n);
+  if (n > 0) IFAC_CK(cudaMemcpyAsync(c.p, b.p, sizeof(T) * n, cudaMemcpyDeviceToDevice, ctx->stream));
+  b = std::move(c);
+}
+
 // The pattern of a job: known >= 0 the number of its blocks where the host
-// knows it (a transposed view), so nothing is read back; guess what it will
-// be about, cap its bound.
-// j's longest[] are set by the caller.
-Pattern run_job(ifac_ctx* ctx, Job j, int64_t in_blocks, int64_t guess, int64_t cap, int64_t known,
+// knows it (a transposed view), so nothing is read back; guess what it will be
+// about.  The one-CTA kernel writes lists of `room` blocks and goes out once more
+// where they are too short.  j's longest[] are set by the caller.
+Pattern run_job(ifac_ctx* ctx, Job j, int64_t in_blocks, int64_t guess, int64_t room, int64_t known,
                 Buf<int32_t>* src, int64_t nnza = 0) {
   Pattern P;
   j.W = words_per_row(j.nb);
@@ -299,9 +310,18 @@ Pattern run_job(ifac_ctx* ctx, Job j, int64_t in_blocks, int64_t guess, int64_t 
     }
   };
   if (rule_small(j.nb, in_blocks, guess)) {
-    alloc(cap);
+    j.cap = (int)room;
+    alloc(room);
     launch_small(ctx, j, nnza);
     P.nnzb = known >= 0 ? known : read_word(ctx, HW_NNZ);
+    if (P.nnzb > j.cap) {
+      j.cap = (int)P.nnzb;
+      j.total = nullptr;
+      j.longest[0] = j.longest[1] = nullptr;
+      alloc(P.nnzb);
+      launch_small(ctx, j, nnza);
+    }
+    shrink(ctx, P.ci, P.nnzb);
     return P;
   }
   const size_t words = (size_t)j.nb * j.W;
@@ -400,9 +420,10 @@ Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const if
   j.arp = arows.rp;
   j.aci = arows.ci;
   j.upper = upper ? 1 : 0;
-  // a row of op(A) with k blocks meets about k nnz(B) / nb of op(B); what the
-  // lists may hold is nb^2 (at most 1 MB where one CTA writes them)
+  // a row of op(A) with k blocks meets about k nnz(B) / nb of op(B)
   const int64_t full = (int64_t)nb * nb, guess = std::min(full, nnza * std::max<int64_t>(1, B.nnzb / nb));
+  // (twice that and at least 64 KB, so that uneven operands seldom need more)
+  const int64_t room = std::min(full, std::max<int64_t>(16384, 2 * nnza * ((B.nnzb + nb - 1) / nb)));
   const bool want_a = want_longest, want_b = want_longest && transB;
   if (want_a) {
     j.lrp[0] = arows.rp;
@@ -412,7 +433,7 @@ Pattern product_pattern(ifac_ctx* ctx, const View& arows, int64_t nnza, const if
     j.lrp[1] = B.row_ptr;
     j.longest[1] = host_word(ctx, HW_LONGEST_B);
   }
-  Pattern P = run_job(ctx, j, std::max(nnza, B.nnzb), guess, full, -1, nullptr, nnza);
+  Pattern P = run_job(ctx, j, std::max(nnza, B.nnzb), guess, room, -1, nullptr, nnza);
   if (want_a) P.longest_a = read_word(ctx, HW_LONGEST_A);  // (written with the total)
   if (want_b) P.longest_b = read_word(ctx, HW_LONGEST_B);
   return P;
@@ -587,12 +608,17 @@ static Kept keep_pattern(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep, 
   k.ci = Buf<int32_t>(ctx, A.nnzb);
   k.norms = Buf<double>(ctx, A.nnzb);
   k.map = Buf<int32_t>(ctx, A.nnzb);
+  const auto finish = [&] {
+    k.n = read_word(ctx, HW_KEPT);
+    shrink(ctx, k.ci, k.n);
+    shrink(ctx, k.norms, k.n);
+  };
   if (A.nnzb <= SMALL_KEEP) {
     k_keep_small<<<1, 1024, 4 * ((size_t)A.nnzb + 1), ctx->stream>>>(A.row_ptr, nb, (int)A.nnzb, keep, A.norms, tau, A.col_idx, k.rp.p,
                                                  k.ci.p, k.norms.p, want_vmap ? nullptr : k.map.p,
                                                  want_vmap ? k.map.p : nullptr, host_word(ctx, HW_KEPT));
     IFAC_CK_LAUNCH();
-    k.n = read_word(ctx, HW_KEPT);
+    finish();
     return k;
   }
   Buf<int32_t> cnt(ctx, nb);
@@ -603,7 +629,7 @@ static Kept keep_pattern(ifac_ctx* ctx, const ifac_bsr& A, const uint8_t* keep, 
                                                     k.norms.p, want_vmap ? nullptr : k.map.p,
                                                     want_vmap ? k.map.p : nullptr);
   IFAC_CK_LAUNCH();
-  k.n = read_word(ctx, HW_KEPT);
+  finish();
   return k;
 }
 

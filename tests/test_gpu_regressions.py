@@ -396,3 +396,85 @@ def test_wide_plan_counted_first(ctx, prec):
     assert not torch.backends.cuda.matmul.allow_tf32
     want = block(D[0] @ D[1])
     assert C.nnzb == nb * nb and torch.equal(ifac.device_tensors(C)[2], want.double())
+
+
+class TrackingAllocator:
+    """torch's caching allocator behind the library's allocator interface:
+    bytes held now and at most."""
+
+    def __init__(self):
+        self.live, self.now, self.peak = {}, 0, 0
+
+    def alloc(self, nbytes, stream):
+        import torch
+        p = torch.cuda.caching_allocator_alloc(nbytes, stream=int(stream))
+        self.live[p] = nbytes
+        self.now += nbytes
+        self.peak = max(self.peak, self.now)
+        return p
+
+    def free(self, ptr, stream):
+        import torch
+        self.now -= self.live.pop(ptr)
+        torch.cuda.caching_allocator_delete(ptr)
+
+
+@pytest.mark.parametrize("bs,nb,prec", [(16, 400, FP64), (32, 900, TF32), (64, 700, BF16), (64, 700, FP64_SPLIT)])
+@pytest.mark.parametrize("tau", [0.0, 1e3])
+def test_memory_of_a_callers_allocator(bs, nb, prec, tau):
+    """From a caller's allocator a product takes what its result, its copies and
+    slices of the operands, and lists of a few words for each block need (here
+    1 KB for each block row beside nb^2 words twice and three bitmaps), and the
+    lists of results, of sums and truncations too, are at most 64 KB too long."""
+    import torch
+    from paper_1901_07993_gb300 import ifac
+    mem = TrackingAllocator()
+    ctx = ifac.Context(allocator=(mem.alloc, mem.free))
+    rows, cols = np.nonzero(np.abs(np.subtract.outer(np.arange(nb), np.arange(nb))) <= 1)
+    rp = np.concatenate([[0], np.cumsum(np.bincount(rows, minlength=nb))]).astype(np.int32)
+    val = np.random.default_rng(1).standard_normal((len(rows), bs, bs)) * np.where(rows == cols, 100.0, 0.01)[:, None, None]
+    A = synth.HostBSR(nb * bs, bs, rp, cols.astype(np.int32), val)
+    dA = ifac.upload(ctx, A)
+    exact = lambda n: 4 * (nb + 1) + max(n, 1) * (4 + 8 + 8 * bs * bs)
+    base = mem.now
+    assert base == exact(A.nnzb)
+    full = 5 * nb - 6
+    copies = {FP64: 0, TF32: 4, BF16: 2, FP64_SPLIT: 14}[prec] * 2 * (A.nnzb + 1) * bs * bs
+    room = exact(full) + copies + 8 * nb * nb + 3 * nb * (nb + 31) // 8 + 1024 * nb + (exact(full) if tau else 0)
+    fits = lambda held, need: need <= held <= need + 2 * 65536
+    mem.peak = mem.now
+    C = ifac.bsr_gemm_trunc(ctx, dA, False, dA, False, 1.0, tau, prec)
+    held = mem.now
+    assert fits(held - base, exact(C.nnzb)) and (C.nnzb == full) == (tau == 0.0)
+    assert mem.peak - base <= room, (mem.peak - base, room)
+    want = oracle.gemm(A, A, False, False, 1.0, tau)
+    got = C.download()
+    assert np.array_equal(got.col_idx, want.col_idx) and np.abs(got.val - want.val).max() <= 4e-3 * np.abs(want.val).max()
+    S = ifac.bsr_add(ctx, 1.0, C, 1.0, dA, 0.0)
+    assert fits(mem.now - held, exact(S.nnzb))
+    held = mem.now
+    T = ifac.bsr_truncate(ctx, dA, 5.0 * bs)
+    assert T.nnzb == nb and fits(mem.now - held, exact(nb))
+    del C, S, T, dA
+    torch.cuda.synchronize()
+    assert not mem.live
+
+
+def test_pattern_longer_than_expected(ctx):
+    """A product whose operands' rows do not meet evenly (a full column times a
+    full row): more blocks than the averages promise, whole all the same."""
+    from paper_1901_07993_gb300 import ifac
+    for nb in (30, 200, 500):
+        col, row = np.zeros((nb, nb), bool), np.zeros((nb, nb), bool)
+        col[:, nb // 3] = True
+        row[nb // 3] = True
+        M = []
+        for k, mask in enumerate((col, row)):
+            r, c = np.nonzero(mask)
+            rp = np.concatenate([[0], np.cumsum(mask.sum(axis=1))]).astype(np.int32)
+            M.append(synth.HostBSR(nb * 16, 16, rp, c.astype(np.int32), np.random.default_rng(k).standard_normal((nb, 16, 16))))
+        dA, dB = ifac.upload(ctx, M[0]), ifac.upload(ctx, M[1])
+        for A, B, hA, hB, t in ((dA, dB, M[0], M[1], False), (dB, dA, M[1], M[0], True)):
+            got, want = ifac.bsr_gemm_trunc(ctx, A, t, B, t, 1.0, 0.0).download(), oracle.gemm(hA, hB, t, t, 1.0, 0.0)
+            assert got.nnzb == nb * nb and np.array_equal(got.col_idx, want.col_idx)
+            assert np.abs(got.val - want.val).max() <= 1e-12 * np.abs(want.val).max()
