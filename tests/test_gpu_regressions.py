@@ -478,3 +478,90 @@ def test_pattern_longer_than_expected(ctx):
             got, want = ifac.bsr_gemm_trunc(ctx, A, t, B, t, 1.0, 0.0).download(), oracle.gemm(hA, hB, t, t, 1.0, 0.0)
             assert got.nnzb == nb * nb and np.array_equal(got.col_idx, want.col_idx)
             assert np.abs(got.val - want.val).max() <= 1e-12 * np.abs(want.val).max()
+
+
+SPECIAL = np.array([np.inf, -np.inf, np.nan, 1e300, -1e39, 3e38, 2.0 ** -126, 2.0 ** -127, 5e-324, -0.0])
+
+
+def _with_specials(nb, bs, seed):
+    """Full matrix of small values with one special value in some columns."""
+    rng = np.random.default_rng(seed)
+    val = rng.standard_normal((nb * nb, bs, bs))
+    for c in range(0, bs, 3):
+        val[rng.integers(nb * nb), rng.integers(bs), c] = SPECIAL[rng.integers(len(SPECIAL))]
+    rp, ci = (np.arange(nb + 1) * nb).astype(np.int32), np.tile(np.arange(nb), nb).astype(np.int32)
+    return synth.HostBSR(nb * bs, bs, rp, ci, val)
+
+
+@pytest.mark.filterwarnings("ignore:invalid value", "ignore:overflow")
+@pytest.mark.parametrize("bs", [5, 16, 32, 64, 128])
+def test_sums_of_infinities_and_nan(ctx, bs):
+    """Sums with infinities and NaN among the operands equal numpy's, value for
+    value; the norms of their blocks are infinite or NaN, and a truncation
+    drops the others only."""
+    from paper_1901_07993_gb300 import ifac
+    nb = 3
+    A, B = _with_specials(nb, bs, 1), _with_specials(nb, bs, 2)
+    dA, dB = ifac.upload(ctx, A), ifac.upload(ctx, B)
+    for alpha, beta in ((1.0, -1.0), (-0.375, 2.0), (3.0, 0.7)):
+        want = alpha * A.val + beta * B.val
+        dev = ifac.bsr_add(ctx, alpha, dA, beta, dB, 0.0)
+        np.testing.assert_array_equal(dev.download().val, want)
+        norms = np.sqrt((want ** 2).sum(axis=(1, 2)))
+        fro = ifac.bsr_fro(ctx, dev)
+        total = np.sqrt((norms ** 2).sum())
+        assert np.isnan(fro) == np.isnan(total) and (np.isnan(total) or fro == total)
+        tau = 4.0 * bs  # above every ordinary block, below infinity
+        assert ifac.bsr_truncate(ctx, dev, tau).nnzb == int((~(norms < tau)).sum())
+
+
+@pytest.mark.filterwarnings("ignore:invalid value", "ignore:overflow")
+@pytest.mark.parametrize("bs", [32, 64, 128])
+@pytest.mark.parametrize("prec", [TF32, BF16])
+@pytest.mark.parametrize("tB", [False, True])
+def test_low_precision_copies_of_special_values(ctx, bs, prec, tB):
+    """The identity times a matrix with infinities, NaN, values past FP32's range
+    and subnormals: the rounded value in its place, and 0 times infinity or NaN
+    elsewhere in its column."""
+    from paper_1901_07993_gb300 import ifac
+    nb = 2
+    n = nb * bs
+    A = _with_specials(nb, bs, 3)
+    eye = synth.HostBSR(n, bs, A.row_ptr, A.col_idx, np.stack([np.eye(bs) * (i == j) for i in range(nb) for j in range(nb)]))
+    if prec == TF32:  # FP32, then ten fraction bits, ties away
+        f = A.val.astype(np.float32)
+        low = ((f.view(np.uint32) + np.uint32(0x1000)) & np.uint32(0xffffe000)).view(np.float32)
+    else:  # seven fraction bits of the FP64 value, ties to even
+        f = A.val
+        u = f.view(np.uint64)
+        u = (u + np.uint64((1 << 44) - 1) + ((u >> np.uint64(45)) & np.uint64(1))) & ~np.uint64((1 << 45) - 1)
+        low = u.view(np.float64).astype(np.float32)
+    low = np.where(np.isfinite(f), low, f).astype(float)
+    low = np.where(np.abs(A.val) < 2.0 ** -126, 0.0, low)
+    D = low.reshape(nb, nb, bs, bs).transpose(0, 2, 1, 3).reshape(n, n)
+    M = D.T if tB else D
+    bad = ~np.isfinite(M)
+    want = np.where(np.isfinite(M), M, 0.0)
+    cols = bad.any(axis=0)
+    want[:, cols] = np.nan
+    want[bad & (bad.sum(axis=0) == 1)[None, :]] = M[bad & (bad.sum(axis=0) == 1)[None, :]]
+    got = ifac.bsr_gemm_trunc(ctx, ifac.upload(ctx, eye), False, ifac.upload(ctx, A), tB, 1.0, 0.0, prec).download()
+    G = got.val.reshape(nb, nb, bs, bs).transpose(0, 2, 1, 3).reshape(n, n)
+    np.testing.assert_array_equal(G, want)
+
+
+@pytest.mark.filterwarnings("ignore:invalid value", "ignore:overflow")
+def test_symmetric_completion_of_infinities_and_nan(ctx):
+    """Symmetric products whose values hold infinities and NaN: the upper
+    blocks are the product's, the lower ones their transposes."""
+    from paper_1901_07993_gb300 import ifac
+    nb, bs = 3, 64
+    A = _with_specials(nb, bs, 5)
+    dA = ifac.upload(ctx, A)
+    full = ifac.bsr_gemm_trunc(ctx, dA, True, dA, False, -0.5, 0.0).download()
+    got = ifac.bsr_gemm_sym_trunc(ctx, dA, True, dA, False, -0.5, 0.0).download()
+    assert not np.isfinite(full.val).all() and np.isfinite(full.val).any()
+    for i in range(nb):
+        for j in range(nb):
+            block = full.val[i * nb + j] if j >= i else full.val[j * nb + i].T
+            np.testing.assert_array_equal(got.val[i * nb + j], block)
