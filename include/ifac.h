@@ -265,8 +265,8 @@ void ifac_bsr_free(ifac_ctx* ctx, ifac_bsr* a);
  * tau_j, f <= 56 chosen so that no partial sum can overflow; the result is
  * converted to FP64 once.  Element error about 2^-(7 s - 3) K_ij sigma_i tau_j
  * (2^-46 for s = 7) plus 2^-f sigma_i tau_j per window.  IFAC_ERR_TIMEOUT if
- * a device pipeline wait expired; IFAC_ERR_CUDA if a fixed-point sum
- * overflowed (not expected: the scale is bounded from the operands). */
+ * a device pipeline wait expired; IFAC_ERR_CUDA if a complete fixed-point sum
+ * is past 2^62 (not expected: the scale is bounded from the operands). */
 int bsr_gemm_trunc(ifac_ctx* ctx, const ifac_bsr* A, int transA, const ifac_bsr* B, int transB,
                    double alpha, double tau, int prec, ifac_bsr* C);
 

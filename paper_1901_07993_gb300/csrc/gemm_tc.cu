@@ -1392,7 +1392,11 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
   const CUtensorMap mapA = make_map<ELT>(la_p, A.nnzb + 1);
   const CUtensorMap mapB = make_map<ELT>(lb_p, B.nnzb + 1);
   // C's blocks fill more tiles of 4 x 4 than half the SMs: 256 x 256 elements a
-  // CTA (gemm_wide.cu); a smaller product spreads over CTA pairs
+  // CTA (gemm_wide.cu); a smaller product spreads over CTA pairs.  Scattered
+  // blocks fill fewer tiles than that, and still: with one block in each tile
+  // (every fourth row and column, 17 to 100 K blocks) TF32 is 1.06 - 1.15 times as
+  // fast as on pairs, BF16 1.3 - 1.8 times; mostly one-pair blocks beside a few
+  // long rows 0.92 times in TF32 (600 block rows), 1.25 in BF16.
   if (C.nnzb > 16 * 76) {
     Plan Pw = make_plan<4, 4>(ctx, arows, A, brows, B, C, crow, pc, false, 0, amap, nullptr, bmap);
     prof_begin(ctx, 1);
@@ -1450,23 +1454,19 @@ static void run(ifac_ctx* ctx, const View& arows, bool tA, const ifac_bsr& A, co
 // likewise the columns of op(B) with tau_j.  A product of two slices
 // (first slices |q| <= 128, later ones |q| <= 64) is a sum of integers, exact
 // in FP32 while its magnitude bound stays <= 2^24.  Slice pairs with equal
-// weight 2^(-7(s+t)), s + t <= NS + 1, are packed greedily into units whose
-// bound over a window stays <= 2^24.  A window holds KW = 16 K blocks (1024
-// terms), or fewer when the product's longest tile has fewer K steps: for
-// NS = 7, 13 units at full windows, 7 when no tile has more than 7 K steps
-// (banded patterns such as a 1D chain).  Per tile and window, each unit is
-// one accumulator that the epilogue adds, scaled, into the FP64 result.
+// weight 2^(-7(s+t)), s + t <= NS + 1, are summed in accumulation units whose
+// bound over a window of K blocks stays <= 2^24.  On narrow tiles every weight
+// class is one unit, and a window as long as that allows (six blocks of 64 with
+// NS = 8); the super-tile kernel's windows hold KW = 16 K blocks (1024 terms),
+// or the longest tile's when fewer, and a class is packed greedily into as many
+// units as it needs (NS = 7: 13 at full windows, 7 up to 7 K steps).  Per tile
+// and window the epilogue adds each unit, scaled, into 64-bit sums.
 // ---------------------------------------------------------------------------
 constexpr int SPLIT_BITS = 7;
 
 // GB300's FP64 pipe is narrow, so the splitting below works on the bit
-// patterns of the FP64 inputs with integer arithmetic only.
+// patterns of the FP64 inputs.
 
-// exponent e of sigma = 2^e for every scalar row of a (possibly transposed)
-// row view: max_k |x_rk| = m 2^e with m in [0.5, 1) (e = 0 for an all-zero row);
-// the largest scaled row 1-norm sum_k |x_rk| / sigma into *l1max and the
-// largest scaled row 2-norm (sum_k x_rk^2)^(1/2) / sigma into *l2max, both
-// bounds from above, as FP32 bits
 // two consecutive values (an even offset into a matrix's values); wide: the
 // values start on a 16-byte boundary (a caller's own array may start on any
 // multiple of eight)
@@ -1552,7 +1552,10 @@ __device__ __forceinline__ void row_scale_max(uint32_t n1, uint32_t n2, unsigned
   }
 }
 
-// Row scales of a view.  While its block rows are short, CTA I reads block row I
+// Row scales of a view: the exponent e of sigma = 2^e for every scalar row of op(X),
+// max_k |x_rk| = m 2^e with m in [0.5, 1) (e = 0 for an all-zero row), the largest
+// scaled 1-norm sum_k |x_rk| / sigma of a row into *l1max and the largest scaled
+// 2-norm into *l2max, both as FP32 bits.  While the block rows are short, CTA I reads block row I
 // (k_row_scale); else CTA c the view's blocks [c L, (c + 1) L), row by row
 // (k_row_parts).  16-byte loads; TR: op(X) row r is column r of the stored blocks, a
 // thread takes two columns and every (512 / B)-th row; else eight lanes share a
@@ -2233,7 +2236,7 @@ __device__ __forceinline__ void class_sums(long long* s, uint32_t (&r)[8][4], co
 
 // v[e] = s[e] 2^E[e] rounded to nearest even from the integer's bits (results
 // outside the normal range: i64_ldexp); `bad` records |s| >= 2^62, which the
-// sums' scale rules out
+// sums' scale rules out (s is complete here; its partial sums are not checked)
 __device__ __forceinline__ void fixed_to_f64(const long long (&s)[4], const int (&E)[4], double (&v)[4], bool& bad) {
   bool odd = false;
 #pragma unroll
@@ -2810,7 +2813,9 @@ static void run_split(ifac_ctx* ctx, int ns, const View& arows, bool tA, const i
   // 2-norm bound is the tight one for dense operands, where every bit of f
   // saved is a rounding the finest accumulation units escape in each window.
   // f <= 56 keeps every weight 2^(f - 7g) of the 7-slice product integral.
-  // An overflow would still be detected and reported.
+  // A sum past 2^62 is an error of the call: the super-tile kernel checks every
+  // addition; the narrow kernel's sums wrap modulo 2^64 and are checked when
+  // complete, so it would miss one of more than three times the bound.
   int lgK = 0;
   while (((int64_t)1 << lgK) < (int64_t)std::max(kmax, 1) * bs) ++lgK;
   const double rk = 0.0125 * std::sqrt((double)std::max(kmax, 1) * bs);
