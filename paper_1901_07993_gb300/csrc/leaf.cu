@@ -22,9 +22,9 @@
 // 1e6 and more.
 // Every step has T^2 / 2 to T tile products (T = nl / 32); the columns of W
 // after all of L would be chains of very different length.  Call times against
-// one CTA per matrix: 8 leaves of 512 rows 15.9 -> 1.65 ms (0.43 TFLOP/s of the
-// FP64 pipe's 1.25), one 15.9 -> 1.30 ms, 32 leaves 16.0 -> 4.1 ms, one of 128
-// rows 572 -> 224 us, one of 1024 rows 113 -> 7.3 ms, 1000 of 32 rows 227 -> 202 us.
+// one CTA per matrix: 8 leaves of 512 rows 15.9 -> 1.54 ms (0.47 TFLOP/s of the
+// FP64 pipe's 1.25), one 15.9 -> 1.17 ms, 32 leaves 16.0 -> 3.9 ms, one of 128
+// rows 572 -> 226 us, one of 1024 rows 113 -> 7.0 ms, 1000 of 32 rows 227 -> 202 us.
 //
 // A non-positive pivot j sets info = j + 1 (the pivot is replaced by 1 so the
 // arithmetic stays finite; that matrix's Z is then meaningless).
@@ -36,8 +36,9 @@ namespace {
 constexpr int TB = 32;
 constexpr int LD = TB + 1;  // padded shared-memory row
 constexpr int NT = 256;
-// CTA 0's update and factorization of the next diagonal tile, in tile products
-constexpr int DIAG_COST = 3;
+// CTA 0's update and factorization of the next diagonal tile, in tile products:
+// eight leaves of 512 rows 1.66 ms with 3, 1.57 with 4, 1.54 with 5 or 6
+constexpr int DIAG_COST = 5;
 
 __device__ __forceinline__ int cluster_rank() {
   int r;
