@@ -149,10 +149,12 @@ __global__ void __launch_bounds__(1024) k_pattern_small(Job j, int nnza) {
       if (lane == 0) wlen[i][wid] = m;
     }
   __syncthreads();
-  if (wid < 2 && j.longest[wid]) {
-    const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)wlen[wid][lane]);
-    if (lane == 0) *j.longest[wid] = m;
-  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (j.longest[i] && wid == i) {
+      const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)wlen[i][lane]);
+      if (lane == 0) *j.longest[i] = m;
+    }
   const int run = (int)__reduce_add_sync(0xffffffffu, (unsigned)(lane < wid ? wsum[lane] : 0)) + x - c;
   if (tid < j.nb) {
     off[tid] = run;
@@ -223,15 +225,21 @@ __global__ void __launch_bounds__(NT) k_rows_scan(Job j, const uint32_t* __restr
   for (int i = 0; i < 2; ++i)
     if (j.longest[i] && lane == 0)
       wlen[i][threadIdx.x >> 5] = row >= j.nb ? 0 : j.lrp[i] ? j.lrp[i][row + 1] - j.lrp[i][row] : c;
-  if (j.longest[0] || j.longest[1]) __syncthreads();
-  if (threadIdx.x < 2 && j.longest[threadIdx.x]) {  // one atomic for each CTA
-    int len = 0;
+  if (j.longest[0] || j.longest[1]) {
+    __syncthreads();
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) len = max(len, wlen[threadIdx.x][w]);
-    atomicMax(lmax + threadIdx.x, len);
+    for (int i = 0; i < 2; ++i)
+      if (j.longest[i] && threadIdx.x == i) {  // one atomic for each CTA
+        int len = 0;
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) len = max(len, wlen[i][w]);
+        atomicMax(lmax + i, len);
+      }
   }
-  if (scan_tail<NT>(cnt, j.rp, j.nb, ticket, j.total) && threadIdx.x < 2 && j.longest[threadIdx.x])
-    *j.longest[threadIdx.x] = atomicExch(lmax + threadIdx.x, 0);
+  const bool last = scan_tail<NT>(cnt, j.rp, j.nb, ticket, j.total);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (last && j.longest[i] && threadIdx.x == i) *j.longest[i] = atomicExch(lmax + i, 0);
 }
 
 // enumerate the set bits of each row in increasing column (warp per row)
